@@ -639,7 +639,7 @@ def run_gpu(args):
 def smoother_kernel_name(p, quad, mg_precision):
     if mg_precision == "tc" and quad == "LGL" and 2 <= p <= 4:
         return f"sem_apply_tc_kernel<P={p}> (SEM-NI, bf16 metric, mma.sync bf16 -> f32; fine-level V-cycle apply)"
-    return (f"{'sem_apply_pipe_kernel' if p <= 4 else 'sem_apply_kernel'}<P={p},{quad},f32,"
+    return (f"sem_apply_plane_kernel<P={p},{quad},f32,"
             f"{'bf16' if mg_precision in ('bf16', 'tc') else 'f32'} metric> (fine-level V-cycle apply)")
 
 

@@ -200,72 +200,11 @@ __device__ __forceinline__ bool finish_reduction(double partial, double* partial
   return threadIdx.x == 0;
 }
 
-// Shared-memory bytes of one CTA: three n^3 tiles per element, plus, when
-// StageMetric is set, the CTA's metric block staged by cp.async at kernel entry
-// (16-byte aligned thanks to the padded metric layout).  Staging is off: on
-// GB300 the extra 36 KB per CTA halves the resident CTAs of the FP32 kernel and
-// measured slower (p = 4: 63 us against 58 us per launch), because the gather
-// and scatter latencies then overlap less.
-template <typename T> struct StageMetric { static constexpr bool value = false; };
-
-template <int P, typename T, typename MT>
+// Shared-memory bytes of one CTA: three n^3 tiles per element.
+template <int P, typename T>
 __host__ __device__ constexpr size_t apply_tile_bytes() {
   return ((size_t)3 * ApplyCfg<P>::E * (P + 1) * (P + 1) * (P + 1) * sizeof(T) + 15) / 16 * 16;
 }
-template <int P, typename T>
-__host__ __device__ constexpr size_t apply_warp_tile_bytes();
-template <int P, typename T, typename MT>
-__host__ __device__ constexpr size_t apply_smem_bytes() {
-  return apply_tile_bytes<P, T, MT>() +
-         (StageMetric<T>::value ? (size_t)ApplyCfg<P>::E * MetricLayout<MT>::block(P + 1) * sizeof(MT) : 0);
-}
-
-__device__ __forceinline__ float ldsmetric(const float* p) { return *p; }
-__device__ __forceinline__ float ldsmetric(const __nv_bfloat16* p) { return __bfloat162float(*p); }
-__device__ __forceinline__ double ldsmetric(const double* p) { return *p; }
-__device__ __forceinline__ df ldsmetric(const df_pair* p) { return df(p->h, p->l); }
-
-// The 7 metric values G00 G01 G02 G11 G12 G22 W of the quadrature points of
-// one column (i, j) of an element, level by level: MetricColumn(block, c) then
-// point(k, g).  SHARED: the block is in shared memory.  The bf16 column is read
-// once, with 64-bit loads, into registers; the other layouts are read point by
-// point.
-__device__ __forceinline__ float bf16_lo(unsigned w) { return __uint_as_float(w << 16); }
-__device__ __forceinline__ float bf16_hi(unsigned w) { return __uint_as_float(w & 0xffff0000u); }
-template <int N, typename MT, bool SHARED>
-struct MetricColumn {  // component-major layouts: point by point
-  using ML = MetricLayout<MT>;
-  const MT* p;
-  __device__ __forceinline__ MetricColumn(const MT* block, int c) : p(block + ML::at(N, c, 0, 0)) {}
-  template <typename T>
-  __device__ __forceinline__ void point(int k, T (&g)[kMetricComps]) const {
-#pragma unroll
-    for (int comp = 0; comp < kMetricComps; ++comp) {
-      const MT* q = p + ML::at(N, 0, k, comp);
-      g[comp] = SHARED ? ldsmetric(q) : ldmetric(q);
-    }
-  }
-};
-template <int N, bool SHARED>
-struct MetricColumn<N, __nv_bfloat16, SHARED> {
-  using ML = MetricLayout<__nv_bfloat16>;
-  static constexpr int NW = ML::col_width(N) / 4;  // 64-bit words of a column
-  uint2 w[NW];
-  __device__ __forceinline__ MetricColumn(const __nv_bfloat16* block, int c) {
-    const uint2* q = reinterpret_cast<const uint2*>(block + ML::at(N, c, 0, 0));
-#pragma unroll
-    for (int t = 0; t < NW; ++t) w[t] = SHARED ? q[t] : __ldg(q + t);
-  }
-  // k is a compile-time constant after unrolling: the selects below resolve to registers
-  __device__ __forceinline__ void point(int k, float (&g)[kMetricComps]) const {
-#pragma unroll
-    for (int comp = 0; comp < kMetricComps; ++comp) {
-      const int v = kMetricComps * k + comp, h = v >> 1;
-      const unsigned u = (h & 1) ? w[h >> 1].y : w[h >> 1].x;
-      g[comp] = (v & 1) ? bf16_hi(u) : bf16_lo(u);
-    }
-  }
-};
 
 // Warp-per-element mode (WARP): each warp of the CTA owns one element and
 // synchronises with __syncwarp only, so the warps of an SM run their gather,
@@ -294,9 +233,7 @@ __global__ void __launch_bounds__(kApplyThreads, (std::is_same<T, df>::value && 
   static_assert(!(WARP && DOT), "the fused inner product needs the CTA-wide mode");
   constexpr int N = P + 1, N2 = N * N, N3 = N2 * N;
   using ML = MetricLayout<MT>;
-  constexpr int BLK = ML::block(N);
   constexpr int E = WARP ? WarpCfg<P>::G : ApplyCfg<P>::E;
-  constexpr bool STAGE = StageMetric<T>::value && !MASS_ONLY && !WARP;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int warp = threadIdx.x >> 5;
   const int tid = WARP ? (threadIdx.x & 31) : threadIdx.x;
@@ -304,7 +241,6 @@ __global__ void __launch_bounds__(kApplyThreads, (std::is_same<T, df>::value && 
   T* sA = reinterpret_cast<T*>(smem_raw) + (WARP ? warp * 3 * E * N3 : 0);
   T* sB = sA + E * N3;
   T* sC = sB + E * N3;
-  MT* sM = reinterpret_cast<MT*>(smem_raw + apply_tile_bytes<P, T, MT>());
   __shared__ double red[32];
   auto group_sync = [] {
     if (WARP) __syncwarp(); else __syncthreads();
@@ -317,26 +253,15 @@ __global__ void __launch_bounds__(kApplyThreads, (std::is_same<T, df>::value && 
   pdl_wait();
   if (a.done != nullptr && *a.done) return;
 
-  if (STAGE) {  // the CTA's metric block: contiguous, 16-byte aligned, a multiple of 16 bytes
-    const int ne = min(E, a.nelem - e0);
-    const size_t bytes = (size_t)ne * BLK * sizeof(MT);
-    const char* src = reinterpret_cast<const char*>(a.metric + (size_t)e0 * BLK);
-    const unsigned dst = (unsigned)__cvta_generic_to_shared(sM);
-    for (size_t off = (size_t)threadIdx.x * 16; off < bytes; off += (size_t)blockDim.x * 16)
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst + (unsigned)off),
-                   "l"(src + off)
-                   : "memory");
-    asm volatile("cp.async.commit_group;\n" ::: "memory");
-  }
-  if (std::is_same<T, df>::value && !STAGE && !MASS_ONLY) {
+  if (std::is_same<T, df>::value && !MASS_ONLY) {
     // Bulk prefetch of the group's metric block (contiguous, 16-byte aligned, a
     // multiple of 16 bytes) into L2, in 16 KB pieces: the quadrature-point stage
     // reads it after the gather and two sweeps, and then hits L2.  Measured
     // faster for the memory-latency-bound double-float kernel only (the FP64
-    // kernel is bound by the FP64 pipe, the FP32 ones stage the metric).
+    // kernel is bound by the FP64 pipe).
     const int ne = min(E, a.nelem - e0);
-    const unsigned bytes = (unsigned)((size_t)ne * BLK * sizeof(MT));
-    const char* src = reinterpret_cast<const char*>(a.metric + (size_t)e0 * BLK);
+    const unsigned bytes = (unsigned)(ML::offset(N, ne, 0, 0, 0) * sizeof(MT));
+    const char* src = reinterpret_cast<const char*>(a.metric + ML::offset(N, e0, 0, 0, 0));
     for (unsigned off = (unsigned)tid * 16384u; off < bytes; off += (unsigned)nth * 16384u)
       asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(src + off),
                    "r"(min(16384u, bytes - off))
@@ -394,7 +319,7 @@ __global__ void __launch_bounds__(kApplyThreads, (std::is_same<T, df>::value && 
     for (int idx = tid; idx < E * N3; idx += nth) {
       const int s = idx / N3, loc = idx - s * N3, e = e0 + s;
       if (e < a.nelem) {
-        const T W = ldmetric(a.metric + (size_t)e * BLK + ML::at(N, loc % N2, loc / N2, 6));
+        const T W = ldmetric(a.metric + ML::offset(N, e, loc % N2, loc / N2, 6));
         sA[idx] = (a.mass_coef * W) * sA[idx];
       }
     }
@@ -403,7 +328,6 @@ __global__ void __launch_bounds__(kApplyThreads, (std::is_same<T, df>::value && 
     // reference gradient along x and y (into sB, sC)
     sweep<N, E, 0, true, false>(tab.D, sA, sB, tid, nth);
     sweep<N, E, 1, true, false>(tab.D, sA, sC, tid, nth);
-    if (STAGE) asm volatile("cp.async.wait_all;\n" ::: "memory");
     group_sync();
     // z-gradient, quadrature-point stage and transposed z-sweep on the columns
     for (int w = tid; w < E * N2; w += nth) {
@@ -416,25 +340,13 @@ __global__ void __launch_bounds__(kApplyThreads, (std::is_same<T, df>::value && 
 #pragma unroll
       for (int k = 0; k < N; ++k) uz[k] = pa[k * N2];
       eo_line<N, true, false>(tab.D, uz, g3);
-      // bf16: the column's values into registers by 64-bit loads (MetricColumn);
-      // the component-major layouts point by point from the column's first value
-      // (measured 17 % faster for the double-float kernel than through MetricColumn)
-      const MT* mblk = STAGE ? sM + (size_t)s * BLK : a.metric + (size_t)e * BLK;
-      const MetricColumn<N, MT, STAGE> mcol(mblk, ML::kColumnMajor ? c : 0);
-      const MT* mp = mblk + c;
+      const MT* mp = a.metric + ML::offset(N, e, c, 0, 0);  // component-major, point by point
 #pragma unroll
       for (int k = 0; k < N; ++k) {
         const T g1 = pb[k * N2], g2 = pc[k * N2];
         T gm[kMetricComps];
-        if constexpr (ML::kColumnMajor) {
-          mcol.point(k, gm);
-        } else {
 #pragma unroll
-          for (int cc = 0; cc < kMetricComps; ++cc) {
-            const MT* q = mp + k * N2 + cc * padded_n3(N);
-            gm[cc] = STAGE ? ldsmetric(q) : ldmetric(q);
-          }
-        }
+        for (int cc = 0; cc < kMetricComps; ++cc) gm[cc] = ldmetric(mp + k * N2 + cc * padded_n3(N));
         const T G00 = gm[0], G01 = gm[1], G02 = gm[2], G11 = gm[3], G12 = gm[4], G22 = gm[5], W = gm[6];
         pb[k * N2] = fma(G02, g3[k], fma(G01, g2, G00 * g1));
         pc[k * N2] = fma(G12, g3[k], fma(G11, g2, G01 * g1));
@@ -515,72 +427,76 @@ __global__ void __launch_bounds__(kApplyThreads, (std::is_same<T, df>::value && 
 }
 
 // ---------------------------------------------------------------------------
-// Pipelined warp kernel of the FP32 operator (p <= 4, stiffness and mass).
+// Plane kernel of the FP32 operator (stiffness and mass, every p).
 //
-// A warp that owns one element at a time waits for the map, then for the
-// gathered values, then for the metric, and has nothing in flight while it
-// computes.  Here each warp loops over "units" of G consecutive elements
-// (unit j of the warp is unit w + j W, W warps in the grid) and keeps the
-// copies of unit j+1 in flight while it computes unit j:
-//   - the unit's metric block, contiguous in the element-blocked layout
-//     (16-byte aligned), by one bulk copy (cp.async.bulk) that lane 0 issues;
-//   - the unit's nodal values, gathered by plain loads into registers from the
-//     map entries (loaded one unit earlier still) and stored to the stage after
-//     this unit's sweeps.  Each lane gathers (and later scatters) the n nodes of
-//     its z-column: for each level the lanes read consecutive map entries.
-// Two stage buffers per warp; a stage's metric is complete when its mbarrier's
-// phase completes (every lane waits on it), its nodal values after __syncwarp.
-// The grid is persistent
-// (the CTAs that are resident at once, 3 per SM), so the pipeline runs over
-// several units.
+// Each lane owns one (i, j) plane of n^2 nodes of one element in registers, a
+// warp the n planes of each of the G = 32 / n elements of a "unit".  The x- and
+// y-sweeps, the quadrature-point stage and their transposes are register
+// arithmetic on the plane; only the two z-sweeps exchange data: every lane
+// reads the n planes of its element from a shared tile by 16-byte loads (the
+// lanes of one element read the same words) and accumulates them with its row
+// of D (or of D^T), kept in registers.  At p = 4 a unit of 6 elements takes
+// about 1,950 warp instructions, 325 an element.  The kernel with one 1-D line
+// of one element per lane that this replaced took 551 and moved every sweep
+// through shared memory (123 wavefronts an element, now 99).  Bound: the shared
+// memory pipe (two z-sweeps read n planes a lane) and latency, at 12 warps an SM.
+// Measured, apply with the clearing of y, SEM-NI, bf16 metric, 2 M nodes, before /
+// after: p = 1..6 76 / 55, 41 / 31, 27 / 23, 27 / 21, 33 / 20, 31 / 25 us; 30 M
+// nodes, p = 4: 307 / 231 us.
 //
-// Every lane owns one line of each sweep (G n^2 <= 32 for p <= 4).  Lanes
-// beyond the unit's G n^2 lines run the same instructions on the line of lane
-// (lane - (32 - G n^2)): their loads are broadcasts of that lane's, their
-// stores are predicated off, so no sweep needs a divergent branch.  The unit
-// tiles use the bank-skewed placement of pipe_word, so that no x-, y- or z-line
-// access conflicts; each lane keeps the tile words of its three lines in
-// registers (80 registers, 3 CTAs per SM: at p = 4 it cut shared-memory
-// wavefronts 14 % and the mixed time step 2.7 % against the plain [k][j][i]
-// tile with 64 registers and 4 CTAs per SM).
+// Each warp loops over units w, w + W, ... (W warps in the persistent grid)
+// with the copies of the next unit in flight:
+//   - its nodal values by 4-byte cp.async into the other of two tiles; the lanes
+//     (s, i) of a copy read one x-row (j, k) of every element s of the unit, and
+//     consecutive elements are neighbours in x, so a copy covers G n consecutive
+//     words.  The nodes of an element follow from its first map entry and the
+//     strides of the slab's lattice (the map is that lattice), so no per-node
+//     map entry is read; the SEM_DEBUG build reads and checks every entry;
+//   - its metric in chunks of rows by bulk copies (cp.async.bulk) into a ring of
+//     kStages chunks, each issued as soon as the chunk before it in its place has
+//     been read (a ring instead of the whole block, which at p = 6 and with the
+//     float metric would leave room for 4 to 8 warps an SM).
+// The result goes through the tile once more, so that the atomic adds have the
+// row pattern of the gather.
 template <int P, typename MT>
-struct PipeCfg {
+struct PlaneCfg {
   static constexpr int N = P + 1, N2 = N * N, N3 = N2 * N;
-  static constexpr int BLK = MetricLayout<MT>::block(N);  // metric values of an element
-  static constexpr int G = WarpCfg<P>::G;
-  static constexpr int NL = G * N2;                  // lines per sweep direction
-  static constexpr int UT = G * N3;                  // nodal values of a unit
-  static constexpr int TW = 32 * N;                  // words of a unit tile (pipe_word)
-  static constexpr int MV = G * BLK;                 // metric values of a unit
-  static constexpr int CH = (int)(MV * sizeof(MT) / 16);  // 16-byte chunks of a unit's metric
-  // two metric stages, two nodal stages, the two work tiles of the sweeps and the
-  // two metric stages' mbarriers
-  static constexpr size_t bar_offset = 2 * (size_t)MV * sizeof(MT) + 4 * (size_t)TW * sizeof(float);
-  static constexpr size_t warp_bytes = bar_offset + 2 * sizeof(uint64_t);
-  static constexpr size_t cta_bytes = kWarpsPerCta * warp_bytes;
-  static_assert(NL <= 32, "a unit must have at most 32 lines per direction");
-  static_assert((MV * sizeof(MT)) % 16 == 0, "stage buffers must stay 16-byte aligned");
-  static_assert(bar_offset % 16 == 0 && warp_bytes % 16 == 0, "mbarriers and warp regions stay aligned");
+  static constexpr int G = 32 / N;            // elements of a unit
+  static constexpr int NL = G * N;            // active lanes
+  static constexpr int CH = (N2 + 3) / 4;     // 16-byte chunks of a plane
+  // plane stride in words: an odd number of 16-byte chunks, so that the 16-byte
+  // accesses of 8 consecutive lanes to their own planes have no bank conflict
+  static constexpr int PS = 4 * (CH | 1);
+  static constexpr int ES = N * PS;           // element stride of a tile
+  static constexpr int TW = G * ES;           // words of a tile
+  using ML = MetricLayout<MT>;
+  static constexpr int NCH = ML::chunks(N), R = ML::rows(N);  // metric chunks of a unit, rows of a chunk
+  static constexpr int kStages = NCH == 1 ? (sizeof(MT) == 2 ? 2 : 1) : (sizeof(MT) == 2 ? 3 : 2);
+  static constexpr unsigned chunk_bytes = ML::chunk(N) * sizeof(MT);
+  static constexpr size_t tile_offset = (size_t)kStages * chunk_bytes;
+  static constexpr size_t bar_offset = tile_offset + 2 * (size_t)TW * sizeof(float);
+  static constexpr size_t warp_bytes = bar_offset + 32;
+  static constexpr int kWarps = 2;            // warps of a CTA
+  static constexpr size_t cta_bytes = kWarps * warp_bytes;
+  // warps an SM keeps resident (registers)
+  static constexpr int kResident = P == 1 ? 24 : P == 2 ? 20 : P == 3 ? 16 : P <= 5 ? 12 : 8;
+  static_assert(chunk_bytes % 16 == 0 && bar_offset % 16 == 0, "stages stay 16-byte aligned");
+  static_assert(kStages <= 4, "four mbarriers of 8 bytes");
 };
 
-// Word of node (i, j, k) of element slot s in a unit tile: row i of 32 words,
-// bank s n^2 + n ((j - i) mod n) + ((k - i) mod n).  For every sweep pattern the
-// warp's lanes run over the slots and two of (i, j, k) with the third fixed, and
-// the banks (i, j, k) -> ((j - i) mod n, (k - i) mod n) are distinct on each such
-// plane (a Latin-square placement), so no line access has a bank conflict; no
-// affine layout of the 5^3 tile does that for x-, y- and z-lines at once.
+// Matrix rows of the z-sweeps, indexed by the lane's plane: D and D^T of the
+// gradient, and for SEM the interpolation B and B^T.
 template <int N>
-__device__ __forceinline__ int pipe_word(int s, int i, int j, int k) {
-  const int jj = j - i + (j < i ? N : 0), kk = k - i + (k < i ? N : 0);
-  return 32 * i + s * N * N + N * jj + kk;
-}
+struct ZTab {
+  float D[N][N], Dt[N][N], B[N][N], Bt[N][N];
+};
 
 // The metric block of a unit reaches shared memory by one bulk copy (the TMA
 // engine, cp.async.bulk) that lane 0 issues; 16-byte cp.async copies from every
 // lane took four load instructions of the warp and about 11 more L1 tag-stage
-// wavefronts per element, in a kernel bound by the L1 pipes and by issue.  Each
-// of a warp's two stages has an mbarrier of count 1: lane 0 arrives with the
-// expected byte count and the copy's completion ends the phase.
+// wavefronts per element, in a kernel bound by the L1 pipes and by issue.  The
+// warp's stage has an mbarrier of count 1: lane 0 arrives with the expected byte
+// count and the copy's completion ends the phase.
 // Shared-memory addresses are passed as 32-bit shared-window offsets.
 __device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void mbar_init(unsigned bar) {
@@ -628,254 +544,399 @@ __device__ __forceinline__ bool mbar_wait(unsigned a, unsigned parity) {
   return mbar_try(a, parity) || mbar_wait_timed(a, parity);
 }
 
-// Map entries of the lane's z-column of unit `unit`: node zc + n^2 t of the unit
-// for t < n (zc = slot s n^3 + column (i + n j)); 0 for elements past the mesh.
+// The warp's sequence of metric chunks: chunk `c` of unit `unit` next, into stage
+// `stage`.  issue() copies it (lane 0) when it lies inside the mesh and steps on.
 template <int P, typename MT>
-__device__ __forceinline__ void pipe_load_map(const ApplyArgs<float, MT>& a, int unit, int nunits, int slot, int zc,
-                                              int (&m)[P + 1]) {
-  using C = PipeCfg<P, MT>;
-  const bool present = unit < nunits && unit * C::G + slot < a.nelem;
-  const int* src = a.map + (size_t)unit * C::UT + zc;
-#pragma unroll
-  for (int t = 0; t < C::N; ++t)
-    m[t] = present ? (int)SEM_IDX(__ldg(src + t * C::N2), a.ndofs, a.dbg, kDbgGather) : 0;
-}
-
-// Lane 0 issues the bulk copy of one unit's metric block (the elements of the unit
-// inside the mesh: a multiple of 16 bytes from a 16-byte aligned address) into a
-// stage.
-template <int P, typename MT>
-__device__ __forceinline__ void pipe_issue_metric(const ApplyArgs<float, MT>& a, int unit, int lane,
-                                                  unsigned sM, unsigned bar) {
-  using C = PipeCfg<P, MT>;
-  const int e0 = unit * C::G;
-  if (lane == 0 && !SEM_HOLD(a, unit))
-    bulk_copy(sM, a.metric + (size_t)e0 * C::BLK, (unsigned)(min(C::G, a.nelem - e0) * C::BLK * (int)sizeof(MT)),
-              bar);
-}
-
-// One 1-D line of n values at tile words off[]: dst = M src (ACC: dst += M src),
-// M in even-odd form.  src may equal dst.
-template <int N, bool ANTI, bool ACC, typename T>
-__device__ __forceinline__ void lane_line(const EoMat<N, T>& M, const T* src, T* dst, const int (&off)[N],
-                                          bool store) {
-  T in[N], out[N];
-#pragma unroll
-  for (int t = 0; t < N; ++t) in[t] = src[off[t]];
-  if (ACC) {
-#pragma unroll
-    for (int t = 0; t < N; ++t) out[t] = dst[off[t]];
+struct PlaneFeed {
+  using C = PlaneCfg<P, MT>;
+  int unit, c, stage;
+  __device__ __forceinline__ void issue(const ApplyArgs<float, MT>& a, int nunits, int tw, int lane, unsigned sM,
+                                        unsigned bar) {
+    if (unit < nunits) {
+      if (lane == 0 && !(SEM_HOLD(a, unit) && c == 0))
+        bulk_copy(sM + stage * C::chunk_bytes, a.metric + ((size_t)unit * C::NCH + c) * C::ML::chunk(C::N),
+                  C::chunk_bytes, bar + 8 * stage);
+      step(tw);
+    }
   }
-  eo_line<N, ANTI, ACC>(M, in, out);
-#pragma unroll
-  for (int t = 0; t < N; ++t)
-    if (store) dst[off[t]] = out[t];
+  __device__ __forceinline__ void step(int tw) {
+    if (++c == C::NCH) {
+      c = 0;
+      unit += tw;
+    }
+    if (++stage == C::kStages) stage = 0;
+  }
+};
+
+// First node of the lane's element of unit `unit` (0 past the mesh).
+template <int P, typename MT>
+__device__ __forceinline__ int plane_base(const ApplyArgs<float, MT>& a, int unit, int nunits, int s) {
+  using C = PlaneCfg<P, MT>;
+  const int e = unit * C::G + s;
+  return (unit < nunits && e < a.nelem) ? __ldg(a.map + (size_t)e * C::N3) : 0;
 }
 
-// 3 CTAs per SM (80 registers) at p = 3, 4; 4 at p <= 2, whose 64 registers hold
-// the shorter lines' offsets without spills (more warps for the small, latency-bound
-// coarse levels: mixed step -0.2 %).
+// Node (i, j, k) of the element e whose first node is `base`.
+template <int N, typename MT>
+__device__ __forceinline__ int plane_node(const ApplyArgs<float, MT>& a, int e, int base, int i, int j, int k,
+                                          unsigned kind) {
+#ifdef SEM_DEBUG
+  return e < a.nelem ? (int)SEM_IDX(__ldg(a.map + (size_t)e * N * N * N + i + N * (j + N * k)), a.ndofs, a.dbg, kind)
+                     : 0;
+#else
+  (void)e;
+  (void)kind;
+  return base + i + j * a.row + k * a.plane;
+#endif
+}
+
+// Copies the unit's nodal values into a tile: lane (s, i) the nodes (i, j, k) of
+// element slot s for every (j, k), one 4-byte cp.async each.
+template <int P, typename MT>
+__device__ __forceinline__ void plane_gather(const ApplyArgs<float, MT>& a, int unit, int base, int s, int r, bool act,
+                                             unsigned tile) {
+  using C = PlaneCfg<P, MT>;
+  constexpr int N = C::N;
+  if (act) {
+    const unsigned dst = tile + 4u * (unsigned)(s * C::ES + r);
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+#pragma unroll
+      for (int j = 0; j < N; ++j) {
+        const float* src = a.u + plane_node<N>(a, unit * C::G + s, base, r, j, k, kDbgGather);
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dst + 4u * (k * C::PS + j * N)), "l"(src)
+                     : "memory");
+      }
+  }
+  asm volatile("cp.async.commit_group;\n" ::: "memory");
+}
+
+// out[m] (+)= sum_l z[l] x_l[m] over the n planes x_l of an element in a tile.
+template <int N, int PS, bool ACC>
+__device__ __forceinline__ void plane_zsweep(const float (&z)[N], const float* elem, float (&out)[N * N]) {
+  constexpr int CH = (N * N + 3) / 4;
+#pragma unroll
+  for (int c = 0; c < CH; ++c) {
+    float4 v[N];
+#pragma unroll
+    for (int l = 0; l < N; ++l) v[l] = *reinterpret_cast<const float4*>(elem + l * PS + 4 * c);
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const int m = 4 * c + t;
+      if (m < N * N) {
+        auto at = [&](int l) { return t == 0 ? v[l].x : t == 1 ? v[l].y : t == 2 ? v[l].z : v[l].w; };
+        float acc = ACC ? fmaf(z[0], at(0), out[m]) : z[0] * at(0);
+#pragma unroll
+        for (int l = 1; l < N; ++l) acc = fmaf(z[l], at(l), acc);
+        out[m] = acc;
+      }
+    }
+  }
+}
+
+// The lane's plane between registers and its place in a tile, by 16-byte accesses.
+template <int N>
+__device__ __forceinline__ void plane_load(const float* p, float (&v)[N * N]) {
+#pragma unroll
+  for (int c = 0; c < (N * N + 3) / 4; ++c) {
+    const float4 q = reinterpret_cast<const float4*>(p)[c];
+    v[4 * c] = q.x;
+    if (4 * c + 1 < N * N) v[4 * c + 1] = q.y;
+    if (4 * c + 2 < N * N) v[4 * c + 2] = q.z;
+    if (4 * c + 3 < N * N) v[4 * c + 3] = q.w;
+  }
+}
+template <int N>
+__device__ __forceinline__ void plane_store(float* p, const float (&v)[N * N]) {
+#pragma unroll
+  for (int c = 0; c < (N * N + 3) / 4; ++c) {
+    auto at = [&](int m) { return m < N * N ? v[m < N * N ? m : 0] : 0.f; };
+    reinterpret_cast<float4*>(p)[c] = make_float4(at(4 * c), at(4 * c + 1), at(4 * c + 2), at(4 * c + 3));
+  }
+}
+
+// v = M along x (DIR 0) or y (DIR 1) of the plane v, in place.
+template <int N, int DIR, bool ANTI>
+__device__ __forceinline__ void plane_sweep(const EoMat<N, float>& M, float (&v)[N * N]) {
+#pragma unroll
+  for (int t = 0; t < N; ++t) {
+    float in[N], out[N];
+#pragma unroll
+    for (int l = 0; l < N; ++l) in[l] = DIR == 0 ? v[t * N + l] : v[l * N + t];
+    eo_line<N, ANTI, false>(M, in, out);
+#pragma unroll
+    for (int l = 0; l < N; ++l) (DIR == 0 ? v[t * N + l] : v[l * N + t]) = out[l];
+  }
+}
+
+// Metric values of row J of the rows at p: point i at g[7 i .. 7 i + 6], read by
+// 8-byte (bf16) or 16-byte (float) loads of four values.
+__device__ __forceinline__ void metric_quad(const __nv_bfloat16* p, float (&g)[4]) {
+  const uint2 w = *reinterpret_cast<const uint2*>(p);
+  g[0] = __uint_as_float(w.x << 16);
+  g[1] = __uint_as_float(w.x & 0xffff0000u);
+  g[2] = __uint_as_float(w.y << 16);
+  g[3] = __uint_as_float(w.y & 0xffff0000u);
+}
+__device__ __forceinline__ void metric_quad(const float* p, float (&g)[4]) {
+  const float4 w = *reinterpret_cast<const float4*>(p);
+  g[0] = w.x;
+  g[1] = w.y;
+  g[2] = w.z;
+  g[3] = w.w;
+}
+template <int N, int J, typename MT>
+__device__ __forceinline__ void metric_row(const MT* p, float (&g)[kMetricComps * N]) {
+  constexpr int v0 = kMetricComps * N * J, v1 = v0 + kMetricComps * N;
+#pragma unroll
+  for (int c = v0 / 4; c < (v1 + 3) / 4; ++c) {
+    float q[4];
+    metric_quad(p + 4 * c, q);
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const int v = 4 * c + t - v0;
+      if (v >= 0 && v < kMetricComps * N) g[v] = q[t];
+    }
+  }
+}
+
+// Quadrature-point stage and x-sweeps of row J (row JC of the chunk whose values of
+// this lane are at `metric`): on entry u the values, gy and gz the y- and
+// z-derivatives of the plane; on exit row J of u holds m + D^T q1 along x, gy and gz
+// hold q2 and q3.
+template <int N, int JC, typename MT>
+__device__ __forceinline__ void plane_row(const EoMat<N, float>& D, const EoMat<N, float>& Dt, const MT* metric,
+                                          float mass, float* u, float* gy, float* gz) {
+  float in[N], g1[N], q1[N], m[N], g[kMetricComps * N];
+  metric_row<N, JC>(metric, g);
+#pragma unroll
+  for (int i = 0; i < N; ++i) in[i] = u[i];
+  eo_line<N, true, false>(D, in, g1);
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const float* G = g + kMetricComps * i;  // G00 G01 G02 G11 G12 G22 W
+    const float x = g1[i], y = gy[i], z = gz[i];
+    q1[i] = fmaf(G[2], z, fmaf(G[1], y, G[0] * x));
+    gy[i] = fmaf(G[4], z, fmaf(G[3], y, G[1] * x));
+    gz[i] = fmaf(G[5], z, fmaf(G[4], y, G[2] * x));
+    m[i] = (mass * G[6]) * in[i];
+  }
+  eo_line<N, true, true>(Dt, q1, m);
+#pragma unroll
+  for (int i = 0; i < N; ++i) u[i] = m[i];
+}
+template <int N, int J, int JC, int R, typename MT>
+__device__ __forceinline__ void plane_chunk(const EoMat<N, float>& D, const EoMat<N, float>& Dt, const MT* metric,
+                                            float mass, float (&u)[N * N], float (&gy)[N * N], float (&gz)[N * N]) {
+  if constexpr (JC < R) {
+    plane_row<N, JC>(D, Dt, metric, mass, u + (J + JC) * N, gy + (J + JC) * N, gz + (J + JC) * N);
+    plane_chunk<N, J, JC + 1, R>(D, Dt, metric, mass, u, gy, gz);
+  }
+}
+
+// The lane's wait for the chunk in stage `use`; when it runs out: report it, let the
+// warp's other copies land, false.
+template <int P, typename MT>
+__device__ __forceinline__ bool plane_wait(const ApplyArgs<float, MT>& a, unsigned bar, int use, unsigned phase,
+                                           int behind, int lane) {
+  using C = PlaneCfg<P, MT>;
+  if (mbar_wait(bar + 8 * use, (phase >> use) & 1u)) return true;
+  if (lane == 0 && a.fault != nullptr) atomicOr(a.fault, 1u);
+  for (int t = 1; t < behind; ++t) {  // `behind` copies issued from this one on
+    const int st = (use + t) % C::kStages;
+    mbar_wait(bar + 8 * st, (phase >> st) & 1u);
+  }
+  asm volatile("cp.async.wait_all;\n" ::: "memory");
+  return false;
+}
+
+// All chunks of a unit, from J = 0: wait, rows, release the stage to the next copy.
+template <int P, int J, typename MT>
+__device__ __forceinline__ bool plane_points(const ApplyArgs<float, MT>& a, const KTab<P + 1, float>& tab,
+                                             PlaneFeed<P, MT>& feed, int& use, unsigned& phase, int& behind, int nunits,
+                                             int tw, int lane, int lidx, unsigned char* wb, unsigned sM, unsigned bar,
+                                             float (&u)[(P + 1) * (P + 1)], float (&gy)[(P + 1) * (P + 1)],
+                                             float (&gz)[(P + 1) * (P + 1)]) {
+  using C = PlaneCfg<P, MT>;
+  if constexpr (J < C::N) {
+    if (!plane_wait<P>(a, bar, use, phase, behind, lane)) return false;
+    phase ^= 1u << use;
+    const MT* m = reinterpret_cast<const MT*>(wb + use * C::chunk_bytes) + lidx * C::ML::stride(C::N);
+    plane_chunk<C::N, J, 0, C::R>(tab.D, tab.Dt, m, a.mass_coef, u, gy, gz);
+    __syncwarp();  // the chunk is read: its stage takes the next copy
+    --behind;
+    if (feed.unit < nunits) ++behind;
+    feed.issue(a, nunits, tw, lane, sM, bar);
+    if (++use == C::kStages) use = 0;
+    return plane_points<P, J + C::R>(a, tab, feed, use, phase, behind, nunits, tw, lane, lidx, wb, sM, bar, u, gy, gz);
+  }
+  return true;
+}
+
 template <int P, int QUAD, typename MT>
-__global__ void __launch_bounds__(kApplyThreads, P <= 2 ? 4 : 3)
-    sem_apply_pipe_kernel(const ApplyArgs<float, MT> a, const __grid_constant__ KTab<P + 1, float> tab,
-                          int nunits) {
+__global__ void __launch_bounds__(32 * PlaneCfg<P, MT>::kWarps, PlaneCfg<P, MT>::kResident / PlaneCfg<P, MT>::kWarps)
+    sem_apply_plane_kernel(const ApplyArgs<float, MT> a, const __grid_constant__ KTab<P + 1, float> tab,
+                           const __grid_constant__ ZTab<P + 1> zt, int nunits) {
   pdl_trigger();
-  using C = PipeCfg<P, MT>;
-  using T = float;
-  constexpr int N = C::N, N2 = C::N2, N3 = C::N3, G = C::G, NL = C::NL;
+  using C = PlaneCfg<P, MT>;
+  constexpr int N = C::N, N2 = C::N2, G = C::G;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int unit = blockIdx.x * kWarpsPerCta + warp;
+  int unit = blockIdx.x * C::kWarps + warp;
   if (unit >= nunits) return;  // no CTA-wide barrier in this kernel
-  {  // while the previous kernel drains: the first unit's map entries and metric into L2
-    const int ne = min(G, a.nelem - unit * G);
-    prefetch_l2_lines(a.map + (size_t)unit * C::UT, (size_t)ne * N3 * sizeof(int), lane, 32);
-    prefetch_l2_lines(a.metric + (size_t)unit * G * C::BLK, (size_t)ne * C::BLK * sizeof(MT), lane, 32);
-  }
-  pdl_wait();
-  if (a.done != nullptr && *a.done) return;
-  const int tw = gridDim.x * kWarpsPerCta;
+  const int tw = gridDim.x * C::kWarps;
   unsigned char* wb = smem_raw + (size_t)warp * C::warp_bytes;
-  MT* sM0 = reinterpret_cast<MT*>(wb);
-  T* sU0 = reinterpret_cast<T*>(wb + 2 * (size_t)C::MV * sizeof(MT));
-  T* sB = sU0 + 2 * C::TW;
-  T* sC = sB + C::TW;
-  // the two metric stages and their mbarriers, as shared-window offsets
-  const unsigned sm_s = smem_u32(sM0), bar_s = smem_u32(wb + C::bar_offset);
-  constexpr unsigned kStageBytes = (unsigned)(C::MV * sizeof(MT));
+  float* tiles = reinterpret_cast<float*>(wb + C::tile_offset);
+  const unsigned sm_s = smem_u32(wb), tile_s = smem_u32(tiles), bar_s = smem_u32(wb + C::bar_offset);
+  // While the previous kernel drains, before pdl_wait: the first metric copies and
+  // the map entries (written by the set-up only).
   if (lane == 0) {
-    mbar_init(bar_s);
-    mbar_init(bar_s + 8);
+    for (int t = 0; t < C::kStages; ++t) mbar_init(bar_s + 8 * t);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
   __syncwarp();
-  unsigned phase = 0;  // bit s: parity of stage s's next completion
-
-  // The lane's lines (those of lane - (32 - NL) for the lanes >= NL, a lane of the
-  // same half-warp, so that the 64-bit metric loads of the idle lanes are
-  // broadcasts within their phase): element slot ls, line ll = r + n q, which is
-  // the x-line (j, k) = (r, q), the y-line (i, k) = (r, q) and the z-line
-  // (i, j) = (r, q); their tile words for t = 0..n-1.
-  static_assert(NL >= 24, "idle lanes must replay a lane of their half-warp");
-  const bool act = lane < NL;
-  const int lw = act ? lane : lane - (32 - NL);
-  const int ls = lw / N2, ll = lw - ls * N2, r = ll % N, q = ll / N;
-  int ox[N], oy[N], oz[N];
+  PlaneFeed<P, MT> feed{unit, 0, 0};
+  int behind = 0;  // copies issued and not yet waited for
 #pragma unroll
-  for (int t = 0; t < N; ++t) {
-    ox[t] = pipe_word<N>(ls, t, r, q);
-    oy[t] = pipe_word<N>(ls, r, t, q);
-    oz[t] = pipe_word<N>(ls, r, q, t);
+  for (int t = 0; t < C::kStages; ++t) {
+    if (feed.unit < nunits) ++behind;
+    feed.issue(a, nunits, tw, lane, sm_s, bar_s);
   }
-  const int zc = ls * N3 + ll;  // first node of the lane's z-column in the unit
-
-  int mc[N], mn[N], mnn[N];  // map entries of the lane's z-column in units j, j+1, j+2
-  pipe_load_map<P>(a, unit, nunits, ls, zc, mc);
-  float gv[N];  // the next unit's gathered values, in flight during this unit's sweeps
-  pipe_issue_metric<P>(a, unit, lane, sm_s, bar_s);
-  {
-    const bool present = unit * G + ls < a.nelem;
+  // lane = slot s of the unit and r: plane k = r of the sweeps, node i = r of the
+  // gather and scatter rows.  Idle lanes (32 - G n) run on the last slot's data
+  // and neither copy nor store.
+  const bool act = lane < C::NL;
+  const int s = act ? lane / N : G - 1, r = act ? lane - s * N : 0;
+  float dz[N], dtz[N];
 #pragma unroll
-    for (int t = 0; t < N; ++t) gv[t] = present ? __ldg(a.u + mc[t]) : 0.f;
-#pragma unroll
-    for (int t = 0; t < N; ++t)
-      if (act) sU0[oz[t]] = gv[t];
+  for (int l = 0; l < N; ++l) {
+    dz[l] = zt.D[r][l];
+    dtz[l] = zt.Dt[r][l];
   }
-  pipe_load_map<P>(a, unit + tw, nunits, ls, zc, mn);
+  int base = plane_base<P>(a, unit, nunits, s);
+  int base_n = plane_base<P>(a, unit + tw, nunits, s);
+  pdl_wait();
+  if (a.done != nullptr && *a.done) {
+    for (int t = 0; t < behind; ++t) mbar_wait(bar_s + 8 * t, 0);  // the CTA must not end under its own copies
+    return;
+  }
+  plane_gather<P>(a, unit, base, s, r, act, tile_s);
+  unsigned phase = 0;  // bit t: parity of stage t's next completion
+  int use = 0;         // stage of the next chunk
   int b = 0;
+  const int lidx = s * N + r;
   for (; unit < nunits; unit += tw) {
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+    __syncwarp();  // every lane's copies of this unit landed
     const int nxt = unit + tw;
-    if (nxt < nunits) {
-      pipe_issue_metric<P>(a, nxt, lane, sm_s + (b ^ 1) * kStageBytes, bar_s + 8 * (b ^ 1));
-      const bool present = nxt * G + ls < a.nelem;
+    if (nxt < nunits) plane_gather<P>(a, nxt, base_n, s, r, act, tile_s + 4u * (unsigned)((b ^ 1) * C::TW));
+    const int base_nn = plane_base<P>(a, nxt + tw, nunits, s);
+    float* elem = tiles + b * C::TW + s * C::ES;
+    float* own = elem + r * C::PS;
+    float u[N2], gy[N2], gz[N2];
+    plane_load<N>(own, u);
+    if (QUAD == SEM_QUAD_LG) {  // values at the Gauss points: x and y in the plane, then z
+      plane_sweep<N, 0, false>(tab.Bi, u);
+      plane_sweep<N, 1, false>(tab.Bi, u);
+      if (act) plane_store<N>(own, u);
+      __syncwarp();
+      float bz[N];
 #pragma unroll
-      for (int t = 0; t < N; ++t) gv[t] = present ? __ldg(a.u + mn[t]) : 0.f;
-    }
-    pipe_load_map<P>(a, nxt + tw, nunits, ls, zc, mnn);
-    if (!mbar_wait(bar_s + 8 * b, (phase >> b) & 1u)) {
-      // the copy did not complete: report it, let the other stage's copy land, stop
-      if (lane == 0 && a.fault != nullptr) atomicOr(a.fault, 1u);
-      if (nxt < nunits) mbar_wait(bar_s + 8 * (b ^ 1), (phase >> (b ^ 1)) & 1u);
-      return;
-    }
-    phase ^= 1u << b;
-    __syncwarp();
-
-    T* sA = sU0 + b * C::TW;
-    const MT* sM = sM0 + b * C::MV;
-    const int e = unit * G + ls;  // the lane's element
-    if (QUAD == SEM_QUAD_LG) {  // values at the Gauss points
-      lane_line<N, false, false>(tab.Bi, sA, sB, ox, act);
+      for (int l = 0; l < N; ++l) bz[l] = zt.B[r][l];
+      plane_zsweep<N, C::PS, false>(bz, elem, u);
       __syncwarp();
-      lane_line<N, false, false>(tab.Bi, sB, sC, oy, act);
-      __syncwarp();
-      lane_line<N, false, false>(tab.Bi, sC, sA, oz, act);
+      if (act) plane_store<N>(own, u);
       __syncwarp();
     }
-    // reference gradient along x and y (into sB, sC)
-    lane_line<N, true, false>(tab.D, sA, sB, ox, act);
-    lane_line<N, true, false>(tab.D, sA, sC, oy, act);
-    __syncwarp();
-    // z-gradient, quadrature-point stage and transposed z-sweep on the lane's column
-    {
-      T uz[N], g3[N], q3[N], m[N];
+    plane_zsweep<N, C::PS, false>(dz, elem, gz);
 #pragma unroll
-      for (int k = 0; k < N; ++k) uz[k] = sA[oz[k]];
-      eo_line<N, true, false>(tab.D, uz, g3);
-      const MetricColumn<N, MT, true> mcol(sM + ls * C::BLK, ll);
+    for (int v = 0; v < N2; ++v) gy[v] = u[v];
+    plane_sweep<N, 1, true>(tab.D, gy);
+    if (!plane_points<P, 0>(a, tab, feed, use, phase, behind, nunits, tw, lane, lidx, wb, sm_s, bar_s, u, gy, gz)) return;
+    __syncwarp();  // the planes of u are read
+    if (act) plane_store<N>(own, gz);
+    plane_sweep<N, 1, true>(tab.Dt, gy);
 #pragma unroll
-      for (int k = 0; k < N; ++k) {
-        const T g1 = sB[oz[k]], g2 = sC[oz[k]];
-        T gm[kMetricComps];
-        mcol.point(k, gm);
-        const T G00 = gm[0], G01 = gm[1], G02 = gm[2], G11 = gm[3], G12 = gm[4], G22 = gm[5], W = gm[6];
-        const T q1 = fma(G02, g3[k], fma(G01, g2, G00 * g1));
-        const T q2 = fma(G12, g3[k], fma(G11, g2, G01 * g1));
-        if (act) {
-          sB[oz[k]] = q1;
-          sC[oz[k]] = q2;
-        }
-        q3[k] = fma(G22, g3[k], fma(G12, g2, G02 * g1));
-        m[k] = (a.mass_coef * W) * uz[k];
-      }
-      eo_line<N, true, true>(tab.Dt, q3, m);
+    for (int v = 0; v < N2; ++v) u[v] += gy[v];
+    __syncwarp();
+    plane_zsweep<N, C::PS, true>(dtz, elem, u);
+    if (QUAD == SEM_QUAD_LG) {  // back from the Gauss points: z, then x and y in the plane
+      __syncwarp();
+      if (act) plane_store<N>(own, u);
+      __syncwarp();
+      float bz[N];
 #pragma unroll
-      for (int k = 0; k < N; ++k)
-        if (act) sA[oz[k]] = m[k];
+      for (int l = 0; l < N; ++l) bz[l] = zt.Bt[r][l];
+      plane_zsweep<N, C::PS, false>(bz, elem, u);
+      plane_sweep<N, 1, false>(tab.Bit, u);
+      plane_sweep<N, 0, false>(tab.Bit, u);
     }
     __syncwarp();
-    lane_line<N, true, true>(tab.Dt, sC, sA, oy, act);
+    if (act) plane_store<N>(own, u);
     __syncwarp();
-    lane_line<N, true, true>(tab.Dt, sB, sA, ox, act);
-    __syncwarp();
-    if (QUAD == SEM_QUAD_LG) {  // back from the Gauss points to the nodes
-      lane_line<N, false, false>(tab.Bit, sA, sB, ox, act);
-      __syncwarp();
-      lane_line<N, false, false>(tab.Bit, sB, sC, oy, act);
-      __syncwarp();
-      lane_line<N, false, false>(tab.Bit, sC, sA, oz, act);
-      __syncwarp();
-    }
-    // scatter-add y += P_e^T y_e along the lane's z-column
-    const T sc = a.scale_out ? a.out_scale : T(1);
+    // scatter-add y += P_e^T y_e, lane (s, i) along the rows of its element
+    const int e = unit * G + s;
     if (act && e < a.nelem) {
+      const float sc = a.scale_out ? a.out_scale : 1.f;
+      const float* row = elem + r;
       if (a.yloc != nullptr) {  // deterministic mode: element-local results
 #pragma unroll
-        for (int t = 0; t < N; ++t) a.yloc[(size_t)unit * C::UT + zc + t * N2] = sA[oz[t]] * sc;
+        for (int v = 0; v < N2; ++v)
+          a.yloc[(size_t)e * C::N3 + r + N * v] = row[(v / N) * C::PS + (v % N) * N] * sc;
       } else {
 #pragma unroll
-        for (int t = 0; t < N; ++t) atomicAdd(a.y + mc[t], sA[oz[t]] * sc);
+        for (int v = 0; v < N2; ++v)
+          atomicAdd(a.y + plane_node<N>(a, e, base, r, v % N, v / N, kDbgScatter),
+                    row[(v / N) * C::PS + (v % N) * N] * sc);
       }
     }
-    if (nxt < nunits) {
-#pragma unroll
-      for (int t = 0; t < N; ++t)
-        if (act) sU0[(b ^ 1) * C::TW + oz[t]] = gv[t];
-    }
-    __syncwarp();  // stage b is refilled by the next iteration's issue
-#pragma unroll
-    for (int t = 0; t < N; ++t) {
-      mc[t] = mn[t];
-      mn[t] = mnn[t];
-    }
+    __syncwarp();  // the next iteration's gather refills this tile
+    base = base_n;
+    base_n = base_nn;
     b ^= 1;
   }
 }
 
-// Persistent grid of the pipelined kernel: the CTAs resident on the device at
-// once (set by prime_t, before any stream capture), at most one warp per unit.
+// Persistent grid of the plane kernel: the CTAs resident on the device at once
+// (set by prime_t, before any stream capture), at most one warp per unit.
 template <int P, int QUAD, typename MT>
-struct PipeGrid {
+struct PlaneGrid {
   static inline int resident = 0;
 };
 
 template <int P, int QUAD, typename MT>
-cudaError_t pipe_prime() {
-  using C = PipeCfg<P, MT>;
-  cudaError_t e = cudaFuncSetAttribute(sem_apply_pipe_kernel<P, QUAD, MT>,
+cudaError_t plane_prime() {
+  using C = PlaneCfg<P, MT>;
+  cudaError_t e = cudaFuncSetAttribute(sem_apply_plane_kernel<P, QUAD, MT>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::cta_bytes);
   int dev = 0, sms = 0, per_sm = 0;
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sem_apply_pipe_kernel<P, QUAD, MT>,
-                                                      kApplyThreads, C::cta_bytes);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sem_apply_plane_kernel<P, QUAD, MT>, 32 * C::kWarps,
+                                                      C::cta_bytes);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  PipeGrid<P, QUAD, MT>::resident = sms * per_sm;
+  PlaneGrid<P, QUAD, MT>::resident = sms * per_sm;
   return cudaSuccess;
 }
 
 template <int P, int QUAD, typename MT>
-cudaError_t launch_apply_pipe(const Level& L, const ApplyArgs<float, MT>& a, const KTab<P + 1, float>& tab,
-                              cudaStream_t s) {
-  using C = PipeCfg<P, MT>;
-  const int resident = PipeGrid<P, QUAD, MT>::resident;
-  if (resident < 1) return cudaErrorInitializationError;  // prime_apply_kernels was not called
+cudaError_t launch_apply_plane(const Level& L, const ApplyArgs<float, MT>& a, const KTab<P + 1, float>& tab,
+                               cudaStream_t s) {
+  using C = PlaneCfg<P, MT>;
+  constexpr int N = P + 1;
+  if (PlaneGrid<P, QUAD, MT>::resident < 1) return cudaErrorInitializationError;  // prime_apply_kernels was not called
   const int nunits = (L.nelem + C::G - 1) / C::G;
-  const int grid = std::min(resident, (nunits + kWarpsPerCta - 1) / kWarpsPerCta);
-  if (grid == 0) return cudaSuccess;
-  launch_k(sem_apply_pipe_kernel<P, QUAD, MT>, grid, kApplyThreads, C::cta_bytes, s, a, tab, nunits);
+  if (nunits == 0) return cudaSuccess;
+  const int grid = std::min(PlaneGrid<P, QUAD, MT>::resident, (nunits + C::kWarps - 1) / C::kWarps);
+  ZTab<N> zt;
+  for (int q = 0; q < N; ++q)
+    for (int l = 0; l < N; ++l) {
+      zt.D[q][l] = zt.Dt[l][q] = (float)(QUAD == SEM_QUAD_LG ? L.tab.Dg : L.tab.D)[q][l];
+      zt.B[q][l] = zt.Bt[l][q] = (float)L.tab.Bi[q][l];
+    }
+  launch_k(sem_apply_plane_kernel<P, QUAD, MT>, grid, 32 * C::kWarps, C::cta_bytes, s, a, tab, zt, nunits);
   return cudaGetLastError();
 }
 
@@ -906,35 +967,33 @@ cudaError_t launch_apply_kernels(const Level& L, const ApplyArgs<T, MT>& a, cons
   constexpr int E = ApplyCfg<P>::E;
   const int grid = (L.nelem + E - 1) / E;
   if (grid == 0) return cudaSuccess;
-  constexpr size_t tiles = apply_tile_bytes<P, T, MT>();
-  constexpr size_t full = apply_smem_bytes<P, T, MT>();
-  // FP32 kernels at p <= 4: elements owned by warps (measured faster; at p = 5, 6
-  // the n^2 = 36, 49 lines fill warps poorly and the CTA-wide mode is faster)
-  constexpr bool warp_mode = sizeof(T) == 4 && P <= 4;
-  if constexpr (std::is_same<T, float>::value && P <= 4) {
-    if (!mass_only && !dot) return launch_apply_pipe<P, QUAD, MT>(L, a, tab, s);
-  }
-  if (warp_mode && !dot) {
-    constexpr int per_cta = kWarpsPerCta * WarpCfg<P>::G;
-    const int wgrid = (L.nelem + per_cta - 1) / per_cta;
-    constexpr size_t wbytes = apply_warp_tile_bytes<P, T>();
-    if (mass_only)
-      launch_k(sem_apply_kernel<P, QUAD, T, MT, false, true, true>, wgrid, kApplyThreads, wbytes, s, a, tab);
-    else
-      launch_k(sem_apply_kernel<P, QUAD, T, MT, false, false, true>, wgrid, kApplyThreads, wbytes, s, a, tab);
+  constexpr size_t tiles = apply_tile_bytes<P, T>();
+  if constexpr (std::is_same<T, float>::value) {
+    if (dot) return cudaErrorInvalidValue;
+    if (!mass_only) return launch_apply_plane<P, QUAD, MT>(L, a, tab, s);
+    // mass only, p <= 4: elements owned by warps (measured faster; at p = 5, 6 the
+    // n^2 = 36, 49 lines fill warps poorly and the CTA-wide mode is faster)
+    if constexpr (P <= 4) {
+      constexpr int per_cta = kWarpsPerCta * WarpCfg<P>::G;
+      launch_k(sem_apply_kernel<P, QUAD, T, MT, false, true, true>, (L.nelem + per_cta - 1) / per_cta, kApplyThreads,
+               apply_warp_tile_bytes<P, T>(), s, a, tab);
+    } else {
+      launch_k(sem_apply_kernel<P, QUAD, T, MT, false, true>, grid, kApplyThreads, tiles, s, a, tab);
+    }
     return cudaGetLastError();
-  }
+  } else {
   if (mass_only) {
     launch_k(sem_apply_kernel<P, QUAD, T, MT, false, true>, grid, kApplyThreads, tiles, s, a, tab);
   } else if (dot) {
-    launch_k(sem_apply_kernel<P, QUAD, T, MT, true, false>, grid, kApplyThreads, full, s, a, tab);
+    launch_k(sem_apply_kernel<P, QUAD, T, MT, true, false>, grid, kApplyThreads, tiles, s, a, tab);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return launch_apply_dot_finish(a.dot_partials, grid, a.cg, a.dot_out, a.done, s);
   } else {
-    launch_k(sem_apply_kernel<P, QUAD, T, MT, false, false>, grid, kApplyThreads, full, s, a, tab);
+    launch_k(sem_apply_kernel<P, QUAD, T, MT, false, false>, grid, kApplyThreads, tiles, s, a, tab);
   }
   return cudaGetLastError();
+  }
 }
 
 // Launch helper shared by the precision-specific translation units.  With
@@ -951,6 +1010,8 @@ cudaError_t launch_apply_t(const Level& L, const ApplyArgs<T, MT>& a, bool mass_
   make_eo(tab.Bit, L.tab.Bi, true);
   ApplyArgs<T, MT> b = a;
   b.ndofs = L.ndofs;
+  b.row = P * L.nx + 1;
+  b.plane = b.row * (P * L.ny + 1);
   b.dbg = L.dbg;
   b.fault = L.fault;
   b.hold = L.hold;
@@ -959,21 +1020,21 @@ cudaError_t launch_apply_t(const Level& L, const ApplyArgs<T, MT>& a, bool mass_
   return launch_assemble(L, a.yloc, a.y, a.done, s);
 }
 
-// Dynamic shared-memory limits of the three variants of one instantiation.
+// Dynamic shared-memory limits of the variants of one instantiation.
 template <int P, int QUAD, typename T, typename MT>
 cudaError_t prime_t() {
-  constexpr int full = (int)apply_smem_bytes<P, T, MT>();
-  cudaError_t e;
-  if constexpr (std::is_same<T, float>::value && P <= 4) {
-    if ((e = pipe_prime<P, QUAD, MT>()) != cudaSuccess) return e;
+  constexpr int tiles = (int)apply_tile_bytes<P, T>();
+  cudaError_t e = cudaFuncSetAttribute(sem_apply_kernel<P, QUAD, T, MT, false, true>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, tiles);
+  if (e != cudaSuccess) return e;
+  if constexpr (std::is_same<T, float>::value) {
+    return plane_prime<P, QUAD, MT>();
+  } else {
+    if ((e = cudaFuncSetAttribute(sem_apply_kernel<P, QUAD, T, MT, false, false>,
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize, tiles)) != cudaSuccess) return e;
+    return cudaFuncSetAttribute(sem_apply_kernel<P, QUAD, T, MT, true, false>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, tiles);
   }
-  if ((e = cudaFuncSetAttribute(sem_apply_kernel<P, QUAD, T, MT, false, false>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, full)) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(sem_apply_kernel<P, QUAD, T, MT, true, false>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, full)) != cudaSuccess) return e;
-  return cudaFuncSetAttribute(sem_apply_kernel<P, QUAD, T, MT, false, true>,
-                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)apply_tile_bytes<P, T, MT>());
 }
 
 template <typename T, typename MT>

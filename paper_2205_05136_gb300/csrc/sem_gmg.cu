@@ -1280,13 +1280,13 @@ int build(sem_ctx* ctx, cudaStream_t s) {
     Level& L = *V.L;
     nmax = std::max(nmax, L.ndofs);
     if (g->precision == SEM_PREC_FP32 && !L.metric32_valid) {
-      if (!L.metric32) GMG_CK(cudaMalloc(&L.metric32, sizeof(float) * metric_count(L)));
+      if (!L.metric32) GMG_CK(cudaMalloc(&L.metric32, sizeof(float) * metric_lowp_count(L)));
       GMG_CK(setup_metric_lowp(L, false, s));
     }
     const bool tc = g->precision == SEM_PREC_BF16_TC && tc_supported(L) && !ctx->deterministic;
     if ((g->precision == SEM_PREC_FP32_BF16 || (g->precision == SEM_PREC_BF16_TC && !tc)) &&
         !L.metric16_valid) {
-      if (!L.metric16) GMG_CK(cudaMalloc(&L.metric16, sizeof(__nv_bfloat16) * metric16_count(L)));
+      if (!L.metric16) GMG_CK(cudaMalloc(&L.metric16, sizeof(__nv_bfloat16) * metric_lowp_count(L)));
       GMG_CK(setup_metric_lowp(L, true, s));
     }
     if (tc && !L.metric_tc_valid) GMG_CK(setup_metric_tc(L, s));

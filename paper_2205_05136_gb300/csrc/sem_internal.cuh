@@ -5,10 +5,8 @@
 //   metric   double [nelem][7][n3p] per quadrature point: G00 G01 G02 G11 G12 G22 W,
 //            n3p = n^3 rounded up to a multiple of 8 (16-byte aligned blocks),
 //            G = w |det J| J^{-1} D J^{-T}, W = w |det J|  (element-blocked SoA)
-//   metric32 float [nelem][7][n3p] copy of the same array (mixed-precision applies)
-//   metric16 bf16  [nelem][n^2][CW] column-major copy: the 7 n values of the
-//            quadrature points of column (i, j) in CW = 7 n rounded up to 4
-//            (p = 4: 36 values, 72 bytes), read by 64-bit loads
+//   metric32 float, metric16 bf16  copies in the order the plane kernel consumes:
+//            [unit][chunk of rows][element of the unit][plane k][RS] (MetricLayout)
 //   mdiag    double [ndofs]  diagonal of the assembled mass matrix
 //   kdiag    double [ndofs]  diagonal of the assembled stiffness matrix
 //   xyz      double [3][ndofs] node coordinates
@@ -203,33 +201,47 @@ inline size_t metric_count(const Level& L) {
 }
 
 // Offset of component `comp` of the quadrature point on column c = i + n j at
-// level k inside one element's metric block.
-//   double, float, float pairs: component-major [7][padded n^3], point c + n^2 k;
-//   bf16: column-major, the 7 values of level k at 7 k .. 7 k + 6 of the
-//   column's CW = 7 n (rounded up to a multiple of 4) values, so that a lane
-//   reads its whole column with CW / 4 aligned 64-bit loads and no point is
-//   padded; the block is rounded up to 16 bytes (cp.async / TMA granularity).
+// level k of element e.
+//   double, float pairs: element-blocked, component-major [7][padded n^3], point
+//   c + n^2 k;
+//   float, bf16: the order in which the plane kernel consumes it.  A unit of
+//   G = 32 / n consecutive elements has n / R chunks of R rows j; a chunk holds, for
+//   each element of the unit and each plane k, the 7 n R values of its points, point
+//   by point, in RS values.  A chunk is one contiguous copy, and RS is an odd number
+//   of the loads of four values that read it (8 bytes bf16, 16 bytes float), so that
+//   the loads of neighbouring lanes, each of its own plane, fall on different banks.
+//   R = n at n <= 3 (one chunk), 1 above: the kernel keeps a short ring of chunks in
+//   shared memory instead of the unit's whole metric.  The last unit is padded.
 template <typename MT>
 struct MetricLayout {
-  static constexpr bool kColumnMajor = false;
   __host__ __device__ static constexpr int block(int n) { return kMetricComps * padded_n3(n); }
-  __host__ __device__ static constexpr int at(int n, int c, int k, int comp) {
-    return comp * padded_n3(n) + c + k * n * n;
+  __host__ __device__ static constexpr size_t offset(int n, int64_t e, int c, int k, int comp) {
+    return (size_t)e * block(n) + comp * padded_n3(n) + c + k * n * n;
   }
 };
-template <>
-struct MetricLayout<__nv_bfloat16> {
-  static constexpr bool kColumnMajor = true;
-  __host__ __device__ static constexpr int col_width(int n) { return (kMetricComps * n + 3) / 4 * 4; }
-  __host__ __device__ static constexpr int block(int n) { return (n * n * col_width(n) + 7) / 8 * 8; }
-  __host__ __device__ static constexpr int at(int n, int c, int k, int comp) {
-    return c * col_width(n) + kMetricComps * k + comp;
+struct PlaneMetricLayout {
+  __host__ __device__ static constexpr int unit(int n) { return 32 / n; }                // G
+  __host__ __device__ static constexpr int rows(int n) { return n <= 3 ? n : 1; }        // R
+  __host__ __device__ static constexpr int chunks(int n) { return n / rows(n); }
+  __host__ __device__ static constexpr int stride(int n) {                               // RS
+    return 4 * (((kMetricComps * n * rows(n) + 3) / 4) | 1);
+  }
+  __host__ __device__ static constexpr int chunk(int n) { return unit(n) * n * stride(n); }
+  __host__ __device__ static constexpr size_t offset(int n, int64_t e, int c, int k, int comp) {
+    const int64_t u = e / unit(n);
+    const int s = (int)(e - u * unit(n)), i = c % n, j = c / n;
+    return (size_t)(u * chunks(n) + j / rows(n)) * chunk(n) + (s * n + k) * stride(n) +
+           kMetricComps * (i + n * (j % rows(n))) + comp;
   }
 };
+template <> struct MetricLayout<float> : PlaneMetricLayout {};
+template <> struct MetricLayout<__nv_bfloat16> : PlaneMetricLayout {};
 
-// Number of values of the bf16 metric of a level.
-inline size_t metric16_count(const Level& L) {
-  return (size_t)L.nelem * MetricLayout<__nv_bfloat16>::block(L.n);
+// Number of values of the float or bf16 metric of a level (whole units).
+inline size_t metric_lowp_count(const Level& L) {
+  using ML = PlaneMetricLayout;
+  const size_t units = ((size_t)L.nelem + ML::unit(L.n) - 1) / ML::unit(L.n);
+  return units * ML::chunks(L.n) * ML::chunk(L.n);
 }
 
 // Arguments of the element kernel y += A_e u_e (scatter-add into y).
@@ -258,9 +270,10 @@ struct ApplyArgs {
   // atomic adds, and a node kernel then adds each node's contributions to y in a
   // fixed order
   typename VecOf<T>::type* yloc;
-  // set by the launcher: the vectors' length, the SEM_DEBUG index-error word and
+  // set by the launcher: the vectors' length and strides, the SEM_DEBUG index-error word and
   // the wait-timeout word
   int64_t ndofs;
+  int row, plane;  // lattice strides: nodes of an x-row and of an (x, y) plane
   unsigned long long* dbg;
   unsigned* fault;
   int hold;  // SEM_DEBUG build: Level::hold

@@ -232,28 +232,25 @@ __global__ void k_region_mask(int64_t ndofs, const double* __restrict__ xyz, int
   }
 }
 
+__device__ __forceinline__ void metric_store(float* p, double v) { *p = __double2float_rn(v); }
+__device__ __forceinline__ void metric_store(__nv_bfloat16* p, double v) { *p = __float2bfloat16_rn(__double2float_rn(v)); }
+
+// FP64 component-major metric -> the plane kernel's low-precision order (MetricLayout);
+// zero in the padding.
 template <typename OT>
-__global__ void k_convert(int64_t n, const double* __restrict__ in, OT* __restrict__ out);
-
-template <>
-__global__ void k_convert<float>(int64_t n, const double* __restrict__ in, float* __restrict__ out) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    out[i] = __double2float_rn(in[i]);
-}
-
-// FP64 component-major metric -> the column-major bf16 layout (MetricLayout).
-__global__ void k_convert_columns_bf16(int64_t n, int np, const double* __restrict__ in,
-                                       __nv_bfloat16* __restrict__ out) {
-  using ML = MetricLayout<__nv_bfloat16>;
-  const int n2 = np * np, cw = ML::col_width(np), blk = ML::block(np), n3p = padded_n3(np);
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t e = i / blk;
-    const int r = (int)(i - e * blk), c = r / cw, s = r - c * cw, k = s / kMetricComps,
-              comp = s - k * kMetricComps;
-    const double v = (c < n2 && k < np) ? in[(e * kMetricComps + comp) * n3p + c + (int64_t)n2 * k] : 0.0;
-    out[i] = __float2bfloat16_rn(__double2float_rn(v));
+__global__ void k_convert_planes(int64_t n, int64_t nelem, int np, const double* __restrict__ in,
+                                 OT* __restrict__ out) {
+  using ML = MetricLayout<OT>;
+  const int rs = ML::stride(np), rows = ML::rows(np), nch = ML::chunks(np), G = ML::unit(np), n3p = padded_n3(np);
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n;
+       t += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t lane = t / rs;  // ((unit, chunk), element slot, plane)
+    const int v = (int)(t - lane * rs), point = v / kMetricComps, comp = v - point * kMetricComps;
+    const int k = (int)(lane % np), slot = (int)((lane / np) % G), chunk = (int)((lane / np / G) % nch);
+    const int64_t e = lane / np / G / nch * G + slot;
+    const int c = chunk * rows * np + point;
+    metric_store(out + t, (e < nelem && point < rows * np) ? in[(e * kMetricComps + comp) * n3p + c + (int64_t)np * np * k]
+                                                           : 0.0);
   }
 }
 
@@ -363,16 +360,14 @@ cudaError_t setup_diagonals(Level& L, cudaStream_t s) {
 }
 
 cudaError_t setup_metric_lowp(Level& L, bool bf16, cudaStream_t s) {
-  const int64_t count = (int64_t)metric_count(L);
+  const int64_t count = (int64_t)metric_lowp_count(L);
   const int threads = 256;
   const int blocks = (int)std::min<int64_t>((count + threads - 1) / threads, 152 * 16);
   if (bf16) {
-    const int64_t count16 = (int64_t)metric16_count(L);
-    const int blocks16 = (int)std::min<int64_t>((count16 + threads - 1) / threads, 152 * 16);
-    k_convert_columns_bf16<<<blocks16, threads, 0, s>>>(count16, L.n, L.metric, L.metric16);
+    k_convert_planes<<<blocks, threads, 0, s>>>(count, L.nelem, L.n, L.metric, L.metric16);
     L.metric16_valid = true;
   } else {
-    k_convert<float><<<blocks, threads, 0, s>>>(count, L.metric, L.metric32);
+    k_convert_planes<<<blocks, threads, 0, s>>>(count, L.nelem, L.n, L.metric, L.metric32);
     L.metric32_valid = true;
   }
   return cudaGetLastError();

@@ -1,0 +1,43 @@
+"""The plane kernel of the FP32 operator at the edges of its units.
+
+A unit is G = 32 // (p + 1) consecutive elements of one warp: meshes of one element, of
+one unit exactly, of one element more or less, of rows that end inside a unit, and vectors
+that start 4 bytes past a 16-byte boundary (the gather copies single words).  The reference
+is the FP64 apply, which the other tests hold to the oracle.  Bounds as in test_gpu_apply:
+FP32 arithmetic with an FP32 metric 6e-7, the bf16 metric 5e-3 (relative, 2-norm).
+"""
+import numpy as np
+import pytest
+import torch
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+gb = pytest.importorskip("paper_2205_05136_gb300")
+
+
+def _dims(p):
+    g = 32 // (p + 1)
+    return [(1, 1, 1), (g, 1, 1), (g - 1, 1, 1), (g + 1, 1, 1), (3, 2, 2), (g + 2, 3, 2)]
+
+
+@pytest.mark.parametrize("quad", ["LGL", "LG"])
+@pytest.mark.parametrize("p", [1, 2, 3, 4, 5, 6])
+def test_plane_kernel_unit_edges(p, quad):
+    for dims in _dims(p):
+        s = W.slab(*dims, (20.0, 7.0, 3.0), perturb=0.1, seed=1)
+        g = gb.Slab(s.flat_vertices(), *dims, p, quad)
+        g.set_tissue(np.full(s.n_elements, 0.12), np.full(s.n_elements, 0.03), W.transmural_fiber_angles(s))
+        buf = torch.tensor(W.uniform_vector(g.ndofs + 1, -1.0, 1.0, seed=2), device="cuda").float()
+        out = torch.empty_like(buf)
+        for off in (0, 1):
+            u = buf[off:off + g.ndofs]
+            y = out[off:off + g.ndofs]
+            for alpha, beta in ((30.0, 1.0), (2.5, -0.7)):
+                ref = g.apply(u.double(), alpha, beta)
+                for prec, tol in ((gb.SEM_PREC_FP32, 6e-7), (gb.SEM_PREC_FP32_BF16, 5e-3)):
+                    g.apply(u, alpha, beta, prec, out=y)
+                    err = float(torch.linalg.norm(y.double() - ref) / torch.linalg.norm(ref))
+                    assert err < tol, (p, quad, dims, off, alpha, prec, err)
+        g.close()
