@@ -14,11 +14,12 @@ cudaError_t launch_apply_fp64(const Level& L, const ApplyArgs64& a, bool mass_on
 __global__ void __launch_bounds__(kApplyThreads)
     k_apply_dot_finish(const double* __restrict__ partials, int n, CgScalars* cg, double* out,
                        const int* done) {
-  pdl_entry();
+  pdl_wait();
   __shared__ double red[32];
   if (done != nullptr && *done) return;
   double v = 0.0;
   for (int b = threadIdx.x; b < n; b += kApplyThreads) v += partials[b];
+  pdl_trigger();
   v = block_sum(v, red);
   if (threadIdx.x == 0) {
     if (cg != nullptr) {
@@ -43,7 +44,7 @@ template <typename V>
 __global__ void __launch_bounds__(256)
     k_assemble(int nx, int ny, int nz, int p, const V* __restrict__ yloc, V* __restrict__ y,
                const int* done) {
-  pdl_entry();
+  pdl_wait();
   if (done != nullptr && *done) return;
   const int n = p + 1, n2 = n * n, n3 = n2 * n;
   const int64_t NX = (int64_t)p * nx + 1, NY = (int64_t)p * ny + 1, nd = NX * NY * ((int64_t)p * nz + 1);
@@ -67,6 +68,7 @@ __global__ void __launch_bounds__(256)
         }
     y[g] += acc;
   }
+  pdl_trigger();
 }
 
 template <typename V>

@@ -229,7 +229,6 @@ __host__ __device__ constexpr size_t apply_warp_tile_bytes() {
 template <int P, int QUAD, typename T, typename MT, bool DOT, bool MASS_ONLY, bool WARP = false>
 __global__ void __launch_bounds__(kApplyThreads, (std::is_same<T, df>::value && P == 4) ? 5 : 1)
     sem_apply_kernel(const ApplyArgs<T, MT> a, const __grid_constant__ KTab<P + 1, T> tab) {
-  pdl_trigger();
   static_assert(!(WARP && DOT), "the fused inner product needs the CTA-wide mode");
   constexpr int N = P + 1, N2 = N * N, N3 = N2 * N;
   using ML = MetricLayout<MT>;
@@ -373,6 +372,7 @@ __global__ void __launch_bounds__(kApplyThreads, (std::is_same<T, df>::value && 
     group_sync();
   }
 
+  pdl_trigger();
   // scatter-add y += P_e^T y_e, and with DOT the partial u_e . y_e
   double dot = 0.0;
   if constexpr (DOT) {
@@ -442,7 +442,8 @@ __global__ void __launch_bounds__(kApplyThreads, (std::is_same<T, df>::value && 
 // memory pipe (two z-sweeps read n planes a lane) and latency, at 12 warps an SM.
 // Measured, apply with the clearing of y, SEM-NI, bf16 metric, 2 M nodes, before /
 // after: p = 1..6 76 / 55, 41 / 31, 27 / 23, 27 / 21, 33 / 20, 31 / 25 us; 30 M
-// nodes, p = 4: 307 / 231 us.
+// nodes, p = 4: 307 / 231 us.  With 16 warps (128 registers) the p = 4 V-cycle on
+// 2 M nodes took 387 us against 362 with 12 (168 registers).
 //
 // Each warp loops over units w, w + W, ... (W warps in the persistent grid)
 // with the copies of the next unit in flight:
@@ -777,7 +778,6 @@ template <int P, int QUAD, typename MT>
 __global__ void __launch_bounds__(32 * PlaneCfg<P, MT>::kWarps, PlaneCfg<P, MT>::kResident / PlaneCfg<P, MT>::kWarps)
     sem_apply_plane_kernel(const ApplyArgs<float, MT> a, const __grid_constant__ KTab<P + 1, float> tab,
                            const __grid_constant__ ZTab<P + 1> zt, int nunits) {
-  pdl_trigger();
   using C = PlaneCfg<P, MT>;
   constexpr int N = C::N, N2 = C::N2, G = C::G;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -789,7 +789,7 @@ __global__ void __launch_bounds__(32 * PlaneCfg<P, MT>::kWarps, PlaneCfg<P, MT>:
   float* tiles = reinterpret_cast<float*>(wb + C::tile_offset);
   const unsigned sm_s = smem_u32(wb), tile_s = smem_u32(tiles), bar_s = smem_u32(wb + C::bar_offset);
   // While the previous kernel drains, before pdl_wait: the first metric copies and
-  // the map entries (written by the set-up only).
+  // the map entries (written by the set-up only, see pdl_trigger).
   if (lane == 0) {
     for (int t = 0; t < C::kStages; ++t) mbar_init(bar_s + 8 * t);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -829,6 +829,7 @@ __global__ void __launch_bounds__(32 * PlaneCfg<P, MT>::kWarps, PlaneCfg<P, MT>:
     asm volatile("cp.async.wait_all;\n" ::: "memory");
     __syncwarp();  // every lane's copies of this unit landed
     const int nxt = unit + tw;
+    if (nxt >= nunits) pdl_trigger();  // the last unit
     if (nxt < nunits) plane_gather<P>(a, nxt, base_n, s, r, act, tile_s + 4u * (unsigned)((b ^ 1) * C::TW));
     const int base_nn = plane_base<P>(a, nxt + tw, nunits, s);
     float* elem = tiles + b * C::TW + s * C::ES;

@@ -211,7 +211,7 @@ __device__ __forceinline__ int64_t line_base(const TcArgs& a, const UnitPos& q, 
 
 template <int P>
 __global__ void __launch_bounds__(TcCfg<P>::WARPS * 32, 3) sem_apply_tc_kernel(const TcArgs a) {
-  pdl_entry();
+  pdl_wait();
   using C = TcCfg<P>;
   constexpr int N = C::N, NP = C::NP, N3 = C::N3, EPT = C::EPT, ROWS = C::ROWS, NG = C::NG;
   constexpr int KS1 = C::KS1, NT1 = C::NT1, NT2 = C::NT2, MTU = C::MTU;
@@ -455,6 +455,7 @@ __global__ void __launch_bounds__(TcCfg<P>::WARPS * 32, 3) sem_apply_tc_kernel(c
     b ^= 1;
   }
   asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+  pdl_trigger();
 }
 
 // ---------------------------------------------------------------------------
@@ -552,7 +553,7 @@ bool tc_fragments(const Tables1D& tab, std::vector<uint32_t>& f) {
 template <int P>
 __global__ void k_metric_tc(int64_t nwords, int nx, int ny, int upr, const double* __restrict__ metric,
                             uint32_t* __restrict__ out) {
-  pdl_entry();
+  pdl_wait();
   using C = TcCfg<P>;
   constexpr int N = C::N, NP = C::NP, N3P = padded_n3(N);
   for (int64_t w = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; w < nwords;

@@ -150,23 +150,25 @@ __host__ __device__ constexpr int k16() { return 16 / (int)sizeof(T); }
 
 template <typename T>
 __global__ void k_zero(int64_t n, T* x, const int* done) {
-  pdl_entry();
+  pdl_wait();
   if (skip(done)) return;
   constexpr int K = k16<T>();
   const int64_t nc = n / K;
   GRID_CHUNKS(c, nc) reinterpret_cast<Pk<T, K>*>(x)[c] = Pk<T, K>{};
   GRID_TAIL(i, nc * K, n) x[i] = T(0);
+  pdl_trigger();
 }
 
 template <typename T>
 __global__ void k_level_inv_diag(int64_t n, double alpha, const double* m, const double* k,
                                  T* inv, double* inv64) {
-  pdl_entry();
+  pdl_wait();
   GRID_LOOP(i, n) {
     const double v = 1.0 / fma(alpha, m[i], k[i]);
     inv[i] = (T)v;
     inv64[i] = v;
   }
+  pdl_trigger();
 }
 
 // Chebyshev step 0 from a zero start: d = D^{-1} b / theta, x = d, t = 0.
@@ -174,7 +176,7 @@ template <typename T>
 __global__ void k_cheb_zero_start(int64_t n, const T* __restrict__ b, const T* __restrict__ invd,
                                   T* __restrict__ x, T* __restrict__ d, T* __restrict__ t,
                                   T inv_theta, const int* done) {
-  pdl_entry();
+  pdl_wait();
   if (skip(done)) return;
   constexpr int K = k16<T>();
   using V = Pk<T, K>;
@@ -194,6 +196,7 @@ __global__ void k_cheb_zero_start(int64_t n, const T* __restrict__ b, const T* _
     x[i] = di;
     t[i] = T(0);
   }
+  pdl_trigger();
 }
 
 // Chebyshev step with t = A x: d = c1 d + c2 D^{-1}(b - t), x += d, t = 0
@@ -208,7 +211,7 @@ template <typename T>
 __global__ void k_cheb_step(int64_t n, const T* __restrict__ b, const T* __restrict__ invd,
                             T* __restrict__ x, T* __restrict__ d, T* __restrict__ t, T c1, T c2,
                             int first, const int* done) {
-  pdl_entry();
+  pdl_wait();
   if (skip(done)) return;
   constexpr int K = k16<T>();
   using V = Pk<T, K>;
@@ -233,6 +236,7 @@ __global__ void k_cheb_step(int64_t n, const T* __restrict__ b, const T* __restr
     x[i] += di;
     t[i] = T(0);
   }
+  pdl_trigger();
 }
 
 // ---------------------------------------------------------------- transfers
@@ -257,7 +261,7 @@ template <typename T>
 __global__ void k_prolong_h(int nfx, int nfy, int nfz, int ncx, int ncy, int ncz,
                             const T* __restrict__ xc, T* __restrict__ xf, T* __restrict__ tf,
                             const int* done) {
-  pdl_entry();
+  pdl_wait();
   if (skip(done)) return;
   const int64_t NX = nfx + 1, NY = nfy + 1, n = NX * NY * (nfz + 1);
   const int64_t CX = ncx + 1, CY = ncy + 1;
@@ -278,13 +282,14 @@ __global__ void k_prolong_h(int nfx, int nfy, int nfz, int ncx, int ncy, int ncz
     xf[g] += s;
     tf[g] = T(0);
   }
+  pdl_trigger();
 }
 
 template <typename T>
 __global__ void k_restrict_h(int nfx, int nfy, int nfz, int ncx, int ncy, int ncz,
                              const T* __restrict__ bf, const T* __restrict__ tf,
                              T* __restrict__ bc, const int* done) {
-  pdl_entry();
+  pdl_wait();
   if (skip(done)) return;
   const int64_t NX = nfx + 1, NY = nfy + 1, n = NX * NY * (nfz + 1);
   const int64_t CX = ncx + 1, CY = ncy + 1;
@@ -303,6 +308,7 @@ __global__ void k_restrict_h(int nfx, int nfy, int nfz, int ncx, int ncy, int nc
           if (w != 0.0) atomicAdd(bc + (kx + a) + CX * ((ky + b) + CY * (kz + c)), (T)w * r);
         }
   }
+  pdl_trigger();
 }
 
 // The same restriction gathered per coarse node (deterministic mode): the fine
@@ -312,7 +318,7 @@ template <typename T>
 __global__ void k_restrict_h_det(int nfx, int nfy, int nfz, int ncx, int ncy, int ncz,
                                  const T* __restrict__ bf, const T* __restrict__ tf,
                                  T* __restrict__ bc, const int* done) {
-  pdl_entry();
+  pdl_wait();
   if (skip(done)) return;
   const int64_t NX = nfx + 1, NY = nfy + 1;
   const int64_t CX = ncx + 1, CY = ncy + 1, nc = CX * CY * (ncz + 1);
@@ -341,12 +347,13 @@ __global__ void k_restrict_h_det(int nfx, int nfy, int nfz, int ncx, int ncy, in
     }
     bc[c] += acc;
   }
+  pdl_trigger();
 }
 
 __global__ void k_coarse_tissue(int ncx, int ncy, int ncz, int nfx, int nfy, const double* sl,
                                 const double* st, const double* th, double* csl, double* cst,
                                 double* cth) {
-  pdl_entry();
+  pdl_wait();
   const int64_t n = (int64_t)ncx * ncy * ncz;
   GRID_LOOP(e, n) {
     const int kx = (int)(e % ncx), ky = (int)((e / ncx) % ncy), kz = (int)(e / ((int64_t)ncx * ncy));
@@ -355,50 +362,56 @@ __global__ void k_coarse_tissue(int ncx, int ncy, int ncz, int nfx, int nfy, con
     cst[e] = st[f];
     cth[e] = th[f];
   }
+  pdl_trigger();
 }
 
 // ---------------------------------------------------------------- reductions
 // Deterministic dot product; the last CTA writes the total to *out.
 __global__ void k_dot(int64_t n, const double* __restrict__ a, const double* __restrict__ b,
                       double* partials, unsigned int* ticket, double* out) {
-  pdl_entry();
+  pdl_wait();
   __shared__ double red[32];
   double v = 0.0;
   GRID_LOOP(i, n) v = fma(a[i], b[i], v);
+  pdl_trigger();
   v = block_sum(v, red);
   double total;
   if (finish_reduction(v, partials, ticket, &total, red)) *out = total;
 }
 
 __global__ void k_fill_start(int64_t n, double* v) {
-  pdl_entry();
+  pdl_wait();
   GRID_LOOP(i, n) {
     const unsigned long long h = ((unsigned long long)i * 2654435761ull) & 0xffffffffull;
     v[i] = (double)h / 4294967296.0 - 0.5;
   }
+  pdl_trigger();
 }
 
 __global__ void k_lanczos_z(int64_t n, const double* dinv, const double* r, double* z) {
-  pdl_entry();
+  pdl_wait();
   GRID_LOOP(i, n) z[i] = dinv[i] * r[i];
+  pdl_trigger();
 }
 
 __global__ void k_lanczos_update(int64_t n, double alpha, const double* Ap, double* r,
                                  const double* dinv, double* z) {
-  pdl_entry();
+  pdl_wait();
   GRID_LOOP(i, n) {
     const double ri = fma(-alpha, Ap[i], r[i]);
     r[i] = ri;
     z[i] = dinv[i] * ri;
   }
+  pdl_trigger();
 }
 
 __global__ void k_lanczos_p(int64_t n, double beta, const double* z, double* p, double* Ap) {
-  pdl_entry();
+  pdl_wait();
   GRID_LOOP(i, n) {
     p[i] = fma(beta, p[i], z[i]);
     Ap[i] = 0.0;
   }
+  pdl_trigger();
 }
 
 // ---------------------------------------------------------------- outer flexible PCG
@@ -439,7 +452,7 @@ __global__ void k_fpcg_init(int64_t n, const double* __restrict__ b, double* Ap_
                             const int* use_main, double* __restrict__ r, T* __restrict__ b0, CgScalars* cg,
                             double* partials, int stride, unsigned int* ticket, double rtol,
                             double atol) {
-  pdl_entry();
+  pdl_wait();
   // A x: Ap_main, or Ap_alt where the flag use_main reads zero
   double* __restrict__ Ap = (use_main == nullptr || *use_main != 0) ? Ap_main : Ap_alt;
   double v[2] = {0.0, 0.0};
@@ -469,6 +482,7 @@ __global__ void k_fpcg_init(int64_t n, const double* __restrict__ b, double* Ap_
     v[0] = fma(ri, ri, v[0]);
     v[1] = fma(bi, bi, v[1]);
   }
+  pdl_trigger();
   double tot[2];
   if (grid_sums_k<2>(v, partials, stride, ticket, tot)) {
     cg->rr = tot[0];
@@ -490,7 +504,7 @@ template <typename T>
 __global__ void k_fpcg_z(int64_t n, const T* __restrict__ x0, double* __restrict__ z,
                          const double* __restrict__ r, double* __restrict__ p, df_pair* __restrict__ p2,
                          CgScalars* cg, double* partials, int stride, unsigned int* ticket) {
-  pdl_entry();
+  pdl_wait();
   if (cg->done) return;
   const bool first = cg->iters == 0;
   double v[2] = {0.0, 0.0};
@@ -528,6 +542,7 @@ __global__ void k_fpcg_z(int64_t n, const T* __restrict__ x0, double* __restrict
     z[i] = zi;
     v[0] = fma(ri, zi, v[0]);
   }
+  pdl_trigger();
   double tot[2];
   if (grid_sums_k<2>(v, partials, stride, ticket, tot)) {
     if (first) {
@@ -545,7 +560,7 @@ __global__ void k_fpcg_z(int64_t n, const T* __restrict__ x0, double* __restrict
 
 __global__ void k_fpcg_p(int64_t n, const double* __restrict__ z, double* __restrict__ p,
                          df_pair* __restrict__ p2, const CgScalars* cg) {
-  pdl_entry();
+  pdl_wait();
   if (cg->done || cg->iters == 0) return;  // first iteration: k_fpcg_z set p = z
   const double beta = cg->beta;
   using D2 = Pk<double, 2>;
@@ -566,6 +581,7 @@ __global__ void k_fpcg_p(int64_t n, const double* __restrict__ z, double* __rest
     p[i] = pi;
     if (p2 != nullptr) p2[i] = split_pair(pi);
   }
+  pdl_trigger();
 }
 
 // x += alpha p, r -= alpha Ap, Ap = 0, b0 = (T) r; r.r; convergence.  VEC: x is
@@ -574,7 +590,7 @@ template <typename T, bool VEC>
 __global__ void k_fpcg_xr(int64_t n, double* __restrict__ x, const double* __restrict__ p,
                           double* __restrict__ Ap, double* __restrict__ r, T* __restrict__ b0,
                           CgScalars* cg, double* partials, int stride, unsigned int* ticket) {
-  pdl_entry();
+  pdl_wait();
   if (cg->done) return;
   const double alpha = cg->alpha;
   double v[1] = {0.0};
@@ -606,6 +622,7 @@ __global__ void k_fpcg_xr(int64_t n, double* __restrict__ x, const double* __res
     b0[i] = (T)ri;
     v[0] = fma(ri, ri, v[0]);
   }
+  pdl_trigger();
   double tot[1];
   if (grid_sums_k<1>(v, partials, stride, ticket, tot)) {
     cg->rr = tot[0];
@@ -715,7 +732,7 @@ __global__ void __launch_bounds__(kThreads, 8)
                  const df_pair* __restrict__ ax2_in, const int* ax2_ok, df_pair* __restrict__ r2,
                  T* __restrict__ b0, CgScalars* cg, double* partials, int stride, unsigned int* ticket,
                  double rtol, double atol) {
-  pdl_entry();
+  pdl_wait();
   // the carried pairs, unless the flag ax2_ok reads zero (then A x is in Ap)
   const df_pair* __restrict__ ax2 = (ax2_ok == nullptr || *ax2_ok != 0) ? ax2_in : nullptr;
   df v[2] = {df(0.f, 0.f), df(0.f, 0.f)};
@@ -747,6 +764,7 @@ __global__ void __launch_bounds__(kThreads, 8)
     }
     init_entry(b[i], ax, r2[i], b0[i], v);
   }
+  pdl_trigger();
   double tot[2];
   if (grid_sums_df<2>(v, partials, stride, ticket, tot)) {
     cg->rr = tot[0];
@@ -775,7 +793,7 @@ template <typename T>
 __global__ void __launch_bounds__(kThreads, 8)
     k_dfpcg_z(int64_t n, const T* __restrict__ x0, T* __restrict__ zs, const df_pair* __restrict__ r2,
               df_pair* __restrict__ p2, CgScalars* cg, double* partials, int stride, unsigned int* ticket) {
-  pdl_entry();
+  pdl_wait();
   if (cg->done) return;
   const bool first = cg->iters == 0;
   df v[2] = {df(0.f, 0.f), df(0.f, 0.f)};
@@ -795,6 +813,7 @@ __global__ void __launch_bounds__(kThreads, 8)
     z_entry(x0[i], zs[i], r2[i], pp, first, v);
     if (first) p2[i] = pp;
   }
+  pdl_trigger();
   double tot[2];
   if (grid_sums_df<2>(v, partials, stride, ticket, tot)) {
     cg->beta = first ? 0.0 : (tot[0] - tot[1]) / cg->rz;
@@ -816,7 +835,7 @@ __device__ __forceinline__ df_pair p_entry(df beta, df_pair pp, T z) {
 template <typename T>
 __global__ void __launch_bounds__(kThreads, 8)
     k_dfpcg_p(int64_t n, const T* __restrict__ zs, df_pair* __restrict__ p2, const CgScalars* cg) {
-  pdl_entry();
+  pdl_wait();
   if (cg->done || cg->iters == 0) return;  // first iteration: k_dfpcg_z set p = z
   const df beta = dfd(cg->beta);
   const int64_t nc = n / 2;
@@ -828,6 +847,7 @@ __global__ void __launch_bounds__(kThreads, 8)
     reinterpret_cast<C2<df_pair>*>(p2)[c] = pp;
   }
   GRID_TAIL(i, nc * 2, n) p2[i] = p_entry(beta, p2[i], zs[i]);
+  pdl_trigger();
 }
 
 // x += alpha p (FP64), r -= alpha Ap, Ap = 0, b0 = r; r.r; convergence.
@@ -847,7 +867,7 @@ __global__ void __launch_bounds__(kThreads, kXrCtasPerSm)
     k_dfpcg_xr(int64_t n, double* __restrict__ x, const df_pair* __restrict__ p2, double* __restrict__ Ap,
                df_pair* __restrict__ r2, T* __restrict__ b0, CgScalars* cg, double* partials, int stride,
                unsigned int* ticket) {
-  pdl_entry();
+  pdl_wait();
   if (cg->done) return;
   const double alpha = cg->alpha;
   const df nalpha = dfneg(dfd(alpha));
@@ -869,6 +889,7 @@ __global__ void __launch_bounds__(kThreads, kXrCtasPerSm)
   GRID_TAIL(i, nc * 2, n) {
     b0[i] = xr_entry<T>(alpha, nalpha, p2[i], x[i], Ap[i], r2[i], v);
   }
+  pdl_trigger();
   double tot[1];
   if (grid_sums_df<1>(v, partials, stride, ticket, tot)) {
     cg->rr = tot[0];
@@ -884,14 +905,16 @@ __global__ void __launch_bounds__(kThreads, kXrCtasPerSm)
 
 template <typename T>
 __global__ void k_to_level0(int64_t n, const double* __restrict__ r, T* __restrict__ b0) {
-  pdl_entry();
+  pdl_wait();
   GRID_LOOP(i, n) b0[i] = (T)r[i];
+  pdl_trigger();
 }
 
 template <typename T>
 __global__ void k_from_level0(int64_t n, const T* __restrict__ x0, double* __restrict__ z) {
-  pdl_entry();
+  pdl_wait();
   GRID_LOOP(i, n) z[i] = (double)x0[i];
+  pdl_trigger();
 }
 
 // ---------------------------------------------------------------- host helpers

@@ -66,29 +66,32 @@ __device__ __forceinline__ bool grid_sums(double (&v)[K], double* partials, unsi
 
 __global__ void k_inv_diag(int64_t n, double alpha, const double* __restrict__ m,
                            const double* __restrict__ k, double* __restrict__ inv) {
-  pdl_entry();
+  pdl_wait();
 #pragma unroll 1
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
     inv[i] = 1.0 / fma(alpha, m[i], k[i]);
+  pdl_trigger();
 }
 
 __global__ void k_scale_mul(int64_t n, double a, const double* __restrict__ d,
                             const double* __restrict__ x, double* __restrict__ y) {
-  pdl_entry();
+  pdl_wait();
 #pragma unroll 1
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
     y[i] = a * d[i] * x[i];
+  pdl_trigger();
 }
 
 __global__ void k_scale_mul32(int64_t n, float a, const double* __restrict__ d,
                               const float* __restrict__ x, float* __restrict__ y) {
-  pdl_entry();
+  pdl_wait();
 #pragma unroll 1
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
     y[i] = a * (float)d[i] * x[i];
+  pdl_trigger();
 }
 
 // r = b - Ap, z = Jacobi(r), p = z, Ap = 0; r.z, r.r, b.b; convergence test.
@@ -97,7 +100,7 @@ __global__ void __launch_bounds__(kVecThreads)
               const double* __restrict__ inv, double* __restrict__ r, double* __restrict__ z,
               double* __restrict__ p, df_pair* __restrict__ p2, CgScalars* cg, double* partials,
               unsigned int* ticket, double rtol, double atol) {
-  pdl_entry();
+  pdl_wait();
   double v[3] = {0.0, 0.0, 0.0};
 #pragma unroll 1
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
@@ -114,6 +117,7 @@ __global__ void __launch_bounds__(kVecThreads)
     v[1] = fma(ri, ri, v[1]);
     v[2] = fma(bi, bi, v[2]);
   }
+  pdl_trigger();
   double tot[3];
   if (grid_sums<3>(v, partials, ticket, tot)) {
     cg->rz = tot[0];
@@ -141,7 +145,7 @@ __global__ void __launch_bounds__(kVecThreads)
     k_cg_xr(int64_t n, double* __restrict__ x, const double* __restrict__ p,
             const double* __restrict__ Ap, double* __restrict__ r, const double* __restrict__ inv,
             double* __restrict__ z, CgScalars* cg, double* partials, unsigned int* ticket) {
-  pdl_entry();
+  pdl_wait();
   if (cg->done) return;
   const double alpha = cg->alpha;
   double v[2] = {0.0, 0.0};
@@ -179,6 +183,7 @@ __global__ void __launch_bounds__(kVecThreads)
     v[0] = fma(ri, zi, v[0]);
     v[1] = fma(ri, ri, v[1]);
   }
+  pdl_trigger();
   double tot[2];
   if (grid_sums<2>(v, partials, ticket, tot)) {
     cg->beta = tot[0] / cg->rz;
@@ -199,7 +204,7 @@ __global__ void __launch_bounds__(kVecThreads)
 __global__ void __launch_bounds__(kVecThreads)
     k_cg_p(int64_t n, const double* __restrict__ z, double* __restrict__ p, df_pair* __restrict__ p2,
            double* __restrict__ Ap, const CgScalars* cg) {
-  pdl_entry();
+  pdl_wait();
   if (cg->done) return;
   const double beta = cg->beta;
   const int64_t g0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -225,6 +230,7 @@ __global__ void __launch_bounds__(kVecThreads)
     Ap[i] = 0.0;
     if (p2 != nullptr) p2[i] = split_pair(pi);
   }
+  pdl_trigger();
 }
 
 // With `same` set (sem_step_host_out), x0 still holds the solution the last call
@@ -263,7 +269,7 @@ __global__ void __launch_bounds__(kVecThreads)
                 double* __restrict__ hnext, double* __restrict__ x0, double* __restrict__ out,
                 const double* __restrict__ mdiag, const double* __restrict__ mask, double iapp,
                 const IonicArgs prm, double dt, int first, int* same) {
-  pdl_entry();
+  pdl_wait();
   const double inv_dt = 1.0 / dt, inv_2dt = 0.5 / dt;
   const double c_open = (first ? dt : 2.0 * dt) * prm.inv_tau_open;
   const double c_close = (first ? dt : 2.0 * dt) * prm.inv_tau_close;
@@ -288,6 +294,7 @@ __global__ void __launch_bounds__(kVecThreads)
     x0[i] = u0;
     out[i] = mdiag ? mdiag[i] * g : g;
   }
+  pdl_trigger();
 }
 
 // The same per-node update in double-float arithmetic on the FP32 pipe (the
@@ -331,7 +338,7 @@ __global__ void __launch_bounds__(kVecThreads)
                    double* __restrict__ hnext, double* __restrict__ x0, double* __restrict__ out,
                    const double* __restrict__ mdiag, const double* __restrict__ mask,
                    const IonicDfArgs P, int first, int* same) {
-  pdl_entry();
+  pdl_wait();
 #pragma unroll 1
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -343,6 +350,7 @@ __global__ void __launch_bounds__(kVecThreads)
                   mdiag != nullptr, stim, P, first, hnext[i], out[i]);
     x0[i] = u0d;
   }
+  pdl_trigger();
 }
 
 // The same on two consecutive nodes per thread with 16-byte loads and stores
@@ -355,7 +363,7 @@ __global__ void __launch_bounds__(kVecThreads)
                     double2* __restrict__ hnext, double2* __restrict__ x0, double2* __restrict__ out,
                     const double2* __restrict__ mdiag, const double2* __restrict__ mask,
                     const IonicDfArgs P, int first, int* same) {
-  pdl_entry();
+  pdl_wait();
   if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0) {
     const int64_t t = n - 1;
     auto r = [](const double2* q, int64_t i) { return reinterpret_cast<const double*>(q)[i]; };
@@ -390,22 +398,24 @@ __global__ void __launch_bounds__(kVecThreads)
     }
     x0[i] = u0;
   }
+  pdl_trigger();
 }
 
 // c = a - b
 __global__ void __launch_bounds__(kVecThreads)
     k_sub(int64_t n, const double* __restrict__ a, const double* __restrict__ b, double* __restrict__ c) {
-  pdl_entry();
+  pdl_wait();
 #pragma unroll 1
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
     c[i] = a[i] - b[i];
+  pdl_trigger();
 }
 
 // c = a - b in double-float, b and c float pairs
 __global__ void __launch_bounds__(kVecThreads)
     k_sub_pairs(int64_t n, const double* __restrict__ a, const df_pair* __restrict__ b, df_pair* __restrict__ c) {
-  pdl_entry();
+  pdl_wait();
 #pragma unroll 1
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -413,16 +423,18 @@ __global__ void __launch_bounds__(kVecThreads)
     const df d = dfnorm(dfd(a[i]) - df(v.h, v.l));
     c[i] = df_pair{d.h, d.l};
   }
+  pdl_trigger();
 }
 
 __global__ void k_fill_pair(int64_t n, double* a, double va, double* b, double vb) {
-  pdl_entry();
+  pdl_wait();
 #pragma unroll 1
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
     a[i] = va;
     b[i] = vb;
   }
+  pdl_trigger();
 }
 
 // Activation time (Eq. tau): du/dt at t1 by the time scheme (BDF1 for the first
@@ -432,7 +444,7 @@ __global__ void __launch_bounds__(kVecThreads)
     k_activation(int64_t n, const double* __restrict__ u1, const double* __restrict__ u0,
                  const double* __restrict__ um1, int first, double dt, double t1,
                  double* __restrict__ dmax, double* __restrict__ tau) {
-  pdl_entry();
+  pdl_wait();
   const double inv_dt = 1.0 / dt, inv_2dt = 0.5 / dt;
 #pragma unroll 1
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
@@ -444,6 +456,7 @@ __global__ void __launch_bounds__(kVecThreads)
       tau[i] = t1;
     }
   }
+  pdl_trigger();
 }
 
 }  // namespace

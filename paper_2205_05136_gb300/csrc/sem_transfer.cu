@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(kTThreads)
     k_ptransfer_pass(int ne, int d0, int d1, int d2, const T* __restrict__ in, const T* __restrict__ in2,
                      T* __restrict__ out, T* __restrict__ out2, const __grid_constant__ PMat<NF, NC, T> pm,
                      const int* done) {
-  pdl_entry();
+  pdl_wait();
   if (done != nullptr && *done) return;
   constexpr int PF = NF - 1, PC = NC - 1;
   constexpr bool PRO = MODE == kProlong || MODE == kProlongAdd;
@@ -92,6 +92,7 @@ __global__ void __launch_bounds__(kTThreads)
       out[o] = acc;
     }
   }
+  pdl_trigger();
 }
 
 // 32 x 8 patches of a plane in x and y; along z as many CTAs as keep the grid
