@@ -62,6 +62,16 @@ __device__ __forceinline__ void store_loc(double* p, double v) { *p = v; }
 __device__ __forceinline__ void store_loc(float* p, float v) { *p = v; }
 __device__ __forceinline__ void store_loc(double* p, df v) { *p = (double)v; }
 
+// The factor on an element result: none, out_scale, or a sign (no FP64 multiplication).
+__device__ __forceinline__ df negated(df v) { return df(-v.h, -v.l); }
+__device__ __forceinline__ double negated(double v) { return -v; }
+__device__ __forceinline__ float negated(float v) { return -v; }
+template <typename T, typename MT>
+__device__ __forceinline__ T scale_result(const ApplyArgs<T, MT>& a, T v) {
+  if (a.scale_out == kScaleOut) v *= a.out_scale;
+  return a.scale_out == kNegateOut ? negated(v) : v;
+}
+
 // Base offset and stride of line l of an n^3 tile along direction DIR
 // (0: x-line (j,k), l = j + n k; 1: y-line (i,k), l = i + n k; 2: z-line (i,j), l = i + n j).
 template <int N, int DIR>
@@ -385,7 +395,7 @@ __global__ void __launch_bounds__(kApplyThreads, (std::is_same<T, df>::value && 
         if (e < a.nelem) {
           const int g = (int)SEM_IDX(__ldg(a.map + (size_t)e * N3 + loc), a.ndofs, a.dbg, kDbgScatter);
           T v = sA[idx];
-          if (a.scale_out) v *= a.out_scale;
+          v = scale_result(a, v);
           if (a.yloc != nullptr) store_loc(a.yloc + (size_t)e * N3 + loc, v);
           else scatter_add(a.y + g, v);
           const float2 uu = __ldg(reinterpret_cast<const float2*>(a.u2) + g);
@@ -399,7 +409,7 @@ __global__ void __launch_bounds__(kApplyThreads, (std::is_same<T, df>::value && 
         if (e < a.nelem) {
           const int g = (int)SEM_IDX(__ldg(a.map + (size_t)e * N3 + loc), a.ndofs, a.dbg, kDbgScatter);
           T v = sA[idx];
-          if (a.scale_out) v *= a.out_scale;
+          v = scale_result(a, v);
           if (a.yloc != nullptr) store_loc(a.yloc + (size_t)e * N3 + loc, v);
           else scatter_add(a.y + g, v);
           dot = fma((double)a.u[g], (double)v, dot);
@@ -414,7 +424,7 @@ __global__ void __launch_bounds__(kApplyThreads, (std::is_same<T, df>::value && 
       const int idx = tid + it * NTH;
       if ((IT * NTH == E * N3 || idx < E * N3) && idx < nv) {
         T v = sA[idx];
-        if (a.scale_out) v *= a.out_scale;
+        v = scale_result(a, v);
         if (a.yloc != nullptr) store_loc(a.yloc + (size_t)e0 * N3 + idx, v);
         else scatter_add(a.y + SEM_IDX(__ldg(gmap + idx), a.ndofs, a.dbg, kDbgScatter), v);
       }

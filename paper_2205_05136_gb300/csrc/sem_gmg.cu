@@ -37,9 +37,8 @@ namespace sem {
 // Separable p-transfers on the slab lattice (sem_transfer.cu); w1, w2 scratch of
 // p_transfer_scratch(F, C, 1) and (F, C, 2) entries.
 template <typename T>
-cudaError_t p_transfer(bool prolong, const Level& F, const Level& C, const double (*P)[kMaxN],
-                       const T* src_b, const T* src_t, T* dst, T* dst_t, T* w1, T* w2, const int* done,
-                       cudaStream_t s);
+cudaError_t p_transfer(bool prolong, const Level& F, const Level& C, const double (*P)[kMaxN], const T* src,
+                       T* dst, T* dst_d, T* w1, T* w2, const int* done, cudaStream_t s);
 size_t p_transfer_scratch(const Level& F, const Level& C, int which);
 
 struct GmgLevel {
@@ -48,7 +47,8 @@ struct GmgLevel {
   int to_next = 0;  // 0: p-transfer to the next level, 1: h-transfer
   double *sl = nullptr, *st = nullptr, *th = nullptr;
   bool owns_tissue = false;
-  void *b = nullptr, *x = nullptr, *t = nullptr, *d = nullptr, *invd = nullptr;
+  // residual (right-hand side at first), iterate, correction, 1 / diagonal
+  void *r = nullptr, *x = nullptr, *d = nullptr, *invd = nullptr;
   void *pw1 = nullptr, *pw2 = nullptr;  // p-transfer scratch towards the next level
   double* dinv64 = nullptr;
   double lam = 0.0;
@@ -171,70 +171,70 @@ __global__ void k_level_inv_diag(int64_t n, double alpha, const double* m, const
   pdl_trigger();
 }
 
-// Chebyshev step 0 from a zero start: d = D^{-1} b / theta, x = d, t = 0.
+// Chebyshev smoothing in residual form.  A level keeps the residual r of its
+// current iterate in place of the right-hand side (the apply subtracts A d from it),
+// so no vector t = A x is written, cleared and read back, and the restriction takes
+// r as it is: a step moves 6 vectors where b, t, x, d moved 8, the first two of a zero
+// start 8 instead of 13, the last one 5 (its d is not stored).  Fine-level vectors of
+// a V-cycle of degree 6 on 2.06 M nodes: 545 MB instead of 768.
+//
+// First step from zero: d = D^{-1} r / theta (x = d follows with the next step, or
+// here with with_x).
 template <typename T>
-__global__ void k_cheb_zero_start(int64_t n, const T* __restrict__ b, const T* __restrict__ invd,
-                                  T* __restrict__ x, T* __restrict__ d, T* __restrict__ t,
-                                  T inv_theta, const int* done) {
+__global__ void k_cheb_zero_start(int64_t n, const T* __restrict__ r, const T* __restrict__ invd,
+                                  T* __restrict__ x, T* __restrict__ d, T inv_theta, int with_x, const int* done) {
   pdl_wait();
   if (skip(done)) return;
   constexpr int K = k16<T>();
   using V = Pk<T, K>;
   const int64_t nc = n / K;
   GRID_CHUNKS(c, nc) {
-    const V bb = reinterpret_cast<const V*>(b)[c], ii = reinterpret_cast<const V*>(invd)[c];
+    const V rr = reinterpret_cast<const V*>(r)[c], ii = reinterpret_cast<const V*>(invd)[c];
     V dd;
 #pragma unroll
-    for (int k = 0; k < K; ++k) dd.e[k] = ii.e[k] * bb.e[k] * inv_theta;
+    for (int k = 0; k < K; ++k) dd.e[k] = ii.e[k] * rr.e[k] * inv_theta;
     reinterpret_cast<V*>(d)[c] = dd;
-    reinterpret_cast<V*>(x)[c] = dd;
-    reinterpret_cast<V*>(t)[c] = V{};
+    if (with_x) reinterpret_cast<V*>(x)[c] = dd;
   }
   GRID_TAIL(i, nc * K, n) {
-    const T di = invd[i] * b[i] * inv_theta;
+    const T di = invd[i] * r[i] * inv_theta;
     d[i] = di;
-    x[i] = di;
-    t[i] = T(0);
+    if (with_x) x[i] = di;
   }
   pdl_trigger();
 }
 
-// Chebyshev step with t = A x: d = c1 d + c2 D^{-1}(b - t), x += d, t = 0
-// (first: d = c2 D^{-1}(b - t)).
+// Chebyshev step from the residual r: d = c1 d + c2 D^{-1} r (kChebFirst: d = c2
+// D^{-1} r), x += d (kChebStartX: x = old d + d, the second step of a zero start);
+// kChebLast: d is not needed any more and not stored.
+constexpr int kChebFirst = 1, kChebStartX = 2, kChebLast = 4;
 template <typename T>
-__device__ __forceinline__ T cheb_d(T b, T t, T invd, T d, T c1, T c2, bool first) {
-  const T ri = b - t;
-  return first ? c2 * invd * ri : fma(c1, d, c2 * invd * ri);
-}
-
-template <typename T>
-__global__ void k_cheb_step(int64_t n, const T* __restrict__ b, const T* __restrict__ invd,
-                            T* __restrict__ x, T* __restrict__ d, T* __restrict__ t, T c1, T c2,
-                            int first, const int* done) {
+__global__ void k_cheb_step(int64_t n, const T* __restrict__ r, const T* __restrict__ invd,
+                            T* __restrict__ x, T* __restrict__ d, T c1, T c2, int mode, const int* done) {
   pdl_wait();
   if (skip(done)) return;
+  const bool first = (mode & kChebFirst) != 0, startx = (mode & kChebStartX) != 0, last = (mode & kChebLast) != 0;
   constexpr int K = k16<T>();
   using V = Pk<T, K>;
   const int64_t nc = n / K;
   GRID_CHUNKS(c, nc) {
-    const V bb = reinterpret_cast<const V*>(b)[c], tt = reinterpret_cast<const V*>(t)[c];
-    const V ii = reinterpret_cast<const V*>(invd)[c];
-    V xx = reinterpret_cast<const V*>(x)[c];
-    V dd = first ? V{} : reinterpret_cast<const V*>(d)[c];
+    const V rr = reinterpret_cast<const V*>(r)[c], ii = reinterpret_cast<const V*>(invd)[c];
+    const V od = first ? V{} : reinterpret_cast<const V*>(d)[c];
+    V xx = startx ? od : reinterpret_cast<const V*>(x)[c];
+    V dd;
 #pragma unroll
     for (int k = 0; k < K; ++k) {
-      dd.e[k] = cheb_d(bb.e[k], tt.e[k], ii.e[k], dd.e[k], c1, c2, first != 0);
+      dd.e[k] = first ? c2 * ii.e[k] * rr.e[k] : fma(c1, od.e[k], c2 * ii.e[k] * rr.e[k]);
       xx.e[k] += dd.e[k];
     }
-    reinterpret_cast<V*>(d)[c] = dd;
+    if (!last) reinterpret_cast<V*>(d)[c] = dd;
     reinterpret_cast<V*>(x)[c] = xx;
-    reinterpret_cast<V*>(t)[c] = V{};
   }
   GRID_TAIL(i, nc * K, n) {
-    const T di = cheb_d(b[i], t[i], invd[i], first ? T(0) : d[i], c1, c2, first != 0);
-    d[i] = di;
-    x[i] += di;
-    t[i] = T(0);
+    const T od = first ? T(0) : d[i];
+    const T di = first ? c2 * invd[i] * r[i] : fma(c1, od, c2 * invd[i] * r[i]);
+    if (!last) d[i] = di;
+    x[i] = (startx ? od : x[i]) + di;
   }
   pdl_trigger();
 }
@@ -259,7 +259,7 @@ __device__ __forceinline__ void hweights(int I, int nf, int nc, int& k, double& 
 
 template <typename T>
 __global__ void k_prolong_h(int nfx, int nfy, int nfz, int ncx, int ncy, int ncz,
-                            const T* __restrict__ xc, T* __restrict__ xf, T* __restrict__ tf,
+                            const T* __restrict__ xc, T* __restrict__ xf, T* __restrict__ df,
                             const int* done) {
   pdl_wait();
   if (skip(done)) return;
@@ -280,15 +280,14 @@ __global__ void k_prolong_h(int nfx, int nfy, int nfz, int ncx, int ncy, int ncz
           if (w != 0.0) s += (T)w * xc[(kx + a) + CX * ((ky + b) + CY * (kz + c))];
         }
     xf[g] += s;
-    tf[g] = T(0);
+    df[g] = s;
   }
   pdl_trigger();
 }
 
 template <typename T>
 __global__ void k_restrict_h(int nfx, int nfy, int nfz, int ncx, int ncy, int ncz,
-                             const T* __restrict__ bf, const T* __restrict__ tf,
-                             T* __restrict__ bc, const int* done) {
+                             const T* __restrict__ rf, T* __restrict__ bc, const int* done) {
   pdl_wait();
   if (skip(done)) return;
   const int64_t NX = nfx + 1, NY = nfy + 1, n = NX * NY * (nfz + 1);
@@ -300,7 +299,7 @@ __global__ void k_restrict_h(int nfx, int nfy, int nfz, int ncx, int ncy, int nc
     hweights(I, nfx, ncx, kx, wx[0], wx[1]);
     hweights(J, nfy, ncy, ky, wy[0], wy[1]);
     hweights(K, nfz, ncz, kz, wz[0], wz[1]);
-    const T r = bf[g] - tf[g];
+    const T r = rf[g];
     for (int c = 0; c < 2; ++c)
       for (int b = 0; b < 2; ++b)
         for (int a = 0; a < 2; ++a) {
@@ -316,8 +315,7 @@ __global__ void k_restrict_h(int nfx, int nfy, int nfz, int ncx, int ncy, int nc
 // trilinear prolongation's weight of that coarse node.
 template <typename T>
 __global__ void k_restrict_h_det(int nfx, int nfy, int nfz, int ncx, int ncy, int ncz,
-                                 const T* __restrict__ bf, const T* __restrict__ tf,
-                                 T* __restrict__ bc, const int* done) {
+                                 const T* __restrict__ rf, T* __restrict__ bc, const int* done) {
   pdl_wait();
   if (skip(done)) return;
   const int64_t NX = nfx + 1, NY = nfy + 1;
@@ -341,7 +339,7 @@ __global__ void k_restrict_h_det(int nfx, int nfy, int nfz, int ncx, int ncy, in
           const double wx = wt(I, nfx, ncx, CI);
           if (wx == 0.0) continue;
           const int64_t g = I + NX * (J + NY * (int64_t)K);
-          acc += (T)(wx * wy * wz) * (bf[g] - tf[g]);
+          acc += (T)(wx * wy * wz) * rf[g];
         }
       }
     }
@@ -953,29 +951,29 @@ double tridiag_max_eig(const std::vector<double>& a, const std::vector<double>& 
   return 0.5 * (lo + hi);
 }
 
-// y += (alpha M + K) x on one level in the V-cycle's precision.
-int level_apply(sem_ctx* ctx, const Level& L, int precision, double alpha, const void* x, void* y,
+// r -= (alpha M + K) d on one level in the V-cycle's precision.
+int level_apply(sem_ctx* ctx, const Level& L, int precision, double alpha, const void* d, void* r,
                 const int* done, cudaStream_t s) {
   cudaError_t e;
   // deterministic mode: element-local results and fixed-order node sums (scalar kernels)
   void* loc = ctx->deterministic ? ctx->det_scratch : nullptr;
   if (precision == SEM_PREC_FP64) {
     ApplyArgs64 a{};
-    a.map = L.map; a.metric = L.metric; a.u = (const double*)x; a.y = (double*)y;
-    a.nelem = L.nelem; a.mass_coef = alpha; a.out_scale = 1.0; a.scale_out = 0; a.done = done;
+    a.map = L.map; a.metric = L.metric; a.u = (const double*)d; a.y = (double*)r;
+    a.nelem = L.nelem; a.mass_coef = alpha; a.out_scale = -1.0; a.scale_out = kNegateOut; a.done = done;
     a.yloc = (double*)loc;
     e = launch_apply_fp64(L, a, false, s);
   } else if (precision == SEM_PREC_FP32_BF16 || precision == SEM_PREC_BF16_TC) {
     ApplyArgs<float, __nv_bfloat16> a{};
-    a.map = L.map; a.metric = L.metric16; a.u = (const float*)x; a.y = (float*)y;
-    a.nelem = L.nelem; a.mass_coef = (float)alpha; a.out_scale = 1.f; a.scale_out = 0; a.done = done;
+    a.map = L.map; a.metric = L.metric16; a.u = (const float*)d; a.y = (float*)r;
+    a.nelem = L.nelem; a.mass_coef = (float)alpha; a.out_scale = -1.f; a.scale_out = kNegateOut; a.done = done;
     a.yloc = (float*)loc;
     e = (precision == SEM_PREC_BF16_TC && tc_supported(L) && loc == nullptr) ? launch_apply_tc(L, a, s)
                                                                              : launch_apply_bf16(L, a, false, s);
   } else {
     ApplyArgs<float, float> a{};
-    a.map = L.map; a.metric = L.metric32; a.u = (const float*)x; a.y = (float*)y;
-    a.nelem = L.nelem; a.mass_coef = (float)alpha; a.out_scale = 1.f; a.scale_out = 0; a.done = done;
+    a.map = L.map; a.metric = L.metric32; a.u = (const float*)d; a.y = (float*)r;
+    a.nelem = L.nelem; a.mass_coef = (float)alpha; a.out_scale = -1.f; a.scale_out = kNegateOut; a.done = done;
     a.yloc = (float*)loc;
     e = launch_apply_fp32(L, a, false, s);
   }
@@ -1011,47 +1009,44 @@ PTab make_ptab(const Level& fine, const Level& coarse) {
   return t;
 }
 
-// Restrict (b_l - t_l) into b_{l+1}.
+// Restrict r_l into r_{l+1}.
 template <typename T>
 int restrict_to(sem_ctx* ctx, Gmg& g, int l, const int* done, cudaStream_t s) {
   GmgLevel& F = g.lv[l];
   GmgLevel& C = g.lv[l + 1];
-  if (F.to_next == 0) {  // three passes that write b_{l+1}
+  if (F.to_next == 0) {  // three passes that write r_{l+1}
     const PTab tab = make_ptab(*F.L, *C.L);
-    GMG_CK(p_transfer<T>(false, *F.L, *C.L, tab.P, (const T*)F.b, (const T*)F.t, (T*)C.b, nullptr,
-                         (T*)F.pw1, (T*)F.pw2, done, s));
+    GMG_CK(p_transfer<T>(false, *F.L, *C.L, tab.P, (const T*)F.r, (T*)C.r, nullptr, (T*)F.pw1, (T*)F.pw2, done, s));
     ctx->launches += 3;
     return SEM_OK;
   }
-  launch_k(k_zero<T>, grid_chunks<T>(C.L->ndofs), kThreads, 0, s, C.L->ndofs, (T*)C.b, done);
+  launch_k(k_zero<T>, grid_chunks<T>(C.L->ndofs), kThreads, 0, s, C.L->ndofs, (T*)C.r, done);
   T* loc = ctx->deterministic ? reinterpret_cast<T*>(ctx->det_scratch) : nullptr;
   if (loc != nullptr) {
     launch_k(k_restrict_h_det<T>, grid1d(C.L->ndofs), kThreads, 0, s,
-        F.L->nx, F.L->ny, F.L->nz, C.L->nx, C.L->ny, C.L->nz, (const T*)F.b, (const T*)F.t,
-        (T*)C.b, done);
+        F.L->nx, F.L->ny, F.L->nz, C.L->nx, C.L->ny, C.L->nz, (const T*)F.r, (T*)C.r, done);
   } else {
     launch_k(k_restrict_h<T>, grid1d(F.L->ndofs), kThreads, 0, s,
-        F.L->nx, F.L->ny, F.L->nz, C.L->nx, C.L->ny, C.L->nz, (const T*)F.b, (const T*)F.t,
-        (T*)C.b, done);
+        F.L->nx, F.L->ny, F.L->nz, C.L->nx, C.L->ny, C.L->nz, (const T*)F.r, (T*)C.r, done);
   }
   GMG_CK(cudaGetLastError());
   ctx->launches += 2;
   return SEM_OK;
 }
 
+// d_l = P x_{l+1}, x_l += d_l.
 template <typename T>
 int prolong_from(sem_ctx* ctx, Gmg& g, int l, const int* done, cudaStream_t s) {
   GmgLevel& F = g.lv[l];
   GmgLevel& C = g.lv[l + 1];
   if (F.to_next == 0) {
     const PTab tab = make_ptab(*F.L, *C.L);
-    GMG_CK(p_transfer<T>(true, *F.L, *C.L, tab.P, (const T*)C.x, nullptr, (T*)F.x, (T*)F.t, (T*)F.pw1,
-                         (T*)F.pw2, done, s));
+    GMG_CK(p_transfer<T>(true, *F.L, *C.L, tab.P, (const T*)C.x, (T*)F.x, (T*)F.d, (T*)F.pw1, (T*)F.pw2, done, s));
     ctx->launches += 3;
     return SEM_OK;
   } else {
     launch_k(k_prolong_h<T>, grid1d(F.L->ndofs), kThreads, 0, s,
-        F.L->nx, F.L->ny, F.L->nz, C.L->nx, C.L->ny, C.L->nz, (const T*)C.x, (T*)F.x, (T*)F.t,
+        F.L->nx, F.L->ny, F.L->nz, C.L->nx, C.L->ny, C.L->nz, (const T*)C.x, (T*)F.x, (T*)F.d,
         done);
   }
   GMG_CK(cudaGetLastError());
@@ -1059,10 +1054,11 @@ int prolong_from(sem_ctx* ctx, Gmg& g, int l, const int* done, cudaStream_t s) {
   return SEM_OK;
 }
 
-// `degree` Chebyshev steps on level l for A x = b (zero start, or from the current x
-// with t = 0).
+// `degree` Chebyshev steps on level l: from a zero start with r the right-hand side,
+// or from the current x with r the residual before its last correction d.  On exit r
+// is the residual before the last correction, which is in d when keep_d.
 template <typename T>
-int chebyshev(sem_ctx* ctx, Gmg& g, int l, int degree, bool zero_start, const int* done,
+int chebyshev(sem_ctx* ctx, Gmg& g, int l, int degree, bool zero_start, bool keep_d, const int* done,
               cudaStream_t s) {
   GmgLevel& V = g.lv[l];
   const Level& L = *V.L;
@@ -1070,24 +1066,26 @@ int chebyshev(sem_ctx* ctx, Gmg& g, int l, int degree, bool zero_start, const in
   const double lo = 0.08 * V.lam, hi = 1.2 * V.lam;
   const double theta = 0.5 * (hi + lo), delta = 0.5 * (hi - lo), sigma = theta / delta;
   double rho_old = 1.0 / sigma;
-  T* b = (T*)V.b; T* x = (T*)V.x; T* t = (T*)V.t; T* d = (T*)V.d; const T* invd = (const T*)V.invd;
+  T* r = (T*)V.r; T* x = (T*)V.x; T* d = (T*)V.d; const T* invd = (const T*)V.invd;
   int k0 = 0;
   if (zero_start) {
-    launch_k(k_cheb_zero_start<T>, grid_chunks<T>(n), kThreads, 0, s, n, b, invd, x, d, t, (T)(1.0 / theta), done);
+    launch_k(k_cheb_zero_start<T>, grid_chunks<T>(n), kThreads, 0, s, n, r, invd, x, d, (T)(1.0 / theta),
+             degree == 1 ? 1 : 0, done);
     GMG_CK(cudaGetLastError());
     ctx->launches += 1;
     k0 = 1;
   }
   for (int k = k0; k < degree; ++k) {
-    int rc = level_apply(ctx, L, g.precision, g.alpha, x, t, done, s);
+    int rc = level_apply(ctx, L, g.precision, g.alpha, d, r, done, s);
     if (rc != SEM_OK) return rc;
+    const int last = (k == degree - 1 && !keep_d) ? kChebLast : 0;
     if (k == 0) {
-      launch_k(k_cheb_step<T>, grid_chunks<T>(n), kThreads, 0, s, n, b, invd, x, d, t, (T)0, (T)(1.0 / theta), 1,
-                                                           done);
+      launch_k(k_cheb_step<T>, grid_chunks<T>(n), kThreads, 0, s, n, r, invd, x, d, (T)0, (T)(1.0 / theta),
+               kChebFirst | last, done);
     } else {
       const double rho = 1.0 / (2.0 * sigma - rho_old);
-      launch_k(k_cheb_step<T>, grid_chunks<T>(n), kThreads, 0, s, n, b, invd, x, d, t, (T)(rho * rho_old),
-                                                           (T)(2.0 * rho / delta), 0, done);
+      launch_k(k_cheb_step<T>, grid_chunks<T>(n), kThreads, 0, s, n, r, invd, x, d, (T)(rho * rho_old),
+               (T)(2.0 * rho / delta), (zero_start && k == 1 ? kChebStartX : 0) | last, done);
       rho_old = rho;
     }
     GMG_CK(cudaGetLastError());
@@ -1100,18 +1098,18 @@ template <typename T>
 int vcycle_level(sem_ctx* ctx, Gmg& g, int l, const int* done, cudaStream_t s, bool record) {
   const int last = (int)g.lv.size() - 1;
   int rc;
-  if (l == last) return chebyshev<T>(ctx, g, l, g.coarse_degree, true, done, s);
-  if ((rc = chebyshev<T>(ctx, g, l, g.degree, true, done, s)) != SEM_OK) return rc;
+  if (l == last) return chebyshev<T>(ctx, g, l, g.coarse_degree, true, false, done, s);
+  if ((rc = chebyshev<T>(ctx, g, l, g.degree, true, true, done, s)) != SEM_OK) return rc;
   GmgLevel& V = g.lv[l];
-  // t = A x (t is zero after the smoother), then b_{l+1} = R (b - t)
+  // r -= A d: the residual of x, then r_{l+1} = R r
   // the fine-level residual apply is bracketed by event nodes when `record`
   if (record && l == 0) GMG_CK(cudaEventRecordWithFlags(g.ev2, s, cudaEventRecordExternal));
-  if ((rc = level_apply(ctx, *V.L, g.precision, g.alpha, V.x, V.t, done, s)) != SEM_OK) return rc;
+  if ((rc = level_apply(ctx, *V.L, g.precision, g.alpha, V.d, V.r, done, s)) != SEM_OK) return rc;
   if (record && l == 0) GMG_CK(cudaEventRecordWithFlags(g.ev3, s, cudaEventRecordExternal));
   if ((rc = restrict_to<T>(ctx, g, l, done, s)) != SEM_OK) return rc;
   if ((rc = vcycle_level<T>(ctx, g, l + 1, done, s, false)) != SEM_OK) return rc;
-  if ((rc = prolong_from<T>(ctx, g, l, done, s)) != SEM_OK) return rc;  // also clears t
-  return chebyshev<T>(ctx, g, l, g.degree, false, done, s);
+  if ((rc = prolong_from<T>(ctx, g, l, done, s)) != SEM_OK) return rc;
+  return chebyshev<T>(ctx, g, l, g.degree, false, false, done, s);
 }
 
 int vcycle(sem_ctx* ctx, Gmg& g, const int* done, cudaStream_t s, bool record = false) {
@@ -1200,7 +1198,7 @@ void free_gmg_struct(Gmg* g) {
     if (V.owns_tissue) {
       cudaFree(V.sl); cudaFree(V.st); cudaFree(V.th);
     }
-    cudaFree(V.b); cudaFree(V.x); cudaFree(V.t); cudaFree(V.d); cudaFree(V.invd);
+    cudaFree(V.r); cudaFree(V.x); cudaFree(V.d); cudaFree(V.invd);
     cudaFree(V.pw1); cudaFree(V.pw2);
     cudaFree(V.dinv64);
   }
@@ -1313,9 +1311,8 @@ int build(sem_ctx* ctx, cudaStream_t s) {
       GMG_CK(setup_metric_lowp(L, true, s));
     }
     if (tc && !L.metric_tc_valid) GMG_CK(setup_metric_tc(L, s));
-    void** vecs[] = {&V.b, &V.x, &V.t, &V.d, &V.invd};
+    void** vecs[] = {&V.r, &V.x, &V.d, &V.invd};
     for (void** v : vecs) GMG_CK(cudaMalloc(v, es * L.ndofs));
-    GMG_CK(cudaMemsetAsync(V.t, 0, es * L.ndofs, s));
     GMG_CK(cudaMalloc(&V.dinv64, sizeof(double) * L.ndofs));
   }
   for (size_t l = 0; l + 1 < g->lv.size(); ++l) {
@@ -1375,7 +1372,7 @@ int pcg_init_seq(sem_ctx* ctx, Gmg& g, double alpha, const double* b, const doub
   Level& L = ctx->L;
   const int64_t n = L.ndofs;
   const int gr = grid1d(n);
-  T* b0 = (T*)g.lv[0].b;
+  T* b0 = (T*)g.lv[0].r;
   const int stride = g.partial_len;
   if (!carried || checked != nullptr) {
     launch_k(k_zero<double>, gr, kThreads, 0, s, n, w.Ap, checked);
@@ -1437,12 +1434,12 @@ int pcg_iter_seq(sem_ctx* ctx, Gmg& g, double alpha, double* x, bool timed, cuda
   if (timed) GMG_CK(cudaEventRecordWithFlags(g.ev1, s, cudaEventRecordExternal));
   if (dfop)
     launch_k(aligned16(x) ? k_dfpcg_xr<T, true> : k_dfpcg_xr<T, false>, std::min(gr, 152 * kXrCtasPerSm),
-             kThreads, 0, s, n, x, p2, w.Ap, r2, (T*)g.lv[0].b, w.cg, g.partials, stride, g.tickets + 2);
+             kThreads, 0, s, n, x, p2, w.Ap, r2, (T*)g.lv[0].r, w.cg, g.partials, stride, g.tickets + 2);
   else if (aligned16(x))
-    launch_k(k_fpcg_xr<T, true>, gr, kThreads, 0, s, n, x, w.p, w.Ap, w.r, (T*)g.lv[0].b, w.cg, g.partials,
+    launch_k(k_fpcg_xr<T, true>, gr, kThreads, 0, s, n, x, w.p, w.Ap, w.r, (T*)g.lv[0].r, w.cg, g.partials,
                                              stride, g.tickets + 2);
   else
-    launch_k(k_fpcg_xr<T, false>, gr, kThreads, 0, s, n, x, w.p, w.Ap, w.r, (T*)g.lv[0].b, w.cg, g.partials,
+    launch_k(k_fpcg_xr<T, false>, gr, kThreads, 0, s, n, x, w.p, w.Ap, w.r, (T*)g.lv[0].r, w.cg, g.partials,
                                               stride, g.tickets + 2);
   GMG_CK(cudaGetLastError());
   return SEM_OK;
@@ -1657,9 +1654,9 @@ int gmg_vcycle(sem_ctx* ctx, double alpha, const double* r, double* z, cudaStrea
   if ((rc = set_alpha(ctx, g, alpha, s)) != SEM_OK) return rc;
   const int64_t n = ctx->L.ndofs;
   if (g.precision == SEM_PREC_FP64)
-    launch_k(k_to_level0<double>, grid1d(n), kThreads, 0, s, n, r, (double*)g.lv[0].b);
+    launch_k(k_to_level0<double>, grid1d(n), kThreads, 0, s, n, r, (double*)g.lv[0].r);
   else
-    launch_k(k_to_level0<float>, grid1d(n), kThreads, 0, s, n, r, (float*)g.lv[0].b);
+    launch_k(k_to_level0<float>, grid1d(n), kThreads, 0, s, n, r, (float*)g.lv[0].r);
   GMG_CK(cudaGetLastError());
   if ((rc = vcycle(ctx, g, nullptr, s)) != SEM_OK) return rc;
   if (g.precision == SEM_PREC_FP64)

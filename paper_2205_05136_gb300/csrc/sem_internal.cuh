@@ -245,6 +245,8 @@ inline size_t metric_lowp_count(const Level& L) {
   return units * ML::chunks(L.n) * ML::chunk(L.n);
 }
 
+constexpr int kScaleOut = 1, kNegateOut = 2;  // ApplyArgs::scale_out
+
 // Arguments of the element kernel y += A_e u_e (scatter-add into y).
 template <typename T, typename MT>
 struct ApplyArgs {
@@ -255,7 +257,7 @@ struct ApplyArgs {
   int nelem;
   T mass_coef;        // coefficient of the mass term inside the element kernel
   T out_scale;        // factor applied to the element result before the scatter
-  int scale_out;      // out_scale != 1
+  int scale_out;      // 0: out_scale is 1; kScaleOut; kNegateOut: it is -1
   const int* done;    // optional: skip all work when *done != 0
   // optional fused u . (A u) (CG's p . A p): every CTA writes its partial sum
   // to dot_partials (one double per CTA of the launch) and a one-CTA kernel

@@ -7,9 +7,9 @@
 // P[i][a] = l^c_a(x^f_i) the 1-D interpolation matrix.  A node on an element
 // boundary gets the same value from either element, because the interpolation
 // is exact at the shared end points (rows 0 and pf of P are unit rows).  So
-//   prolongation  x_f += P x_c, t_f = 0: three 1-D passes, coarse lattice ->
+//   prolongation  d_f = P x_c, x_f += d_f: three 1-D passes, coarse lattice ->
 //                 (NXc, NYc, NZf) -> (NXc, NYf, NZf) -> fine lattice;
-//   restriction   b_c = P^T (b_f - t_f): three 1-D passes the other way,
+//   restriction   r_c = P^T r_f: three 1-D passes the other way,
 //                 coarse node A summing P1[I][A] over the fine nodes I of the
 //                 elements that hold it, each fine node once.
 // Each pass is one thread per output node reading a short run along one
@@ -33,18 +33,16 @@ struct PMat {
   T P[NF][NC];
 };
 
-enum { kProlong = 0, kProlongAdd = 1, kRestrict = 2, kRestrictDiff = 3 };
+enum { kProlong = 0, kProlongAdd = 1, kRestrict = 2 };
 constexpr int kPassX = 32, kPassY = kTThreads / kPassX;  // CTA of a pass: 32 x 8 output nodes
 
 // One 1-D pass along lattice axis AX (0 x, 1 y, 2 z) between degree pf = NF - 1
 // and pc = NC - 1 on ne elements along that axis.  Output lattice d[0..2]; the
 // input lattice is the same except along AX.
-//   kProlong:      out = P in;           kProlongAdd:   out += P in, out2 = 0;
-//   kRestrict:     out = P^T in;         kRestrictDiff: out = P^T (in - in2).
+//   kProlong: out = P in;   kProlongAdd: out2 = P in, out += out2;   kRestrict: out = P^T in.
 template <int NF, int NC, int AX, int MODE, typename T>
 __global__ void __launch_bounds__(kTThreads)
-    k_ptransfer_pass(int ne, int d0, int d1, int d2, const T* __restrict__ in, const T* __restrict__ in2,
-                     T* __restrict__ out, T* __restrict__ out2, const __grid_constant__ PMat<NF, NC, T> pm,
+    k_ptransfer_pass(int ne, int d0, int d1, int d2, const T* __restrict__ in, T* __restrict__ out, T* __restrict__ out2, const __grid_constant__ PMat<NF, NC, T> pm,
                      const int* done) {
   pdl_wait();
   if (done != nullptr && *done) return;
@@ -73,14 +71,13 @@ __global__ void __launch_bounds__(kTThreads)
       for (int a = 0; a < NC; ++a) acc = fma(pm.P[i][a], src[a * stride], acc);
       if constexpr (MODE == kProlongAdd) {
         out[o] += acc;
-        out2[o] = T(0);
+        out2[o] = acc;
       } else {
         out[o] = acc;
       }
     } else {
       auto val = [&](int I) {
-        const int64_t k = base + (int64_t)I * stride;
-        return MODE == kRestrictDiff ? in[k] - in2[k] : in[k];
+        return in[base + (int64_t)I * stride];
       };
       const int e = min(q / PC, ne - 1), a = q - PC * e;
 #pragma unroll
@@ -105,7 +102,7 @@ dim3 pass_grid(int d0, int d1, int d2) {
 
 template <int NF, int NC, typename T>
 cudaError_t launch_passes(bool prolong, const Level& F, const Level& C, const double (*P)[kMaxN],
-                          const T* src_b, const T* src_t, T* dst, T* dst_t, T* w1, T* w2,
+                          const T* src, T* dst, T* dst_d, T* w1, T* w2,
                           const int* done, cudaStream_t s) {
   PMat<NF, NC, T> pm;
   for (int i = 0; i < NF; ++i)
@@ -117,38 +114,38 @@ cudaError_t launch_passes(bool prolong, const Level& F, const Level& C, const do
   cudaError_t e;
   if (prolong) {  // coarse -> (xc, yc, zf) -> (xc, yf, zf) -> fine
     e = launch_k(k_ptransfer_pass<NF, NC, 2, kProlong, T>, pass_grid(xc, yc, zf), dim3(kPassX, kPassY), 0, s,
-                 nz, xc, yc, zf, src_b, nullptr, w2, nullptr, pm, done);
+                 nz, xc, yc, zf, src, w2, nullptr, pm, done);
     if (e == cudaSuccess)
       e = launch_k(k_ptransfer_pass<NF, NC, 1, kProlong, T>, pass_grid(xc, yf, zf), dim3(kPassX, kPassY), 0,
-                   s, ny, xc, yf, zf, w2, nullptr, w1, nullptr, pm, done);
+                   s, ny, xc, yf, zf, w2, w1, nullptr, pm, done);
     if (e == cudaSuccess)
       e = launch_k(k_ptransfer_pass<NF, NC, 0, kProlongAdd, T>, pass_grid(xf, yf, zf), dim3(kPassX, kPassY),
-                   0, s, nx, xf, yf, zf, w1, nullptr, dst, dst_t, pm, done);
+                   0, s, nx, xf, yf, zf, w1, dst, dst_d, pm, done);
   } else {  // fine -> (xc, yf, zf) -> (xc, yc, zf) -> coarse
-    e = launch_k(k_ptransfer_pass<NF, NC, 0, kRestrictDiff, T>, pass_grid(xc, yf, zf), dim3(kPassX, kPassY),
-                 0, s, nx, xc, yf, zf, src_b, src_t, w1, nullptr, pm, done);
+    e = launch_k(k_ptransfer_pass<NF, NC, 0, kRestrict, T>, pass_grid(xc, yf, zf), dim3(kPassX, kPassY),
+                 0, s, nx, xc, yf, zf, src, w1, nullptr, pm, done);
     if (e == cudaSuccess)
       e = launch_k(k_ptransfer_pass<NF, NC, 1, kRestrict, T>, pass_grid(xc, yc, zf), dim3(kPassX, kPassY), 0,
-                   s, ny, xc, yc, zf, w1, nullptr, w2, nullptr, pm, done);
+                   s, ny, xc, yc, zf, w1, w2, nullptr, pm, done);
     if (e == cudaSuccess)
       e = launch_k(k_ptransfer_pass<NF, NC, 2, kRestrict, T>, pass_grid(xc, yc, zc), dim3(kPassX, kPassY), 0,
-                   s, nz, xc, yc, zc, w2, nullptr, dst, nullptr, pm, done);
+                   s, nz, xc, yc, zc, w2, dst, nullptr, pm, done);
   }
   return e;
 }
 
 }  // namespace
 
-// prolong: dst (fine x) += P src_b (coarse x), dst_t (fine t) cleared.
-// restrict: dst (coarse b) = P^T (src_b - src_t) (fine b, fine t).
+// prolong: dst_d (fine d) = P src (coarse x), dst (fine x) += dst_d.
+// restrict: dst (coarse r) = P^T src (fine r).
 // w1, w2: scratch of (NXc NYf NZf) and (NXc NYc NZf) entries.
 template <typename T>
 cudaError_t p_transfer(bool prolong, const Level& F, const Level& C, const double (*P)[kMaxN],
-                       const T* src_b, const T* src_t, T* dst, T* dst_t, T* w1, T* w2, const int* done,
+                       const T* src, T* dst, T* dst_d, T* w1, T* w2, const int* done,
                        cudaStream_t s) {
   const int nf = F.n, nc = C.n;
 #define SEM_PAIR(A, B) \
-  if (nf == A && nc == B) return launch_passes<A, B, T>(prolong, F, C, P, src_b, src_t, dst, dst_t, w1, w2, done, s);
+  if (nf == A && nc == B) return launch_passes<A, B, T>(prolong, F, C, P, src, dst, dst_d, w1, w2, done, s);
   SEM_PAIR(7, 4)
   SEM_PAIR(6, 3)
   SEM_PAIR(5, 3)
@@ -169,10 +166,10 @@ size_t p_transfer_scratch(const Level& F, const Level& C, int which) {
 }
 
 template cudaError_t p_transfer<float>(bool, const Level&, const Level&, const double (*)[kMaxN],
-                                       const float*, const float*, float*, float*, float*, float*,
-                                       const int*, cudaStream_t);
+                                       const float*, float*, float*, float*, float*, const int*,
+                                       cudaStream_t);
 template cudaError_t p_transfer<double>(bool, const Level&, const Level&, const double (*)[kMaxN],
-                                        const double*, const double*, double*, double*, double*, double*,
-                                        const int*, cudaStream_t);
+                                        const double*, double*, double*, double*, double*, const int*,
+                                        cudaStream_t);
 
 }  // namespace sem
