@@ -34,12 +34,10 @@
 
 namespace sem {
 
-// Separable p-transfers on the slab lattice (sem_transfer.cu); w1, w2 scratch of
-// p_transfer_scratch(F, C, 1) and (F, C, 2) entries.
+// p-transfers on the slab lattice (sem_transfer.cu).
 template <typename T>
-cudaError_t p_transfer(bool prolong, const Level& F, const Level& C, const double (*P)[kMaxN], const T* src,
-                       T* dst, T* dst_d, T* w1, T* w2, const int* done, cudaStream_t s);
-size_t p_transfer_scratch(const Level& F, const Level& C, int which);
+cudaError_t p_transfer(bool prolong, const Level& F, const Level& C, const double (*P)[kMaxN], const T* src, T* dst,
+                       T* dst_d, const int* done, cudaStream_t s);
 
 struct GmgLevel {
   Level* L = nullptr;
@@ -49,7 +47,6 @@ struct GmgLevel {
   bool owns_tissue = false;
   // residual (right-hand side at first), iterate, correction, 1 / diagonal
   void *r = nullptr, *x = nullptr, *d = nullptr, *invd = nullptr;
-  void *pw1 = nullptr, *pw2 = nullptr;  // p-transfer scratch towards the next level
   double* dinv64 = nullptr;
   double lam = 0.0;
 };
@@ -1014,10 +1011,10 @@ template <typename T>
 int restrict_to(sem_ctx* ctx, Gmg& g, int l, const int* done, cudaStream_t s) {
   GmgLevel& F = g.lv[l];
   GmgLevel& C = g.lv[l + 1];
-  if (F.to_next == 0) {  // three passes that write r_{l+1}
+  if (F.to_next == 0) {
     const PTab tab = make_ptab(*F.L, *C.L);
-    GMG_CK(p_transfer<T>(false, *F.L, *C.L, tab.P, (const T*)F.r, (T*)C.r, nullptr, (T*)F.pw1, (T*)F.pw2, done, s));
-    ctx->launches += 3;
+    GMG_CK(p_transfer<T>(false, *F.L, *C.L, tab.P, (const T*)F.r, (T*)C.r, nullptr, done, s));
+    ctx->launches += 1;
     return SEM_OK;
   }
   launch_k(k_zero<T>, grid_chunks<T>(C.L->ndofs), kThreads, 0, s, C.L->ndofs, (T*)C.r, done);
@@ -1041,8 +1038,8 @@ int prolong_from(sem_ctx* ctx, Gmg& g, int l, const int* done, cudaStream_t s) {
   GmgLevel& C = g.lv[l + 1];
   if (F.to_next == 0) {
     const PTab tab = make_ptab(*F.L, *C.L);
-    GMG_CK(p_transfer<T>(true, *F.L, *C.L, tab.P, (const T*)C.x, (T*)F.x, (T*)F.d, (T*)F.pw1, (T*)F.pw2, done, s));
-    ctx->launches += 3;
+    GMG_CK(p_transfer<T>(true, *F.L, *C.L, tab.P, (const T*)C.x, (T*)F.x, (T*)F.d, done, s));
+    ctx->launches += 1;
     return SEM_OK;
   } else {
     launch_k(k_prolong_h<T>, grid1d(F.L->ndofs), kThreads, 0, s,
@@ -1199,7 +1196,6 @@ void free_gmg_struct(Gmg* g) {
       cudaFree(V.sl); cudaFree(V.st); cudaFree(V.th);
     }
     cudaFree(V.r); cudaFree(V.x); cudaFree(V.d); cudaFree(V.invd);
-    cudaFree(V.pw1); cudaFree(V.pw2);
     cudaFree(V.dinv64);
   }
   cudaFree(g->z);
@@ -1314,12 +1310,6 @@ int build(sem_ctx* ctx, cudaStream_t s) {
     void** vecs[] = {&V.r, &V.x, &V.d, &V.invd};
     for (void** v : vecs) GMG_CK(cudaMalloc(v, es * L.ndofs));
     GMG_CK(cudaMalloc(&V.dinv64, sizeof(double) * L.ndofs));
-  }
-  for (size_t l = 0; l + 1 < g->lv.size(); ++l) {
-    GmgLevel& V = g->lv[l];
-    if (V.to_next != 0) continue;
-    GMG_CK(cudaMalloc(&V.pw1, es * p_transfer_scratch(*V.L, *g->lv[l + 1].L, 1)));
-    GMG_CK(cudaMalloc(&V.pw2, es * p_transfer_scratch(*V.L, *g->lv[l + 1].L, 2)));
   }
   const int64_t nf = ctx->L.ndofs;
   GMG_CK(cudaMalloc(&g->z, sizeof(double) * nf));
