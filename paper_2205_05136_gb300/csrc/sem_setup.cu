@@ -4,14 +4,13 @@
 //
 // Metric (Section 4: "the Jacobian of the transformation ... is cached";
 // Section 4.2: D evaluated at every quadrature point, Eq. diffusiontensor):
-//   J[d][c] = dx_d / dxi_c at each quadrature point, obtained by
-//   differentiating the element's nodal coordinate field (SEM-NI: D on the
-//   GLL nodes; SEM: interpolate to the Gauss points, then the Gauss
-//   collocation derivative),
+//   J[d][c] = dx_d / dxi_c at each quadrature point, the derivative of the
+//   element's trilinear map,
 //   D_e = sigma_t I + (sigma_l - sigma_t) f f^T,  f = (cos theta, sin theta, 0),
 //   G   = w |det J| J^{-1} D_e J^{-T}  (6 entries),  W = w |det J|.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 #include "sem_internal.cuh"
@@ -22,20 +21,19 @@ namespace {
 struct SetupTab {
   int n;
   double xg[kMaxN];          // LGL nodes
+  double xq[kMaxN];          // quadrature nodes
   double wq[kMaxN];          // quadrature weights
   double Bq[kMaxN][kMaxN];   // GLL basis at the quadrature points (identity for SEM-NI)
   double Dq[kMaxN][kMaxN];   // derivative of the GLL basis at the quadrature points
-  double Dc[kMaxN][kMaxN];   // collocation derivative on the quadrature points
 };
 
 SetupTab make_setup_tab(const Tables1D& t) {
   SetupTab s{};
   s.n = t.n;
-  for (int i = 0; i < t.n; ++i) { s.xg[i] = t.xg[i]; s.wq[i] = t.wq[i]; }
+  for (int i = 0; i < t.n; ++i) { s.xg[i] = t.xg[i]; s.xq[i] = t.xq[i]; s.wq[i] = t.wq[i]; }
   for (int q = 0; q < t.n; ++q)
     for (int l = 0; l < t.n; ++l) {
       s.Bq[q][l] = t.Bi[q][l];
-      s.Dc[q][l] = t.Dg[q][l];
       double d = 0.0;
       if (t.quad == SEM_QUAD_LGL) {
         d = t.D[q][l];
@@ -59,104 +57,95 @@ __device__ __forceinline__ double trilinear(const double (*V)[3], int d, double 
   return acc;
 }
 
-// One CTA per element.
-__global__ void k_metric(int nelem, const double* __restrict__ evert,
-                         const double* __restrict__ sigma_l, const double* __restrict__ sigma_t,
-                         const double* __restrict__ theta, const __grid_constant__ SetupTab tab,
-                         int lg, double* __restrict__ metric, int* bad) {
-  const int e = blockIdx.x;
-  if (e >= nelem) return;
-  const int n = tab.n, n2 = n * n, n3 = n2 * n;
-  __shared__ double V[8][3];
-  __shared__ double X[3][kMaxN * kMaxN * kMaxN];
-  __shared__ double Y[3][kMaxN * kMaxN * kMaxN];
-  if (threadIdx.x < 24) V[threadIdx.x / 3][threadIdx.x % 3] = evert[(size_t)e * 24 + threadIdx.x];
-  __syncthreads();
-  for (int a = threadIdx.x; a < n3; a += blockDim.x) {
-    const int i = a % n, j = (a / n) % n, k = a / n2;
-    for (int d = 0; d < 3; ++d) X[d][a] = trilinear(V, d, tab.xg[i], tab.xg[j], tab.xg[k]);
+constexpr int kSetupThreads = 256;
+// Elements of a CTA of the metric and diagonal kernels: about four points a thread.
+__host__ __device__ constexpr int setup_elems(int n3) { return n3 < 1024 ? 1024 / n3 : 1; }
+
+// Metric of E elements per CTA, one quadrature point a thread and turn.  The trilinear
+// map x_d = c0 + c1 xi + c2 eta + c3 zeta + c4 xi eta + c5 eta zeta + c6 xi zeta +
+// c7 xi eta zeta is kept by its coefficients, so a column of J takes three
+// multiply-adds an entry; with A = adj J = det J J^{-1} (rows the cross products of
+// J's columns), G = w / det A D_e A^T takes one division.  About 100 FP64 operations a
+// point, which bound the kernel (2 a clock and SM); differentiating the nodal
+// coordinates and dividing nine entries took about 400 (2.0 ms on 15,410 elements at
+// p = 5, now 0.56 ms).
+template <int N>
+__global__ void __launch_bounds__(kSetupThreads)
+    k_metric(int nelem, const double* __restrict__ evert, const double* __restrict__ sigma_l,
+             const double* __restrict__ sigma_t, const double* __restrict__ theta,
+             const __grid_constant__ SetupTab tab, double* __restrict__ metric, int* bad) {
+  constexpr int N2 = N * N, N3 = N2 * N, E = setup_elems(N3), N3P = padded_n3(N);
+  __shared__ double coef[E][3][8];
+  __shared__ double tens[E][4];  // sigma_t, sigma_l - sigma_t, cos theta, sin theta
+  __shared__ double xq[N], wq[N];
+  const int e0 = blockIdx.x * E, ne = min(E, nelem - e0);
+  if (threadIdx.x < N) {
+    xq[threadIdx.x] = tab.xq[threadIdx.x];
+    wq[threadIdx.x] = tab.wq[threadIdx.x];
+  }
+  for (int t = threadIdx.x; t < ne * 3; t += kSetupThreads) {
+    const int el = t / 3, d = t - 3 * el;
+    const double* v = evert + (size_t)(e0 + el) * 24 + d;
+    double x[8];
+    for (int i = 0; i < 8; ++i) x[i] = v[3 * i];
+    // sums and differences over the corners' bits (1: xi, 2: eta, 4: zeta)
+    for (int bit = 1; bit < 8; bit <<= 1)
+      for (int i = 0; i < 8; ++i)
+        if (!(i & bit)) {
+          const double lo = x[i], hi = x[i | bit];
+          x[i] = 0.5 * (hi + lo);
+          x[i | bit] = 0.5 * (hi - lo);
+        }
+    for (int i = 0; i < 8; ++i) coef[el][d][i] = x[i];
+  }
+  for (int el = threadIdx.x; el < ne; el += kSetupThreads) {
+    const double st = sigma_t[e0 + el], th = theta[e0 + el];
+    tens[el][0] = st;
+    tens[el][1] = sigma_l[e0 + el] - st;
+    tens[el][2] = cos(th);
+    tens[el][3] = sin(th);
   }
   __syncthreads();
-  if (lg) {  // coordinates at the Gauss points: X -> Y (x), Y -> X (y), X -> Y (z)
-    for (int a = threadIdx.x; a < n3; a += blockDim.x) {
-      const int q = a % n, j = (a / n) % n, k = a / n2;
-      for (int d = 0; d < 3; ++d) {
-        double s = 0.0;
-        for (int l = 0; l < n; ++l) s += tab.Bq[q][l] * X[d][k * n2 + j * n + l];
-        Y[d][a] = s;
-      }
-    }
-    __syncthreads();
-    for (int a = threadIdx.x; a < n3; a += blockDim.x) {
-      const int i = a % n, q = (a / n) % n, k = a / n2;
-      for (int d = 0; d < 3; ++d) {
-        double s = 0.0;
-        for (int l = 0; l < n; ++l) s += tab.Bq[q][l] * Y[d][k * n2 + l * n + i];
-        X[d][a] = s;
-      }
-    }
-    __syncthreads();
-    for (int a = threadIdx.x; a < n3; a += blockDim.x) {
-      const int i = a % n, j = (a / n) % n, q = a / n2;
-      for (int d = 0; d < 3; ++d) {
-        double s = 0.0;
-        for (int l = 0; l < n; ++l) s += tab.Bq[q][l] * X[d][l * n2 + j * n + i];
-        Y[d][a] = s;
-      }
-    }
-    __syncthreads();
-  }
-  const double(*Xq)[kMaxN * kMaxN * kMaxN] = lg ? Y : X;
-  const double sl = sigma_l[e], st = sigma_t[e], th = theta[e];
-  const double f0 = cos(th), f1 = sin(th);
-  double Dm[3][3];
-  const double fv[3] = {f0, f1, 0.0};
-  for (int r = 0; r < 3; ++r)
-    for (int c = 0; c < 3; ++c) Dm[r][c] = (r == c ? st : 0.0) + (sl - st) * fv[r] * fv[c];
-  for (int a = threadIdx.x; a < n3; a += blockDim.x) {
-    const int qx = a % n, qy = (a / n) % n, qz = a / n2;
+  for (int t = threadIdx.x; t < ne * N3; t += kSetupThreads) {
+    const int el = t / N3, a = t - el * N3, qx = a % N, qy = a / N % N, qz = a / N2;
+    const double x = xq[qx], y = xq[qy], z = xq[qz];
     double J[3][3];
+#pragma unroll
     for (int d = 0; d < 3; ++d) {
-      double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-      for (int l = 0; l < n; ++l) {
-        s0 += tab.Dc[qx][l] * Xq[d][qz * n2 + qy * n + l];
-        s1 += tab.Dc[qy][l] * Xq[d][qz * n2 + l * n + qx];
-        s2 += tab.Dc[qz][l] * Xq[d][l * n2 + qy * n + qx];
-      }
-      J[d][0] = s0; J[d][1] = s1; J[d][2] = s2;
+      const double* c = coef[el][d];  // index bits: 1 xi, 2 eta, 4 zeta
+      J[d][0] = fma(z, fma(y, c[7], c[5]), fma(y, c[3], c[1]));
+      J[d][1] = fma(z, fma(x, c[7], c[6]), fma(x, c[3], c[2]));
+      J[d][2] = fma(y, fma(x, c[7], c[6]), fma(x, c[5], c[4]));
     }
-    const double det = J[0][0] * (J[1][1] * J[2][2] - J[1][2] * J[2][1]) -
-                       J[0][1] * (J[1][0] * J[2][2] - J[1][2] * J[2][0]) +
-                       J[0][2] * (J[1][0] * J[2][1] - J[1][1] * J[2][0]);
+    double A[3][3];
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      const int p = (r + 1) % 3, q = (r + 2) % 3;
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        const int u = (d + 1) % 3, v = (d + 2) % 3;
+        A[r][d] = fma(J[u][p], J[v][q], -(J[v][p] * J[u][q]));
+      }
+    }
+    const double det = fma(J[2][0], A[0][2], fma(J[1][0], A[0][1], J[0][0] * A[0][0]));
     if (!(det > 0.0)) atomicExch(bad, 1);
-    double inv[3][3];
-    inv[0][0] = (J[1][1] * J[2][2] - J[1][2] * J[2][1]) / det;
-    inv[0][1] = (J[0][2] * J[2][1] - J[0][1] * J[2][2]) / det;
-    inv[0][2] = (J[0][1] * J[1][2] - J[0][2] * J[1][1]) / det;
-    inv[1][0] = (J[1][2] * J[2][0] - J[1][0] * J[2][2]) / det;
-    inv[1][1] = (J[0][0] * J[2][2] - J[0][2] * J[2][0]) / det;
-    inv[1][2] = (J[0][2] * J[1][0] - J[0][0] * J[1][2]) / det;
-    inv[2][0] = (J[1][0] * J[2][1] - J[1][1] * J[2][0]) / det;
-    inv[2][1] = (J[0][1] * J[2][0] - J[0][0] * J[2][1]) / det;
-    inv[2][2] = (J[0][0] * J[1][1] - J[0][1] * J[1][0]) / det;
-    const double W = tab.wq[qx] * tab.wq[qy] * tab.wq[qz] * det;
-    double T[3][3];  // inv * Dm
-    for (int r = 0; r < 3; ++r)
-      for (int c = 0; c < 3; ++c)
-        T[r][c] = inv[r][0] * Dm[0][c] + inv[r][1] * Dm[1][c] + inv[r][2] * Dm[2][c];
-    double G[3][3];  // W * T * inv^T
-    for (int r = 0; r < 3; ++r)
-      for (int c = 0; c < 3; ++c)
-        G[r][c] = W * (T[r][0] * inv[c][0] + T[r][1] * inv[c][1] + T[r][2] * inv[c][2]);
-    const int n3p = padded_n3(n);
-    double* out = metric + (size_t)e * kMetricComps * n3p + a;
-    out[0 * n3p] = G[0][0];
-    out[1 * n3p] = 0.5 * (G[0][1] + G[1][0]);
-    out[2 * n3p] = 0.5 * (G[0][2] + G[2][0]);
-    out[3 * n3p] = G[1][1];
-    out[4 * n3p] = 0.5 * (G[1][2] + G[2][1]);
-    out[5 * n3p] = G[2][2];
-    out[6 * n3p] = W;
+    const double w = wq[qx] * wq[qy] * wq[qz], s = w / det;
+    const double st = s * tens[el][0], sd = s * tens[el][1], f0 = tens[el][2], f1 = tens[el][3];
+    double af[3];
+#pragma unroll
+    for (int r = 0; r < 3; ++r) af[r] = fma(A[r][1], f1, A[r][0] * f0);
+    double* out = metric + (size_t)(e0 + el) * kMetricComps * N3P + a;
+    auto g = [&](int r, int c) {
+      const double aa = fma(A[r][2], A[c][2], fma(A[r][1], A[c][1], A[r][0] * A[c][0]));
+      return fma(sd * af[r], af[c], st * aa);
+    };
+    out[0 * N3P] = g(0, 0);
+    out[1 * N3P] = g(0, 1);
+    out[2 * N3P] = g(0, 2);
+    out[3 * N3P] = g(1, 1);
+    out[4 * N3P] = g(1, 2);
+    out[5 * N3P] = g(2, 2);
+    out[6 * N3P] = w * det;
   }
 }
 
@@ -183,35 +172,106 @@ __global__ void k_nodes(int nelem, int nx, int ny, int nz, const double* __restr
 
 // Assembled diagonals of M and K: per element and local node a,
 //   M_aa = sum_q W_q phi_a(q)^2,  K_aa = sum_q grad phi_a(q) . G_q grad phi_a(q)
-// (reference gradients; G already holds J^{-1} D J^{-T} w |det J|).
-__global__ void k_diagonals(int nelem, const int* __restrict__ map,
-                            const double* __restrict__ metric, const __grid_constant__ SetupTab tab,
-                            double* __restrict__ mdiag, double* __restrict__ kdiag) {
-  const int e = blockIdx.x;
-  if (e >= nelem) return;
-  const int n = tab.n, n2 = n * n, n3 = n2 * n;
-  const int n3p = padded_n3(n);
-  const double* me = metric + (size_t)e * kMetricComps * n3p;
-  for (int a = threadIdx.x; a < n3; a += blockDim.x) {
-    const int i = a % n, j = (a / n) % n, k = a / n2;
-    double Msum = 0.0, Ksum = 0.0;
-    for (int qz = 0; qz < n; ++qz)
-      for (int qy = 0; qy < n; ++qy)
-        for (int qx = 0; qx < n; ++qx) {
-          const int q = qx + n * qy + n2 * qz;
-          const double b0 = tab.Bq[qx][i], b1 = tab.Bq[qy][j], b2 = tab.Bq[qz][k];
-          const double d0 = tab.Dq[qx][i], d1 = tab.Dq[qy][j], d2 = tab.Dq[qz][k];
-          const double gx = d0 * b1 * b2, gy = b0 * d1 * b2, gz = b0 * b1 * d2, ph = b0 * b1 * b2;
-          const double G00 = me[0 * n3p + q], G01 = me[1 * n3p + q], G02 = me[2 * n3p + q];
-          const double G11 = me[3 * n3p + q], G12 = me[4 * n3p + q], G22 = me[5 * n3p + q];
-          const double W = me[6 * n3p + q];
-          Ksum += G00 * gx * gx + G11 * gy * gy + G22 * gz * gz +
-                  2.0 * (G01 * gx * gy + G02 * gx * gz + G12 * gy * gz);
-          Msum += W * ph * ph;
-        }
-    const int g = map[(size_t)e * n3 + a];
-    atomicAdd(mdiag + g, Msum);
-    atomicAdd(kdiag + g, Ksum);
+// (reference gradients; G already holds J^{-1} D J^{-T} w |det J|).  With the 1-D
+// tables' products bb = B^2, bd = B D, dd = D^2 every term is separable:
+//   K_aa: G00 (dd bb bb) + G11 (bb dd bb) + G22 (bb bb dd)
+//         + 2 G01 (bd bd bb) + 2 G02 (bd bb bd) + 2 G12 (bb bd bd),
+//   M_aa: W (bb bb bb)                                       (factors along x y z).
+// SEM-NI (k_diagonals_ni): B is the identity, so a node sums three lines of points and
+// its own point.  SEM (k_diagonals): three sweeps over 7, 7 and 4 fields.  The direct
+// sum over all points of every node took n^6 terms an element: 31.9 ms on 15,410
+// elements at p = 5, now 0.17 ms (SEM-NI) and 0.67 ms (SEM).
+template <int N>
+__global__ void __launch_bounds__(kSetupThreads)
+    k_diagonals_ni(int nelem, const int* __restrict__ map, const double* __restrict__ metric,
+                   const __grid_constant__ SetupTab tab, double* __restrict__ mdiag, double* __restrict__ kdiag) {
+  constexpr int N2 = N * N, N3 = N2 * N, E = setup_elems(N3), N3P = padded_n3(N);
+  __shared__ double dd[N][N], dq[N];  // D[q][a]^2, D[a][a]
+  const int e0 = blockIdx.x * E, ne = min(E, nelem - e0);
+  if (threadIdx.x < N2) {
+    const int q = threadIdx.x / N, a = threadIdx.x % N;
+    dd[q][a] = tab.Dq[q][a] * tab.Dq[q][a];
+    if (q == a) dq[a] = tab.Dq[a][a];
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < ne * N3; t += kSetupThreads) {
+    const int el = t / N3, a = t - el * N3, i = a % N, j = a / N % N, k = a / N2;
+    const double* me = metric + (size_t)(e0 + el) * kMetricComps * N3P;
+    const double *mx = me + (a - i), *my = me + 3 * N3P + (a - j * N), *mz = me + 5 * N3P + (a - k * N2);
+    double s = 2.0 * (me[1 * N3P + a] * dq[i] * dq[j] + me[2 * N3P + a] * dq[i] * dq[k] + me[4 * N3P + a] * dq[j] * dq[k]);
+#pragma unroll
+    for (int q = 0; q < N; ++q)
+      s = fma(mz[q * N2], dd[q][k], fma(my[q * N], dd[q][j], fma(mx[q], dd[q][i], s)));
+    const int g = map[(size_t)(e0 + el) * N3 + a];
+    atomicAdd(mdiag + g, me[6 * N3P + a]);
+    atomicAdd(kdiag + g, s);
+  }
+}
+
+template <int N>
+__global__ void __launch_bounds__(kSetupThreads)
+    k_diagonals(int nelem, const int* __restrict__ map, const double* __restrict__ metric,
+                const __grid_constant__ SetupTab tab, double* __restrict__ mdiag, double* __restrict__ kdiag) {
+  constexpr int N2 = N * N, N3 = N2 * N, N3P = padded_n3(N), E = N3 < 256 ? 256 / N3 : 1;
+  // [0..2]: bb, bd, dd; fields after the x-sweep (7) and after the y-sweep (4)
+  __shared__ double T[3][N][N];
+  __shared__ double X[7][E * N3];
+  __shared__ double Y[4][E * N3];
+  const int e0 = blockIdx.x * E, ne = min(E, nelem - e0);
+  if (threadIdx.x < N2) {
+    const int q = threadIdx.x / N, a = threadIdx.x % N;
+    const double B = tab.Bq[q][a], D = tab.Dq[q][a];
+    T[0][q][a] = B * B;
+    T[1][q][a] = B * D;
+    T[2][q][a] = D * D;
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < ne * N3; t += kSetupThreads) {
+    const int el = t / N3, a = t - el * N3, i = a % N;
+    const double* me = metric + (size_t)(e0 + el) * kMetricComps * N3P + (a - i);
+    double s[7] = {0, 0, 0, 0, 0, 0, 0};  // G00 dd, G01 bd, G02 bd, G11 bb, G12 bb, G22 bb, W bb
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      const double bb = T[0][q][i], bd = T[1][q][i], dd = T[2][q][i];
+      s[0] = fma(me[q], dd, s[0]);
+      s[1] = fma(me[N3P + q], bd, s[1]);
+      s[2] = fma(me[2 * N3P + q], bd, s[2]);
+#pragma unroll
+      for (int c = 3; c < 7; ++c) s[c] = fma(me[c * N3P + q], bb, s[c]);
+    }
+    for (int c = 0; c < 7; ++c) X[c][t] = s[c];
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < ne * N3; t += kSetupThreads) {
+    const int j = t / N % N, b = t - j * N;
+    double v0 = 0, v1 = 0, v2 = 0, v3 = 0;  // with bb, bd, dd along z, and the mass
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      const double bb = T[0][q][j], bd = T[1][q][j], dd = T[2][q][j];
+      const int p = b + q * N;
+      v0 = fma(X[0][p], bb, fma(X[3][p], dd, fma(2.0 * X[1][p], bd, v0)));
+      v1 = fma(X[2][p], bb, fma(X[4][p], bd, v1));
+      v2 = fma(X[5][p], bb, v2);
+      v3 = fma(X[6][p], bb, v3);
+    }
+    Y[0][t] = v0;
+    Y[1][t] = 2.0 * v1;
+    Y[2][t] = v2;
+    Y[3][t] = v3;
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < ne * N3; t += kSetupThreads) {
+    const int k = t / N2 % N, b = t - k * N2;
+    double ks = 0, ms = 0;
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      const int p = b + q * N2;
+      ks = fma(Y[0][p], T[0][q][k], fma(Y[1][p], T[1][q][k], fma(Y[2][p], T[2][q][k], ks)));
+      ms = fma(Y[3][p], T[0][q][k], ms);
+    }
+    const int g = map[(size_t)e0 * N3 + t];
+    atomicAdd(mdiag + g, ms);
+    atomicAdd(kdiag + g, ks);
   }
 }
 
@@ -326,17 +386,33 @@ void level_free(Level& L) {
   L = Level();
 }
 
+// The instantiation of one degree: f(std::integral_constant<int, n>).
+template <typename F>
+cudaError_t for_points(int n, F f) {
+  switch (n) {
+    case 2: f(std::integral_constant<int, 2>()); break;
+    case 3: f(std::integral_constant<int, 3>()); break;
+    case 4: f(std::integral_constant<int, 4>()); break;
+    case 5: f(std::integral_constant<int, 5>()); break;
+    case 6: f(std::integral_constant<int, 6>()); break;
+    case 7: f(std::integral_constant<int, 7>()); break;
+    default: return cudaErrorInvalidValue;
+  }
+  return cudaGetLastError();
+}
+
 cudaError_t setup_geometry(Level& L, const double* sigma_l, const double* sigma_t,
                            const double* theta, int* d_bad, cudaStream_t s) {
   const SetupTab tab = make_setup_tab(L.tab);
-  const int n3 = L.n * L.n * L.n;
-  k_metric<<<L.nelem, setup_threads(n3), 0, s>>>(L.nelem, L.evert, sigma_l, sigma_t, theta, tab,
-                                                 L.quad == SEM_QUAD_LG, L.metric, d_bad);
   L.metric32_valid = false;
   L.metric16_valid = false;
   L.metric2_valid = false;
   L.metric_tc_valid = false;
-  return cudaGetLastError();
+  return for_points(L.n, [&](auto n) {
+    constexpr int N = decltype(n)::value, E = setup_elems(N * N * N);
+    k_metric<N><<<(L.nelem + E - 1) / E, kSetupThreads, 0, s>>>(L.nelem, L.evert, sigma_l, sigma_t, theta, tab, L.metric,
+                                                                d_bad);
+  });
 }
 
 cudaError_t setup_node_coords(Level& L, cudaStream_t s) {
@@ -349,14 +425,20 @@ cudaError_t setup_node_coords(Level& L, cudaStream_t s) {
 
 cudaError_t setup_diagonals(Level& L, cudaStream_t s) {
   const SetupTab tab = make_setup_tab(L.tab);
-  const int n3 = L.n * L.n * L.n;
   cudaError_t err = cudaMemsetAsync(L.mdiag, 0, sizeof(double) * L.ndofs, s);
   if (err != cudaSuccess) return err;
   err = cudaMemsetAsync(L.kdiag, 0, sizeof(double) * L.ndofs, s);
   if (err != cudaSuccess) return err;
-  k_diagonals<<<L.nelem, setup_threads(n3), 0, s>>>(L.nelem, L.map, L.metric, tab, L.mdiag,
-                                                    L.kdiag);
-  return cudaGetLastError();
+  return for_points(L.n, [&](auto n) {
+    constexpr int N = decltype(n)::value, N3 = N * N * N;
+    if (L.quad == SEM_QUAD_LGL) {
+      constexpr int E = setup_elems(N3);
+      k_diagonals_ni<N><<<(L.nelem + E - 1) / E, kSetupThreads, 0, s>>>(L.nelem, L.map, L.metric, tab, L.mdiag, L.kdiag);
+    } else {
+      constexpr int E = N3 < 256 ? 256 / N3 : 1;
+      k_diagonals<N><<<(L.nelem + E - 1) / E, kSetupThreads, 0, s>>>(L.nelem, L.map, L.metric, tab, L.mdiag, L.kdiag);
+    }
+  });
 }
 
 cudaError_t setup_metric_lowp(Level& L, bool bf16, cudaStream_t s) {
