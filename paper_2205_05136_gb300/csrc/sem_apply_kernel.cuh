@@ -68,8 +68,8 @@ __device__ __forceinline__ double negated(double v) { return -v; }
 __device__ __forceinline__ float negated(float v) { return -v; }
 template <typename T, typename MT>
 __device__ __forceinline__ T scale_result(const ApplyArgs<T, MT>& a, T v) {
-  if (a.scale_out == kScaleOut) v *= a.out_scale;
-  return a.scale_out == kNegateOut ? negated(v) : v;
+  if (a.scale_out) v = a.scale_out == kNegateOut ? negated(v) : v * a.out_scale;
+  return v;
 }
 
 // Base offset and stride of line l of an n^3 tile along direction DIR

@@ -68,7 +68,7 @@ __host__ __device__ constexpr int setup_elems(int n3) { return n3 < 1024 ? 1024 
 // J's columns), G = w / det A D_e A^T takes one division.  About 100 FP64 operations a
 // point, which bound the kernel (2 a clock and SM); differentiating the nodal
 // coordinates and dividing nine entries took about 400 (2.0 ms on 15,410 elements at
-// p = 5, now 0.56 ms).
+// p = 5, now 0.60 ms).
 template <int N>
 __global__ void __launch_bounds__(kSetupThreads)
     k_metric(int nelem, const double* __restrict__ evert, const double* __restrict__ sigma_l,
@@ -180,7 +180,7 @@ __global__ void k_nodes(int nelem, int nx, int ny, int nz, const double* __restr
 // SEM-NI (k_diagonals_ni): B is the identity, so a node sums three lines of points and
 // its own point.  SEM (k_diagonals): three sweeps over 7, 7 and 4 fields.  The direct
 // sum over all points of every node took n^6 terms an element: 31.9 ms on 15,410
-// elements at p = 5, now 0.17 ms (SEM-NI) and 0.67 ms (SEM).
+// elements at p = 5, now 0.15 ms (SEM-NI) and 0.67 ms (SEM).
 template <int N>
 __global__ void __launch_bounds__(kSetupThreads)
     k_diagonals_ni(int nelem, const int* __restrict__ map, const double* __restrict__ metric,
