@@ -40,6 +40,21 @@ template <> struct ApplyCfg<4> { static constexpr int E = 10; };
 template <> struct ApplyCfg<5> { static constexpr int E = 7; };
 template <> struct ApplyCfg<6> { static constexpr int E = 5; };
 
+// Threads and elements of a CTA of the plain and the fused-inner-product apply.  Up
+// to p = 4 a CTA of 128 threads is the faster one (more CTAs of an SM are in different
+// phases between barriers): double-float, SEM-NI, 2 M nodes, 256 / 128 threads:
+// p = 1 330 / 265, p = 2 144 / 129, p = 3 124 / 100, p = 4 88 / 85 us; FP64 p = 2
+// 344 / 334, p = 4 292 / 291.  At p = 5, 6 128 threads hold 3 and 2 elements (84, 77 %
+// of the lines): 97 and 102 us against 96 and 95.  The FP64 apply with the inner
+// product keeps 256: sem_apply_dot_static's scratch holds one partial a CTA.
+template <int P, typename T, bool DOT>
+struct ApplyCta {
+  static constexpr bool kNarrow = P <= 4 && !(std::is_same<T, double>::value && DOT);
+  static constexpr int kThreads = kNarrow ? kApplyThreads / 2 : kApplyThreads;
+  static constexpr int E = kNarrow ? ApplyCfg<P>::E / 2 : ApplyCfg<P>::E;
+  static constexpr size_t smem = ((size_t)3 * E * (P + 1) * (P + 1) * (P + 1) * sizeof(T) + 15) / 16 * 16;
+};
+
 __device__ __forceinline__ double ldmetric(const double* p) { return __ldg(p); }
 __device__ __forceinline__ float ldmetric(const float* p) { return __ldg(p); }
 __device__ __forceinline__ float ldmetric(const __nv_bfloat16* p) {
@@ -89,7 +104,18 @@ __device__ __forceinline__ void line_geom(int l, int& base, int& stride) {
 // At n = 5 that is 12 multiply-adds and 8 additions instead of 25 multiply-adds.
 template <int N, bool ANTI, bool ACC, typename T>
 __device__ __forceinline__ void eo_line(const EoMat<N, T>& M, const T (&in)[N], T (&out)[N]) {
-  if constexpr (EoMat<N, T>::kDirect) {  // out_q (+)= sum_l m[q][l] in_l
+  if constexpr (N == 2 && ANTI) {
+    // derivative of a linear function: both rows of D are (-d, d) (a = 0), and both
+    // columns of D^T; D is only applied without ACC and D^T with it
+    if constexpr (!ACC) {
+      out[0] = out[1] = M.b[0][0] * (in[0] - in[1]);
+    } else {
+      const T y = M.a[0][0] * (in[0] + in[1]);
+      out[0] = out[0] + y;
+      out[1] = out[1] - y;
+    }
+    return;
+  } else if constexpr (EoMat<N, T>::kDirect) {  // out_q (+)= sum_l m[q][l] in_l
 #pragma unroll
     for (int q = 0; q < N; ++q) {
       T acc = ACC ? fma(M.m[q][0], in[0], out[q]) : M.m[q][0] * in[0];
@@ -166,6 +192,28 @@ __device__ __forceinline__ void sweep(const EoMat<N, T>& M, const T* src, T* dst
   }
 }
 
+// The same along a direction known at run time (one copy of the code for several
+// directions).
+template <int N, int E, bool ANTI, bool ACC, typename T>
+__device__ __forceinline__ void sweep_dir(const EoMat<N, T>& M, const T* src, T* dst, int dir, int tid, int nth) {
+  constexpr int N2 = N * N, N3 = N2 * N;
+  const int stride = dir == 0 ? 1 : dir == 1 ? N : N2;
+  for (int w = tid; w < E * N2; w += nth) {
+    const int s = w / N2, l = w - s * N2;
+    const int base = s * N3 + (dir == 0 ? l * N : dir == 1 ? (l / N) * N2 + l % N : l);
+    T in[N], out[N];
+#pragma unroll
+    for (int t = 0; t < N; ++t) in[t] = src[base + t * stride];
+    if (ACC) {
+#pragma unroll
+      for (int t = 0; t < N; ++t) out[t] = dst[base + t * stride];
+    }
+    eo_line<N, ANTI, ACC>(M, in, out);
+#pragma unroll
+    for (int t = 0; t < N; ++t) dst[base + t * stride] = out[t];
+  }
+}
+
 // Block-wide sum of v (all threads must call); result valid in thread 0.
 __device__ __forceinline__ double block_sum(double v, double* red) {
 #pragma unroll
@@ -234,15 +282,22 @@ __host__ __device__ constexpr size_t apply_warp_tile_bytes() {
 }
 
 // The double-float kernel at p = 4 (the outer operator of the benchmark's mixed
-// step) is bound by issue and memory latency: 5 CTAs per SM at 48 registers, with
-// small spills, measured faster than 4 at 62 (at p = 3, 5, 6 it would spill far more).
+// step) is bound by issue and memory latency: 10 CTAs per SM at 48 registers, with
+// small spills (8 measure the same in the plain apply, 1 % slower with the inner
+// product; at p = 3, 5, 6 it would spill far more).
 template <int P, int QUAD, typename T, typename MT, bool DOT, bool MASS_ONLY, bool WARP = false>
-__global__ void __launch_bounds__(kApplyThreads, (std::is_same<T, df>::value && P == 4) ? 5 : 1)
+__global__ void __launch_bounds__(MASS_ONLY ? kApplyThreads : ApplyCta<P, T, DOT>::kThreads,
+                                  (std::is_same<T, df>::value && !MASS_ONLY && P == 4)
+                                      ? 5 * kApplyThreads / ApplyCta<P, T, DOT>::kThreads : 1)
     sem_apply_kernel(const ApplyArgs<T, MT> a, const __grid_constant__ KTab<P + 1, T> tab) {
   static_assert(!(WARP && DOT), "the fused inner product needs the CTA-wide mode");
   constexpr int N = P + 1, N2 = N * N, N3 = N2 * N;
   using ML = MetricLayout<MT>;
-  constexpr int E = WARP ? WarpCfg<P>::G : ApplyCfg<P>::E;
+  constexpr int E = WARP ? WarpCfg<P>::G : MASS_ONLY ? ApplyCfg<P>::E : ApplyCta<P, T, DOT>::E;
+  // One copy of the sweep code for the directions: double-float at p = 4 (85 -> 80 us,
+  // SEM 120 -> 112) and FP64 at p = 1 (668 -> 644, SEM 1023 -> 975) gain by the shorter
+  // code; at p = 6 the run-time strides cost more (95 -> 130 us).
+  constexpr bool kRolled = (std::is_same<T, df>::value && P == 4) || (std::is_same<T, double>::value && P == 1 && !MASS_ONLY);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int warp = threadIdx.x >> 5;
   const int tid = WARP ? (threadIdx.x & 31) : threadIdx.x;
@@ -282,7 +337,7 @@ __global__ void __launch_bounds__(kApplyThreads, (std::is_same<T, df>::value && 
   // the plain apply have compile-time trip counts: they unroll and keep the
   // loads of all their iterations in flight at once.  The apply with the fused
   // inner product keeps the rolled loops (both measured faster that way).
-  constexpr int NTH = WARP ? 32 : kApplyThreads;
+  constexpr int NTH = WARP ? 32 : MASS_ONLY ? kApplyThreads : ApplyCta<P, T, DOT>::kThreads;
   constexpr int IT = (E * N3 + NTH - 1) / NTH;
 
   // gather u_e = P_e u
@@ -316,12 +371,20 @@ __global__ void __launch_bounds__(kApplyThreads, (std::is_same<T, df>::value && 
   group_sync();
 
   if (QUAD == SEM_QUAD_LG) {  // values at the Gauss points
-    sweep<N, E, 0, false, false>(tab.Bi, sA, sB, tid, nth);
-    group_sync();
-    sweep<N, E, 1, false, false>(tab.Bi, sB, sC, tid, nth);
-    group_sync();
-    sweep<N, E, 2, false, false>(tab.Bi, sC, sA, tid, nth);
-    group_sync();
+    if constexpr (kRolled) {
+#pragma unroll 1
+      for (int d = 0; d < 3; ++d) {
+        sweep_dir<N, E, false, false>(tab.Bi, sA, sA, d, tid, nth);
+        group_sync();
+      }
+    } else {
+      sweep<N, E, 0, false, false>(tab.Bi, sA, sB, tid, nth);
+      group_sync();
+      sweep<N, E, 1, false, false>(tab.Bi, sB, sC, tid, nth);
+      group_sync();
+      sweep<N, E, 2, false, false>(tab.Bi, sC, sA, tid, nth);
+      group_sync();
+    }
   }
 
   if (MASS_ONLY) {
@@ -335,8 +398,13 @@ __global__ void __launch_bounds__(kApplyThreads, (std::is_same<T, df>::value && 
     group_sync();
   } else {
     // reference gradient along x and y (into sB, sC)
-    sweep<N, E, 0, true, false>(tab.D, sA, sB, tid, nth);
-    sweep<N, E, 1, true, false>(tab.D, sA, sC, tid, nth);
+    if constexpr (kRolled) {
+#pragma unroll 1
+      for (int d = 0; d < 2; ++d) sweep_dir<N, E, true, false>(tab.D, sA, d == 0 ? sB : sC, d, tid, nth);
+    } else {
+      sweep<N, E, 0, true, false>(tab.D, sA, sB, tid, nth);
+      sweep<N, E, 1, true, false>(tab.D, sA, sC, tid, nth);
+    }
     group_sync();
     // z-gradient, quadrature-point stage and transposed z-sweep on the columns
     for (int w = tid; w < E * N2; w += nth) {
@@ -367,19 +435,35 @@ __global__ void __launch_bounds__(kApplyThreads, (std::is_same<T, df>::value && 
       for (int k = 0; k < N; ++k) pa[k * N2] = m[k];
     }
     group_sync();
-    sweep<N, E, 1, true, true>(tab.Dt, sC, sA, tid, nth);
-    group_sync();
-    sweep<N, E, 0, true, true>(tab.Dt, sB, sA, tid, nth);
-    group_sync();
+    if constexpr (kRolled) {
+#pragma unroll 1
+      for (int d = 1; d >= 0; --d) {
+        sweep_dir<N, E, true, true>(tab.Dt, d == 0 ? sB : sC, sA, d, tid, nth);
+        group_sync();
+      }
+    } else {
+      sweep<N, E, 1, true, true>(tab.Dt, sC, sA, tid, nth);
+      group_sync();
+      sweep<N, E, 0, true, true>(tab.Dt, sB, sA, tid, nth);
+      group_sync();
+    }
   }
 
   if (QUAD == SEM_QUAD_LG) {  // back from the Gauss points to the nodes
-    sweep<N, E, 0, false, false>(tab.Bit, sA, sB, tid, nth);
-    group_sync();
-    sweep<N, E, 1, false, false>(tab.Bit, sB, sC, tid, nth);
-    group_sync();
-    sweep<N, E, 2, false, false>(tab.Bit, sC, sA, tid, nth);
-    group_sync();
+    if constexpr (kRolled) {
+#pragma unroll 1
+      for (int d = 0; d < 3; ++d) {
+        sweep_dir<N, E, false, false>(tab.Bit, sA, sA, d, tid, nth);
+        group_sync();
+      }
+    } else {
+      sweep<N, E, 0, false, false>(tab.Bit, sA, sB, tid, nth);
+      group_sync();
+      sweep<N, E, 1, false, false>(tab.Bit, sB, sC, tid, nth);
+      group_sync();
+      sweep<N, E, 2, false, false>(tab.Bit, sC, sA, tid, nth);
+      group_sync();
+    }
   }
 
   pdl_trigger();
@@ -866,9 +950,18 @@ __global__ void __launch_bounds__(32 * PlaneCfg<P, MT>::kWarps, PlaneCfg<P, MT>:
     if (!plane_points<P, 0>(a, tab, feed, use, phase, behind, nunits, tw, lane, lidx, wb, sm_s, bar_s, u, gy, gz)) return;
     __syncwarp();  // the planes of u are read
     if (act) plane_store<N>(own, gz);
-    plane_sweep<N, 1, true>(tab.Dt, gy);
 #pragma unroll
-    for (int v = 0; v < N2; ++v) u[v] += gy[v];
+    for (int i = 0; i < N; ++i) {  // u += D^T q2 along y
+      float in[N], out[N];
+#pragma unroll
+      for (int j = 0; j < N; ++j) {
+        in[j] = gy[j * N + i];
+        out[j] = u[j * N + i];
+      }
+      eo_line<N, true, true>(tab.Dt, in, out);
+#pragma unroll
+      for (int j = 0; j < N; ++j) u[j * N + i] = out[j];
+    }
     __syncwarp();
     plane_zsweep<N, C::PS, true>(dtz, elem, u);
     if (QUAD == SEM_QUAD_LG) {  // back from the Gauss points: z, then x and y in the plane
@@ -996,12 +1089,16 @@ cudaError_t launch_apply_kernels(const Level& L, const ApplyArgs<T, MT>& a, cons
   if (mass_only) {
     launch_k(sem_apply_kernel<P, QUAD, T, MT, false, true>, grid, kApplyThreads, tiles, s, a, tab);
   } else if (dot) {
-    launch_k(sem_apply_kernel<P, QUAD, T, MT, true, false>, grid, kApplyThreads, tiles, s, a, tab);
+    using C = ApplyCta<P, T, true>;
+    const int dgrid = (L.nelem + C::E - 1) / C::E;
+    launch_k(sem_apply_kernel<P, QUAD, T, MT, true, false>, dgrid, C::kThreads, C::smem, s, a, tab);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return launch_apply_dot_finish(a.dot_partials, grid, a.cg, a.dot_out, a.done, s);
+    return launch_apply_dot_finish(a.dot_partials, dgrid, a.cg, a.dot_out, a.done, s);
   } else {
-    launch_k(sem_apply_kernel<P, QUAD, T, MT, false, false>, grid, kApplyThreads, tiles, s, a, tab);
+    using C = ApplyCta<P, T, false>;
+    launch_k(sem_apply_kernel<P, QUAD, T, MT, false, false>, (L.nelem + C::E - 1) / C::E, C::kThreads, C::smem, s, a,
+             tab);
   }
   return cudaGetLastError();
   }

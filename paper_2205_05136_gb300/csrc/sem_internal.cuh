@@ -17,6 +17,7 @@
 #include <stdint.h>
 
 #include <string>
+#include <type_traits>
 #include <utility>
 
 #include "sem.h"
@@ -131,11 +132,13 @@ void build_tables(int p, int quad, Tables1D* t);
 // and for odd n the middle column a[q][H] = M[q][H] and the middle row
 // c[l] = M[H][l] (l <= H).  A product y = M x then takes about half the
 // multiplications (see eo_line).  For n = 2 and 4 the split saves no
-// multiplication, so the matrix itself (m) is kept and multiplied directly.
+// multiplication, so the matrix itself (m) is kept and multiplied directly; but in
+// double-float, where a multiply-add takes 13 instructions and an addition 8, the
+// split is shorter at n = 4 (132 instead of 172 instructions a line).
 template <int N, typename T>
 struct EoMat {
   static constexpr int H = N / 2;
-  static constexpr bool kDirect = (N == 2 || N == 4);
+  static constexpr bool kDirect = (N == 2 || (N == 4 && !std::is_same<T, df>::value));
   static constexpr int NM = kDirect ? N : 1;
   T a[H][H + 1];
   T b[H][H];

@@ -499,7 +499,7 @@ int ensure_workspace(sem_ctx* ctx) {
   SEM_CK(cudaMalloc(&w.vec_partials, sizeof(double) * kReduceSlots * kVecBlocksMax));
   SEM_CK(cudaMalloc(&w.tickets, sizeof(unsigned int) * 4));
   SEM_CK(cudaMemset(w.tickets, 0, sizeof(unsigned int) * 4));
-  const int ag = std::max(1, apply_grid_blocks(ctx->L));
+  const int ag = 2 * std::max(1, apply_grid_blocks(ctx->L));  // the double-float apply has up to twice the CTAs
   SEM_CK(cudaMalloc(&w.apply_partials, sizeof(double) * ag));
   SEM_CK(cudaMalloc(&w.dot_result, sizeof(double)));
   SEM_CK(cudaMalloc(&w.same, sizeof(int)));
