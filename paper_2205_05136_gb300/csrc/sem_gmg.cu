@@ -236,6 +236,202 @@ __global__ void k_cheb_step(int64_t n, const T* __restrict__ r, const T* __restr
   pdl_trigger();
 }
 
+// ---- all Chebyshev steps of a small coarsest level in one CTA
+//
+// Steps of a level of a few hundred nodes cost two launches each, about 1 us a launch
+// whatever the level's size.  One CTA of kCoarseThreads threads runs all of them with
+// everything on chip: the metric (in its storage type, word by word across the
+// elements so that the lanes' reads do not conflict), d and the element results in
+// shared memory, r, x, 1 / diagonal and the elements' node numbers in registers.  A
+// step is two phases between barriers: every thread evaluates its elements (Q_1 in
+// registers); every thread sums the results of its nodes' elements in a fixed order
+// (the deterministic mode needs no variant) and updates.  The metric is copied before
+// the wait for the previous kernel.  The launcher takes it for a Q_1 level in FP32 of
+// at most kCoarseNodes nodes whose metric fits.  One PCG iteration, before / now,
+// with coarsest levels of 608, 108, 30 and 990 nodes: 113 / 102, 145 / 125, 103 / 81,
+// 437 / 430 us (degree 10, with the one-launch restriction below).  (With the metric read from L1 at every step, lane by lane, a step of the
+// 608-node level took as long as its two launches.)
+constexpr int kCoarseThreads = 512, kCoarseNodes = 1024, kCoarsePer = kCoarseNodes / kCoarseThreads;
+constexpr int kCoarseDegree = 200;
+constexpr size_t kCoarseSmem = 227 * 1024;
+
+struct ChebCoef {
+  float c1[kCoarseDegree], c2[kCoarseDegree];
+};
+
+// Shared-memory words of an element's metric: 56 values of the storage type.
+template <typename MT> __host__ __device__ constexpr int coarse_words() { return 56 * (int)sizeof(MT) / 4; }
+__device__ __forceinline__ void coarse_point(const unsigned* w, int nep, int pt, float (&G)[kMetricComps],
+                                             const __nv_bfloat16*) {
+#pragma unroll
+  for (int c = 0; c < kMetricComps; ++c) {
+    const int v = kMetricComps * pt + c;
+    const unsigned u = w[(v >> 1) * nep];
+    G[c] = __uint_as_float((v & 1) ? u & 0xffff0000u : u << 16);
+  }
+}
+__device__ __forceinline__ void coarse_point(const unsigned* w, int nep, int pt, float (&G)[kMetricComps], const float*) {
+#pragma unroll
+  for (int c = 0; c < kMetricComps; ++c) G[c] = __uint_as_float(w[(kMetricComps * pt + c) * nep]);
+}
+
+// Element results y = (mass M + K) u of one Q_1 element, in place; w: its first
+// metric word, nep words between its words.
+template <int QUAD, typename MT>
+__device__ __forceinline__ void q1_element(const KTab<2, float>& tab, const unsigned* w, int nep, float mass,
+                                           float (&u)[8]) {
+  // f(node, node) for the four lines of a direction; nodes a = i + 2 j + 4 k
+  auto lines = [](int dir, auto f) {
+#pragma unroll
+    for (int l = 0; l < 4; ++l) {
+      const int base = dir == 0 ? 2 * l : dir == 1 ? (l & 1) + 4 * (l >> 1) : l;
+      f(base, base + (1 << dir));
+    }
+  };
+  auto interpolate = [&](const EoMat<2, float>& M) {
+#pragma unroll
+    for (int dir = 0; dir < 3; ++dir)
+      lines(dir, [&](int p, int q) {
+        const float in[2] = {u[p], u[q]};
+        float out[2];
+        eo_line<2, false, false>(M, in, out);
+        u[p] = out[0];
+        u[q] = out[1];
+      });
+  };
+  if (QUAD == SEM_QUAD_LG) interpolate(tab.Bi);
+  float g[3][8];
+#pragma unroll
+  for (int dir = 0; dir < 3; ++dir)
+    lines(dir, [&](int p, int q) {
+      const float in[2] = {u[p], u[q]};
+      float out[2];
+      eo_line<2, true, false>(tab.D, in, out);
+      g[dir][p] = out[0];
+      g[dir][q] = out[1];
+    });
+#pragma unroll
+  for (int a = 0; a < 8; ++a) {
+    float G[kMetricComps];
+    coarse_point(w, nep, a, G, static_cast<const MT*>(nullptr));
+    const float x = g[0][a], y = g[1][a], z = g[2][a];
+    g[0][a] = fmaf(G[2], z, fmaf(G[1], y, G[0] * x));
+    g[1][a] = fmaf(G[4], z, fmaf(G[3], y, G[1] * x));
+    g[2][a] = fmaf(G[5], z, fmaf(G[4], y, G[2] * x));
+    u[a] = (mass * G[6]) * u[a];
+  }
+#pragma unroll
+  for (int dir = 2; dir >= 0; --dir)
+    lines(dir, [&](int p, int q) {
+      const float in[2] = {g[dir][p], g[dir][q]};
+      float out[2] = {u[p], u[q]};
+      eo_line<2, true, true>(tab.Dt, in, out);
+      u[p] = out[0];
+      u[q] = out[1];
+    });
+  if (QUAD == SEM_QUAD_LG) interpolate(tab.Bit);
+}
+
+template <int QUAD, typename MT>
+__global__ void __launch_bounds__(kCoarseThreads, 1)
+    k_cheb_coarse(int nx, int ny, int nz, const int* __restrict__ map, const MT* __restrict__ metric, float mass,
+                  const __grid_constant__ KTab<2, float> tab, const __grid_constant__ ChebCoef cf, int degree,
+                  const float* __restrict__ rhs, const float* __restrict__ invd, float* __restrict__ x_out,
+                  int64_t ndofs, unsigned long long* dbg, const int* done) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  constexpr int W = coarse_words<MT>();
+  static_assert(MetricLayout<MT>::unit(2) * 2 * MetricLayout<MT>::stride(2) == MetricLayout<MT>::chunk(2) &&
+                    2 * MetricLayout<MT>::stride(2) == 56, "the elements' 56 values follow one another at n = 2");
+  const int n = (nx + 1) * (ny + 1) * (nz + 1), ne = nx * ny * nz, nep = ne | 1;
+  float* sd = reinterpret_cast<float*>(smem_raw);  // d on the nodes
+  float* sy = sd + n;                              // element results [8][nep]
+  unsigned* sm = reinterpret_cast<unsigned*>(sy + 8 * nep);  // metric [W][nep]
+  const unsigned* gm = reinterpret_cast<const unsigned*>(metric);
+#pragma unroll 8
+  for (int t = threadIdx.x; t < ne * W; t += kCoarseThreads) sm[(t % W) * nep + t / W] = __ldg(gm + t);
+  unsigned short node[kCoarsePer][8];
+#pragma unroll
+  for (int q = 0; q < kCoarsePer; ++q) {
+    const int e = threadIdx.x + q * kCoarseThreads;
+#pragma unroll
+    for (int a = 0; a < 8; ++a)
+      node[q][a] = e < ne ? (unsigned short)SEM_IDX(__ldg(map + 8 * e + a), ndofs, dbg, kDbgGather) : 0;
+  }
+  pdl_wait();
+  if (skip(done)) return;
+  float r[kCoarsePer], x[kCoarsePer], inv[kCoarsePer];
+  const float c0 = cf.c2[0];  // 1 / theta
+#pragma unroll
+  for (int t = 0; t < kCoarsePer; ++t) {
+    const int i = threadIdx.x + t * kCoarseThreads;
+    if (i < n) {
+      r[t] = rhs[i];
+      inv[t] = invd[i];
+      x[t] = inv[t] * r[t] * c0;
+      sd[i] = x[t];
+    }
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int s = 1; s < degree; ++s) {
+#pragma unroll
+    for (int q = 0; q < kCoarsePer; ++q) {
+      const int e = threadIdx.x + q * kCoarseThreads;
+      if (e < ne) {
+        float u[8];
+#pragma unroll
+        for (int a = 0; a < 8; ++a) u[a] = sd[node[q][a]];
+        q1_element<QUAD, MT>(tab, sm + e, nep, mass, u);
+#pragma unroll
+        for (int a = 0; a < 8; ++a) sy[a * nep + e] = u[a];
+      }
+    }
+    __syncthreads();
+    const float c1 = cf.c1[s], c2 = cf.c2[s];
+#pragma unroll
+    for (int t = 0; t < kCoarsePer; ++t) {
+      const int i = threadIdx.x + t * kCoarseThreads;
+      if (i < n) {
+        const int I = i % (nx + 1), J = i / (nx + 1) % (ny + 1), K = i / ((nx + 1) * (ny + 1));
+        float y = 0.f;
+#pragma unroll
+        for (int a = 7; a >= 0; --a) {  // the node is local node a of the element below it by a's bits
+          const int ex = I - (a & 1), ey = J - (a >> 1 & 1), ez = K - (a >> 2);
+          if (ex >= 0 && ex < nx && ey >= 0 && ey < ny && ez >= 0 && ez < nz)
+            y += sy[a * nep + ex + nx * (ey + ny * ez)];
+        }
+        r[t] -= y;
+        const float d = fmaf(c1, sd[i], c2 * inv[t] * r[t]);
+        sd[i] = d;
+        x[t] += d;
+      }
+    }
+    __syncthreads();
+  }
+  pdl_trigger();
+#pragma unroll
+  for (int t = 0; t < kCoarsePer; ++t) {
+    const int i = threadIdx.x + t * kCoarseThreads;
+    if (i < n) x_out[i] = x[t];
+  }
+}
+
+template <typename MT>
+size_t coarse_smem(const Level& L) {
+  const size_t nep = (size_t)L.nelem | 1;
+  return 4 * ((size_t)L.ndofs + 8 * nep + coarse_words<MT>() * nep);
+}
+cudaError_t prime_coarse() {
+  auto set = [](auto kern) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoarseSmem);
+  };
+  cudaError_t e = set(k_cheb_coarse<SEM_QUAD_LG, float>);
+  if (e == cudaSuccess) e = set(k_cheb_coarse<SEM_QUAD_LGL, float>);
+  if (e == cudaSuccess) e = set(k_cheb_coarse<SEM_QUAD_LG, __nv_bfloat16>);
+  if (e == cudaSuccess) e = set(k_cheb_coarse<SEM_QUAD_LGL, __nv_bfloat16>);
+  return e;
+}
+
 // ---------------------------------------------------------------- transfers
 struct PTab {
   int nf, nc;
@@ -282,65 +478,41 @@ __global__ void k_prolong_h(int nfx, int nfy, int nfz, int ncx, int ncy, int ncz
   pdl_trigger();
 }
 
+// Restriction gathered per coarse node: the fine nodes within 1 of 2 C in each
+// direction (also at a trailing single element), in a fixed order, weighted by the
+// trilinear prolongation's weight of that coarse node.  Every coarse node is written
+// once: nothing is cleared before and the result is the same in every run.
 template <typename T>
 __global__ void k_restrict_h(int nfx, int nfy, int nfz, int ncx, int ncy, int ncz,
-                             const T* __restrict__ rf, T* __restrict__ bc, const int* done) {
-  pdl_wait();
-  if (skip(done)) return;
-  const int64_t NX = nfx + 1, NY = nfy + 1, n = NX * NY * (nfz + 1);
-  const int64_t CX = ncx + 1, CY = ncy + 1;
-  GRID_LOOP(g, n) {
-    const int I = (int)(g % NX), J = (int)((g / NX) % NY), K = (int)(g / (NX * NY));
-    int kx, ky, kz;
-    double wx[2], wy[2], wz[2];
-    hweights(I, nfx, ncx, kx, wx[0], wx[1]);
-    hweights(J, nfy, ncy, ky, wy[0], wy[1]);
-    hweights(K, nfz, ncz, kz, wz[0], wz[1]);
-    const T r = rf[g];
-    for (int c = 0; c < 2; ++c)
-      for (int b = 0; b < 2; ++b)
-        for (int a = 0; a < 2; ++a) {
-          const double w = wx[a] * wy[b] * wz[c];
-          if (w != 0.0) atomicAdd(bc + (kx + a) + CX * ((ky + b) + CY * (kz + c)), (T)w * r);
-        }
-  }
-  pdl_trigger();
-}
-
-// The same restriction gathered per coarse node (deterministic mode): the fine
-// nodes within 3 of 2 C in each direction, in a fixed order, weighted by the
-// trilinear prolongation's weight of that coarse node.
-template <typename T>
-__global__ void k_restrict_h_det(int nfx, int nfy, int nfz, int ncx, int ncy, int ncz,
-                                 const T* __restrict__ rf, T* __restrict__ bc, const int* done) {
+                             const T* __restrict__ rf, T* __restrict__ rc, const int* done) {
   pdl_wait();
   if (skip(done)) return;
   const int64_t NX = nfx + 1, NY = nfy + 1;
   const int64_t CX = ncx + 1, CY = ncy + 1, nc = CX * CY * (ncz + 1);
   GRID_LOOP(c, nc) {
     const int CI = (int)(c % CX), CJ = (int)((c / CX) % CY), CK = (int)(c / (CX * CY));
-    auto wt = [](int I, int nf, int ncoarse, int C) {
-      int k;
-      double w0, w1;
-      hweights(I, nf, ncoarse, k, w0, w1);
-      return k == C ? w0 : (k + 1 == C ? w1 : 0.0);
+    // weights of the fine nodes 2 C - 1, 2 C, 2 C + 1: 1/2 beside C, 1 on it; a trailing
+    // single element has its only inner neighbour at the mesh's end, weight 1
+    auto weights = [](int C, int nf, T (&w)[3]) {
+      const bool odd_end = 2 * C > nf;  // C is the closing node of an odd nf: fine node nf is 2 C - 1
+      w[0] = C == 0 ? T(0) : (odd_end ? T(1) : T(0.5));
+      w[1] = odd_end ? T(0) : T(1);
+      w[2] = 2 * C + 2 <= nf ? T(0.5) : T(0);
     };
-    T acc = T(0);
-    for (int K = max(0, 2 * CK - 3); K <= min(nfz, 2 * CK + 3); ++K) {
-      const double wz = wt(K, nfz, ncz, CK);
-      if (wz == 0.0) continue;
-      for (int J = max(0, 2 * CJ - 3); J <= min(nfy, 2 * CJ + 3); ++J) {
-        const double wy = wt(J, nfy, ncy, CJ);
-        if (wy == 0.0) continue;
-        for (int I = max(0, 2 * CI - 3); I <= min(nfx, 2 * CI + 3); ++I) {
-          const double wx = wt(I, nfx, ncx, CI);
-          if (wx == 0.0) continue;
-          const int64_t g = I + NX * (J + NY * (int64_t)K);
-          acc += (T)(wx * wy * wz) * rf[g];
-        }
-      }
+    T wx[3], wy[3], wz[3], v[27];
+    weights(CI, nfx, wx);
+    weights(CJ, nfy, wy);
+    weights(CK, nfz, wz);
+    const int64_t base = (2 * CI - 1) + NX * ((2 * CJ - 1) + NY * (int64_t)(2 * CK - 1));
+#pragma unroll
+    for (int a = 0; a < 27; ++a) {  // all loads in flight
+      const int i = a % 3, j = a / 3 % 3, k = a / 9;
+      v[a] = (wx[i] != T(0) && wy[j] != T(0) && wz[k] != T(0)) ? rf[base + i + NX * (j + NY * (int64_t)k)] : T(0);
     }
-    bc[c] += acc;
+    T acc = T(0);
+#pragma unroll
+    for (int a = 0; a < 27; ++a) acc = fma(wx[a % 3] * wy[a / 3 % 3] * wz[a / 9], v[a], acc);
+    rc[c] = acc;
   }
   pdl_trigger();
 }
@@ -1017,17 +1189,10 @@ int restrict_to(sem_ctx* ctx, Gmg& g, int l, const int* done, cudaStream_t s) {
     ctx->launches += 1;
     return SEM_OK;
   }
-  launch_k(k_zero<T>, grid_chunks<T>(C.L->ndofs), kThreads, 0, s, C.L->ndofs, (T*)C.r, done);
-  T* loc = ctx->deterministic ? reinterpret_cast<T*>(ctx->det_scratch) : nullptr;
-  if (loc != nullptr) {
-    launch_k(k_restrict_h_det<T>, grid1d(C.L->ndofs), kThreads, 0, s,
-        F.L->nx, F.L->ny, F.L->nz, C.L->nx, C.L->ny, C.L->nz, (const T*)F.r, (T*)C.r, done);
-  } else {
-    launch_k(k_restrict_h<T>, grid1d(F.L->ndofs), kThreads, 0, s,
-        F.L->nx, F.L->ny, F.L->nz, C.L->nx, C.L->ny, C.L->nz, (const T*)F.r, (T*)C.r, done);
-  }
+  launch_k(k_restrict_h<T>, grid1d(C.L->ndofs), kThreads, 0, s, F.L->nx, F.L->ny, F.L->nz, C.L->nx, C.L->ny, C.L->nz,
+           (const T*)F.r, (T*)C.r, done);
   GMG_CK(cudaGetLastError());
-  ctx->launches += 2;
+  ctx->launches += 1;
   return SEM_OK;
 }
 
@@ -1091,11 +1256,58 @@ int chebyshev(sem_ctx* ctx, Gmg& g, int l, int degree, bool zero_start, bool kee
   return SEM_OK;
 }
 
+// Whether k_cheb_coarse takes the coarsest level.
+bool coarse_in_one_cta(const Gmg& g) {
+  const Level& L = *g.lv.back().L;
+  if (g.precision == SEM_PREC_FP64 || L.p != 1 || L.ndofs > kCoarseNodes || g.coarse_degree > kCoarseDegree) return false;
+  return (g.precision == SEM_PREC_FP32 ? coarse_smem<float>(L) : coarse_smem<__nv_bfloat16>(L)) <= kCoarseSmem;
+}
+
+template <int QUAD, typename MT>
+cudaError_t launch_coarse(const GmgLevel& V, const MT* metric, double alpha, int degree, const int* done, cudaStream_t s) {
+  const Level& L = *V.L;
+  const double lo = 0.08 * V.lam, hi = 1.2 * V.lam;
+  const double theta = 0.5 * (hi + lo), delta = 0.5 * (hi - lo), sigma = theta / delta;
+  ChebCoef cf;
+  double rho_old = 1.0 / sigma;
+  cf.c1[0] = 0.f;
+  cf.c2[0] = (float)(1.0 / theta);
+  for (int k = 1; k < degree; ++k) {
+    const double rho = 1.0 / (2.0 * sigma - rho_old);
+    cf.c1[k] = (float)(rho * rho_old);
+    cf.c2[k] = (float)(2.0 * rho / delta);
+    rho_old = rho;
+  }
+  KTab<2, float> tab;
+  make_eo(tab.D, QUAD == SEM_QUAD_LG ? L.tab.Dg : L.tab.D, false);
+  make_eo(tab.Dt, QUAD == SEM_QUAD_LG ? L.tab.Dg : L.tab.D, true);
+  make_eo(tab.Bi, L.tab.Bi, false);
+  make_eo(tab.Bit, L.tab.Bi, true);
+  return launch_k(k_cheb_coarse<QUAD, MT>, 1, kCoarseThreads, coarse_smem<MT>(L), s, L.nx, L.ny, L.nz, L.map, metric,
+                  (float)alpha, tab, cf, degree, (const float*)V.r, (const float*)V.invd, (float*)V.x, L.ndofs, L.dbg,
+                  done);
+}
+
+int chebyshev_coarse(sem_ctx* ctx, Gmg& g, const int* done, cudaStream_t s) {
+  const GmgLevel& V = g.lv.back();
+  const bool lg = V.L->quad == SEM_QUAD_LG;
+  if (g.precision == SEM_PREC_FP32)
+    GMG_CK((lg ? launch_coarse<SEM_QUAD_LG, float> : launch_coarse<SEM_QUAD_LGL, float>)(V, V.L->metric32, g.alpha,
+                                                                                        g.coarse_degree, done, s));
+  else
+    GMG_CK((lg ? launch_coarse<SEM_QUAD_LG, __nv_bfloat16> : launch_coarse<SEM_QUAD_LGL, __nv_bfloat16>)(
+        V, V.L->metric16, g.alpha, g.coarse_degree, done, s));
+  ctx->launches += 1;
+  return SEM_OK;
+}
+
 template <typename T>
 int vcycle_level(sem_ctx* ctx, Gmg& g, int l, const int* done, cudaStream_t s, bool record) {
   const int last = (int)g.lv.size() - 1;
   int rc;
-  if (l == last) return chebyshev<T>(ctx, g, l, g.coarse_degree, true, false, done, s);
+  if (l == last)
+    return coarse_in_one_cta(g) ? chebyshev_coarse(ctx, g, done, s)
+                                : chebyshev<T>(ctx, g, l, g.coarse_degree, true, false, done, s);
   if ((rc = chebyshev<T>(ctx, g, l, g.degree, true, true, done, s)) != SEM_OK) return rc;
   GmgLevel& V = g.lv[l];
   // r -= A d: the residual of x, then r_{l+1} = R r
@@ -1221,6 +1433,7 @@ void free_gmg_struct(Gmg* g) {
 
 int build(sem_ctx* ctx, cudaStream_t s) {
   if (ctx->gmg) return SEM_OK;
+  GMG_CK(prime_coarse());
   Gmg* g = new Gmg();
   g->precision = ctx->gmg_precision;
   g->degree = ctx->gmg_degree;
