@@ -910,11 +910,13 @@ __global__ void __launch_bounds__(32 * PlaneCfg<P, MT>::kWarps, PlaneCfg<P, MT>:
   int base = plane_base<P>(a, unit, nunits, s);
   int base_n = plane_base<P>(a, unit + tw, nunits, s);
   pdl_wait();
-  if (a.done != nullptr && *a.done) {
-    for (int t = 0; t < behind; ++t) mbar_wait(bar_s + 8 * t, 0);  // the CTA must not end under its own copies
+  const bool stop = a.done != nullptr && *a.done;
+  plane_gather<P>(a, unit, base, s, r, act, tile_s);
+  if (stop) {  // the CTA must not end under its own copies
+    for (int t = 0; t < behind; ++t) mbar_wait(bar_s + 8 * t, 0);
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
     return;
   }
-  plane_gather<P>(a, unit, base, s, r, act, tile_s);
   unsigned phase = 0;  // bit t: parity of stage t's next completion
   int use = 0;         // stage of the next chunk
   int b = 0;

@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(BrickCfg<NF, NC>::kThreads)
   const BrickPos<NF, NC> q(nx, ny, nz);
   const int xf = PF * nx + 1, yf = PF * ny + 1, zf = PF * nz + 1;
   pdl_wait();
-  if (done != nullptr && *done) return;
+  const bool stop = done != nullptr && *done;  // acted on before the first store (sem_gmg.cu, skip)
   {  // z: the lane's column (x, y) of the fine nodes
     const int x = PF * (q.ex - 1) + 1 + lane, y = PF * (q.ey - 1) + 1 + warp, z0 = PF * (q.ez - 1) + 1;
     const bool col = lane < C::RX && x >= 0 && x < xf && y >= 0 && y < yf;
@@ -154,6 +154,7 @@ __global__ void __launch_bounds__(BrickCfg<NF, NC>::kThreads)
     T f[C::RZ];
 #pragma unroll
     for (int k = 0; k < C::RZ; ++k) f[k] = (col && z0 + k >= 0 && z0 + k < zf) ? p[(int64_t)xf * yf * k] : T(0);
+    if (stop) return;
     restrict_line<NF, NC, B::Z>(pm, f, [&](int c, T v) { s1[c][warp][lane] = v; });
   }
   __syncthreads();
@@ -193,7 +194,15 @@ __global__ void __launch_bounds__(BrickCfg<NF, NC>::kThreads)
   const BrickPos<NF, NC> q(nx, ny, nz);
   const int xc = PC * nx + 1, yc = PC * ny + 1;
   pdl_wait();
-  if (done != nullptr && *done) return;
+  const bool stop = done != nullptr && *done;  // acted on before the first store (sem_gmg.cu, skip)
+  // the fine column (x, y) of the lane, read while the coarse nodes are
+  const int xf = PF * nx + 1, yf = PF * ny + 1;
+  const int64_t o = PF * q.ex + lane + (int64_t)xf * (PF * q.ey + warp + (int64_t)yf * (PF * q.ez)),
+                zs = (int64_t)xf * yf;
+  const bool col = warp < q.fy && lane < q.fx;
+  T x[C::FZ];
+#pragma unroll
+  for (int i = 0; i < C::FZ; ++i) x[i] = col && i < q.fz ? out[o + zs * i] : T(0);
   for (int t = threadIdx.x; t < C::CZ * C::CY * B::X; t += C::kThreads) {  // x: one element of one row a thread
     const int e = t % B::X, y = t / B::X % C::CY, z = t / (B::X * C::CY);
     if (e >= q.lx) continue;
@@ -206,6 +215,7 @@ __global__ void __launch_bounds__(BrickCfg<NF, NC>::kThreads)
       if (i < PF || e == q.lx - 1) s1[z][y][PF * e + i] = v;
     });
   }
+  if (stop) return;
   __syncthreads();
   for (int t = threadIdx.x; t < C::CZ * 32; t += C::kThreads) {  // y: one (z, x) a thread
     T c[C::CY];
@@ -214,13 +224,8 @@ __global__ void __launch_bounds__(BrickCfg<NF, NC>::kThreads)
     prolong_line<NF, NC, B::Y>(pm, c, [&](int i, T v) { s2[t >> 5][i][t & 31] = v; });
   }
   __syncthreads();
-  if (warp < q.fy && lane < q.fx) {  // z: the lane's column (x, y) of the fine nodes
-    const int xf = PF * nx + 1, yf = PF * ny + 1;
-    const int64_t o = PF * q.ex + lane + (int64_t)xf * (PF * q.ey + warp + (int64_t)yf * (PF * q.ez)),
-                  zs = (int64_t)xf * yf;
-    T c[C::CZ], x[C::FZ];
-#pragma unroll
-    for (int i = 0; i < C::FZ; ++i) x[i] = i < q.fz ? out[o + zs * i] : T(0);
+  if (col) {  // z
+    T c[C::CZ];
 #pragma unroll
     for (int k = 0; k < C::CZ; ++k) c[k] = s2[k][warp][lane];
     prolong_line<NF, NC, B::Z>(pm, c, [&](int i, T v) {
