@@ -146,10 +146,29 @@ def _check(rc: int, ctx=None):
     return rc
 
 
+class Context(_P):
+    """A sem_ctx handle with its node and element counts, fixed when it is created (the
+    array checks of every call need them)."""
+    ndofs = None
+    nelem = None
+
+
+def _ndofs(ctx) -> int:
+    n = getattr(ctx, "ndofs", None)
+    return sem_num_dofs(ctx) if n is None else n
+
+
+# the current stream's handle without the Stream object around it (a call on a small mesh
+# takes about as long on the host as that object's construction several times over)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream=None):
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return _P(stream.cuda_stream)
+    if stream is not None:
+        return _P(stream.cuda_stream)
+    if _raw_stream is not None:
+        return _P(_raw_stream(torch.cuda.current_device()))
+    return _P(torch.cuda.current_stream().cuda_stream)
 
 
 def _dev(t: torch.Tensor, dtype, n=None, name="tensor"):
@@ -173,9 +192,11 @@ def sem_create(nx, ny, nz, vertices, p, quad, device=0):
     v = np.ascontiguousarray(vertices, dtype=np.float64).reshape(-1)
     if v.size != (nx + 1) * (ny + 1) * (nz + 1) * 3:
         raise ValueError("vertices must hold (nx+1)(ny+1)(nz+1) points")
-    out = _P()
+    out = Context()
     rc = lib().sem_create(ctypes.byref(out), nx, ny, nz, v.ctypes.data_as(_DP), p, quad, device)
     _check(rc, None)
+    out.ndofs = sem_num_dofs(out)
+    out.nelem = sem_num_elements(out)
     return out
 
 
@@ -212,20 +233,20 @@ def sem_set_tissue(ctx, sigma_l, sigma_t, theta, stream=None):
 
 def sem_apply(ctx, alpha, beta, u, y, precision=SEM_PREC_FP64, stream=None):
     dt = torch.float64 if precision in (SEM_PREC_FP64, SEM_PREC_DF64) else torch.float32
-    n = sem_num_dofs(ctx)
+    n = _ndofs(ctx)
     return _check(lib().sem_apply(ctx, float(alpha), float(beta), _dev(u, dt, n, "u"),
                                   _dev(y, dt, n, "y"), int(precision), _stream(stream)), ctx)
 
 
 def sem_diagonal(ctx, alpha, beta, d, stream=None):
-    n = sem_num_dofs(ctx)
+    n = _ndofs(ctx)
     return _check(lib().sem_diagonal(ctx, float(alpha), float(beta), _dev(d, torch.float64, n, "d"),
                                      _stream(stream)), ctx)
 
 
 def sem_cg_solve(ctx, alpha, b, x, rtol, atol, maxit, precond=SEM_PC_JACOBI, stream=None,
                  raise_on_error=True):
-    n = sem_num_dofs(ctx)
+    n = _ndofs(ctx)
     it = _I()
     res = _D()
     rc = lib().sem_cg_solve(ctx, float(alpha), _dev(b, torch.float64, n, "b"),
@@ -258,13 +279,13 @@ def sem_state_destroy(st):
 
 
 def sem_state_set(ctx, st, u0, h0, stream=None):
-    n = sem_num_dofs(ctx)
+    n = _ndofs(ctx)
     return _check(lib().sem_state_set(st, _dev(u0, torch.float64, n, "u0"),
                                       _dev(h0, torch.float64, n, "h0"), _stream(stream)), ctx)
 
 
 def sem_state_get(ctx, st, u=None, u_prev=None, h=None, h_prev=None, stream=None):
-    n = sem_num_dofs(ctx)
+    n = _ndofs(ctx)
     nout = _I64()
     ptrs = [_dev(t, torch.float64, n, nm) if t is not None else _P()
             for t, nm in ((u, "u"), (u_prev, "u_prev"), (h, "h"), (h_prev, "h_prev"))]
@@ -325,7 +346,7 @@ def sem_state_track_activation(ctx, st, enable=True, stream=None):
 
 def sem_state_get_activation(ctx, st, tau, dudt_max, stream=None):
     """tau, dudt_max: float64 CUDA tensors of ndofs entries (or None)."""
-    n = sem_num_dofs(ctx)
+    n = _ndofs(ctx)
     t = _dev(tau, torch.float64, n, "tau") if tau is not None else None
     d = _dev(dudt_max, torch.float64, n, "dudt_max") if dudt_max is not None else None
     return _check(lib().sem_state_get_activation(st, t, d, _stream(stream)), ctx)
@@ -338,7 +359,7 @@ def sem_set_timing(ctx, enable: bool):
 def sem_apply_dot_static(ctx, alpha, beta, u, y, dot, stream=None):
     """y = alpha M u + beta K u and dot[0] = u . y with no allocation inside libsem
     (static device scratch; see include/sem.h)."""
-    n = sem_num_dofs(ctx)
+    n = _ndofs(ctx)
     return _check(lib().sem_apply_dot_static(ctx, float(alpha), float(beta),
                                              _dev(u, torch.float64, n, "u"),
                                              _dev(y, torch.float64, n, "y"),
@@ -369,7 +390,7 @@ def sem_set_gmg(ctx, degree=3, coarse_degree=10, min_coarse_dofs=2000, precision
 
 
 def sem_vcycle(ctx, alpha, r, z, stream=None):
-    n = sem_num_dofs(ctx)
+    n = _ndofs(ctx)
     return _check(lib().sem_vcycle(ctx, float(alpha), _dev(r, torch.float64, n, "r"),
                                    _dev(z, torch.float64, n, "z"), _stream(stream)), ctx)
 

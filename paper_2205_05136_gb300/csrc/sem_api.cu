@@ -319,7 +319,7 @@ int sem_set_tissue(sem_ctx* ctx, const double* sigma_l, const double* sigma_t,
   SEM_CK(setup_geometry(ctx->L, ctx->sigma_l, ctx->sigma_t, ctx->theta, ctx->d_flag, s));
   SEM_CK(setup_diagonals(ctx->L, s));
   ctx->ws.inv_alpha = -1.0;
-  gmg_free(ctx);  // coarse levels inherit the tissue: rebuilt on next use
+  gmg_tissue_changed(ctx);  // coarse levels inherit the tissue
   return SEM_OK;
 }
 

@@ -162,6 +162,7 @@ cudaError_t launch_operator(sem_ctx* ctx, const ApplyArgs64& a, cudaStream_t s);
 
 // Geometric multigrid (sem_gmg.cu).
 void gmg_free(sem_ctx* ctx);
+void gmg_tissue_changed(sem_ctx* ctx);  // the hierarchy is renewed on its next use
 int gmg_vcycle(sem_ctx* ctx, double alpha, const double* r, double* z, cudaStream_t s);
 int gmg_pcg(sem_ctx* ctx, double alpha, const double* b, double* x, double rtol, double atol,
             int maxit, int* iters, double* final_res, sem_stats* stats, cudaStream_t s,

@@ -61,30 +61,37 @@ struct LanczosScalars {
 struct Gmg {
   std::vector<GmgLevel> lv;
   double alpha = -1.0;
+  bool stale = false;  // the tissue changed: metrics, diagonals and estimates are renewed on the next use
   int precision = SEM_PREC_FP32;
   int degree = 3, coarse_degree = 10;
   double* z = nullptr;                                 // outer PCG preconditioned residual
   // CUDA graphs of the PCG set-up and of one PCG iteration (V-cycle included),
   // keyed by the solution pointer and alpha; captured on a private stream.
   struct Graphs {
+    bool used = false;
     const double* x = nullptr;
     const double* b = nullptr;
     double alpha = 0.0;
     double rtol = 0.0, atol = 0.0;
-    cudaGraphExec_t init = nullptr, iter = nullptr;
-    cudaGraphExec_t init_carried = nullptr;  // set-up from the carried A x (ws.Ax)
-    cudaGraphExec_t init_checked = nullptr;  // the same where ws.same reads nonzero, else applied
-    cudaGraphExec_t iter_timed = nullptr;    // an iteration with event nodes around two applies
-    int64_t init_kernels = 0, iter_kernels = 0, init_carried_kernels = 0, init_checked_kernels = 0;
-    int64_t iter_timed_kernels = 0;
-    int last_iters = 0;  // iterations the previous solve with these graphs took
-    // the set-up (variant v: applied, carried, checked) and its first `n` iterations
-    // (the first one timed when t = 1) as one graph: one launch where five were
-    struct Combo {
+    // one executable graph and its kernel count, captured when it is first launched
+    struct Exec {
       cudaGraphExec_t exec = nullptr;
-      int n = 0;
       int64_t kernels = 0;
-    } combo[3][2];
+    };
+    Exec init[3];     // the set-up: A x applied, carried (ws.Ax), carried where ws.same reads nonzero
+    Exec iter[2];     // an iteration; [1] with event nodes around two applies
+    int last_iters = 0;  // iterations the previous solve with these graphs took
+    // the set-up (variant v) and its first `n` iterations as one graph: one launch
+    // where n + 1 were.  Captured once two solves in a row took n iterations.
+    struct Combo : Exec {
+      int n = 0, seen = 0;
+    } combo[3];
+    void drop() {
+      for (Exec& e : init) if (e.exec) cudaGraphExecDestroy(e.exec);
+      for (Exec& e : iter) if (e.exec) cudaGraphExecDestroy(e.exec);
+      for (Combo& c : combo) if (c.exec) cudaGraphExecDestroy(c.exec);
+      *this = Graphs();
+    }
   };
   Graphs graphs[16];
   int next_graph = 0;
@@ -1467,16 +1474,7 @@ void free_gmg_struct(Gmg* g) {
     cudaFree(V.dinv64);
   }
   cudaFree(g->z);
-  for (auto& gr : g->graphs) {
-    if (gr.init) cudaGraphExecDestroy(gr.init);
-    if (gr.iter) cudaGraphExecDestroy(gr.iter);
-    if (gr.init_carried) cudaGraphExecDestroy(gr.init_carried);
-    if (gr.init_checked) cudaGraphExecDestroy(gr.init_checked);
-    if (gr.iter_timed) cudaGraphExecDestroy(gr.iter_timed);
-    for (auto& cv : gr.combo)
-      for (auto& c : cv)
-        if (c.exec) cudaGraphExecDestroy(c.exec);
-  }
+  for (auto& gr : g->graphs) gr.drop();
   if (g->capture) cudaStreamDestroy(g->capture);
   if (g->ev0) cudaEventDestroy(g->ev0);
   if (g->ev1) cudaEventDestroy(g->ev1);
@@ -1487,8 +1485,49 @@ void free_gmg_struct(Gmg* g) {
   delete g;
 }
 
+// The low-precision metrics of every level that the V-cycle reads.
+int level_metrics(sem_ctx* ctx, Gmg& g, cudaStream_t s) {
+  for (GmgLevel& V : g.lv) {
+    Level& L = *V.L;
+    if (g.precision == SEM_PREC_FP32 && !L.metric32_valid) {
+      if (!L.metric32) GMG_CK(cudaMalloc(&L.metric32, sizeof(float) * metric_lowp_count(L)));
+      GMG_CK(setup_metric_lowp(L, false, s));
+    }
+    const bool tc = g.precision == SEM_PREC_BF16_TC && tc_supported(L) && !ctx->deterministic;
+    if ((g.precision == SEM_PREC_FP32_BF16 || (g.precision == SEM_PREC_BF16_TC && !tc)) &&
+        !L.metric16_valid) {
+      if (!L.metric16) GMG_CK(cudaMalloc(&L.metric16, sizeof(__nv_bfloat16) * metric_lowp_count(L)));
+      GMG_CK(setup_metric_lowp(L, true, s));
+    }
+    if (tc && !L.metric_tc_valid) GMG_CK(setup_metric_tc(L, s));
+  }
+  return SEM_OK;
+}
+
+// New tissue on a standing hierarchy: the coarse levels' tissue, metrics and diagonals
+// (the fine level's are sem_set_tissue's), the estimates (alpha = -1) and the graphs,
+// whose launches hold the smoother's coefficients.
+int refresh(sem_ctx* ctx, Gmg& g, cudaStream_t s) {
+  for (auto& gr : g.graphs) gr.drop();
+  g.alpha = -1.0;
+  for (size_t l = 1; l < g.lv.size(); ++l) {
+    GmgLevel &F = g.lv[l - 1], &V = g.lv[l];
+    Level& L = *V.L;
+    if (V.owns_tissue) {
+      launch_k(k_coarse_tissue, grid1d(L.nelem), kThreads, 0, s, L.nx, L.ny, L.nz, F.L->nx, F.L->ny, F.sl, F.st, F.th,
+               V.sl, V.st, V.th);
+      GMG_CK(cudaGetLastError());
+    }
+    GMG_CK(setup_geometry(L, V.sl, V.st, V.th, ctx->d_flag, s));
+    GMG_CK(setup_diagonals(L, s));
+  }
+  const int rc = level_metrics(ctx, g, s);
+  if (rc == SEM_OK) g.stale = false;
+  return rc;
+}
+
 int build(sem_ctx* ctx, cudaStream_t s) {
-  if (ctx->gmg) return SEM_OK;
+  if (ctx->gmg) return ctx->gmg->stale ? refresh(ctx, *ctx->gmg, s) : SEM_OK;
   GMG_CK(prime_coarse());
   Gmg* g = new Gmg();
   g->precision = ctx->gmg_precision;
@@ -1560,22 +1599,12 @@ int build(sem_ctx* ctx, cudaStream_t s) {
   GMG_CK(cudaMemcpyAsync(&bad, ctx->d_flag, sizeof(int), cudaMemcpyDeviceToHost, s));
   GMG_CK(cudaStreamSynchronize(s));
   if (bad) return fail(ctx, SEM_ERR_BAD_MESH, "a coarsened multigrid level has an inverted element");
+  if (const int rc = level_metrics(ctx, *g, s); rc != SEM_OK) return rc;
   const size_t es = elem_size(g->precision);
   int64_t nmax = 0;
   for (GmgLevel& V : g->lv) {
     Level& L = *V.L;
     nmax = std::max(nmax, L.ndofs);
-    if (g->precision == SEM_PREC_FP32 && !L.metric32_valid) {
-      if (!L.metric32) GMG_CK(cudaMalloc(&L.metric32, sizeof(float) * metric_lowp_count(L)));
-      GMG_CK(setup_metric_lowp(L, false, s));
-    }
-    const bool tc = g->precision == SEM_PREC_BF16_TC && tc_supported(L) && !ctx->deterministic;
-    if ((g->precision == SEM_PREC_FP32_BF16 || (g->precision == SEM_PREC_BF16_TC && !tc)) &&
-        !L.metric16_valid) {
-      if (!L.metric16) GMG_CK(cudaMalloc(&L.metric16, sizeof(__nv_bfloat16) * metric_lowp_count(L)));
-      GMG_CK(setup_metric_lowp(L, true, s));
-    }
-    if (tc && !L.metric_tc_valid) GMG_CK(setup_metric_tc(L, s));
     void** vecs[] = {&V.r, &V.x, &V.d, &V.invd};
     for (void** v : vecs) GMG_CK(cudaMalloc(v, es * L.ndofs));
     GMG_CK(cudaMalloc(&V.dinv64, sizeof(double) * L.ndofs));
@@ -1704,94 +1733,45 @@ int pcg_iter_seq(sem_ctx* ctx, Gmg& g, double alpha, double* x, bool timed, cuda
   return SEM_OK;
 }
 
-// Captures (once per solution pointer, right-hand side, alpha and tolerances) the
-// set-up and iteration sequences as CUDA graphs; sixteen are cached.
-template <typename T>
-int get_graphs(sem_ctx* ctx, Gmg& g, double alpha, const double* b, double* x, double rtol,
-               double atol, Gmg::Graphs** out) {
+// The graphs of one solution pointer, right-hand side, alpha and tolerances (all baked
+// into the captured launches); sixteen are cached.
+Gmg::Graphs& get_graphs(Gmg& g, double alpha, const double* b, double* x, double rtol, double atol) {
   for (auto& gr : g.graphs)
-    if (gr.iter && gr.x == x && gr.b == b && gr.alpha == alpha && gr.rtol == rtol && gr.atol == atol) {
-      *out = &gr;
-      return SEM_OK;
-    }
+    if (gr.used && gr.x == x && gr.b == b && gr.alpha == alpha && gr.rtol == rtol && gr.atol == atol) return gr;
   Gmg::Graphs& gr = g.graphs[g.next_graph];
   g.next_graph = (g.next_graph + 1) % 16;
-  if (gr.init) { cudaGraphExecDestroy(gr.init); gr.init = nullptr; }
-  if (gr.iter) { cudaGraphExecDestroy(gr.iter); gr.iter = nullptr; }
-  if (gr.init_carried) { cudaGraphExecDestroy(gr.init_carried); gr.init_carried = nullptr; }
-  if (gr.init_checked) { cudaGraphExecDestroy(gr.init_checked); gr.init_checked = nullptr; }
-  if (gr.iter_timed) { cudaGraphExecDestroy(gr.iter_timed); gr.iter_timed = nullptr; }
-  for (auto& cv : gr.combo)
-    for (auto& c : cv) {
-      if (c.exec) cudaGraphExecDestroy(c.exec);
-      c = Gmg::Graphs::Combo();
-    }
-  cudaStream_t cs = g.capture;
-  const int64_t l0 = ctx->launches;
-  for (int which = 0; which < 5; ++which) {
-    GMG_CK(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-    int rc = (which == 1 || which == 4) ? pcg_iter_seq<T>(ctx, g, alpha, x, which == 4, cs)
-                                        : pcg_init_seq<T>(ctx, g, alpha, b, x, rtol, atol, which >= 2,
-                                                          which == 3 ? ctx->ws.same : nullptr, cs);
-    cudaGraph_t graph = nullptr;
-    const cudaError_t ec = cudaStreamEndCapture(cs, &graph);
-    if (rc != SEM_OK) {
-      if (graph) cudaGraphDestroy(graph);
-      return rc;
-    }
-    if (ec != cudaSuccess) return cuda_fail(ctx, ec, "cudaStreamEndCapture");
-    cudaGraphExec_t exec = nullptr;
-    const cudaError_t ei = cudaGraphInstantiate(&exec, graph, 0);
-    const int64_t nk = count_kernels(graph);
-    cudaGraphDestroy(graph);
-    if (ei != cudaSuccess) return cuda_fail(ctx, ei, "cudaGraphInstantiate");
-    if (which == 0) { gr.init = exec; gr.init_kernels = nk; }
-    else if (which == 1) { gr.iter = exec; gr.iter_kernels = nk; }
-    else if (which == 2) { gr.init_carried = exec; gr.init_carried_kernels = nk; }
-    else if (which == 3) { gr.init_checked = exec; gr.init_checked_kernels = nk; }
-    else { gr.iter_timed = exec; gr.iter_timed_kernels = nk; }
-  }
-  ctx->launches = l0;  // capture launched nothing; replays are counted
+  gr.drop();
+  gr.used = true;
   gr.x = x;
   gr.b = b;
   gr.alpha = alpha;
-  gr.rtol = rtol;  // the stopping tolerances are baked into the set-up graph
+  gr.rtol = rtol;
   gr.atol = atol;
-  *out = &gr;
-  return SEM_OK;
+  return gr;
 }
 
-// The combined graph of set-up variant v and n iterations (the first timed when
-// timed), captured on first use and again when n changes.
-template <typename T>
-int get_combo(sem_ctx* ctx, Gmg& g, Gmg::Graphs& gr, int v, bool timed, int n, double alpha, const double* b,
-              double* x, double rtol, double atol, Gmg::Graphs::Combo** out) {
-  Gmg::Graphs::Combo& c = gr.combo[v][timed ? 1 : 0];
-  if (c.exec == nullptr || c.n != n) {
-    if (c.exec) { cudaGraphExecDestroy(c.exec); c = Gmg::Graphs::Combo(); }
-    cudaStream_t cs = g.capture;
-    const int64_t l0 = ctx->launches;
-    GMG_CK(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-    int rc = pcg_init_seq<T>(ctx, g, alpha, b, x, rtol, atol, v >= 1, v == 2 ? ctx->ws.same : nullptr, cs);
-    for (int i = 0; i < n && rc == SEM_OK; ++i) rc = pcg_iter_seq<T>(ctx, g, alpha, x, timed && i == 0, cs);
-    cudaGraph_t graph = nullptr;
-    const cudaError_t ec = cudaStreamEndCapture(cs, &graph);
-    ctx->launches = l0;
-    if (rc != SEM_OK) {
-      if (graph) cudaGraphDestroy(graph);
-      return rc;
-    }
-    if (ec != cudaSuccess) return cuda_fail(ctx, ec, "cudaStreamEndCapture");
-    const cudaError_t ei = cudaGraphInstantiate(&c.exec, graph, 0);
-    c.kernels = count_kernels(graph);
-    cudaGraphDestroy(graph);
-    if (ei != cudaSuccess) {
-      c.exec = nullptr;
-      return cuda_fail(ctx, ei, "cudaGraphInstantiate");
-    }
-    c.n = n;
+// Captures what seq issues on the private stream into e.
+template <typename F>
+int capture(sem_ctx* ctx, Gmg& g, Gmg::Graphs::Exec& e, F seq) {
+  cudaStream_t cs = g.capture;
+  const int64_t l0 = ctx->launches;
+  GMG_CK(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
+  const int rc = seq(cs);
+  cudaGraph_t graph = nullptr;
+  const cudaError_t ec = cudaStreamEndCapture(cs, &graph);
+  ctx->launches = l0;  // capture launched nothing; replays are counted
+  if (rc != SEM_OK) {
+    if (graph) cudaGraphDestroy(graph);
+    return rc;
   }
-  *out = &c;
+  if (ec != cudaSuccess) return cuda_fail(ctx, ec, "cudaStreamEndCapture");
+  cudaGraphExec_t exec = nullptr;
+  const cudaError_t ei = cudaGraphInstantiate(&exec, graph, 0);
+  const int64_t nk = count_kernels(graph);
+  cudaGraphDestroy(graph);
+  if (ei != cudaSuccess) return cuda_fail(ctx, ei, "cudaGraphInstantiate");
+  e.exec = exec;
+  e.kernels = nk;
   return SEM_OK;
 }
 
@@ -1800,35 +1780,54 @@ int pcg_t(sem_ctx* ctx, Gmg& g, double alpha, const double* b, double* x, double
           double atol, int maxit, int* iters, double* final_res, sem_stats* stats, bool carried,
           bool checked, cudaStream_t s) {
   Workspace& w = ctx->ws;
-  Gmg::Graphs* gr = nullptr;
-  int rc = get_graphs<T>(ctx, g, alpha, b, x, rtol, atol, &gr);
-  if (rc != SEM_OK) return rc;
+  Gmg::Graphs& gr = get_graphs(g, alpha, b, x, rtol, atol);
   Timing& tm = ctx->timing;
   bool done_h = false;
   int launched = 0;
   // with timing on, the first iteration of one solve in kTimingEvery is the timed one
   bool sample = tm.enabled && (tm.solves++ % kTimingEvery) == 0;
-  auto launch_iter = [&]() -> cudaError_t {
-    const bool timed = sample && launched == 0;
-    const cudaError_t e = cudaGraphLaunch(timed ? gr->iter_timed : gr->iter, s);
-    ctx->launches += timed ? gr->iter_timed_kernels : gr->iter_kernels;
-    return e;
-  };
-  // Successive solves (time steps) take about the same number of iterations:
-  // the set-up and the previous count go out as one graph before the scalars are
-  // read, so that a solve that needs no more costs one launch and one host round
-  // trip.  An iteration launched after convergence runs kernels that return at once.
-  const int ahead = std::min(maxit, std::max(0, gr->last_iters));
   const int variant = !carried ? 0 : (checked ? 2 : 1);
-  if (ahead > 0) {
-    Gmg::Graphs::Combo* c = nullptr;
-    if ((rc = get_combo<T>(ctx, g, *gr, variant, sample, ahead, alpha, b, x, rtol, atol, &c)) != SEM_OK) return rc;
-    GMG_CK(cudaGraphLaunch(c->exec, s));
-    ctx->launches += c->kernels;
+  auto seq_init = [&](cudaStream_t cs) {
+    return pcg_init_seq<T>(ctx, g, alpha, b, x, rtol, atol, variant >= 1, variant == 2 ? w.same : nullptr, cs);
+  };
+  auto launch = [&](Gmg::Graphs::Exec& e, auto seq) -> int {
+    if (e.exec == nullptr) {
+      const int rc = capture(ctx, g, e, seq);
+      if (rc != SEM_OK) return rc;
+    }
+    GMG_CK(cudaGraphLaunch(e.exec, s));
+    ctx->launches += e.kernels;
+    return SEM_OK;
+  };
+  auto launch_iter = [&]() -> int {
+    const bool timed = sample && launched == 0;
+    return launch(gr.iter[timed ? 1 : 0], [&](cudaStream_t cs) { return pcg_iter_seq<T>(ctx, g, alpha, x, timed, cs); });
+  };
+  // Successive solves (time steps) take about the same number of iterations: the
+  // set-up and the previous count go out before the scalars are read, as one graph
+  // once the count has repeated, so that a solve that needs no more costs one launch
+  // and one host round trip.  An iteration launched after convergence runs kernels
+  // that return at once.
+  const int ahead = std::min(maxit, std::max(0, gr.last_iters));
+  Gmg::Graphs::Combo& c = gr.combo[variant];
+  if (c.n != ahead) {
+    if (c.exec) cudaGraphExecDestroy(c.exec);
+    c = Gmg::Graphs::Combo();
+    c.n = ahead;
+  }
+  int rc;
+  if (ahead > 0 && !sample && (c.exec != nullptr || c.seen++ > 0)) {
+    rc = launch(c, [&](cudaStream_t cs) {
+      int r = seq_init(cs);
+      for (int i = 0; i < ahead && r == SEM_OK; ++i) r = pcg_iter_seq<T>(ctx, g, alpha, x, false, cs);
+      return r;
+    });
+    if (rc != SEM_OK) return rc;
     launched = ahead;
   } else {
-    GMG_CK(cudaGraphLaunch(variant == 0 ? gr->init : (variant == 2 ? gr->init_checked : gr->init_carried), s));
-    ctx->launches += variant == 0 ? gr->init_kernels : (variant == 2 ? gr->init_checked_kernels : gr->init_carried_kernels);
+    if ((rc = launch(gr.init[variant], seq_init)) != SEM_OK) return rc;
+    for (; launched < ahead; ++launched)
+      if ((rc = launch_iter()) != SEM_OK) return rc;
   }
   while (true) {
     GMG_CK(cudaMemcpyAsync(w.cg_host, w.cg, sizeof(CgScalars), cudaMemcpyDeviceToHost, s));
@@ -1858,11 +1857,11 @@ int pcg_t(sem_ctx* ctx, Gmg& g, double alpha, const double* b, double* x, double
     }
     if (w.cg_host->done) { done_h = true; break; }
     if (launched >= maxit) break;
-    GMG_CK(launch_iter());
+    if ((rc = launch_iter()) != SEM_OK) return rc;
     ++launched;
   }
   const CgScalars& h = *w.cg_host;
-  gr->last_iters = h.iters;
+  gr.last_iters = h.iters;
   if (iters) *iters = h.iters;
   if (final_res) *final_res = std::sqrt(h.rr);
   if (stats) {
@@ -1878,6 +1877,10 @@ int pcg_t(sem_ctx* ctx, Gmg& g, double alpha, const double* b, double* x, double
 }
 
 }  // namespace
+
+void gmg_tissue_changed(sem_ctx* ctx) {
+  if (ctx->gmg) ctx->gmg->stale = true;
+}
 
 void gmg_free(sem_ctx* ctx) {
   if (ctx->gmg) {

@@ -1,4 +1,4 @@
-"""The coarsest multigrid level's smoother in one CTA, at the edges of its range.
+"""Coarse multigrid levels: the one-CTA smoother at the edges of its range, h-transfers, new tissue.
 
 It takes a Q_1 level of at most 1024 nodes whose metric fits in shared memory: levels of a few
 nodes, of one element, near 1024 nodes (taken), above (the launch-per-step path), thin ones, and
@@ -61,3 +61,39 @@ def test_h_transfers_odd_and_even(dims):
     ref = H.vcycle(r)
     assert np.linalg.norm(z.cpu().numpy() - ref) / np.linalg.norm(ref) < 1e-10
     g.close()
+
+
+@pytest.mark.parametrize("precision,tol", [(capi.SEM_PREC_FP64, 1e-12), (capi.SEM_PREC_FP32, 1e-6),
+                                           (capi.SEM_PREC_FP32_BF16, 1e-6), (capi.SEM_PREC_BF16_TC, 2e-6)])
+def test_hierarchy_follows_new_tissue(precision, tol):
+    """A standing hierarchy (p- and h-levels, captured solves) after sem_set_tissue is that of a context made
+    with the new tissue: the same V-cycle up to the order of the atomic sums, and the same solution."""
+    dims, p = (9, 5, 4), 4
+    s = W.slab(*dims, (20.0, 7.0, 3.0), perturb=0.1, seed=1)
+    ne = s.n_elements
+    rng = np.random.default_rng(5)
+    old = (np.full(ne, 0.12), np.full(ne, 0.03), W.transmural_fiber_angles(s))
+    new = (0.2 * rng.uniform(0.8, 1.2, ne), 0.05 * rng.uniform(0.8, 1.2, ne), -W.transmural_fiber_angles(s))
+    out = []
+    for first in (old, new):
+        g = gb.Slab(s.flat_vertices(), *dims, p, "LGL")
+        g.set_tissue(*first)
+        capi.sem_set_gmg(g.ctx, 3, 6, 60, precision)
+        r = torch.tensor(W.uniform_vector(g.ndofs, -1.0, 1.0, seed=3), device="cuda")
+        x = torch.zeros_like(r)
+        if first is old:
+            for _ in range(4):  # captures the set-up, an iteration, and both as one graph
+                x.zero_()
+                g.cg_solve(ALPHA, r, x, rtol=1e-12, precond=capi.SEM_PC_GMG)
+            g.set_tissue(*new)
+        z = torch.empty_like(r)
+        capi.sem_vcycle(g.ctx, ALPHA, r, z)
+        x.zero_()
+        it, _ = g.cg_solve(ALPHA, r, x, rtol=1e-12, precond=capi.SEM_PC_GMG)
+        out.append((z, x.clone(), it, capi.sem_gmg_info(g.ctx, ALPHA)["lambda_max"]))
+        g.close()
+    (z0, x0, it0, l0), (z1, x1, it1, l1) = out
+    assert np.allclose(l0, l1, rtol=1e-12, atol=0)
+    assert float(torch.linalg.norm(z0 - z1) / torch.linalg.norm(z1)) < tol
+    assert float(torch.linalg.norm(x0 - x1) / torch.linalg.norm(x1)) < 1e-10
+    assert abs(it0 - it1) <= 1
