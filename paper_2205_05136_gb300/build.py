@@ -29,6 +29,7 @@ SOURCES = [
     "sem_apply_fp32.cu",
     "sem_apply_df64.cu",
     "sem_solver.cu",
+    "sem_cg_small.cu",
     "sem_api.cu",
     "sem_noalloc.cu",
     "sem_apply_tc.cu",

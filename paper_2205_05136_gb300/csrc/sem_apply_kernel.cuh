@@ -168,12 +168,12 @@ __device__ __forceinline__ void eo_line(const EoMat<N, T>& M, const T (&in)[N], 
   }
 }
 
-// dst = M along DIR of src (ACC: dst += ...), for every line of the E element
-// tiles (thread tid of a group of nth threads).  src may equal dst.
-template <int N, int E, int DIR, bool ANTI, bool ACC, typename T>
-__device__ __forceinline__ void sweep(const EoMat<N, T>& M, const T* src, T* dst, int tid, int nth) {
+// dst = M along DIR of src (ACC: dst += ...), for every line of ne element tiles
+// (thread tid of a group of nth threads).  src may equal dst.
+template <int N, int DIR, bool ANTI, bool ACC, typename T>
+__device__ __forceinline__ void sweep(const EoMat<N, T>& M, const T* src, T* dst, int ne, int tid, int nth) {
   constexpr int N2 = N * N, N3 = N2 * N;
-  for (int w = tid; w < E * N2; w += nth) {
+  for (int w = tid; w < ne * N2; w += nth) {
     const int s = w / N2, l = w - s * N2;
     int base, stride;
     line_geom<N, DIR>(l, base, stride);
@@ -194,11 +194,11 @@ __device__ __forceinline__ void sweep(const EoMat<N, T>& M, const T* src, T* dst
 
 // The same along a direction known at run time (one copy of the code for several
 // directions).
-template <int N, int E, bool ANTI, bool ACC, typename T>
-__device__ __forceinline__ void sweep_dir(const EoMat<N, T>& M, const T* src, T* dst, int dir, int tid, int nth) {
+template <int N, bool ANTI, bool ACC, typename T>
+__device__ __forceinline__ void sweep_dir(const EoMat<N, T>& M, const T* src, T* dst, int dir, int ne, int tid, int nth) {
   constexpr int N2 = N * N, N3 = N2 * N;
   const int stride = dir == 0 ? 1 : dir == 1 ? N : N2;
-  for (int w = tid; w < E * N2; w += nth) {
+  for (int w = tid; w < ne * N2; w += nth) {
     const int s = w / N2, l = w - s * N2;
     const int base = s * N3 + (dir == 0 ? l * N : dir == 1 ? (l / N) * N2 + l % N : l);
     T in[N], out[N];
@@ -281,6 +281,114 @@ __host__ __device__ constexpr size_t apply_warp_tile_bytes() {
   return (size_t)3 * kWarpsPerCta * WarpCfg<P>::G * (P + 1) * (P + 1) * (P + 1) * sizeof(T);
 }
 
+// The element results (mass M_e + K_e) u_e (MASS_ONLY: mass M_e u_e) of ne element
+// tiles, from the gathered values in sA into sA; sB, sC scratch of the same size.  Tile
+// s is element e0 + s, and those from e_end on have no metric (their values are zero).
+template <int P, int QUAD, bool MASS_ONLY, bool ROLLED, bool WARP, typename T, typename MT>
+__device__ __forceinline__ void element_results(const KTab<P + 1, T>& tab, const MT* metric, T mass, int e0, int e_end,
+                                                int ne, T* sA, T* sB, T* sC, int tid, int nth) {
+  constexpr int N = P + 1, N2 = N * N, N3 = N2 * N;
+  using ML = MetricLayout<MT>;
+  auto group_sync = [] {
+    if (WARP) __syncwarp(); else __syncthreads();
+  };
+  if (QUAD == SEM_QUAD_LG) {  // values at the Gauss points
+    if constexpr (ROLLED) {
+#pragma unroll 1
+      for (int d = 0; d < 3; ++d) {
+        sweep_dir<N, false, false>(tab.Bi, sA, sA, d, ne, tid, nth);
+        group_sync();
+      }
+    } else {
+      sweep<N, 0, false, false>(tab.Bi, sA, sB, ne, tid, nth);
+      group_sync();
+      sweep<N, 1, false, false>(tab.Bi, sB, sC, ne, tid, nth);
+      group_sync();
+      sweep<N, 2, false, false>(tab.Bi, sC, sA, ne, tid, nth);
+      group_sync();
+    }
+  }
+
+  if (MASS_ONLY) {
+    for (int idx = tid; idx < ne * N3; idx += nth) {
+      const int s = idx / N3, loc = idx - s * N3, e = e0 + s;
+      if (e < e_end) {
+        const T W = ldmetric(metric + ML::offset(N, e, loc % N2, loc / N2, 6));
+        sA[idx] = (mass * W) * sA[idx];
+      }
+    }
+    group_sync();
+  } else {
+    // reference gradient along x and y (into sB, sC)
+    if constexpr (ROLLED) {
+#pragma unroll 1
+      for (int d = 0; d < 2; ++d) sweep_dir<N, true, false>(tab.D, sA, d == 0 ? sB : sC, d, ne, tid, nth);
+    } else {
+      sweep<N, 0, true, false>(tab.D, sA, sB, ne, tid, nth);
+      sweep<N, 1, true, false>(tab.D, sA, sC, ne, tid, nth);
+    }
+    group_sync();
+    // z-gradient, quadrature-point stage and transposed z-sweep on the columns
+    for (int w = tid; w < ne * N2; w += nth) {
+      const int s = w / N2, c = w - s * N2, e = e0 + s;
+      if (e >= e_end) continue;
+      T* pa = sA + s * N3 + c;
+      T* pb = sB + s * N3 + c;
+      T* pc = sC + s * N3 + c;
+      T uz[N], g3[N], q3[N], m[N];
+#pragma unroll
+      for (int k = 0; k < N; ++k) uz[k] = pa[k * N2];
+      eo_line<N, true, false>(tab.D, uz, g3);
+      const MT* mp = metric + ML::offset(N, e, c, 0, 0);  // component-major, point by point
+#pragma unroll
+      for (int k = 0; k < N; ++k) {
+        const T g1 = pb[k * N2], g2 = pc[k * N2];
+        T gm[kMetricComps];
+#pragma unroll
+        for (int cc = 0; cc < kMetricComps; ++cc) gm[cc] = ldmetric(mp + k * N2 + cc * padded_n3(N));
+        const T G00 = gm[0], G01 = gm[1], G02 = gm[2], G11 = gm[3], G12 = gm[4], G22 = gm[5], W = gm[6];
+        pb[k * N2] = fma(G02, g3[k], fma(G01, g2, G00 * g1));
+        pc[k * N2] = fma(G12, g3[k], fma(G11, g2, G01 * g1));
+        q3[k] = fma(G22, g3[k], fma(G12, g2, G02 * g1));
+        m[k] = (mass * W) * uz[k];
+      }
+      eo_line<N, true, true>(tab.Dt, q3, m);
+#pragma unroll
+      for (int k = 0; k < N; ++k) pa[k * N2] = m[k];
+    }
+    group_sync();
+    if constexpr (ROLLED) {
+#pragma unroll 1
+      for (int d = 1; d >= 0; --d) {
+        sweep_dir<N, true, true>(tab.Dt, d == 0 ? sB : sC, sA, d, ne, tid, nth);
+        group_sync();
+      }
+    } else {
+      sweep<N, 1, true, true>(tab.Dt, sC, sA, ne, tid, nth);
+      group_sync();
+      sweep<N, 0, true, true>(tab.Dt, sB, sA, ne, tid, nth);
+      group_sync();
+    }
+  }
+
+  if (QUAD == SEM_QUAD_LG) {  // back from the Gauss points to the nodes
+    if constexpr (ROLLED) {
+#pragma unroll 1
+      for (int d = 0; d < 3; ++d) {
+        sweep_dir<N, false, false>(tab.Bit, sA, sA, d, ne, tid, nth);
+        group_sync();
+      }
+    } else {
+      sweep<N, 0, false, false>(tab.Bit, sA, sB, ne, tid, nth);
+      group_sync();
+      sweep<N, 1, false, false>(tab.Bit, sB, sC, ne, tid, nth);
+      group_sync();
+      sweep<N, 2, false, false>(tab.Bit, sC, sA, ne, tid, nth);
+      group_sync();
+    }
+  }
+}
+
 // The double-float kernel at p = 4 (the outer operator of the benchmark's mixed
 // step) is bound by issue and memory latency: 10 CTAs per SM at 48 registers, with
 // small spills (8 measure the same in the plain apply, 1 % slower with the inner
@@ -291,7 +399,7 @@ __global__ void __launch_bounds__(MASS_ONLY ? kApplyThreads : ApplyCta<P, T, DOT
                                       ? 5 * kApplyThreads / ApplyCta<P, T, DOT>::kThreads : 1)
     sem_apply_kernel(const ApplyArgs<T, MT> a, const __grid_constant__ KTab<P + 1, T> tab) {
   static_assert(!(WARP && DOT), "the fused inner product needs the CTA-wide mode");
-  constexpr int N = P + 1, N2 = N * N, N3 = N2 * N;
+  constexpr int N = P + 1, N3 = N * N * N;
   using ML = MetricLayout<MT>;
   constexpr int E = WARP ? WarpCfg<P>::G : MASS_ONLY ? ApplyCfg<P>::E : ApplyCta<P, T, DOT>::E;
   // One copy of the sweep code for the directions: double-float at p = 4 (85 -> 80 us,
@@ -370,101 +478,7 @@ __global__ void __launch_bounds__(MASS_ONLY ? kApplyThreads : ApplyCta<P, T, DOT
   }
   group_sync();
 
-  if (QUAD == SEM_QUAD_LG) {  // values at the Gauss points
-    if constexpr (kRolled) {
-#pragma unroll 1
-      for (int d = 0; d < 3; ++d) {
-        sweep_dir<N, E, false, false>(tab.Bi, sA, sA, d, tid, nth);
-        group_sync();
-      }
-    } else {
-      sweep<N, E, 0, false, false>(tab.Bi, sA, sB, tid, nth);
-      group_sync();
-      sweep<N, E, 1, false, false>(tab.Bi, sB, sC, tid, nth);
-      group_sync();
-      sweep<N, E, 2, false, false>(tab.Bi, sC, sA, tid, nth);
-      group_sync();
-    }
-  }
-
-  if (MASS_ONLY) {
-    for (int idx = tid; idx < E * N3; idx += nth) {
-      const int s = idx / N3, loc = idx - s * N3, e = e0 + s;
-      if (e < a.nelem) {
-        const T W = ldmetric(a.metric + ML::offset(N, e, loc % N2, loc / N2, 6));
-        sA[idx] = (a.mass_coef * W) * sA[idx];
-      }
-    }
-    group_sync();
-  } else {
-    // reference gradient along x and y (into sB, sC)
-    if constexpr (kRolled) {
-#pragma unroll 1
-      for (int d = 0; d < 2; ++d) sweep_dir<N, E, true, false>(tab.D, sA, d == 0 ? sB : sC, d, tid, nth);
-    } else {
-      sweep<N, E, 0, true, false>(tab.D, sA, sB, tid, nth);
-      sweep<N, E, 1, true, false>(tab.D, sA, sC, tid, nth);
-    }
-    group_sync();
-    // z-gradient, quadrature-point stage and transposed z-sweep on the columns
-    for (int w = tid; w < E * N2; w += nth) {
-      const int s = w / N2, c = w - s * N2, e = e0 + s;
-      if (e >= a.nelem) continue;
-      T* pa = sA + s * N3 + c;
-      T* pb = sB + s * N3 + c;
-      T* pc = sC + s * N3 + c;
-      T uz[N], g3[N], q3[N], m[N];
-#pragma unroll
-      for (int k = 0; k < N; ++k) uz[k] = pa[k * N2];
-      eo_line<N, true, false>(tab.D, uz, g3);
-      const MT* mp = a.metric + ML::offset(N, e, c, 0, 0);  // component-major, point by point
-#pragma unroll
-      for (int k = 0; k < N; ++k) {
-        const T g1 = pb[k * N2], g2 = pc[k * N2];
-        T gm[kMetricComps];
-#pragma unroll
-        for (int cc = 0; cc < kMetricComps; ++cc) gm[cc] = ldmetric(mp + k * N2 + cc * padded_n3(N));
-        const T G00 = gm[0], G01 = gm[1], G02 = gm[2], G11 = gm[3], G12 = gm[4], G22 = gm[5], W = gm[6];
-        pb[k * N2] = fma(G02, g3[k], fma(G01, g2, G00 * g1));
-        pc[k * N2] = fma(G12, g3[k], fma(G11, g2, G01 * g1));
-        q3[k] = fma(G22, g3[k], fma(G12, g2, G02 * g1));
-        m[k] = (a.mass_coef * W) * uz[k];
-      }
-      eo_line<N, true, true>(tab.Dt, q3, m);
-#pragma unroll
-      for (int k = 0; k < N; ++k) pa[k * N2] = m[k];
-    }
-    group_sync();
-    if constexpr (kRolled) {
-#pragma unroll 1
-      for (int d = 1; d >= 0; --d) {
-        sweep_dir<N, E, true, true>(tab.Dt, d == 0 ? sB : sC, sA, d, tid, nth);
-        group_sync();
-      }
-    } else {
-      sweep<N, E, 1, true, true>(tab.Dt, sC, sA, tid, nth);
-      group_sync();
-      sweep<N, E, 0, true, true>(tab.Dt, sB, sA, tid, nth);
-      group_sync();
-    }
-  }
-
-  if (QUAD == SEM_QUAD_LG) {  // back from the Gauss points to the nodes
-    if constexpr (kRolled) {
-#pragma unroll 1
-      for (int d = 0; d < 3; ++d) {
-        sweep_dir<N, E, false, false>(tab.Bit, sA, sA, d, tid, nth);
-        group_sync();
-      }
-    } else {
-      sweep<N, E, 0, false, false>(tab.Bit, sA, sB, tid, nth);
-      group_sync();
-      sweep<N, E, 1, false, false>(tab.Bit, sB, sC, tid, nth);
-      group_sync();
-      sweep<N, E, 2, false, false>(tab.Bit, sC, sA, tid, nth);
-      group_sync();
-    }
-  }
+  element_results<P, QUAD, MASS_ONLY, kRolled, WARP>(tab, a.metric, a.mass_coef, e0, a.nelem, E, sA, sB, sC, tid, nth);
 
   pdl_trigger();
   // scatter-add y += P_e^T y_e, and with DOT the partial u_e . y_e

@@ -335,6 +335,14 @@ cudaError_t setup_node_coords(Level& L, cudaStream_t s);
 cudaError_t setup_region_mask(const Level& L, int region, const double* prm, double* mask,
                               cudaStream_t s);
 
+// CG of a small mesh in one kernel (sem_cg_small.cu): the solve of cg_solve with the FP64
+// operator, inv = 1 / diagonal or nullptr.  At most 64 iterations a launch; resume
+// continues from x, r, p and *sc.  p and Ap are scratch.
+bool cg_small_fits(const Level& L);
+cudaError_t launch_cg_small(const Level& L, double alpha, const double* b, const double* inv, const double* ax0, double* x,
+                            double* r, double* p, double* Ap, CgScalars* sc, double rtol, double atol, int maxit,
+                            bool resume, cudaStream_t s);
+
 // Vector kernels (sem_solver.cu).
 int vec_blocks(int64_t n);
 cudaError_t vec_axpby_diag(int64_t n, double a, const double* x, double b, const double* y,

@@ -652,6 +652,24 @@ int apply_tc(sem_ctx* ctx, double alpha, double beta, const float* u, float* y, 
   return SEM_OK;
 }
 
+// Reports the solve whose scalars the host has read.
+static int cg_result(sem_ctx* ctx, bool done, int maxit, int* iters, double* final_res, sem_stats* stats) {
+  const CgScalars& h = *ctx->ws.cg_host;
+  if (iters) *iters = h.iters;
+  if (final_res) *final_res = std::sqrt(h.rr);
+  if (stats) {
+    stats->cg_iters += h.iters;
+    stats->last_residual = std::sqrt(h.rr);
+  }
+  if (h.status == SEM_ERR_NONFINITE)
+    return fail(ctx, SEM_ERR_NONFINITE, "non-finite value in a CG inner product");
+  if (!done)
+    return fail(ctx, SEM_ERR_NOT_CONVERGED,
+                "CG did not converge in " + std::to_string(maxit) + " iterations (|r| = " +
+                    std::to_string(std::sqrt(h.rr)) + ")");
+  return SEM_OK;
+}
+
 int cg_solve(sem_ctx* ctx, double alpha, const double* b, double* x, double rtol, double atol,
              int maxit, int precond, int* iters, double* final_res, sem_stats* stats,
              cudaStream_t s, double* ax0, const int* ax0_ok) {
@@ -677,6 +695,18 @@ int cg_solve(sem_ctx* ctx, double alpha, const double* b, double* x, double rtol
     return fail(ctx, SEM_ERR_ARG, "unknown preconditioner");
   }
   if (ax0_ok != nullptr) ax0 = nullptr;  // no device-side choice here: apply the operator
+  Timing& tm = ctx->timing;
+  if (ctx->op_precision == SEM_PREC_FP64 && !ctx->deterministic && !tm.enabled && cg_small_fits(L)) {
+    bool resume = false;
+    do {
+      SEM_CK(launch_cg_small(L, alpha, b, inv, ax0, x, w.r, w.p, w.Ap, w.cg, rtol, atol, maxit, resume, s));
+      ctx->launches += 1;
+      SEM_CK(cudaMemcpyAsync(w.cg_host, w.cg, sizeof(CgScalars), cudaMemcpyDeviceToHost, s));
+      SEM_CK(cudaStreamSynchronize(s));
+      resume = true;
+    } while (!w.cg_host->done && w.cg_host->iters < maxit);
+    return cg_result(ctx, w.cg_host->done != 0, maxit, iters, final_res, stats);
+  }
   // Ap = A x (or the carried ax0), then the initial residual; Ap is zero for the iterations
   SEM_CK(cudaMemsetAsync(w.Ap, 0, sizeof(double) * n, s));
   if (ax0 == nullptr) {
@@ -697,7 +727,6 @@ int cg_solve(sem_ctx* ctx, double alpha, const double* b, double* x, double rtol
   ap.cg = w.cg;
   ap.u2 = p2;
 
-  Timing& tm = ctx->timing;
   constexpr int kChunkMax = 16;
   // with timing on, the apply of the first iteration of one solve in kTimingEvery
   // is bracketed by events (they interrupt the programmatic dependent launch)
@@ -709,7 +738,6 @@ int cg_solve(sem_ctx* ctx, double alpha, const double* b, double* x, double rtol
   int launched = 0;
   int chunk = 4;
   bool done = false;
-  int rc_out = SEM_OK;
   while (true) {
     const int this_chunk = std::min(chunk, maxit - launched);
     if (this_chunk > 0) {
@@ -744,20 +772,7 @@ int cg_solve(sem_ctx* ctx, double alpha, const double* b, double* x, double rtol
     if (launched >= maxit) break;
     chunk = std::min(kChunkMax, chunk * 2);
   }
-  const CgScalars& h = *w.cg_host;
-  if (iters) *iters = h.iters;
-  if (final_res) *final_res = std::sqrt(h.rr);
-  if (stats) {
-    stats->cg_iters += h.iters;
-    stats->last_residual = std::sqrt(h.rr);
-  }
-  if (h.status == SEM_ERR_NONFINITE)
-    rc_out = fail(ctx, SEM_ERR_NONFINITE, "non-finite value in a CG inner product");
-  else if (!done)
-    rc_out = fail(ctx, SEM_ERR_NOT_CONVERGED,
-                  "CG did not converge in " + std::to_string(maxit) + " iterations (|r| = " +
-                      std::to_string(std::sqrt(h.rr)) + ")");
-  return rc_out;
+  return cg_result(ctx, done, maxit, iters, final_res, stats);
 }
 
 // Constants of dfexp: ln2 split for Cody and Waite's reduction (c1, c2 with 16
