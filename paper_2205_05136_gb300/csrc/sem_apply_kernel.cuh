@@ -558,9 +558,13 @@ __global__ void __launch_bounds__(MASS_ONLY ? kApplyThreads : ApplyCta<P, T, DOT
 //   - its nodal values by 4-byte cp.async into the other of two tiles; the lanes
 //     (s, i) of a copy read one x-row (j, k) of every element s of the unit, and
 //     consecutive elements are neighbours in x, so a copy covers G n consecutive
-//     words.  The nodes of an element follow from its first map entry and the
-//     strides of the slab's lattice (the map is that lattice), so no per-node
-//     map entry is read; the SEM_DEBUG build reads and checks every entry;
+//     words.  The nodes of an element follow from its first node and the strides of
+//     the slab's lattice (the map is that lattice), so no per-node map entry is
+//     read; the SEM_DEBUG build reads and checks every entry.  The first nodes are
+//     an array of their own: read from the map they cost a 32-byte sector an
+//     element, at p = 1 an eighth of the FP32 kernel's traffic (2.0 M DOFs,
+//     FP32, SEM-NI: p = 1 84.7 -> 75.4 us, p = 2 44.2 -> 42.6; BF16 metric
+//     55.4 -> 52.9 and 31.8 -> 28.8);
 //   - its metric in chunks of rows by bulk copies (cp.async.bulk) into a ring of
 //     kStages chunks, each issued as soon as the chunk before it in its place has
 //     been read (a ring instead of the whole block, which at p = 6 and with the
@@ -682,7 +686,7 @@ template <int P, typename MT>
 __device__ __forceinline__ int plane_base(const ApplyArgs<float, MT>& a, int unit, int nunits, int s) {
   using C = PlaneCfg<P, MT>;
   const int e = unit * C::G + s;
-  return (unit < nunits && e < a.nelem) ? __ldg(a.map + (size_t)e * C::N3) : 0;
+  return (unit < nunits && e < a.nelem) ? __ldg(a.first + e) : 0;
 }
 
 // Node (i, j, k) of the element e whose first node is `base`.
@@ -1135,6 +1139,7 @@ cudaError_t launch_apply_t(const Level& L, const ApplyArgs<T, MT>& a, bool mass_
   ApplyArgs<T, MT> b = a;
   b.ndofs = L.ndofs;
   b.row = P * L.nx + 1;
+  b.first = L.first;
   b.plane = b.row * (P * L.ny + 1);
   b.dbg = L.dbg;
   b.fault = L.fault;

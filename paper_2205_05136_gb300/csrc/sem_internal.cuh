@@ -183,6 +183,7 @@ struct Level {
   int64_t ndofs = 0;
   Tables1D tab;
   int* map = nullptr;
+  int* first = nullptr;      // [nelem] first node of each element (map[e][0])
   double* evert = nullptr;   // [nelem][8][3] element vertices
   double* metric = nullptr;  // [nelem][7][n^3]
   float* metric32 = nullptr;
@@ -276,10 +277,12 @@ struct ApplyArgs {
   // atomic adds, and a node kernel then adds each node's contributions to y in a
   // fixed order
   typename VecOf<T>::type* yloc;
-  // set by the launcher: the vectors' length and strides, the SEM_DEBUG index-error word and
+  // set by the launcher: the vectors' length and strides, the elements' first
+  // nodes, the SEM_DEBUG index-error word and
   // the wait-timeout word
   int64_t ndofs;
   int row, plane;  // lattice strides: nodes of an x-row and of an (x, y) plane
+  const int* first;  // Level::first
   unsigned long long* dbg;
   unsigned* fault;
   int hold;  // SEM_DEBUG build: Level::hold

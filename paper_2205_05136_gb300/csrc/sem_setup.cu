@@ -338,6 +338,7 @@ cudaError_t level_create(Level& L, int nx, int ny, int nz, const double* vertice
   build_tables(p, quad, &L.tab);
   const int n = L.n, n3 = n * n * n;
   std::vector<int> map((size_t)L.nelem * n3);
+  std::vector<int> first((size_t)L.nelem);
   std::vector<double> ev((size_t)L.nelem * 24);
   for (int ez = 0; ez < nz; ++ez)
     for (int ey = 0; ey < ny; ++ey)
@@ -349,6 +350,7 @@ cudaError_t level_create(Level& L, int nx, int ny, int nz, const double* vertice
               const int64_t g = (ex * (int64_t)p + i) + NX * ((ey * (int64_t)p + j) + NY * (ez * (int64_t)p + k));
               map[e * n3 + i + n * (j + n * k)] = (int)g;
             }
+        first[e] = map[e * n3];
         for (int c = 0; c < 2; ++c)
           for (int b = 0; b < 2; ++b)
             for (int a = 0; a < 2; ++a) {
@@ -359,6 +361,7 @@ cudaError_t level_create(Level& L, int nx, int ny, int nz, const double* vertice
   const size_t nm = metric_count(L);
   cudaError_t e;
   if ((e = cudaMalloc(&L.map, sizeof(int) * map.size())) != cudaSuccess) return e;
+  if ((e = cudaMalloc(&L.first, sizeof(int) * first.size())) != cudaSuccess) return e;
   if ((e = cudaMalloc(&L.evert, sizeof(double) * ev.size())) != cudaSuccess) return e;
   if ((e = cudaMalloc(&L.metric, sizeof(double) * nm)) != cudaSuccess) return e;
   if ((e = cudaMemsetAsync(L.metric, 0, sizeof(double) * nm, s)) != cudaSuccess) return e;  // padding
@@ -366,6 +369,7 @@ cudaError_t level_create(Level& L, int nx, int ny, int nz, const double* vertice
   if ((e = cudaMalloc(&L.kdiag, sizeof(double) * L.ndofs)) != cudaSuccess) return e;
   if (coords && (e = cudaMalloc(&L.xyz, sizeof(double) * 3 * L.ndofs)) != cudaSuccess) return e;
   if ((e = cudaMemcpyAsync(L.map, map.data(), sizeof(int) * map.size(), cudaMemcpyHostToDevice, s)) != cudaSuccess) return e;
+  if ((e = cudaMemcpyAsync(L.first, first.data(), sizeof(int) * first.size(), cudaMemcpyHostToDevice, s)) != cudaSuccess) return e;
   if ((e = cudaMemcpyAsync(L.evert, ev.data(), sizeof(double) * ev.size(), cudaMemcpyHostToDevice, s)) != cudaSuccess) return e;
   // the host vectors must outlive the copies
   return cudaStreamSynchronize(s);
@@ -373,6 +377,7 @@ cudaError_t level_create(Level& L, int nx, int ny, int nz, const double* vertice
 
 void level_free(Level& L) {
   cudaFree(L.map);
+  cudaFree(L.first);
   cudaFree(L.evert);
   cudaFree(L.metric);
   cudaFree(L.metric32);
