@@ -292,25 +292,44 @@ __global__ void k_region_mask(int64_t ndofs, const double* __restrict__ xyz, int
   }
 }
 
-__device__ __forceinline__ void metric_store(float* p, double v) { *p = __double2float_rn(v); }
-__device__ __forceinline__ void metric_store(__nv_bfloat16* p, double v) { *p = __float2bfloat16_rn(__double2float_rn(v)); }
+template <typename OT>
+__device__ __forceinline__ OT metric_round(double v);
+template <>
+__device__ __forceinline__ float metric_round<float>(double v) { return __double2float_rn(v); }
+template <>
+__device__ __forceinline__ __nv_bfloat16 metric_round<__nv_bfloat16>(double v) {
+  return __float2bfloat16_rn(__double2float_rn(v));
+}
 
 // FP64 component-major metric -> the plane kernel's low-precision order (MetricLayout);
-// zero in the padding.
-template <typename OT>
-__global__ void k_convert_planes(int64_t n, int64_t nelem, int np, const double* __restrict__ in,
-                                 OT* __restrict__ out) {
+// zero in the padding.  A CTA rounds the values of E elements into shared memory as it
+// reads them (coalesced: an element is one contiguous block) and writes them in the
+// target's order, four values a thread and store; every index is split by constants.
+// DRAM bounds it.  A thread per target value, with 64-bit divisions by run-time sizes
+// and 8-byte loads seven components apart, took 2.46 ms on 462,024 elements at p = 4 for
+// bf16 and 2.36 for FP32; now 0.69 and 0.88 (6.2 TB/s both).
+template <int N, typename OT>
+__global__ void __launch_bounds__(kSetupThreads)
+    k_convert_planes(int nelem, int padded, const double* __restrict__ in, OT* __restrict__ out) {
   using ML = MetricLayout<OT>;
-  const int rs = ML::stride(np), rows = ML::rows(np), nch = ML::chunks(np), G = ML::unit(np), n3p = padded_n3(np);
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t lane = t / rs;  // ((unit, chunk), element slot, plane)
-    const int v = (int)(t - lane * rs), point = v / kMetricComps, comp = v - point * kMetricComps;
-    const int k = (int)(lane % np), slot = (int)((lane / np) % G), chunk = (int)((lane / np / G) % nch);
-    const int64_t e = lane / np / G / nch * G + slot;
-    const int c = chunk * rows * np + point;
-    metric_store(out + t, (e < nelem && point < rows * np) ? in[(e * kMetricComps + comp) * n3p + c + (int64_t)np * np * k]
-                                                           : 0.0);
+  constexpr int N2 = N * N, N3P = padded_n3(N), E = setup_elems(N2 * N), block = kMetricComps * N3P;
+  constexpr int R = ML::rows(N), chunks = ML::chunks(N), RS = ML::stride(N), G = ML::unit(N);
+  constexpr int vectors = chunks * N * (RS / 4);  // an element's stores of four values
+  struct alignas(4 * sizeof(OT)) Four { OT v[4]; };
+  __shared__ OT m[E * block];
+  const int e0 = blockIdx.x * E, ne = min(E, nelem - e0), nout = min(E, padded - e0);
+#pragma unroll 8
+  for (int t = threadIdx.x; t < ne * block; t += kSetupThreads) m[t] = metric_round<OT>(__ldcs(in + (size_t)e0 * block + t));
+  __syncthreads();
+  for (int t = threadIdx.x; t < nout * vectors; t += kSetupThreads) {
+    const int el = t / vectors, q = t - el * vectors, v0 = 4 * (q % (RS / 4)), k = q / (RS / 4) % N,
+              chunk = q / (RS / 4) / N, e = e0 + el, unit = e / G, slot = e - unit * G;
+    Four w;
+    for (int i = 0; i < 4; ++i) {
+      const int point = (v0 + i) / kMetricComps, comp = (v0 + i) - kMetricComps * point;
+      w.v[i] = el < ne && point < R * N ? m[el * block + comp * N3P + chunk * R * N + point + N2 * k] : metric_round<OT>(0.0);
+    }
+    *(Four*)(out + (size_t)(unit * (int64_t)chunks + chunk) * ML::chunk(N) + (slot * N + k) * RS + v0) = w;
   }
 }
 
@@ -447,17 +466,16 @@ cudaError_t setup_diagonals(Level& L, cudaStream_t s) {
 }
 
 cudaError_t setup_metric_lowp(Level& L, bool bf16, cudaStream_t s) {
-  const int64_t count = (int64_t)metric_lowp_count(L);
-  const int threads = 256;
-  const int blocks = (int)std::min<int64_t>((count + threads - 1) / threads, 152 * 16);
-  if (bf16) {
-    k_convert_planes<<<blocks, threads, 0, s>>>(count, L.nelem, L.n, L.metric, L.metric16);
-    L.metric16_valid = true;
-  } else {
-    k_convert_planes<<<blocks, threads, 0, s>>>(count, L.nelem, L.n, L.metric, L.metric32);
-    L.metric32_valid = true;
-  }
-  return cudaGetLastError();
+  const int G = PlaneMetricLayout::unit(L.n), padded = (L.nelem + G - 1) / G * G;
+  (bf16 ? L.metric16_valid : L.metric32_valid) = true;
+  return for_points(L.n, [&](auto n) {
+    constexpr int N = decltype(n)::value, E = setup_elems(N * N * N);
+    const int ctas = (padded + E - 1) / E;
+    if (bf16)
+      k_convert_planes<N><<<ctas, kSetupThreads, 0, s>>>(L.nelem, padded, L.metric, L.metric16);
+    else
+      k_convert_planes<N><<<ctas, kSetupThreads, 0, s>>>(L.nelem, padded, L.metric, L.metric32);
+  });
 }
 
 cudaError_t setup_metric_df(Level& L, cudaStream_t s) {
