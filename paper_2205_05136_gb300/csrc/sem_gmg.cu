@@ -191,9 +191,11 @@ __global__ void k_level_inv_diag(int64_t n, double alpha, const double* m, const
 // Chebyshev smoothing in residual form.  A level keeps the residual r of its
 // current iterate in place of the right-hand side (the apply subtracts A d from it),
 // so no vector t = A x is written, cleared and read back, and the restriction takes
-// r as it is: a step moves 6 vectors where b, t, x, d moved 8, the first two of a zero
-// start 8 instead of 13, the last one 5 (its d is not stored).  Fine-level vectors of
-// a V-cycle of degree 6 on 2.06 M nodes: 545 MB instead of 768.
+// r as it is.  x takes its corrections two at a time, so a pair of steps moves 10
+// vectors where b, t, x, d moved 16, the first two of a zero start 8 instead of 13, the
+// last one 5 (its d is not stored).  Fine-level vectors of a V-cycle of degree 6 on
+// 2.06 M nodes: 462 MB; 545 with x updated in every step, 768 with b and t.  The
+// V-cycle there (bf16 metric): 310 us, 317 with x updated in every step.
 //
 // First step from zero: d = D^{-1} r / theta (x = d follows with the next step, or
 // here with with_x).
@@ -224,39 +226,42 @@ __global__ void k_cheb_zero_start(int64_t n, const T* __restrict__ r, const T* _
 }
 
 // Chebyshev step from the residual r: d = c1 d + c2 D^{-1} r (kChebFirst: d = c2
-// D^{-1} r), x += d (kChebStartX: x = old d + d, the second step of a zero start);
-// kChebLast: d is not needed any more and not stored.
-constexpr int kChebFirst = 1, kChebStartX = 2, kChebLast = 4;
+// D^{-1} r).  A step reads the d before it in any case, so x takes two corrections
+// every second step: it is left alone with kChebDefer, gains old d + d with kChebPair,
+// becomes old d + d with kChebStartX (the second step of a zero start) and gains d with
+// none of these.  kChebLast: d is not needed any more and not stored.
+constexpr int kChebFirst = 1, kChebStartX = 2, kChebLast = 4, kChebDefer = 8, kChebPair = 16;
 template <typename T>
 __global__ void k_cheb_step(int64_t n, const T* __restrict__ r, const T* __restrict__ invd,
                             T* __restrict__ x, T* __restrict__ d, T c1, T c2, int mode, const int* done) {
   pdl_wait();
   const bool stop = skip(done);
   const bool first = (mode & kChebFirst) != 0, startx = (mode & kChebStartX) != 0, last = (mode & kChebLast) != 0;
+  const bool defer = (mode & kChebDefer) != 0, pair = (mode & (kChebPair | kChebStartX)) != 0;
   constexpr int K = k16<T>();
   using V = Pk<T, K>;
   const int64_t nc = n / K;
   GRID_CHUNKS(c, nc) {
     const V rr = reinterpret_cast<const V*>(r)[c], ii = reinterpret_cast<const V*>(invd)[c];
     const V od = first ? V{} : reinterpret_cast<const V*>(d)[c];
-    V xx = startx ? od : reinterpret_cast<const V*>(x)[c];
+    V xx = startx || defer ? V{} : reinterpret_cast<const V*>(x)[c];
     if (stop) return;
     V dd;
 #pragma unroll
     for (int k = 0; k < K; ++k) {
       dd.e[k] = first ? c2 * ii.e[k] * rr.e[k] : fma(c1, od.e[k], c2 * ii.e[k] * rr.e[k]);
-      xx.e[k] += dd.e[k];
+      xx.e[k] += pair ? od.e[k] + dd.e[k] : dd.e[k];
     }
     if (!last) reinterpret_cast<V*>(d)[c] = dd;
-    reinterpret_cast<V*>(x)[c] = xx;
+    if (!defer) reinterpret_cast<V*>(x)[c] = xx;
   }
   GRID_TAIL(i, nc * K, n) {
     const T od = first ? T(0) : d[i];
     const T di = first ? c2 * invd[i] * r[i] : fma(c1, od, c2 * invd[i] * r[i]);
-    const T xi = startx ? od : x[i];
+    const T xi = startx || defer ? T(0) : x[i];
     if (stop) return;
     if (!last) d[i] = di;
-    x[i] = xi + di;
+    if (!defer) x[i] = xi + (pair ? od + di : di);
   }
   pdl_trigger();
 }
@@ -1300,7 +1305,9 @@ int chebyshev(sem_ctx* ctx, Gmg& g, int l, int degree, bool zero_start, bool kee
   double rho_old = 1.0 / sigma;
   T* r = (T*)V.r; T* x = (T*)V.x; T* d = (T*)V.d; const T* invd = (const T*)V.invd;
   int k0 = 0;
+  bool owed = false;  // the correction in d is not in x yet
   if (zero_start) {
+    owed = degree > 1;
     launch_k(k_cheb_zero_start<T>, grid_chunks<T>(n), kThreads, 0, s, n, r, invd, x, d, (T)(1.0 / theta),
              degree == 1 ? 1 : 0, done);
     GMG_CK(cudaGetLastError());
@@ -1310,16 +1317,21 @@ int chebyshev(sem_ctx* ctx, Gmg& g, int l, int degree, bool zero_start, bool kee
   for (int k = k0; k < degree; ++k) {
     int rc = level_apply(ctx, L, g.precision, g.alpha, d, r, done, s);
     if (rc != SEM_OK) return rc;
-    const int last = (k == degree - 1 && !keep_d) ? kChebLast : 0;
+    const bool end = k == degree - 1;
+    int mode = end && !keep_d ? kChebLast : 0;
+    if (owed) mode |= zero_start && k == 1 ? kChebStartX : kChebPair;
+    else if (!end) mode |= kChebDefer;
+    owed = !owed && !end;
+    double c1 = 0.0, c2 = 1.0 / theta;
     if (k == 0) {
-      launch_k(k_cheb_step<T>, grid_chunks<T>(n), kThreads, 0, s, n, r, invd, x, d, (T)0, (T)(1.0 / theta),
-               kChebFirst | last, done);
+      mode |= kChebFirst;
     } else {
       const double rho = 1.0 / (2.0 * sigma - rho_old);
-      launch_k(k_cheb_step<T>, grid_chunks<T>(n), kThreads, 0, s, n, r, invd, x, d, (T)(rho * rho_old),
-               (T)(2.0 * rho / delta), (zero_start && k == 1 ? kChebStartX : 0) | last, done);
+      c1 = rho * rho_old;
+      c2 = 2.0 * rho / delta;
       rho_old = rho;
     }
+    launch_k(k_cheb_step<T>, grid_chunks<T>(n), kThreads, 0, s, n, r, invd, x, d, (T)c1, (T)c2, mode, done);
     GMG_CK(cudaGetLastError());
     ctx->launches += 1;
   }
