@@ -86,6 +86,23 @@ cudaError_t launch_assemble(const Level& L, const float* yloc, float* y, const i
   return assemble_t(L, yloc, y, done, s);
 }
 
+template <int P>
+static int dot_elems(bool df64) { return df64 ? ApplyCta<P, df, true>::E : ApplyCta<P, double, true>::E; }
+
+int dot_blocks(const Level& L, bool df64) {
+  int E = 1;
+  switch (L.p) {
+    case 1: E = dot_elems<1>(df64); break;
+    case 2: E = dot_elems<2>(df64); break;
+    case 3: E = dot_elems<3>(df64); break;
+    case 4: E = dot_elems<4>(df64); break;
+    case 5: E = dot_elems<5>(df64); break;
+    case 6: E = dot_elems<6>(df64); break;
+    default: return 0;
+  }
+  return (L.nelem + E - 1) / E;
+}
+
 int apply_grid_blocks(const Level& L) {
   int E = 1;
   switch (L.p) {

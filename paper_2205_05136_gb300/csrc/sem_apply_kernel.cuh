@@ -528,7 +528,7 @@ __global__ void __launch_bounds__(MASS_ONLY ? kApplyThreads : ApplyCta<P, T, DOT
       }
     }
   }
-  if (DOT) {  // this CTA's partial; k_apply_dot_finish sums them after the launch
+  if (DOT) {  // this CTA's partial; the next kernel sums them
     const double bs = block_sum(dot, red);
     if (threadIdx.x == 0) a.dot_partials[blockIdx.x] = bs;
   }
@@ -1113,7 +1113,7 @@ cudaError_t launch_apply_kernels(const Level& L, const ApplyArgs<T, MT>& a, cons
     const int dgrid = (L.nelem + C::E - 1) / C::E;
     launch_k(sem_apply_kernel<P, QUAD, T, MT, true, false>, dgrid, C::kThreads, C::smem, s, a, tab);
     const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess || (a.cg == nullptr && a.dot_out == nullptr)) return e;
     return launch_apply_dot_finish(a.dot_partials, dgrid, a.cg, a.dot_out, a.done, s);
   } else {
     using C = ApplyCta<P, T, false>;

@@ -20,7 +20,7 @@ struct Workspace {
   CgScalars* cg = nullptr;   // device
   CgScalars* cg_host = nullptr;  // page-locked mirror
   double* vec_partials = nullptr;     // [kReduceSlots][kVecBlocksMax]
-  unsigned int* tickets = nullptr;    // [4]: [0] the CG vector kernels' reductions, the rest spare
+  unsigned int* tickets = nullptr;    // [4]: [0] the CG vector kernels' reductions, [1], [2] k_cg_update's grid barrier
   double* apply_partials = nullptr;   // [apply grid]
   double* dot_result = nullptr;       // 1 double
   int* same = nullptr;        // device flag of sem_step_host_out's carry check (sem_ctx::carry)

@@ -264,11 +264,11 @@ struct ApplyArgs {
   int scale_out;      // 0: out_scale is 1; kScaleOut; kNegateOut: it is -1
   const int* done;    // optional: skip all work when *done != 0
   // optional fused u . (A u) (CG's p . A p): every CTA writes its partial sum
-  // to dot_partials (one double per CTA of the launch) and a one-CTA kernel
-  // launched after the apply adds them up
+  // to dot_partials (one double per CTA of the launch, dot_blocks of them) and a
+  // one-CTA kernel launched after the apply adds them up
   double* dot_partials;
   CgScalars* cg;      // when set, the sum goes to pAp, and alpha = rz / pAp
-  double* dot_out;    // otherwise the sum goes here
+  double* dot_out;    // otherwise the sum goes here; with neither the caller sums
   // optional (double-float operator with the fused inner product): u split into
   // float pairs by the kernel that formed u; the gather then reads the pairs and
   // converts nothing
@@ -298,6 +298,8 @@ cudaError_t launch_apply_bf16(const Level& L, const ApplyArgs<float, __nv_bfloat
 cudaError_t launch_apply_df64(const Level& L, const ApplyArgs<df, df_pair>& a, bool mass_only,
                               cudaStream_t s);
 int apply_grid_blocks(const Level& L);
+// Partials the FP64 (or, df64 set, the double-float) apply with the inner product writes.
+int dot_blocks(const Level& L, bool df64);
 // y[g] += the element contributions yloc[e][n^3] of node g, elements in a fixed
 // order (ez, ey, ex ascending): the deterministic assembly of the apply kernels'
 // element results (and of the p-restriction's coarse-element results).

@@ -233,6 +233,184 @@ __global__ void __launch_bounds__(kVecThreads)
   pdl_trigger();
 }
 
+// Both vector updates of a CG iteration and their scalars in one cooperative kernel:
+// every CTA sums the apply's partials of p . A p (in one fixed order, so all CTAs hold
+// the same alpha), updates x and r, and after a grid barrier over the partial sums of
+// r . z and r . r updates p from the values it kept in registers.  Up to kUpdateNodes
+// nodes the vectors stay in L2 and the three kernels it replaces (the sum of the
+// partials, k_cg_xr, k_cg_p) are launches, reduction tails and FP64 instructions (2 a
+// clock and SM): both sums share one shuffle tree (half the lanes each), the divisions
+// are one thread's, and the nodes are spread over all SMs.  A Jacobi-CG step, three
+// launches / one: p = 3 SEM 299 k nodes 2.15 / 2.05 ms, SEM-NI 1.55 / 1.43; p = 6 SEM
+// 267 k 2.63 / 2.49; p = 1 SEM-NI 287 k 1.81 / 1.74; 633 k nodes 4.16 / 4.15.  Below
+// kUpdateMin the programmatic launches hide as much (p = 1 SEM 46 k nodes 983 / 1007 us,
+// 99 k 1388 / 1394).  Cooperative, since its CTAs wait for one another; at most one CTA
+// an SM.  No pdl_trigger: with it the apply's CTAs crowd on the SMs that come free first
+// (p = 3, 50 k nodes 361 -> 551 us a step).
+constexpr int kUpdThreads = 512, kUpdCtas = 152;
+template <int PAIRS>
+__global__ void __launch_bounds__(kUpdThreads, 1)
+    k_cg_update(int64_t n, double* __restrict__ x, double* __restrict__ p, df_pair* __restrict__ p2,
+                double* __restrict__ Ap, double* __restrict__ r, const double* __restrict__ inv, CgScalars* cg,
+                const double* __restrict__ dot, int ndot, double* partials, unsigned* bar) {
+  if (cg->done) return;
+  __shared__ double red[2][32], bc[2];
+  __shared__ int gave_up;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const double rz = cg->rz;
+  const int64_t c0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+  auto load = [n](const double* v, int64_t c) {
+    if (2 * c + 1 < n) return reinterpret_cast<const D2*>(v)[c];
+    return D2{{2 * c < n ? v[2 * c] : 0.0, 0.0}};
+  };
+  auto store = [n](double* v, int64_t c, const D2& a) {
+    if (2 * c + 1 < n) reinterpret_cast<D2*>(v)[c] = a;
+    else if (2 * c < n) v[2 * c] = a.e[0];
+  };
+  D2 pp[PAIRS], rr[PAIRS], zz[PAIRS];
+#pragma unroll
+  for (int k = 0; k < PAIRS; ++k) {
+    pp[k] = load(p, c0 + k * stride);
+    rr[k] = load(r, c0 + k * stride);
+    zz[k] = load(Ap, c0 + k * stride);
+  }
+  double s = 0.0;
+  for (int b = threadIdx.x; b < ndot; b += blockDim.x) s += dot[b];
+  s = block_sum(s, red[0]);
+  if (threadIdx.x == 0) {
+    bc[0] = s;
+    bc[1] = rz / s;
+    gave_up = 0;
+  }
+  __syncthreads();
+  const double pAp = bc[0], alpha = bc[1];
+  double v0 = 0.0, v1 = 0.0;
+#pragma unroll
+  for (int k = 0; k < PAIRS; ++k) {
+    const int64_t c = c0 + k * stride;
+    D2 xx = load(x, c), ii;
+    if (inv) ii = load(inv, c);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      xx.e[j] = fma(alpha, pp[k].e[j], xx.e[j]);
+      rr[k].e[j] = fma(-alpha, zz[k].e[j], rr[k].e[j]);
+      zz[k].e[j] = inv ? ii.e[j] * rr[k].e[j] : rr[k].e[j];
+      if (2 * c + j < n) {
+        v0 = fma(rr[k].e[j], zz[k].e[j], v0);
+        v1 = fma(rr[k].e[j], rr[k].e[j], v1);
+      }
+    }
+    store(x, c, xx);
+    store(r, c, rr[k]);
+  }
+  // lanes 0..15 sum v0, lanes 16..31 v1
+  auto pair_tree = [lane](double a0, double a1) {
+    double v = lane < 16 ? a0 : a1;
+    v += __shfl_xor_sync(0xffffffffu, lane < 16 ? a1 : a0, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+  };
+  double v = pair_tree(v0, v1);
+  if ((lane & 15) == 0) red[1][2 * warp + (lane >> 4)] = v;
+  __syncthreads();
+  if (warp == 0) {
+    const int W = blockDim.x / 32;
+    v = pair_tree(lane < W ? red[1][2 * lane] : 0.0, lane < W ? red[1][2 * lane + 1] : 0.0);
+    if ((lane & 15) == 0) {
+      __stcg(partials + 2 * blockIdx.x + (lane >> 4), v);
+      __threadfence();
+    }
+    __syncwarp();
+    if (lane == 0) {
+      volatile unsigned* gen = bar + 1;
+      const unsigned mine = *gen;
+      __threadfence();
+      if (atomicAdd(bar, 1u) == gridDim.x - 1) {
+        *(volatile unsigned*)bar = 0u;
+        __threadfence();
+        *gen = mine + 1u;
+      } else {
+        int left = 1 << 22;  // seconds; the CTAs of a cooperative launch run at the same time
+        while (*gen == mine && --left) {}
+        if (left == 0) gave_up = 1;
+      }
+      __threadfence();
+    }
+    __syncwarp();
+    double t0 = 0.0, t1 = 0.0;
+    for (int b = lane; b < (int)gridDim.x; b += 32) {
+      t0 += __ldcg(partials + 2 * b);
+      t1 += __ldcg(partials + 2 * b + 1);
+    }
+    v = pair_tree(t0, t1);
+    if ((lane & 15) == 0) bc[lane >> 4] = v;
+  }
+  __syncthreads();
+  const double nrz = bc[0], nrr = bc[1];
+  const bool finite = isfinite(nrz) && isfinite(nrr) && isfinite(alpha);
+  if (threadIdx.x == 0) red[0][0] = nrz / rz;
+  __syncthreads();
+  const double beta = red[0][0];
+  const bool stop = !finite || nrr <= cg->tol2;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    cg->pAp = pAp;
+    cg->alpha = alpha;
+    cg->beta = beta;
+    cg->rz = nrz;
+    cg->rr = nrr;
+    cg->iters += 1;
+    if (!finite) cg->status = SEM_ERR_NONFINITE;
+    if (stop) cg->done = 1;
+  }
+  if (gave_up && threadIdx.x == 0) {
+    cg->status = SEM_ERR_CUDA;
+    cg->done = 1;
+  }
+  if (stop || gave_up) return;
+#pragma unroll
+  for (int k = 0; k < PAIRS; ++k) {
+    const int64_t c = c0 + k * stride;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) pp[k].e[j] = fma(beta, pp[k].e[j], zz[k].e[j]);
+    store(p, c, pp[k]);
+    store(Ap, c, D2{});
+    if (p2 != nullptr) {
+      const df_pair a0 = split_pair(pp[k].e[0]), a1 = split_pair(pp[k].e[1]);
+      if (2 * c + 1 < n) reinterpret_cast<float4*>(p2)[c] = make_float4(a0.h, a0.l, a1.h, a1.l);
+      else if (2 * c < n) p2[2 * c] = a0;
+    }
+  }
+}
+
+constexpr int64_t kUpdateMin = 100000, kUpdateNodes = (int64_t)kUpdCtas * kUpdThreads * 2 * 4;
+
+cudaError_t launch_cg_update(int64_t n, double* x, double* p, df_pair* p2, double* Ap, double* r, const double* inv,
+                             CgScalars* cg, const double* dot, int ndot, double* partials, unsigned* bar, cudaStream_t s) {
+  const int64_t pairs = (n + 1) / 2, each = (pairs + kUpdCtas - 1) / kUpdCtas;  // of a CTA
+  const int per = each <= kUpdThreads ? 1 : each <= 2 * kUpdThreads ? 2 : 4;
+  const int threads = (int)std::max<int64_t>(128, (each + per - 1) / per + 31) / 32 * 32;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = (unsigned)std::min<int64_t>((pairs + threads * per - 1) / (threads * per), kUpdCtas);
+  cfg.blockDim = threads;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeCooperative;
+  at[0].val.cooperative = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  auto* k = per == 1 ? k_cg_update<1> : per == 2 ? k_cg_update<2> : k_cg_update<4>;
+  return cudaLaunchKernelEx(&cfg, k, n, x, p, p2, Ap, r, inv, cg, dot, ndot, partials, bar);
+}
+
+// Whether the device runs k_cg_update's CTAs side by side.
+bool cg_update_fits(int64_t n, const double* x) {
+  int dev = 0, sms = 0, coop = 0;
+  return n >= kUpdateMin && n <= kUpdateNodes && (reinterpret_cast<uintptr_t>(x) & 15u) == 0 && cudaGetDevice(&dev) == cudaSuccess &&
+         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms >= kUpdCtas &&
+         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop != 0;
+}
+
 // With `same` set (sem_step_host_out), x0 still holds the solution the last call
 // left there: a value that differs from the incoming u^n, bit for bit, clears *same.
 __device__ __forceinline__ void check_same(int* same, double old, double u) {
@@ -663,6 +841,10 @@ static int cg_result(sem_ctx* ctx, bool done, int maxit, int* iters, double* fin
   }
   if (h.status == SEM_ERR_NONFINITE)
     return fail(ctx, SEM_ERR_NONFINITE, "non-finite value in a CG inner product");
+  if (h.status == SEM_ERR_CUDA) {
+    cudaMemset(ctx->ws.tickets, 0, sizeof(unsigned) * 4);
+    return fail(ctx, SEM_ERR_CUDA, "the CG update gave up waiting for its grid barrier");
+  }
   if (!done)
     return fail(ctx, SEM_ERR_NOT_CONVERGED,
                 "CG did not converge in " + std::to_string(maxit) + " iterations (|r| = " +
@@ -724,8 +906,10 @@ int cg_solve(sem_ctx* ctx, double alpha, const double* b, double* x, double rtol
   ApplyArgs64 ap = base_args(ctx, alpha, 1.0, w.p, w.Ap);
   ap.done = &w.cg->done;
   ap.dot_partials = w.apply_partials;
-  ap.cg = w.cg;
   ap.u2 = p2;
+  const bool one = cg_update_fits(n, x);
+  const int ndot = dot_blocks(L, p2 != nullptr);
+  if (!one) ap.cg = w.cg;
 
   constexpr int kChunkMax = 16;
   // with timing on, the apply of the first iteration of one solve in kTimingEvery
@@ -746,6 +930,11 @@ int cg_solve(sem_ctx* ctx, double alpha, const double* b, double* x, double rtol
         if (timed) SEM_CK(cudaEventRecord(tm.start, s));
         SEM_CK(launch_operator(ctx, ap, s));
         if (timed) SEM_CK(cudaEventRecord(tm.stop, s));
+        if (one) {
+          SEM_CK(launch_cg_update(n, x, w.p, p2, w.Ap, w.r, inv, w.cg, w.apply_partials, ndot, w.vec_partials,
+                                  w.tickets + 1, s));
+          continue;
+        }
         if ((reinterpret_cast<uintptr_t>(x) & 15u) == 0)
           launch_k(k_cg_xr<true>, vg, kVecThreads, 0, s, n, x, w.p, w.Ap, w.r, inv, w.z, w.cg, w.vec_partials,
                                                    w.tickets + 0);
@@ -756,7 +945,8 @@ int cg_solve(sem_ctx* ctx, double alpha, const double* b, double* x, double rtol
       }
       SEM_CK(cudaGetLastError());
       launched += this_chunk;
-      ctx->launches += 4 * this_chunk;  // apply, its inner-product sum, x/r update, p update
+      // apply and update, or apply, its inner-product sum, x/r update, p update
+      ctx->launches += (one ? 2 : 4) * this_chunk;
     }
     SEM_CK(cudaMemcpyAsync(w.cg_host, w.cg, sizeof(CgScalars), cudaMemcpyDeviceToHost, s));
     SEM_CK(cudaStreamSynchronize(s));
