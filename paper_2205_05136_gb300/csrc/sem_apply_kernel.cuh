@@ -1064,6 +1064,171 @@ cudaError_t launch_apply_plane(const Level& L, const ApplyArgs<float, MT>& a, co
   return cudaGetLastError();
 }
 
+// The FP32 operator on few elements (p >= 3): one 1-D line of an element per thread,
+// an element (two at p = 3) per CTA.  Below about a warp of the plane kernel an SM the
+// apply takes as long as one warp takes for its unit, and a lane of that kernel works
+// through a whole plane; here a thread works through one line a sweep, the column's
+// metric waits in registers before pdl_wait, and the z-sweeps are registers only.
+// An apply, FP32 metric, plane kernel / this one, on 288 elements: SEM-NI p = 3..6
+// 3.1 / 2.6, 3.9 / 2.8, 6.1 / 3.0, 7.1 / 3.4 us, SEM 3.5 / 2.9, 5.5 / 3.2, 8.0 / 3.5,
+// 10.1 / 3.9; on 1,250 elements 3.2 / 3.0, 4.0 / 3.8, 6.6 / 4.7, 8.0 / 6.0 and 3.6 / 3.3,
+// 6.0 / 4.1, 8.8 / 5.6, 11.5 / 6.9; on 2,808 elements 3.5 / 4.3, 4.7 / 5.9, 7.2 / 7.6,
+// 9.1 / 10.3 and 4.0 / 4.9, 6.4 / 6.4, 9.4 / 9.3, 12.4 / 12.2.  The line (kElements)
+// lies where the two meet.  At p = 1 and 2 the plane kernel is as fast on any mesh.
+template <int P, int QUAD>
+struct FewCfg {
+  static constexpr int N2 = (P + 1) * (P + 1), E = P == 3 ? 2 : 1;
+  static constexpr int kThreads = (E * N2 + 31) / 32 * 32;
+  static constexpr bool kSem = QUAD == SEM_QUAD_LG;
+  static constexpr int kElements = P == 3 ? 1500 : P == 4 ? (kSem ? 2500 : 1500) : P == 5 ? (kSem ? 2800 : 2400) : kSem ? 2800 : 2200;
+};
+
+template <int P, int QUAD, typename MT>
+__global__ void __launch_bounds__(FewCfg<P, QUAD>::kThreads)
+    sem_apply_few_kernel(const ApplyArgs<float, MT> a, const __grid_constant__ KTab<P + 1, float> tab) {
+  constexpr int N = P + 1, N2 = N * N, N3 = N2 * N, E = FewCfg<P, QUAD>::E;
+  using ML = MetricLayout<MT>;
+  __shared__ float sA[E * N3], sB[E * N3], sC[E * N3];
+  const int slot = threadIdx.x / N2, c = threadIdx.x - slot * N2, e = blockIdx.x * E + slot;
+  const bool act = slot < E && e < a.nelem;
+  const int i = c % N, q = c / N;  // of the thread's column (i, j = q) and of its y-line (i, k = q)
+  float* A = sA + (slot < E ? slot * N3 : 0);
+  float* B = sB + (slot < E ? slot * N3 : 0);
+  float* C = sC + (slot < E ? slot * N3 : 0);
+  const int xl = N * c, yl = i + N2 * q;
+  MT G[N][kMetricComps];
+  int g0 = 0;
+  if (act) {
+    g0 = __ldg(a.first + e);
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+#pragma unroll
+      for (int m = 0; m < kMetricComps; ++m) G[k][m] = __ldg(a.metric + ML::offset(N, e, c, k, m));
+  }
+  auto line = [](float* p, int stride, float (&v)[N]) {
+#pragma unroll
+    for (int t = 0; t < N; ++t) v[t] = p[t * stride];
+  };
+  auto put = [](float* p, int stride, const float (&v)[N]) {
+#pragma unroll
+    for (int t = 0; t < N; ++t) p[t * stride] = v[t];
+  };
+  auto result = [&](int ii, int jj, int kk, float v) {
+    v = scale_result(a, v);
+    if (a.yloc != nullptr) store_loc(a.yloc + (size_t)e * N3 + ii + N * jj + N2 * kk, v);
+    else scatter_add(a.y + plane_node<N>(a, e, g0, ii, jj, kk, kDbgScatter), v);
+  };
+  pdl_wait();
+  const bool stop = a.done != nullptr && *a.done;
+  float z[N], w[N], v[N];
+  if (act) {
+#pragma unroll
+    for (int k = 0; k < N; ++k) z[k] = a.u[plane_node<N>(a, e, g0, i, q, k, kDbgGather)];
+  }
+  if (stop) return;
+  if (act) {
+    if (QUAD == SEM_QUAD_LG) {
+      eo_line<N, false, false>(tab.Bi, z, w);
+      put(A + c, N2, w);
+    } else {
+      put(A + c, N2, z);
+    }
+  }
+  __syncthreads();
+  if (QUAD == SEM_QUAD_LG) {  // values at the Gauss points
+    if (act) {
+      line(A + xl, 1, v);
+      eo_line<N, false, false>(tab.Bi, v, w);
+      put(A + xl, 1, w);
+    }
+    __syncthreads();
+  }
+  if (act) {
+    line(A + yl, N, v);
+    if (QUAD == SEM_QUAD_LG) {
+      eo_line<N, false, false>(tab.Bi, v, w);
+      put(A + yl, N, w);
+      eo_line<N, true, false>(tab.D, w, v);
+      put(C + yl, N, v);
+    } else {
+      eo_line<N, true, false>(tab.D, v, w);
+      put(C + yl, N, w);
+    }
+  }
+  if (QUAD == SEM_QUAD_LG) __syncthreads();
+  if (act) {
+    line(A + xl, 1, v);
+    eo_line<N, true, false>(tab.D, v, w);
+    put(B + xl, 1, w);
+    if (QUAD == SEM_QUAD_LG) line(A + c, N2, z);
+  }
+  __syncthreads();
+  float m[N];
+  if (act) {
+    eo_line<N, true, false>(tab.D, z, v);
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      const float g1 = B[c + k * N2], g2 = C[c + k * N2], g3 = v[k];
+      float g[kMetricComps];
+#pragma unroll
+      for (int t = 0; t < kMetricComps; ++t) g[t] = (float)G[k][t];
+      B[c + k * N2] = fmaf(g[2], g3, fmaf(g[1], g2, g[0] * g1));
+      C[c + k * N2] = fmaf(g[4], g3, fmaf(g[3], g2, g[1] * g1));
+      w[k] = fmaf(g[5], g3, fmaf(g[4], g2, g[2] * g1));
+      m[k] = (a.mass_coef * g[6]) * z[k];
+    }
+    eo_line<N, true, true>(tab.Dt, w, m);
+  }
+  __syncthreads();
+  if (act) {
+    line(B + xl, 1, v);
+    for (int t = 0; t < N; ++t) w[t] = 0.f;
+    eo_line<N, true, true>(tab.Dt, v, w);
+    put(B + xl, 1, w);
+    line(C + yl, N, v);
+    for (int t = 0; t < N; ++t) w[t] = 0.f;
+    eo_line<N, true, true>(tab.Dt, v, w);
+    put(C + yl, N, w);
+  }
+  __syncthreads();
+  if (act) {
+#pragma unroll
+    for (int k = 0; k < N; ++k) m[k] += B[c + k * N2] + C[c + k * N2];
+  }
+  if (QUAD == SEM_QUAD_LG) {  // back to the nodes
+    if (act) {
+      eo_line<N, false, false>(tab.Bit, m, w);
+      put(A + c, N2, w);
+    }
+    __syncthreads();
+    if (act) {
+      line(A + xl, 1, v);
+      eo_line<N, false, false>(tab.Bit, v, w);
+      put(A + xl, 1, w);
+    }
+    __syncthreads();
+    if (act) {
+      line(A + yl, N, v);
+      eo_line<N, false, false>(tab.Bit, v, w);
+    }
+  }
+  pdl_trigger();
+  if (act) {
+#pragma unroll
+    for (int t = 0; t < N; ++t) {
+      if (QUAD == SEM_QUAD_LG) result(i, t, q, w[t]);
+      else result(i, q, t, m[t]);
+    }
+  }
+}
+
+template <int P, int QUAD, typename MT>
+cudaError_t launch_apply_few(const Level& L, const ApplyArgs<float, MT>& a, const KTab<P + 1, float>& tab, cudaStream_t s) {
+  using C = FewCfg<P, QUAD>;
+  launch_k(sem_apply_few_kernel<P, QUAD, MT>, (L.nelem + C::E - 1) / C::E, C::kThreads, 0, s, a, tab);
+  return cudaGetLastError();
+}
+
 // Even-odd form (EoMat) of the n x n matrix M (or of its transpose), from the
 // host tables; the mirrored rows are implied by the symmetry of M.
 template <int N, typename T>
@@ -1094,6 +1259,10 @@ cudaError_t launch_apply_kernels(const Level& L, const ApplyArgs<T, MT>& a, cons
   constexpr size_t tiles = apply_tile_bytes<P, T>();
   if constexpr (std::is_same<T, float>::value) {
     if (dot) return cudaErrorInvalidValue;
+    if constexpr (P >= 3) {
+      // (the plane kernel where a metric copy is to be held back)
+      if (!mass_only && L.nelem <= FewCfg<P, QUAD>::kElements && L.hold < 0) return launch_apply_few<P, QUAD, MT>(L, a, tab, s);
+    }
     if (!mass_only) return launch_apply_plane<P, QUAD, MT>(L, a, tab, s);
     // mass only, p <= 4: elements owned by warps (measured faster; at p = 5, 6 the
     // n^2 = 36, 49 lines fill warps poorly and the CTA-wide mode is faster)

@@ -1,9 +1,11 @@
-"""The plane kernel of the FP32 operator at the edges of its units.
+"""The plane kernel of the FP32 operator at the edges of its units, and the kernel for few elements.
 
 A unit is G = 32 // (p + 1) consecutive elements of one warp: meshes of one element, of
 one unit exactly, of one element more or less, of rows that end inside a unit, of more
 elements than one CTA of the metric's conversion takes, and vectors
-that start 4 bytes past a 16-byte boundary (the gather copies single words).  The reference
+that start 4 bytes past a 16-byte boundary (the gather copies single words).  From p = 3 the
+meshes of up to some 2,000 elements take the kernel of one line per thread; 2,989 and 3,360
+elements (no multiple and a multiple of every unit) take the plane kernel.  The reference
 is the FP64 apply, which the other tests hold to the oracle.  Bounds as in test_gpu_apply:
 FP32 arithmetic with an FP32 metric 6e-7, the bf16 metric 5e-3 (relative, 2-norm).
 """
@@ -20,7 +22,8 @@ gb = pytest.importorskip("paper_2205_05136_gb300")
 
 def _dims(p):
     g = 32 // (p + 1)
-    return [(1, 1, 1), (g, 1, 1), (g - 1, 1, 1), (g + 1, 1, 1), (3, 2, 2), (g + 2, 3, 2), (8 * g + 1, 1, 1)]
+    large = [(61, 7, 7), (60, 7, 8)] if p >= 3 else []  # above the sizes of the kernel for few elements
+    return large + [(1, 1, 1), (g, 1, 1), (g - 1, 1, 1), (g + 1, 1, 1), (3, 2, 2), (g + 2, 3, 2), (8 * g + 1, 1, 1)]
 
 
 @pytest.mark.parametrize("quad", ["LGL", "LG"])
