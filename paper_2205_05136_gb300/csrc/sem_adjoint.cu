@@ -133,109 +133,157 @@ struct GradTab {
 };
 
 // One CTA per element: g_k[e] -= sum_q W_q grad w . dD_k grad u at the quadrature points.
-__global__ void k_param_grad(int nelem, const int* __restrict__ map, const double* __restrict__ evert,
-                             const double* __restrict__ sigma_l, const double* __restrict__ sigma_t,
-                             const double* __restrict__ theta, const __grid_constant__ GradTab tab,
-                             const double* __restrict__ w, const double* __restrict__ u,
-                             double* __restrict__ g_sl, double* __restrict__ g_st,
-                             double* __restrict__ g_th) {
+// The FP64 pipe bounds it (2 operations a clock and SM): the trilinear map by its
+// coefficients, the adjugate A = det J J^{-1} in place of nine divided entries (one
+// division a point, by det), one cos and sin an element, about 150
+// operations a point.  2,340 elements, p = 3 SEM-NI: 50 us; 135 with the corner sums,
+// nine divisions and a cos and sin in every thread.
+__host__ __device__ constexpr int grad_threads(int n3) { return n3 >= 128 ? 128 : (n3 + 31) / 32 * 32; }
+template <int N>
+__global__ void __launch_bounds__(grad_threads(N * N * N))
+    k_param_grad(int nelem, const int* __restrict__ map, const double* __restrict__ evert,
+                 const double* __restrict__ sigma_l, const double* __restrict__ sigma_t,
+                 const double* __restrict__ theta, const __grid_constant__ GradTab tab, const double* __restrict__ w,
+                 const double* __restrict__ u, double* __restrict__ g_sl, double* __restrict__ g_st,
+                 double* __restrict__ g_th) {
   const int e = blockIdx.x;
   if (e >= nelem) return;
-  const int n = tab.n, n2 = n * n, n3 = n2 * n;
-  __shared__ double V[8][3];
-  __shared__ double F[2][kMaxN * kMaxN * kMaxN];
-  __shared__ double G[2][kMaxN * kMaxN * kMaxN];
-  __shared__ double red[3][32];
-  if (threadIdx.x < 24) V[threadIdx.x / 3][threadIdx.x % 3] = evert[(size_t)e * 24 + threadIdx.x];
-  for (int a = threadIdx.x; a < n3; a += blockDim.x) {
-    const int gidx = map[(size_t)e * n3 + a];
+  constexpr int N2 = N * N, N3 = N2 * N, kCta = grad_threads(N3);
+  __shared__ double coef[3][8];
+  __shared__ double F[2][N3], G[2][N3];
+  __shared__ double Dc[N][N + 1], xq[N], wq[N], dir[2], red[3][kCta / 32];
+  const int t = threadIdx.x;
+  if (t < 3) {
+    double x[8];
+    for (int i = 0; i < 8; ++i) x[i] = evert[(size_t)e * 24 + 3 * i + t];
+    // sums and differences over the corners' bits (1: xi, 2: eta, 4: zeta)
+    for (int bit = 1; bit < 8; bit <<= 1)
+      for (int i = 0; i < 8; ++i)
+        if (!(i & bit)) {
+          const double lo = x[i], hi = x[i | bit];
+          x[i] = 0.5 * (hi + lo);
+          x[i | bit] = 0.5 * (hi - lo);
+        }
+    for (int i = 0; i < 8; ++i) coef[t][i] = x[i];
+  }
+  if (t == kCta - 1) {
+    const double th = theta[e];
+    dir[0] = cos(th);
+    dir[1] = sin(th);
+  }
+  for (int a = t; a < N2; a += kCta) Dc[a / N][a % N] = tab.Dc[a / N][a % N];
+  if (t < N) {
+    xq[t] = tab.xq[t];
+    wq[t] = tab.wq[t];
+  }
+  for (int a = t; a < N3; a += kCta) {
+    const int gidx = map[(size_t)e * N3 + a];
     F[0][a] = w[gidx];
     F[1][a] = u[gidx];
   }
   __syncthreads();
   if (tab.lg) {  // values at the Gauss points: F -> G (x), G -> F (y), F -> G (z), G -> F copy
-    for (int a = threadIdx.x; a < 2 * n3; a += blockDim.x) {
-      const int c = a / n3, r = a % n3, q = r % n, j = (r / n) % n, k = r / n2;
+    for (int a = t; a < 2 * N3; a += kCta) {
+      const int c = a / N3, r = a % N3, q = r % N, j = (r / N) % N, k = r / N2;
       double s = 0.0;
-      for (int l = 0; l < n; ++l) s += tab.Bi[q][l] * F[c][k * n2 + j * n + l];
+      for (int l = 0; l < N; ++l) s += tab.Bi[q][l] * F[c][k * N2 + j * N + l];
       G[c][r] = s;
     }
     __syncthreads();
-    for (int a = threadIdx.x; a < 2 * n3; a += blockDim.x) {
-      const int c = a / n3, r = a % n3, i = r % n, q = (r / n) % n, k = r / n2;
+    for (int a = t; a < 2 * N3; a += kCta) {
+      const int c = a / N3, r = a % N3, i = r % N, q = (r / N) % N, k = r / N2;
       double s = 0.0;
-      for (int l = 0; l < n; ++l) s += tab.Bi[q][l] * G[c][k * n2 + l * n + i];
+      for (int l = 0; l < N; ++l) s += tab.Bi[q][l] * G[c][k * N2 + l * N + i];
       F[c][r] = s;
     }
     __syncthreads();
-    for (int a = threadIdx.x; a < 2 * n3; a += blockDim.x) {
-      const int c = a / n3, r = a % n3, i = r % n, j = (r / n) % n, q = r / n2;
+    for (int a = t; a < 2 * N3; a += kCta) {
+      const int c = a / N3, r = a % N3, i = r % N, j = (r / N) % N, q = r / N2;
       double s = 0.0;
-      for (int l = 0; l < n; ++l) s += tab.Bi[q][l] * F[c][l * n2 + j * n + i];
+      for (int l = 0; l < N; ++l) s += tab.Bi[q][l] * F[c][l * N2 + j * N + i];
       G[c][r] = s;
     }
     __syncthreads();
-    for (int a = threadIdx.x; a < 2 * n3; a += blockDim.x) F[a / n3][a % n3] = G[a / n3][a % n3];
+    for (int a = t; a < 2 * N3; a += kCta) F[a / N3][a % N3] = G[a / N3][a % N3];
     __syncthreads();
   }
-  const double sl = sigma_l[e], st = sigma_t[e], th = theta[e];
-  const double f[3] = {cos(th), sin(th), 0.0};
-  const double fp[3] = {-sin(th), cos(th), 0.0};
+  const double f0 = dir[0], f1 = dir[1];
   double acc[3] = {0.0, 0.0, 0.0};
-  for (int a = threadIdx.x; a < n3; a += blockDim.x) {
-    const int qx = a % n, qy = (a / n) % n, qz = a / n2;
-    const double xi[3] = {tab.xq[qx], tab.xq[qy], tab.xq[qz]};
-    // Jacobian of the trilinear map at xi
-    double J[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
-    for (int v = 0; v < 8; ++v) {
-      const double sg[3] = {(v & 1) ? 1.0 : -1.0, (v & 2) ? 1.0 : -1.0, (v & 4) ? 1.0 : -1.0};
-      const double fa[3] = {0.5 * (1.0 + sg[0] * xi[0]), 0.5 * (1.0 + sg[1] * xi[1]), 0.5 * (1.0 + sg[2] * xi[2])};
-      const double dN[3] = {0.5 * sg[0] * fa[1] * fa[2], fa[0] * 0.5 * sg[1] * fa[2], fa[0] * fa[1] * 0.5 * sg[2]};
-      for (int d = 0; d < 3; ++d)
-        for (int c = 0; c < 3; ++c) J[d][c] += V[v][d] * dN[c];
+  for (int a = t; a < N3; a += kCta) {
+    const int qx = a % N, qy = (a / N) % N, qz = a / N2;
+    const double x = xq[qx], y = xq[qy], z = xq[qz];
+    double J[3][3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const double* c = coef[d];
+      J[d][0] = fma(z, fma(y, c[7], c[5]), fma(y, c[3], c[1]));
+      J[d][1] = fma(z, fma(x, c[7], c[6]), fma(x, c[3], c[2]));
+      J[d][2] = fma(y, fma(x, c[7], c[6]), fma(x, c[5], c[4]));
     }
-    const double det = J[0][0] * (J[1][1] * J[2][2] - J[1][2] * J[2][1]) -
-                       J[0][1] * (J[1][0] * J[2][2] - J[1][2] * J[2][0]) +
-                       J[0][2] * (J[1][0] * J[2][1] - J[1][1] * J[2][0]);
-    double inv[3][3];
-    inv[0][0] = (J[1][1] * J[2][2] - J[1][2] * J[2][1]) / det;
-    inv[0][1] = (J[0][2] * J[2][1] - J[0][1] * J[2][2]) / det;
-    inv[0][2] = (J[0][1] * J[1][2] - J[0][2] * J[1][1]) / det;
-    inv[1][0] = (J[1][2] * J[2][0] - J[1][0] * J[2][2]) / det;
-    inv[1][1] = (J[0][0] * J[2][2] - J[0][2] * J[2][0]) / det;
-    inv[1][2] = (J[0][2] * J[1][0] - J[0][0] * J[1][2]) / det;
-    inv[2][0] = (J[1][0] * J[2][1] - J[1][1] * J[2][0]) / det;
-    inv[2][1] = (J[0][1] * J[2][0] - J[0][0] * J[2][1]) / det;
-    inv[2][2] = (J[0][0] * J[1][1] - J[0][1] * J[1][0]) / det;
-    const double W = tab.wq[qx] * tab.wq[qy] * tab.wq[qz] * det;
-    double gw[3], gu[3];
+    double A[3][3];  // row r, column d: det (dxi_r / dx_d)
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      const int p = (r + 1) % 3, q = (r + 2) % 3;
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        const int m = (d + 1) % 3, v = (d + 2) % 3;
+        A[r][d] = fma(J[m][p], J[v][q], -(J[v][p] * J[m][q]));
+      }
+    }
+    const double det = fma(J[2][0], A[0][2], fma(J[1][0], A[0][1], J[0][0] * A[0][0]));
+    double g[2][3];  // det grad w, det grad u
+#pragma unroll
     for (int c = 0; c < 2; ++c) {
       double ref[3] = {0.0, 0.0, 0.0};
-      for (int l = 0; l < n; ++l) {
-        ref[0] += tab.Dc[qx][l] * F[c][qz * n2 + qy * n + l];
-        ref[1] += tab.Dc[qy][l] * F[c][qz * n2 + l * n + qx];
-        ref[2] += tab.Dc[qz][l] * F[c][l * n2 + qy * n + qx];
+#pragma unroll
+      for (int l = 0; l < N; ++l) {
+        ref[0] = fma(Dc[qx][l], F[c][qz * N2 + qy * N + l], ref[0]);
+        ref[1] = fma(Dc[qy][l], F[c][qz * N2 + l * N + qx], ref[1]);
+        ref[2] = fma(Dc[qz][l], F[c][l * N2 + qy * N + qx], ref[2]);
       }
-      double* out = c == 0 ? gw : gu;
-      for (int d = 0; d < 3; ++d) out[d] = inv[0][d] * ref[0] + inv[1][d] * ref[1] + inv[2][d] * ref[2];
+#pragma unroll
+      for (int d = 0; d < 3; ++d) g[c][d] = fma(A[2][d], ref[2], fma(A[1][d], ref[1], A[0][d] * ref[0]));
     }
-    const double wf = gw[0] * f[0] + gw[1] * f[1];
-    const double uf = gu[0] * f[0] + gu[1] * f[1];
-    const double wfp = gw[0] * fp[0] + gw[1] * fp[1];
-    const double ufp = gu[0] * fp[0] + gu[1] * fp[1];
-    const double wu = gw[0] * gu[0] + gw[1] * gu[1] + gw[2] * gu[2];
-    acc[0] += W * wf * uf;
-    acc[1] += W * (wu - wf * uf);
-    acc[2] += W * (sl - st) * (wfp * uf + wf * ufp);
+    const double s = wq[qx] * wq[qy] * wq[qz] / det;
+    const double wf = fma(g[0][1], f1, g[0][0] * f0), uf = fma(g[1][1], f1, g[1][0] * f0);
+    const double wfp = fma(g[0][1], f0, -(g[0][0] * f1)), ufp = fma(g[1][1], f0, -(g[1][0] * f1));
+    const double wu = fma(g[0][2], g[1][2], fma(g[0][1], g[1][1], g[0][0] * g[1][0]));
+    acc[0] = fma(s, wf * uf, acc[0]);
+    acc[1] = fma(s, fma(-wf, uf, wu), acc[1]);
+    acc[2] = fma(s, fma(wfp, uf, wf * ufp), acc[2]);
   }
+#pragma unroll
   for (int k = 0; k < 3; ++k) {
-    const double s = block_sum(acc[k], red[k]);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      if (k == 0) g_sl[e] -= s;
-      if (k == 1) g_st[e] -= s;
-      if (k == 2) g_th[e] -= s;
-    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
+    if ((t & 31) == 0) red[k][t >> 5] = acc[k];
+  }
+  __syncthreads();
+  if (t < 3) {
+    double s = 0.0;
+    for (int i = 0; i < kCta / 32; ++i) s += red[t][i];
+    if (t == 2) s *= sigma_l[e] - sigma_t[e];
+    double* g = t == 0 ? g_sl : t == 1 ? g_st : g_th;
+    g[e] -= s;
+  }
+}
+
+cudaError_t launch_param_grad(sem_ctx* ctx, const GradTab& tab, const double* w, const double* u, double* g_sl,
+                              double* g_st, double* g_th, cudaStream_t s) {
+  const Level& L = ctx->L;
+  auto run = [&](auto k, int threads) {
+    k<<<L.nelem, threads, 0, s>>>(L.nelem, L.map, L.evert, ctx->sigma_l, ctx->sigma_t, ctx->theta, tab, w, u, g_sl,
+                                  g_st, g_th);
+    return cudaGetLastError();
+  };
+  switch (L.n) {
+    case 2: return run(k_param_grad<2>, grad_threads(8));
+    case 3: return run(k_param_grad<3>, grad_threads(27));
+    case 4: return run(k_param_grad<4>, grad_threads(64));
+    case 5: return run(k_param_grad<5>, grad_threads(125));
+    case 6: return run(k_param_grad<6>, grad_threads(216));
+    case 7: return run(k_param_grad<7>, grad_threads(343));
+    default: return cudaErrorInvalidValue;
   }
 }
 
@@ -377,10 +425,7 @@ int adjoint_grad(sem_ctx* ctx, const double* trace_bar, double* g_sl, double* g_
       int rc = cg_solve(ctx, alpha, UB(k + 1), tp->w, rtol, atol, maxit, precond, nullptr, nullptr,
                         stats, s);
       if (rc != SEM_OK) return rc;
-      k_param_grad<<<L.nelem, 128, 0, s>>>(L.nelem, L.map, L.evert, ctx->sigma_l, ctx->sigma_t,
-                                           ctx->theta, gtab, tp->w, tp->seg_u + (j + 2) * n, g_sl,
-                                           g_st, g_th);
-      ADJ_CK(cudaGetLastError());
+      ADJ_CK(launch_param_grad(ctx, gtab, tp->w, tp->seg_u + (j + 2) * n, g_sl, g_st, g_th, s));
       if (L.quad == SEM_QUAD_LGL) {
         k_scale_mul<<<gr, kThreads, 0, s>>>(n, L.mdiag, tp->w, tp->gbar);
         ADJ_CK(cudaGetLastError());
