@@ -60,9 +60,9 @@ FP64_PEAK_TFLOPS = 1.25  # nominal GB300 FP64: 152 SMs x 2 DFMA/clk x 2 flop x ~
 # p = 4 SEM-NI slab of 2,064,933 nodes, each with the hash of the kernel sources it
 # was taken from: a figure whose kernel code has changed since is reported as null
 # (kernel_source_hash below; comments do not count).
-NCU_TRAFFIC = {(4, "LGL"): (273.026304e6 + 12.97408e6, "apply")}
-NCU_TRAFFIC_SMOOTHER = {(4, "LGL", "bf16"): (88.765696e6 + 1.543936e6, "apply")}
-NCU_SOURCE_HASH = {"apply": "9c6bd0526832d33d"}
+NCU_TRAFFIC = {(4, "LGL"): (273.02656e6 + 13.325056e6, "apply")}
+NCU_TRAFFIC_SMOOTHER = {(4, "LGL", "bf16"): (73.033472e6 + 1.024256e6, "apply")}
+NCU_SOURCE_HASH = {"apply": "43384910de6fa8b5"}
 KERNEL_SOURCES = {"apply": ("sem_apply_kernel.cuh", "sem_apply_fp32.cu", "sem_apply_fp64.cu",
                             "sem_internal.cuh")}
 
@@ -126,6 +126,14 @@ def apply_bytes_per_element_fp32(p: int, metric: str = "fp32") -> int:
     mb = 2 if metric in ("bf16", "tc") else 4
     mapb = 0 if metric == "tc" else 4 * n ** 3
     return 7 * mb * n ** 3 + mapb + 8 * p ** 3
+
+
+def smoother_bytes_per_element(p: int, metric: str) -> int:
+    """The same of the kernel that runs: it takes node indices from the lattice and reads
+    one int32 an element (its first node) in place of the map."""
+    if metric == "tc":
+        return apply_bytes_per_element_fp32(p, metric)
+    return apply_bytes_per_element_fp32(p, metric) - 4 * (p + 1) ** 3 + 4
 
 
 def apply_bytes_per_element(p: int) -> int:
@@ -468,7 +476,7 @@ def run_gpu(args):
     dominant = "outer_apply"
     if stats.n_smoother_apply > 0:
         sm_ms = stats.smoother_apply_ms / stats.n_smoother_apply
-        sm_bytes = n_e * apply_bytes_per_element_fp32(p, args.mg_precision)
+        sm_bytes = n_e * smoother_bytes_per_element(p, args.mg_precision)
         per_vcycle = 2 * args.mg_degree  # fine-level applies per V-cycle (one V-cycle per PCG iteration)
         kernels["smoother_apply"] = {
             "kernel": smoother_kernel_name(p, quad, args.mg_precision),

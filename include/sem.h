@@ -353,7 +353,7 @@ int sem_apply_dot_static(sem_ctx* ctx, double alpha, double beta, const double* 
 int sem_debug_set_map_entry(sem_ctx* ctx, int64_t entry, int value, int* previous);
 
 /* SEM_DEBUG build only (the normal build returns SEM_ERR_UNSUPPORTED): the
- * pipelined FP32 apply of the fine level leaves out the metric copy of element
+ * FP32 apply of the fine level (the plane kernel, whatever the mesh size) leaves out the metric copy of element
  * group `group` (its group index; -1: none), so that the warp's bounded wait
  * for that copy runs out.  That warp then sets the context's wait-timeout word,
  * lets its other copy in flight land and returns, and the next multigrid solve

@@ -375,7 +375,7 @@ def sem_debug_set_map_entry(ctx, entry: int, value: int) -> int:
 
 
 def sem_debug_hold_copy(ctx, group: int):
-    """SEM_DEBUG build only: the pipelined FP32 apply leaves out the metric copy of
+    """SEM_DEBUG build only: the FP32 apply leaves out the metric copy of
     element group `group` (-1: none), so that its bounded wait runs out."""
     return _check(lib().sem_debug_hold_copy(ctx, int(group)), ctx)
 

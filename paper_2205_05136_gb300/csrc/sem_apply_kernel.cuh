@@ -901,7 +901,7 @@ __global__ void __launch_bounds__(32 * PlaneCfg<P, MT>::kWarps, PlaneCfg<P, MT>:
   float* tiles = reinterpret_cast<float*>(wb + C::tile_offset);
   const unsigned sm_s = smem_u32(wb), tile_s = smem_u32(tiles), bar_s = smem_u32(wb + C::bar_offset);
   // While the previous kernel drains, before pdl_wait: the first metric copies and
-  // the map entries (written by the set-up only, see pdl_trigger).
+  // the first nodes (written by the set-up only, see pdl_trigger).
   if (lane == 0) {
     for (int t = 0; t < C::kStages; ++t) mbar_init(bar_s + 8 * t);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");

@@ -8,10 +8,9 @@
 // tissue of its first fine child.
 //
 // Transfers (matrix-vector products, Section 4.3):
-//   p-levels: per element, nodal interpolation Q_pc -> Q_pf by three 1-D
-//     sweeps; restriction is its transpose, with each fine node's residual
-//     divided by the number of elements sharing it so that the element-wise
-//     sum equals P^T r;
+//   p-levels: nodal interpolation Q_pc -> Q_pf, the tensor product of 1-D
+//     prolongations on the lattice (sem_transfer.cu); restriction is its
+//     transpose;
 //   h-levels: per fine vertex, the coarse trilinear function evaluated at the
 //     reference coordinates -1, 0, +1 of the coarse element (a trailing odd
 //     element spans one fine element: -1, +1); restriction by the transpose.

@@ -194,7 +194,7 @@ struct Level {
   bool metric32_valid = false, metric16_valid = false, metric2_valid = false, metric_tc_valid = false;
   unsigned long long* dbg = nullptr;  // SEM_DEBUG build: the context's index-error word
   unsigned* fault = nullptr;  // the context's wait-timeout word (nonzero: a kernel gave up a wait)
-  int hold = -1;  // SEM_DEBUG build: element group whose metric copy the pipelined apply skips
+  int hold = -1;  // SEM_DEBUG build: element group whose metric copy the plane kernel skips
   double* mdiag = nullptr;
   double* kdiag = nullptr;
   double* xyz = nullptr;
@@ -278,8 +278,7 @@ struct ApplyArgs {
   // fixed order
   typename VecOf<T>::type* yloc;
   // set by the launcher: the vectors' length and strides, the elements' first
-  // nodes, the SEM_DEBUG index-error word and
-  // the wait-timeout word
+  // nodes, the SEM_DEBUG index-error word and the wait-timeout word
   int64_t ndofs;
   int row, plane;  // lattice strides: nodes of an x-row and of an (x, y) plane
   const int* first;  // Level::first
@@ -302,7 +301,7 @@ int apply_grid_blocks(const Level& L);
 int dot_blocks(const Level& L, bool df64);
 // y[g] += the element contributions yloc[e][n^3] of node g, elements in a fixed
 // order (ez, ey, ex ascending): the deterministic assembly of the apply kernels'
-// element results (and of the p-restriction's coarse-element results).
+// element results.
 cudaError_t launch_assemble(const Level& L, const double* yloc, double* y, const int* done, cudaStream_t s);
 cudaError_t launch_assemble(const Level& L, const float* yloc, float* y, const int* done, cudaStream_t s);
 // Sum, in a fixed order, of the n per-CTA partials of a fused inner product:
