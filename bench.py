@@ -62,7 +62,7 @@ FP64_PEAK_TFLOPS = 1.25  # nominal GB300 FP64: 152 SMs x 2 DFMA/clk x 2 flop x ~
 # (kernel_source_hash below; comments do not count).
 NCU_TRAFFIC = {(4, "LGL"): (273.02656e6 + 13.325056e6, "apply")}
 NCU_TRAFFIC_SMOOTHER = {(4, "LGL", "bf16"): (73.033472e6 + 1.024256e6, "apply")}
-NCU_SOURCE_HASH = {"apply": "43384910de6fa8b5"}
+NCU_SOURCE_HASH = {"apply": "ef6141e672304f3f"}
 KERNEL_SOURCES = {"apply": ("sem_apply_kernel.cuh", "sem_apply_fp32.cu", "sem_apply_fp64.cu",
                             "sem_internal.cuh")}
 

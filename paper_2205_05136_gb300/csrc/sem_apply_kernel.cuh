@@ -1064,23 +1064,29 @@ cudaError_t launch_apply_plane(const Level& L, const ApplyArgs<float, MT>& a, co
   return cudaGetLastError();
 }
 
-// The FP32 operator on few elements (p >= 3): one 1-D line of an element per thread,
-// an element (two at p = 3) per CTA.  Below about a warp of the plane kernel an SM the
-// apply takes as long as one warp takes for its unit, and a lane of that kernel works
-// through a whole plane; here a thread works through one line a sweep, the column's
-// metric waits in registers before pdl_wait, and the z-sweeps are registers only.
-// An apply, FP32 metric, plane kernel / this one, on 288 elements: SEM-NI p = 3..6
+// The FP32 operator on few elements (p >= 3): one 1-D line of an element per thread, E
+// elements a CTA.  Below about a warp of the plane kernel an SM the apply takes as long
+// as one warp takes for its unit, and a lane of that kernel works through a whole plane;
+// here a thread works through one line a sweep, the column's metric waits in registers
+// before pdl_wait, and the z-sweeps are registers only.  E fills the warps where that
+// pays: one element a CTA took 5.9 instead of 5.1 us at p = 4 (2,808 elements, SEM-NI),
+// 7.5 instead of 7.2 at p = 5; three a CTA at p = 6 lose by the wider barriers (88
+// elements 3.5 us against 3.0).
+// An apply, FP32 metric, plane kernel / this one, p = 3..6: 288 elements, SEM-NI
 // 3.1 / 2.6, 3.9 / 2.8, 6.1 / 3.0, 7.1 / 3.4 us, SEM 3.5 / 2.9, 5.5 / 3.2, 8.0 / 3.5,
-// 10.1 / 3.9; on 1,250 elements 3.2 / 3.0, 4.0 / 3.8, 6.6 / 4.7, 8.0 / 6.0 and 3.6 / 3.3,
-// 6.0 / 4.1, 8.8 / 5.6, 11.5 / 6.9; on 2,808 elements 3.5 / 4.3, 4.7 / 5.9, 7.2 / 7.6,
-// 9.1 / 10.3 and 4.0 / 4.9, 6.4 / 6.4, 9.4 / 9.3, 12.4 / 12.2.  The line (kElements)
-// lies where the two meet.  At p = 1 and 2 the plane kernel is as fast on any mesh.
+// 10.1 / 3.9; 1,250 elements 3.2 / 2.9, 4.0 / 3.4, 6.6 / 4.4, 8.0 / 5.9 and 3.6 / 3.3,
+// 6.0 / 3.8, 8.8 / 5.0, 11.5 / 6.9; 2,808 elements 3.5 / 3.8, 4.6 / 5.1, 7.2 / 7.2,
+// 9.0 / 10.2 and 4.0 / 4.5, 6.4 / 5.6, 9.4 / 8.5, 12.3 / 12.1; 5,760 elements
+// 4.0 / 5.9, 6.1 / 8.0, 8.5 / 12.1 and 4.8 / 7.0, 7.8 / 9.3, 10.7 / 14.4 (p = 3..5).
+// The line (kElements) lies where the two meet.  At p = 1 and 2 the plane kernel is as
+// fast on any mesh.
 template <int P, int QUAD>
 struct FewCfg {
-  static constexpr int N2 = (P + 1) * (P + 1), E = P == 3 ? 2 : 1;
+  static constexpr int N2 = (P + 1) * (P + 1), E = P == 3 ? 4 : P == 4 ? 5 : P == 5 ? 3 : 1;
   static constexpr int kThreads = (E * N2 + 31) / 32 * 32;
   static constexpr bool kSem = QUAD == SEM_QUAD_LG;
-  static constexpr int kElements = P == 3 ? 1500 : P == 4 ? (kSem ? 2500 : 1500) : P == 5 ? (kSem ? 2800 : 2400) : kSem ? 2800 : 2200;
+  static constexpr int kElements =
+      P == 3 ? 1600 : P == 4 ? (kSem ? 3800 : 2200) : P == 5 ? (kSem ? 3400 : 2600) : kSem ? 2800 : 2200;
 };
 
 template <int P, int QUAD, typename MT>

@@ -4,7 +4,7 @@ A unit is G = 32 // (p + 1) consecutive elements of one warp: meshes of one elem
 one unit exactly, of one element more or less, of rows that end inside a unit, of more
 elements than one CTA of the metric's conversion takes, and vectors
 that start 4 bytes past a 16-byte boundary (the gather copies single words).  From p = 3 the
-meshes of up to some 2,000 elements take the kernel of one line per thread; 2,989 and 3,360
+meshes of up to some 3,000 elements take the kernel of one line per thread; 4,067 and 4,320
 elements (no multiple and a multiple of every unit) take the plane kernel.  The reference
 is the FP64 apply, which the other tests hold to the oracle.  Bounds as in test_gpu_apply:
 FP32 arithmetic with an FP32 metric 6e-7, the bf16 metric 5e-3 (relative, 2-norm).
@@ -22,7 +22,7 @@ gb = pytest.importorskip("paper_2205_05136_gb300")
 
 def _dims(p):
     g = 32 // (p + 1)
-    large = [(61, 7, 7), (60, 7, 8)] if p >= 3 else []  # above the sizes of the kernel for few elements
+    large = [(83, 7, 7), (60, 8, 9)] if p >= 3 else []  # above the sizes of the kernel for few elements
     return large + [(1, 1, 1), (g, 1, 1), (g - 1, 1, 1), (g + 1, 1, 1), (3, 2, 2), (g + 2, 3, 2), (8 * g + 1, 1, 1)]
 
 
