@@ -52,8 +52,9 @@ extern "C" {
 #define SEM_ERR_NONFINITE (-5)     /* NaN or Inf met in a CG inner product */
 #define SEM_ERR_UNSUPPORTED (-6)   /* valid request that this library does not provide */
 #define SEM_ERR_NOMEM (-7)         /* device allocation failed */
-#define SEM_ERR_TIMEOUT (-8)       /* a kernel's bounded wait for its own copy gave up (reported by the
-                                      next multigrid solve; the context stays usable) */
+#define SEM_ERR_TIMEOUT (-8)       /* a kernel's bounded wait gave up: for its own copy (reported by the next
+                                      multigrid solve) or at the grid barrier of the CG vector update
+                                      (reported by that solve); the context stays usable */
 
 #define SEM_QUAD_LG 0  /* SEM: (p+1)-point Legendre-Gauss quadrature */
 #define SEM_QUAD_LGL 1 /* SEM-NI: (p+1)-point Legendre-Gauss-Lobatto quadrature */
@@ -361,6 +362,13 @@ int sem_debug_set_map_entry(sem_ctx* ctx, int64_t entry, int value, int* previou
  * path without any fault.  Drops the multigrid hierarchy (its captured graphs
  * hold the launch arguments); the next solve rebuilds it.  Synchronous. */
 int sem_debug_hold_copy(sem_ctx* ctx, int group);
+
+/* SEM_DEBUG build only (the normal build returns SEM_ERR_UNSUPPORTED): CTA `cta`
+ * (-1: none) of the one-kernel CG vector update does not arrive at its grid
+ * barrier, so that the others' bounded wait runs out.  The kernel returns and
+ * the solve gives SEM_ERR_TIMEOUT; with the hook off again the next solve is as
+ * before. */
+int sem_debug_hold_update(sem_ctx* ctx, int cta);
 
 /* Enable (1) or disable (0) CUDA-event timing of the operator-apply kernels
  * inside sem_step / sem_cg_solve (reported in sem_stats).  One solve in ten

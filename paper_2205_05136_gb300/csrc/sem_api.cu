@@ -808,6 +808,18 @@ int sem_debug_hold_copy(sem_ctx* ctx, int group) {
 #endif
 }
 
+int sem_debug_hold_update(sem_ctx* ctx, int cta) {
+  CK_CTX(ctx);
+#ifdef SEM_DEBUG
+  if (cta < -1) return fail(ctx, SEM_ERR_ARG, "cta must be >= -1");
+  ctx->hold_update = cta;
+  return SEM_OK;
+#else
+  (void)cta;
+  return fail(ctx, SEM_ERR_UNSUPPORTED, "sem_debug_hold_update needs the SEM_DEBUG build");
+#endif
+}
+
 int sem_gmg_info(sem_ctx* ctx, double alpha, int max_levels, int* nlevels, int* p, int* dims,
                  int64_t* ndofs, double* lambda_max, void* stream) {
   CK_CTX(ctx);

@@ -65,6 +65,7 @@ struct sem_ctx {
   sem::Workspace ws;
   sem::Timing timing;
   int64_t launches = 0;             // libsem kernels launched so far
+  int hold_update = -1;             // SEM_DEBUG build: CTA of k_cg_update that does not arrive
   sem::Gmg* gmg = nullptr;          // built on first use of the multigrid preconditioner
   sem::Tape* tape = nullptr;        // recorded forward run for the adjoint
   int gmg_degree = 3, gmg_coarse_degree = 10, gmg_min_coarse_dofs = 2000;

@@ -43,9 +43,12 @@ __device__ __forceinline__ int64_t dbg_index(int64_t g, int64_t n, unsigned long
 // a copy the SEM_DEBUG build leaves out on request (sem_debug_hold_copy), so that
 // the wait for it runs out and the timeout path runs
 #define SEM_HOLD(a, unit) ((unit) == (a).hold)
+// the same for a CTA's arrival at a grid barrier (sem_debug_hold_update)
+#define SEM_HOLD_CTA(hold) ((int)blockIdx.x == (hold))
 #else
 #define SEM_IDX(g, n, word, kind) (g)
 #define SEM_HOLD(a, unit) false
+#define SEM_HOLD_CTA(hold) ((void)(hold), false)
 #endif
 
 // Programmatic dependent launch (PDL).  A kernel launched by launch_k may be

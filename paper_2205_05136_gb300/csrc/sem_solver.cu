@@ -233,6 +233,18 @@ __global__ void __launch_bounds__(kVecThreads)
   pdl_trigger();
 }
 
+// Waits until *gen leaves `mine`; false when it has not within kMbarTimeoutNs (the CTAs of
+// a cooperative launch run at the same time, so the bound only turns a barrier that never
+// opens into an error status).
+static __device__ __noinline__ bool grid_wait(const volatile unsigned* gen, unsigned mine) {
+  const unsigned long long t0 = global_ns();
+  while (true) {
+    for (int i = 0; i < 64; ++i)
+      if (*gen != mine) return true;
+    if (global_ns() - t0 > kMbarTimeoutNs) return false;
+  }
+}
+
 // Both vector updates of a CG iteration and their scalars in one cooperative kernel:
 // every CTA sums the apply's partials of p . A p (in one fixed order, so all CTAs hold
 // the same alpha), updates x and r, and after a grid barrier over the partial sums of
@@ -252,7 +264,7 @@ template <int PAIRS>
 __global__ void __launch_bounds__(kUpdThreads, 1)
     k_cg_update(int64_t n, double* __restrict__ x, double* __restrict__ p, df_pair* __restrict__ p2,
                 double* __restrict__ Ap, double* __restrict__ r, const double* __restrict__ inv, CgScalars* cg,
-                const double* __restrict__ dot, int ndot, double* partials, unsigned* bar) {
+                const double* __restrict__ dot, int ndot, double* partials, unsigned* bar, int hold) {
   if (cg->done) return;
   __shared__ double red[2][32], bc[2];
   __shared__ int gave_up;
@@ -326,14 +338,14 @@ __global__ void __launch_bounds__(kUpdThreads, 1)
       volatile unsigned* gen = bar + 1;
       const unsigned mine = *gen;
       __threadfence();
-      if (atomicAdd(bar, 1u) == gridDim.x - 1) {
+      if (SEM_HOLD_CTA(hold)) {
+        gave_up = 1;  // this CTA does not arrive
+      } else if (atomicAdd(bar, 1u) == gridDim.x - 1) {
         *(volatile unsigned*)bar = 0u;
         __threadfence();
         *gen = mine + 1u;
-      } else {
-        int left = 1 << 22;  // seconds; the CTAs of a cooperative launch run at the same time
-        while (*gen == mine && --left) {}
-        if (left == 0) gave_up = 1;
+      } else if (!grid_wait(gen, mine)) {
+        gave_up = 1;
       }
       __threadfence();
     }
@@ -353,7 +365,7 @@ __global__ void __launch_bounds__(kUpdThreads, 1)
   __syncthreads();
   const double beta = red[0][0];
   const bool stop = !finite || nrr <= cg->tol2;
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
+  if (blockIdx.x == 0 && threadIdx.x == 0 && !gave_up) {
     cg->pAp = pAp;
     cg->alpha = alpha;
     cg->beta = beta;
@@ -363,8 +375,8 @@ __global__ void __launch_bounds__(kUpdThreads, 1)
     if (!finite) cg->status = SEM_ERR_NONFINITE;
     if (stop) cg->done = 1;
   }
-  if (gave_up && threadIdx.x == 0) {
-    cg->status = SEM_ERR_CUDA;
+  if (gave_up && threadIdx.x == 0) {  // cg_result clears the barrier's words
+    cg->status = SEM_ERR_TIMEOUT;
     cg->done = 1;
   }
   if (stop || gave_up) return;
@@ -386,7 +398,8 @@ __global__ void __launch_bounds__(kUpdThreads, 1)
 constexpr int64_t kUpdateMin = 100000, kUpdateNodes = (int64_t)kUpdCtas * kUpdThreads * 2 * 4;
 
 cudaError_t launch_cg_update(int64_t n, double* x, double* p, df_pair* p2, double* Ap, double* r, const double* inv,
-                             CgScalars* cg, const double* dot, int ndot, double* partials, unsigned* bar, cudaStream_t s) {
+                             CgScalars* cg, const double* dot, int ndot, double* partials, unsigned* bar, int hold,
+                             cudaStream_t s) {
   const int64_t pairs = (n + 1) / 2, each = (pairs + kUpdCtas - 1) / kUpdCtas;  // of a CTA
   const int per = each <= kUpdThreads ? 1 : each <= 2 * kUpdThreads ? 2 : 4;
   const int threads = (int)std::max<int64_t>(128, (each + per - 1) / per + 31) / 32 * 32;
@@ -400,7 +413,7 @@ cudaError_t launch_cg_update(int64_t n, double* x, double* p, df_pair* p2, doubl
   cfg.attrs = at;
   cfg.numAttrs = 1;
   auto* k = per == 1 ? k_cg_update<1> : per == 2 ? k_cg_update<2> : k_cg_update<4>;
-  return cudaLaunchKernelEx(&cfg, k, n, x, p, p2, Ap, r, inv, cg, dot, ndot, partials, bar);
+  return cudaLaunchKernelEx(&cfg, k, n, x, p, p2, Ap, r, inv, cg, dot, ndot, partials, bar, hold);
 }
 
 // Whether the device runs k_cg_update's CTAs side by side.
@@ -831,7 +844,8 @@ int apply_tc(sem_ctx* ctx, double alpha, double beta, const float* u, float* y, 
 }
 
 // Reports the solve whose scalars the host has read.
-static int cg_result(sem_ctx* ctx, bool done, int maxit, int* iters, double* final_res, sem_stats* stats) {
+static int cg_result(sem_ctx* ctx, bool done, int maxit, int* iters, double* final_res, sem_stats* stats,
+                     cudaStream_t s) {
   const CgScalars& h = *ctx->ws.cg_host;
   if (iters) *iters = h.iters;
   if (final_res) *final_res = std::sqrt(h.rr);
@@ -841,9 +855,12 @@ static int cg_result(sem_ctx* ctx, bool done, int maxit, int* iters, double* fin
   }
   if (h.status == SEM_ERR_NONFINITE)
     return fail(ctx, SEM_ERR_NONFINITE, "non-finite value in a CG inner product");
-  if (h.status == SEM_ERR_CUDA) {
-    cudaMemset(ctx->ws.tickets, 0, sizeof(unsigned) * 4);
-    return fail(ctx, SEM_ERR_CUDA, "the CG update gave up waiting for its grid barrier");
+  if (h.status == SEM_ERR_TIMEOUT) {
+    // the arrivals it left would open the next solve's barrier too early: cleared on the
+    // solve's stream, and complete before any other stream can follow
+    SEM_CK(cudaMemsetAsync(ctx->ws.tickets, 0, sizeof(unsigned) * 4, s));
+    SEM_CK(cudaStreamSynchronize(s));
+    return fail(ctx, SEM_ERR_TIMEOUT, "the CG update's wait for its grid barrier timed out");
   }
   if (!done)
     return fail(ctx, SEM_ERR_NOT_CONVERGED,
@@ -887,7 +904,7 @@ int cg_solve(sem_ctx* ctx, double alpha, const double* b, double* x, double rtol
       SEM_CK(cudaStreamSynchronize(s));
       resume = true;
     } while (!w.cg_host->done && w.cg_host->iters < maxit);
-    return cg_result(ctx, w.cg_host->done != 0, maxit, iters, final_res, stats);
+    return cg_result(ctx, w.cg_host->done != 0, maxit, iters, final_res, stats, s);
   }
   // Ap = A x (or the carried ax0), then the initial residual; Ap is zero for the iterations
   SEM_CK(cudaMemsetAsync(w.Ap, 0, sizeof(double) * n, s));
@@ -932,7 +949,7 @@ int cg_solve(sem_ctx* ctx, double alpha, const double* b, double* x, double rtol
         if (timed) SEM_CK(cudaEventRecord(tm.stop, s));
         if (one) {
           SEM_CK(launch_cg_update(n, x, w.p, p2, w.Ap, w.r, inv, w.cg, w.apply_partials, ndot, w.vec_partials,
-                                  w.tickets + 1, s));
+                                  w.tickets + 1, ctx->hold_update, s));
           continue;
         }
         if ((reinterpret_cast<uintptr_t>(x) & 15u) == 0)
@@ -962,7 +979,7 @@ int cg_solve(sem_ctx* ctx, double alpha, const double* b, double* x, double rtol
     if (launched >= maxit) break;
     chunk = std::min(kChunkMax, chunk * 2);
   }
-  return cg_result(ctx, done, maxit, iters, final_res, stats);
+  return cg_result(ctx, done, maxit, iters, final_res, stats, s);
 }
 
 // Constants of dfexp: ln2 split for Cody and Waite's reduction (c1, c2 with 16
