@@ -282,11 +282,13 @@ __host__ __device__ constexpr size_t apply_warp_tile_bytes() {
 }
 
 // The element results (mass M_e + K_e) u_e (MASS_ONLY: mass M_e u_e) of ne element
-// tiles, from the gathered values in sA into sA; sB, sC scratch of the same size.  Tile
+// tiles, from the gathered values in sA into sA; sB, sC scratch of the same size.
+// weight: W alone (float and bf16 metrics, MASS_ONLY), [element][padded n^3].  Tile
 // s is element e0 + s, and those from e_end on have no metric (their values are zero).
 template <int P, int QUAD, bool MASS_ONLY, bool ROLLED, bool WARP, typename T, typename MT>
-__device__ __forceinline__ void element_results(const KTab<P + 1, T>& tab, const MT* metric, T mass, int e0, int e_end,
-                                                int ne, T* sA, T* sB, T* sC, int tid, int nth) {
+__device__ __forceinline__ void element_results(const KTab<P + 1, T>& tab, const MT* metric,
+                                                const MT* weight, T mass, int e0, int e_end, int ne, T* sA, T* sB,
+                                                T* sC, int tid, int nth) {
   constexpr int N = P + 1, N2 = N * N, N3 = N2 * N;
   using ML = MetricLayout<MT>;
   auto group_sync = [] {
@@ -313,7 +315,8 @@ __device__ __forceinline__ void element_results(const KTab<P + 1, T>& tab, const
     for (int idx = tid; idx < ne * N3; idx += nth) {
       const int s = idx / N3, loc = idx - s * N3, e = e0 + s;
       if (e < e_end) {
-        const T W = ldmetric(metric + ML::offset(N, e, loc % N2, loc / N2, 6));
+        const T W = ldmetric(std::is_same<T, float>::value ? weight + (size_t)e * padded_n3(N) + loc
+                                                           : metric + ML::offset(N, e, loc % N2, loc / N2, 6));
         sA[idx] = (mass * W) * sA[idx];
       }
     }
@@ -478,7 +481,8 @@ __global__ void __launch_bounds__(MASS_ONLY ? kApplyThreads : ApplyCta<P, T, DOT
   }
   group_sync();
 
-  element_results<P, QUAD, MASS_ONLY, kRolled, WARP>(tab, a.metric, a.mass_coef, e0, a.nelem, E, sA, sB, sC, tid, nth);
+  element_results<P, QUAD, MASS_ONLY, kRolled, WARP>(tab, a.metric, a.weight, a.mass_coef, e0, a.nelem, E, sA, sB, sC,
+                                                     tid, nth);
 
   pdl_trigger();
   // scatter-add y += P_e^T y_e, and with DOT the partial u_e . y_e
@@ -1315,6 +1319,7 @@ cudaError_t launch_apply_t(const Level& L, const ApplyArgs<T, MT>& a, bool mass_
   b.ndofs = L.ndofs;
   b.row = P * L.nx + 1;
   b.first = L.first;
+  b.weight = std::is_same<T, float>::value && weight_lowp_count(L) > 0 ? a.metric + metric_lowp_count(L) : nullptr;
   b.plane = b.row * (P * L.ny + 1);
   b.dbg = L.dbg;
   b.fault = L.fault;

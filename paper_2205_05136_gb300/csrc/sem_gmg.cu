@@ -1501,13 +1501,13 @@ int level_metrics(sem_ctx* ctx, Gmg& g, cudaStream_t s) {
   for (GmgLevel& V : g.lv) {
     Level& L = *V.L;
     if (g.precision == SEM_PREC_FP32 && !L.metric32_valid) {
-      if (!L.metric32) GMG_CK(cudaMalloc(&L.metric32, sizeof(float) * metric_lowp_count(L)));
+      if (!L.metric32) GMG_CK(cudaMalloc(&L.metric32, sizeof(float) * metric_lowp_values(L)));
       GMG_CK(setup_metric_lowp(L, false, s));
     }
     const bool tc = g.precision == SEM_PREC_BF16_TC && tc_supported(L) && !ctx->deterministic;
     if ((g.precision == SEM_PREC_FP32_BF16 || (g.precision == SEM_PREC_BF16_TC && !tc)) &&
         !L.metric16_valid) {
-      if (!L.metric16) GMG_CK(cudaMalloc(&L.metric16, sizeof(__nv_bfloat16) * metric_lowp_count(L)));
+      if (!L.metric16) GMG_CK(cudaMalloc(&L.metric16, sizeof(__nv_bfloat16) * metric_lowp_values(L)));
       GMG_CK(setup_metric_lowp(L, true, s));
     }
     if (tc && !L.metric_tc_valid) GMG_CK(setup_metric_tc(L, s));

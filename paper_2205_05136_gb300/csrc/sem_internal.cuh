@@ -195,6 +195,7 @@ struct Level {
   uint32_t* metric_tc = nullptr;  // bf16 metric in the tensor-core kernel's order (sem_apply_tc.cu)
   uint32_t* tc_frag = nullptr;    // constant MMA fragments of the tensor-core kernel
   bool metric32_valid = false, metric16_valid = false, metric2_valid = false, metric_tc_valid = false;
+  bool weight32_valid = false, weight16_valid = false;  // the weights behind them (geometry only: written once)
   unsigned long long* dbg = nullptr;  // SEM_DEBUG build: the context's index-error word
   unsigned* fault = nullptr;  // the context's wait-timeout word (nonzero: a kernel gave up a wait)
   int hold = -1;  // SEM_DEBUG build: element group whose metric copy the plane kernel skips
@@ -251,6 +252,15 @@ inline size_t metric_lowp_count(const Level& L) {
   const size_t units = ((size_t)L.nelem + ML::unit(L.n) - 1) / ML::unit(L.n);
   return units * ML::chunks(L.n) * ML::chunk(L.n);
 }
+// Behind them, on a SEM fine level, the weights W alone, [nelem][n3p]: the FP32 mass
+// operator reads nothing else, and taken from the seven values of each point they cost
+// it the whole metric.  An apply on 2 M nodes, p = 1..6: FP32 99 58 40 38 35 34 us so, 92
+// 49 31 25 25 25 from the FP64 metric, 82 41 29 23 23 23 from here; bf16 90 53 35 29 30 30
+// and 76 40 29 23 23 23.  The other levels only apply alpha M + K.
+inline size_t weight_lowp_count(const Level& L) {
+  return L.quad == SEM_QUAD_LG && L.xyz != nullptr ? (size_t)L.nelem * padded_n3(L.n) : 0;
+}
+inline size_t metric_lowp_values(const Level& L) { return metric_lowp_count(L) + weight_lowp_count(L); }
 
 constexpr int kScaleOut = 1, kNegateOut = 2;  // ApplyArgs::scale_out
 
@@ -285,6 +295,7 @@ struct ApplyArgs {
   int64_t ndofs;
   int row, plane;  // lattice strides: nodes of an x-row and of an (x, y) plane
   const int* first;  // Level::first
+  const MT* weight;  // mass-only FP32 kernels: W of every point (weight_lowp_count)
   unsigned long long* dbg;
   unsigned* fault;
   int hold;  // SEM_DEBUG build: Level::hold

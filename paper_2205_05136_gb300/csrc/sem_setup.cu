@@ -307,10 +307,12 @@ __device__ __forceinline__ __nv_bfloat16 metric_round<__nv_bfloat16>(double v) {
 // target's order, four values a thread and store; every index is split by constants.
 // DRAM bounds it.  A thread per target value, with 64-bit divisions by run-time sizes
 // and 8-byte loads seven components apart, took 2.46 ms on 462,024 elements at p = 4 for
-// bf16 and 2.36 for FP32; now 0.69 and 0.88 (6.2 TB/s both).
+// bf16 and 2.36 for FP32; now 0.69 and 0.88 (6.2 TB/s both).  weight: where W alone goes
+// too (weight_lowp_count), or nullptr.
 template <int N, typename OT>
 __global__ void __launch_bounds__(kSetupThreads)
-    k_convert_planes(int nelem, int padded, const double* __restrict__ in, OT* __restrict__ out) {
+    k_convert_planes(int nelem, int padded, const double* __restrict__ in, OT* __restrict__ out,
+                     OT* __restrict__ weight) {
   using ML = MetricLayout<OT>;
   constexpr int N2 = N * N, N3P = padded_n3(N), E = setup_elems(N2 * N), block = kMetricComps * N3P;
   constexpr int R = ML::rows(N), chunks = ML::chunks(N), RS = ML::stride(N), G = ML::unit(N);
@@ -321,6 +323,9 @@ __global__ void __launch_bounds__(kSetupThreads)
 #pragma unroll 8
   for (int t = threadIdx.x; t < ne * block; t += kSetupThreads) m[t] = metric_round<OT>(__ldcs(in + (size_t)e0 * block + t));
   __syncthreads();
+  if (weight != nullptr)
+    for (int t = threadIdx.x; t < ne * N3P; t += kSetupThreads)
+      weight[(size_t)e0 * N3P + t] = m[t / N3P * block + 6 * N3P + t % N3P];
   for (int t = threadIdx.x; t < nout * vectors; t += kSetupThreads) {
     const int el = t / vectors, q = t - el * vectors, v0 = 4 * (q % (RS / 4)), k = q / (RS / 4) % N,
               chunk = q / (RS / 4) / N, e = e0 + el, unit = e / G, slot = e - unit * G;
@@ -468,13 +473,19 @@ cudaError_t setup_diagonals(Level& L, cudaStream_t s) {
 cudaError_t setup_metric_lowp(Level& L, bool bf16, cudaStream_t s) {
   const int G = PlaneMetricLayout::unit(L.n), padded = (L.nelem + G - 1) / G * G;
   (bf16 ? L.metric16_valid : L.metric32_valid) = true;
+  bool& written = bf16 ? L.weight16_valid : L.weight32_valid;
+  const bool weights = weight_lowp_count(L) > 0 && !written;
+  const size_t at = metric_lowp_count(L);
+  written = written || weights;
   return for_points(L.n, [&](auto n) {
     constexpr int N = decltype(n)::value, E = setup_elems(N * N * N);
     const int ctas = (padded + E - 1) / E;
     if (bf16)
-      k_convert_planes<N><<<ctas, kSetupThreads, 0, s>>>(L.nelem, padded, L.metric, L.metric16);
+      k_convert_planes<N><<<ctas, kSetupThreads, 0, s>>>(L.nelem, padded, L.metric, L.metric16,
+                                                 weights ? L.metric16 + at : nullptr);
     else
-      k_convert_planes<N><<<ctas, kSetupThreads, 0, s>>>(L.nelem, padded, L.metric, L.metric32);
+      k_convert_planes<N><<<ctas, kSetupThreads, 0, s>>>(L.nelem, padded, L.metric, L.metric32,
+                                                 weights ? L.metric32 + at : nullptr);
   });
 }
 
