@@ -370,6 +370,12 @@ int sem_debug_hold_copy(sem_ctx* ctx, int group);
  * before. */
 int sem_debug_hold_update(sem_ctx* ctx, int cta);
 
+/* SEM_DEBUG build only (the normal build returns SEM_ERR_UNSUPPORTED): the context
+ * takes the device for one that can place at most `ctas` CTAs in a cluster, so that
+ * the CG solves of small meshes fall back to a kernel per step as they do on such a
+ * device (a partition of a GPU, for instance). */
+int sem_debug_limit_cluster(sem_ctx* ctx, int ctas);
+
 /* Enable (1) or disable (0) CUDA-event timing of the operator-apply kernels
  * inside sem_step / sem_cg_solve (reported in sem_stats).  One solve in ten
  * (the first after enabling, then every tenth) times the operator apply of its

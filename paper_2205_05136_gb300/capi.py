@@ -54,6 +54,7 @@ EXPORTS = [
     "sem_set_timing", "sem_apply_dot_static", "sem_set_gmg", "sem_vcycle", "sem_gmg_info",
     "sem_forward_record", "sem_adjoint_grad", "sem_set_operator_precision", "sem_set_deterministic",
     "sem_debug_set_map_entry", "sem_debug_hold_copy", "sem_debug_hold_update",
+    "sem_debug_limit_cluster",
 ]
 
 
@@ -125,6 +126,7 @@ def lib():
             "sem_debug_set_map_entry": (_I, [_P, _I64, _I, ctypes.POINTER(_I)]),
             "sem_debug_hold_copy": (_I, [_P, _I]),
             "sem_debug_hold_update": (_I, [_P, _I]),
+            "sem_debug_limit_cluster": (_I, [_P, _I]),
             "sem_forward_record": (_I, [_P, _P, _D, _I, _I, _P, _I, _P, _D, _D, _I, _I,
                                         ctypes.POINTER(sem_stats), _P]),
             "sem_adjoint_grad": (_I, [_P, _P, _P, _P, _P, _D, _D, _I, _I, ctypes.POINTER(sem_stats), _P]),
@@ -385,6 +387,12 @@ def sem_debug_hold_update(ctx, cta: int):
     """SEM_DEBUG build only: CTA `cta` (-1: none) of the one-kernel CG vector update does not
     arrive at its grid barrier, so that the others' bounded wait runs out."""
     return _check(lib().sem_debug_hold_update(ctx, int(cta)), ctx)
+
+
+def sem_debug_limit_cluster(ctx, ctas: int):
+    """SEM_DEBUG build only: treat the device as one that can place at most `ctas` CTAs in a
+    cluster (the CG solves of small meshes then take a kernel per step)."""
+    return _check(lib().sem_debug_limit_cluster(ctx, int(ctas)), ctx)
 
 
 def sem_set_deterministic(ctx, enable: bool):

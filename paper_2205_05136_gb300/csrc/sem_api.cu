@@ -820,6 +820,19 @@ int sem_debug_hold_update(sem_ctx* ctx, int cta) {
 #endif
 }
 
+int sem_debug_limit_cluster(sem_ctx* ctx, int ctas) {
+  CK_CTX(ctx);
+#ifdef SEM_DEBUG
+  if (ctas < 0) return fail(ctx, SEM_ERR_ARG, "ctas must be >= 0");
+  ctx->max_cluster = ctas;
+  ctx->cg_small = -1;
+  return SEM_OK;
+#else
+  (void)ctas;
+  return fail(ctx, SEM_ERR_UNSUPPORTED, "sem_debug_limit_cluster needs the SEM_DEBUG build");
+#endif
+}
+
 int sem_gmg_info(sem_ctx* ctx, double alpha, int max_levels, int* nlevels, int* p, int* dims,
                  int64_t* ndofs, double* lambda_max, void* stream) {
   CK_CTX(ctx);

@@ -274,6 +274,43 @@ __global__ void __launch_bounds__(kThreads)
   cluster_sync();  // no CTA ends while another may write to its shared memory
 }
 
+// CTAs of the cluster: 8 up to 1,500 nodes (20 time steps of 765 nodes: 1.61 ms, 1.84 with
+// 16: cheaper barriers and sums), above and at p = 1 (most elements a node) the 16 SMs pay.
+int small_ctas(const Level& L) { return L.p >= 2 && L.ndofs <= 1500 ? 8 : kCtasMax; }
+
+template <int P>
+constexpr size_t small_smem() {
+  return (size_t)3 * ApplyCfg<P>::E * (P + 1) * (P + 1) * (P + 1) * sizeof(double);
+}
+
+// Grid, block, shared memory and cluster of nc CTAs (at[0]).
+template <int P>
+void small_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at, int nc) {
+  static_assert(small_smem<P>() <= 46 * 1024, "within the default limit beside the static arrays");
+  cfg.gridDim = dim3((unsigned)nc);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = small_smem<P>();
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)nc;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+}
+
+// Whether the device can hold the cluster (a partition of a GPU may have no 16 SMs in one
+// GPC); also allows the kernel the cluster size beyond the portable 8.
+template <int P, int QUAD>
+bool small_placeable(int nc) {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at[1];
+  small_config<P>(cfg, at, nc);
+  int clusters = 0;
+  const bool ok = cudaFuncSetAttribute(k_cg_small<P, QUAD>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                  cudaOccupancyMaxActiveClusters(&clusters, k_cg_small<P, QUAD>, &cfg) == cudaSuccess;
+  if (!ok) cudaGetLastError();  // the launches of cg_solve take the mesh instead
+  return ok && clusters > 0;
+}
+
 template <int P, int QUAD>
 cudaError_t launch_small(const Level& L, const SmallArgs& a, cudaStream_t s) {
   constexpr int N = P + 1;
@@ -282,42 +319,44 @@ cudaError_t launch_small(const Level& L, const SmallArgs& a, cudaStream_t s) {
   make_eo(tab.Dt, QUAD == SEM_QUAD_LG ? L.tab.Dg : L.tab.D, true);
   make_eo(tab.Bi, L.tab.Bi, false);
   make_eo(tab.Bit, L.tab.Bi, true);
-  constexpr size_t smem = (size_t)3 * ApplyCfg<P>::E * N * N * N * sizeof(double);
-  static_assert(smem <= 46 * 1024, "within the default limit beside the static arrays");
-  cudaError_t e = cudaFuncSetAttribute(k_cg_small<P, QUAD>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (e != cudaSuccess) return e;
-  // 8 CTAs up to 1,500 nodes (20 time steps of 765 nodes: 1.61 ms, 1.84 with 16: cheaper
-  // barriers and sums), above and at p = 1 (most elements a node) the 16 SMs pay
-  const int nc = L.p >= 2 && L.ndofs <= 1500 ? 8 : kCtasMax;
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)nc);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
   cudaLaunchAttribute at[2];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = (unsigned)nc;
-  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  small_config<P>(cfg, at, small_ctas(L));
+  cfg.stream = s;
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
   cfg.numAttrs = pdl_enabled() ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, k_cg_small<P, QUAD>, a, tab);
 }
 
 }  // namespace
 
-// Whether the one-kernel solve takes a mesh: up to where it measured even with the
-// launches of cg_solve (us a time step, launches / one kernel): p = 1 SEM-NI 177 / 173 at
-// 4,816 nodes, SEM 768 / 791 at 3,108; p = 2 SEM-NI 213 / 216 at 9,405, SEM 600 / 594 at
+// Whether the one-kernel solve takes a mesh on the current device: up to where it
+// measured even with the launches of cg_solve (us a time step, launches / one kernel):
+// p = 1 SEM-NI 177 / 173 at 4,816 nodes, SEM 768 / 791 at 3,108; p = 2 SEM-NI 213 / 216 at 9,405, SEM 600 / 594 at
 // 7,497; p = 3 SEM 749 / 781 at 10,450; p = 4 SEM 817 / 868 at 14,625; p = 6 SEM still
 // 1,172 / 661 at 8,113.
-bool cg_small_fits(const Level& L) {
+bool cg_small_fits(const Level& L, int max_ctas) {
   static constexpr int64_t kNodes[2][kMaxP + 1] = {
       {0, 2500, 6000, 9000, 12000, 14000, 14000},    // SEM
       {0, 4500, 8000, 10000, 12000, 14000, 14000}};  // SEM-NI
   static_assert(14000 <= kCtasMax * kThreads * kPer, "every node has a place");
-  return L.p >= 1 && L.p <= kMaxP && L.ndofs <= kNodes[L.quad == SEM_QUAD_LGL ? 1 : 0][L.p];
+  if (L.p < 1 || L.p > kMaxP || L.ndofs > kNodes[L.quad == SEM_QUAD_LGL ? 1 : 0][L.p]) return false;
+  const int nc = small_ctas(L);
+  if (nc > max_ctas) return false;
+#define SEM_CASE(PP) \
+  case PP:           \
+    return L.quad == SEM_QUAD_LG ? small_placeable<PP, SEM_QUAD_LG>(nc) : small_placeable<PP, SEM_QUAD_LGL>(nc);
+  switch (L.p) {
+    SEM_CASE(1)
+    SEM_CASE(2)
+    SEM_CASE(3)
+    SEM_CASE(4)
+    SEM_CASE(5)
+    SEM_CASE(6)
+  }
+#undef SEM_CASE
+  return false;
 }
 
 cudaError_t launch_cg_small(const Level& L, double alpha, const double* b, const double* inv, const double* ax0, double* x,

@@ -65,6 +65,8 @@ struct sem_ctx {
   sem::Workspace ws;
   sem::Timing timing;
   int64_t launches = 0;             // libsem kernels launched so far
+  int cg_small = -1;                // whether k_cg_small takes the mesh on this device (-1: not asked yet)
+  int max_cluster = 16;             // CTAs a cluster may have (fewer only by the SEM_DEBUG build's hook)
   int hold_update = -1;             // SEM_DEBUG build: CTA of k_cg_update that does not arrive
   sem::Gmg* gmg = nullptr;          // built on first use of the multigrid preconditioner
   sem::Tape* tape = nullptr;        // recorded forward run for the adjoint

@@ -355,8 +355,10 @@ cudaError_t setup_region_mask(const Level& L, int region, const double* prm, dou
 
 // CG of a small mesh in one kernel (sem_cg_small.cu): the solve of cg_solve with the FP64
 // operator, inv = 1 / diagonal or nullptr.  At most 64 iterations a launch; resume
-// continues from x, r, p and *sc.  p and Ap are scratch.
-bool cg_small_fits(const Level& L);
+// continues from x, r, p and *sc.  p and Ap are scratch.  cg_small_fits: whether it takes
+// the mesh and the current device can place its cluster (of at most max_ctas CTAs); it
+// must have returned true before launch_cg_small.
+bool cg_small_fits(const Level& L, int max_ctas);
 cudaError_t launch_cg_small(const Level& L, double alpha, const double* b, const double* inv, const double* ax0, double* x,
                             double* r, double* p, double* Ap, CgScalars* sc, double rtol, double atol, int maxit,
                             bool resume, cudaStream_t s);

@@ -895,7 +895,11 @@ int cg_solve(sem_ctx* ctx, double alpha, const double* b, double* x, double rtol
   }
   if (ax0_ok != nullptr) ax0 = nullptr;  // no device-side choice here: apply the operator
   Timing& tm = ctx->timing;
-  if (ctx->op_precision == SEM_PREC_FP64 && !ctx->deterministic && !tm.enabled && cg_small_fits(L)) {
+  auto small = [&] {  // mesh and device are the context's for good: asked once
+    if (ctx->cg_small < 0) ctx->cg_small = cg_small_fits(L, ctx->max_cluster) ? 1 : 0;
+    return ctx->cg_small != 0;
+  };
+  if (ctx->op_precision == SEM_PREC_FP64 && !ctx->deterministic && !tm.enabled && small()) {
     bool resume = false;
     do {
       SEM_CK(launch_cg_small(L, alpha, b, inv, ax0, x, w.r, w.p, w.Ap, w.cg, rtol, atol, maxit, resume, s));
