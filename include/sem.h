@@ -381,7 +381,8 @@ int sem_debug_limit_cluster(sem_ctx* ctx, int ctas);
  * (the first after enabling, then every tenth) times the operator apply of its
  * first iteration, and with the multigrid preconditioner also the fine-level
  * residual apply of that iteration's V-cycle: the events that bracket them cost
- * a few microseconds each, so the other solves run without them. */
+ * a few microseconds each, so the other solves run without them.  On a small mesh,
+ * where a whole solve is one kernel, the timed solve runs a kernel per step. */
 int sem_set_timing(sem_ctx* ctx, int enable);
 
 #ifdef __cplusplus

@@ -894,12 +894,16 @@ int cg_solve(sem_ctx* ctx, double alpha, const double* b, double* x, double rtol
     return fail(ctx, SEM_ERR_ARG, "unknown preconditioner");
   }
   if (ax0_ok != nullptr) ax0 = nullptr;  // no device-side choice here: apply the operator
+  // with timing on, the apply of the first iteration of one solve in kTimingEvery
+  // is bracketed by events (they interrupt the programmatic dependent launch; the
+  // one-kernel solve has no apply of its own, so that solve takes a kernel per step)
   Timing& tm = ctx->timing;
+  bool sample = tm.enabled && (tm.solves++ % kTimingEvery) == 0;
   auto small = [&] {  // mesh and device are the context's for good: asked once
     if (ctx->cg_small < 0) ctx->cg_small = cg_small_fits(L, ctx->max_cluster) ? 1 : 0;
     return ctx->cg_small != 0;
   };
-  if (ctx->op_precision == SEM_PREC_FP64 && !ctx->deterministic && !tm.enabled && small()) {
+  if (ctx->op_precision == SEM_PREC_FP64 && !ctx->deterministic && !sample && small()) {
     bool resume = false;
     do {
       SEM_CK(launch_cg_small(L, alpha, b, inv, ax0, x, w.r, w.p, w.Ap, w.cg, rtol, atol, maxit, resume, s));
@@ -933,9 +937,6 @@ int cg_solve(sem_ctx* ctx, double alpha, const double* b, double* x, double rtol
   if (!one) ap.cg = w.cg;
 
   constexpr int kChunkMax = 16;
-  // with timing on, the apply of the first iteration of one solve in kTimingEvery
-  // is bracketed by events (they interrupt the programmatic dependent launch)
-  bool sample = tm.enabled && (tm.solves++ % kTimingEvery) == 0;
   if (sample && (tm.start == nullptr || tm.stop == nullptr)) {
     if (tm.start == nullptr) SEM_CK(cudaEventCreate(&tm.start));
     if (tm.stop == nullptr) SEM_CK(cudaEventCreate(&tm.stop));

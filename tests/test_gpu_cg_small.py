@@ -79,3 +79,22 @@ def test_small_steps_match_launched_steps(quad):
     assert float(torch.linalg.norm(u0 - u1) / torch.linalg.norm(u1)) < 1e-10
     assert float(torch.linalg.norm(h0 - h1) / torch.linalg.norm(h1)) < 1e-11
     assert abs(i0 - i1) <= 2, (i0, i1)
+
+
+def test_timing_changes_the_timed_solve_only():
+    """With timing on, one solve in ten runs a kernel per step to bracket its apply; the nine after it
+    launch what they launch with timing off (three kernels a time step)."""
+    s, tissue, g = _problem((9, 5, 4), 2, "LGL")
+    g.set_ionic()
+    g.set_stimulus("box", (0.0, 0.0, 0.0, 3.0, 3.0, 3.0), 50.0, 0.0, 1.0)
+    st = g.new_state(-85.0, 1.0)
+    st.step(0.05, 2, rtol=1e-12)  # both alphas' diagonals
+    assert st.step(0.05, 9, rtol=1e-12).kernel_launches == 3 * 9
+    capi.sem_set_timing(g.ctx, True)
+    timed = st.step(0.05, 1, rtol=1e-12)
+    assert timed.n_apply == 1 and timed.apply_ms > 0.0 and timed.kernel_launches > 3
+    rest = st.step(0.05, 9, rtol=1e-12)
+    assert rest.n_apply == 0 and rest.kernel_launches == 3 * 9
+    assert st.step(0.05, 1, rtol=1e-12).n_apply == 1
+    st.close()
+    g.close()
