@@ -45,3 +45,24 @@ def test_plane_kernel_unit_edges(p, quad):
                     err = float(torch.linalg.norm(y.double() - ref) / torch.linalg.norm(ref))
                     assert err < tol, (p, quad, dims, off, alpha, prec, err)
         g.close()
+
+
+@pytest.mark.parametrize("quad", ["LGL", "LG"])
+@pytest.mark.parametrize("p,dims", [(1, (20, 12, 9)), (2, (12, 8, 5)), (3, (83, 7, 7)), (4, (83, 7, 7)), (5, (60, 8, 9)),
+                                    (6, (60, 8, 9)), (3, (9, 5, 3)), (5, (6, 4, 3))])
+def test_deterministic_element_results(p, quad, dims):
+    """Deterministic mode of the plane kernel at every degree (from p = 3 on 4,067 and 4,320 elements) and of
+    the kernel for few elements at odd degrees: bitwise repeat, and the FP64 operator within the bounds above."""
+    s = W.slab(*dims, (20.0, 7.0, 3.0), perturb=0.1, seed=1)
+    g = gb.Slab(s.flat_vertices(), *dims, p, quad)
+    g.set_tissue(np.full(s.n_elements, 0.12), np.full(s.n_elements, 0.03), W.transmural_fiber_angles(s))
+    gb.capi.sem_set_deterministic(g.ctx, True)
+    u = torch.tensor(W.uniform_vector(g.ndofs, -1.0, 1.0, seed=2), device="cuda").float()
+    for alpha, beta in ((30.0, 1.0), (2.5, -0.7)):
+        ref = g.apply(u.double(), alpha, beta)
+        for prec, tol in ((gb.SEM_PREC_FP32, 6e-7), (gb.SEM_PREC_FP32_BF16, 5e-3)):
+            y = g.apply(u, alpha, beta, prec)
+            assert torch.equal(y, g.apply(u, alpha, beta, prec))
+            err = float(torch.linalg.norm(y.double() - ref) / torch.linalg.norm(ref))
+            assert err < tol, (p, quad, dims, alpha, prec, err)
+    g.close()
