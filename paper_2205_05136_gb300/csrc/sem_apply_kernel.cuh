@@ -282,13 +282,12 @@ __host__ __device__ constexpr size_t apply_warp_tile_bytes() {
 }
 
 // The element results (mass M_e + K_e) u_e (MASS_ONLY: mass M_e u_e) of ne element
-// tiles, from the gathered values in sA into sA; sB, sC scratch of the same size.
-// weight: W alone (float and bf16 metrics, MASS_ONLY), [element][padded n^3].  Tile
+// tiles, from the gathered values in sA into sA; sB, sC scratch of the same size.  The
+// FP32 mass operator's metric is W alone, [element][padded n^3] (weight_lowp_count).  Tile
 // s is element e0 + s, and those from e_end on have no metric (their values are zero).
 template <int P, int QUAD, bool MASS_ONLY, bool ROLLED, bool WARP, typename T, typename MT>
-__device__ __forceinline__ void element_results(const KTab<P + 1, T>& tab, const MT* metric,
-                                                const MT* weight, T mass, int e0, int e_end, int ne, T* sA, T* sB,
-                                                T* sC, int tid, int nth) {
+__device__ __forceinline__ void element_results(const KTab<P + 1, T>& tab, const MT* metric, T mass, int e0, int e_end,
+                                                int ne, T* sA, T* sB, T* sC, int tid, int nth) {
   constexpr int N = P + 1, N2 = N * N, N3 = N2 * N;
   using ML = MetricLayout<MT>;
   auto group_sync = [] {
@@ -315,8 +314,8 @@ __device__ __forceinline__ void element_results(const KTab<P + 1, T>& tab, const
     for (int idx = tid; idx < ne * N3; idx += nth) {
       const int s = idx / N3, loc = idx - s * N3, e = e0 + s;
       if (e < e_end) {
-        const T W = ldmetric(std::is_same<T, float>::value ? weight + (size_t)e * padded_n3(N) + loc
-                                                           : metric + ML::offset(N, e, loc % N2, loc / N2, 6));
+        const T W = ldmetric(metric + (std::is_same<T, float>::value ? (size_t)e * padded_n3(N) + loc
+                                                                     : ML::offset(N, e, loc % N2, loc / N2, 6)));
         sA[idx] = (mass * W) * sA[idx];
       }
     }
@@ -481,8 +480,7 @@ __global__ void __launch_bounds__(MASS_ONLY ? kApplyThreads : ApplyCta<P, T, DOT
   }
   group_sync();
 
-  element_results<P, QUAD, MASS_ONLY, kRolled, WARP>(tab, a.metric, a.weight, a.mass_coef, e0, a.nelem, E, sA, sB, sC,
-                                                     tid, nth);
+  element_results<P, QUAD, MASS_ONLY, kRolled, WARP>(tab, a.metric, a.mass_coef, e0, a.nelem, E, sA, sB, sC, tid, nth);
 
   pdl_trigger();
   // scatter-add y += P_e^T y_e, and with DOT the partial u_e . y_e
@@ -1274,14 +1272,18 @@ cudaError_t launch_apply_kernels(const Level& L, const ApplyArgs<T, MT>& a, cons
       if (!mass_only && L.nelem <= FewCfg<P, QUAD>::kElements && L.hold < 0) return launch_apply_few<P, QUAD, MT>(L, a, tab, s);
     }
     if (!mass_only) return launch_apply_plane<P, QUAD, MT>(L, a, tab, s);
-    // mass only, p <= 4: elements owned by warps (measured faster; at p = 5, 6 the
-    // n^2 = 36, 49 lines fill warps poorly and the CTA-wide mode is faster)
+    // mass only (Gauss quadrature; without it the mass is a diagonal), on the weights
+    if (weight_lowp_count(L) == 0) return cudaErrorInvalidValue;
+    ApplyArgs<T, MT> m = a;
+    m.metric = a.metric + metric_lowp_count(L);
+    // p <= 4: elements owned by warps (measured faster; at p = 5, 6 the n^2 = 36, 49
+    // lines fill warps poorly and the CTA-wide mode is faster)
     if constexpr (P <= 4) {
       constexpr int per_cta = kWarpsPerCta * WarpCfg<P>::G;
       launch_k(sem_apply_kernel<P, QUAD, T, MT, false, true, true>, (L.nelem + per_cta - 1) / per_cta, kApplyThreads,
-               apply_warp_tile_bytes<P, T>(), s, a, tab);
+               apply_warp_tile_bytes<P, T>(), s, m, tab);
     } else {
-      launch_k(sem_apply_kernel<P, QUAD, T, MT, false, true>, grid, kApplyThreads, tiles, s, a, tab);
+      launch_k(sem_apply_kernel<P, QUAD, T, MT, false, true>, grid, kApplyThreads, tiles, s, m, tab);
     }
     return cudaGetLastError();
   } else {
@@ -1319,7 +1321,6 @@ cudaError_t launch_apply_t(const Level& L, const ApplyArgs<T, MT>& a, bool mass_
   b.ndofs = L.ndofs;
   b.row = P * L.nx + 1;
   b.first = L.first;
-  b.weight = std::is_same<T, float>::value && weight_lowp_count(L) > 0 ? a.metric + metric_lowp_count(L) : nullptr;
   b.plane = b.row * (P * L.ny + 1);
   b.dbg = L.dbg;
   b.fault = L.fault;

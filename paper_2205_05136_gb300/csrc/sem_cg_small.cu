@@ -137,8 +137,7 @@ __global__ void __launch_bounds__(kThreads)
       for (int i = tid + (kept ? KEEP * kThreads : 0); i < ne * N3; i += kThreads)
         sA[i] = __ldcg(u + at(i, kDbgGather));
       __syncthreads();
-      element_results<P, QUAD, false, false, false>(tab, a.metric, a.metric, a.mass, e0, last, ne, sA, sB, sC, tid,
-                                                    kThreads);
+      element_results<P, QUAD, false, false, false>(tab, a.metric, a.mass, e0, last, ne, sA, sB, sC, tid, kThreads);
       if (kept) {
 #pragma unroll
         for (int k = 0; k < KEEP; ++k) {

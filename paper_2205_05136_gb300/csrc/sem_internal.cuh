@@ -255,8 +255,8 @@ inline size_t metric_lowp_count(const Level& L) {
 // Behind them, on a SEM fine level, the weights W alone, [nelem][n3p]: the FP32 mass
 // operator reads nothing else, and taken from the seven values of each point they cost
 // it the whole metric.  An apply on 2 M nodes, p = 1..6: FP32 99 58 40 38 35 34 us so, 92
-// 49 31 25 25 25 from the FP64 metric, 82 41 29 23 23 23 from here; bf16 90 53 35 29 30 30
-// and 76 40 29 23 23 23.  The other levels only apply alpha M + K.
+// 49 31 25 25 25 from the FP64 metric, 83 41 29 23 23 25 from here; bf16 90 53 35 29 30 30
+// and 76 40 29 23 23 24.  The other levels only apply alpha M + K.
 inline size_t weight_lowp_count(const Level& L) {
   return L.quad == SEM_QUAD_LG && L.xyz != nullptr ? (size_t)L.nelem * padded_n3(L.n) : 0;
 }
@@ -295,7 +295,6 @@ struct ApplyArgs {
   int64_t ndofs;
   int row, plane;  // lattice strides: nodes of an x-row and of an (x, y) plane
   const int* first;  // Level::first
-  const MT* weight;  // mass-only FP32 kernels: W of every point (weight_lowp_count)
   unsigned long long* dbg;
   unsigned* fault;
   int hold;  // SEM_DEBUG build: Level::hold
