@@ -342,11 +342,12 @@ int sem_apply_dot_static(sem_ctx* ctx, double alpha, double beta, const double* 
 
 /* Fault injection for the SEM_DEBUG build (paper_2205_05136_gb300.build with
  * debug=True: -DSEM_DEBUG).  That build checks every node index the apply
- * and transfer kernels read from the element-to-DOF map (or compute from the
- * node lattice) against [0, ndofs); an index outside is not used (node 0 is
- * read or written instead), the first one is recorded in a device word, and
- * sem_apply, sem_cg_solve, sem_step and sem_vcycle then synchronise their
- * stream and return SEM_ERR_ARG naming it.  This entry point overwrites entry
+ * kernels (the one-kernel CG and the one-CTA coarsest level among them) read from
+ * the element-to-DOF map, or (tensor-core kernel) compute from the node lattice,
+ * against [0, ndofs); an index outside is not used (node 0 is read or written
+ * instead), the first one is recorded in a device word, and sem_apply,
+ * sem_cg_solve, sem_step and sem_vcycle then synchronise their stream and return
+ * SEM_ERR_ARG naming it.  This entry point overwrites entry
  * `entry` (element e, local node a at e (p+1)^3 + a) of the context's fine
  * level map with `value` and returns the old value in *previous (may be
  * NULL), so a test can plant a bad index.  The normal build returns
@@ -354,9 +355,9 @@ int sem_apply_dot_static(sem_ctx* ctx, double alpha, double beta, const double* 
 int sem_debug_set_map_entry(sem_ctx* ctx, int64_t entry, int value, int* previous);
 
 /* SEM_DEBUG build only (the normal build returns SEM_ERR_UNSUPPORTED): the
- * FP32 apply of the fine level (the plane kernel, whatever the mesh size) leaves out the metric copy of element
- * group `group` (its group index; -1: none), so that the warp's bounded wait
- * for that copy runs out.  That warp then sets the context's wait-timeout word,
+ * FP32 apply of the fine level (the plane kernel, whatever the mesh size) leaves
+ * out the metric copy of element group `group` (its group index; -1: none), so
+ * that the warp's bounded wait for that copy runs out.  That warp then sets the context's wait-timeout word,
  * lets its other copy in flight land and returns, and the next multigrid solve
  * returns SEM_ERR_TIMEOUT (its result is not used).  Exercises the timeout
  * path without any fault.  Drops the multigrid hierarchy (its captured graphs

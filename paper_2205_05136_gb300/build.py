@@ -18,7 +18,7 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libsem.so")
-# the SEM_DEBUG build: index checks in the apply and transfer kernels
+# the SEM_DEBUG build: index checks in the apply kernels, injected waits that run out
 BUILD_DEBUG = os.path.join(HERE, "_build_debug")
 LIB_DEBUG = os.path.join(HERE, "libsem_debug.so")
 

@@ -193,10 +193,10 @@ int debug_check(sem_ctx* ctx, int rc, cudaStream_t s) {
     return cuda_fail(ctx, cudaGetLastError(), "SEM_DEBUG index-error word");
   if (w == 0) return rc;
   cudaMemset(ctx->L.dbg, 0, sizeof(w));
-  static const char* kinds[] = {"?", "gather", "scatter", "node line", "transfer"};
+  static const char* kinds[] = {"?", "gather", "scatter", "node line"};
   const unsigned kind = (unsigned)(w >> 56);
   const int idx = (int)(uint32_t)(w & 0xffffffffull);
-  return fail(ctx, SEM_ERR_ARG, std::string("SEM_DEBUG: ") + kinds[kind < 5 ? kind : 0] +
+  return fail(ctx, SEM_ERR_ARG, std::string("SEM_DEBUG: ") + kinds[kind < 4 ? kind : 0] +
                                     " node index " + std::to_string(idx) + " outside [0, " +
                                     std::to_string(ctx->L.ndofs) + ") (access skipped)");
 #else
@@ -382,7 +382,7 @@ int sem_set_deterministic(sem_ctx* ctx, int enable) {
     }
   }
   ctx->deterministic = enable != 0;
-  gmg_free(ctx);  // captured graphs embed the apply and transfer kernels
+  gmg_free(ctx);  // captured graphs embed the apply kernels
   return SEM_OK;
 }
 

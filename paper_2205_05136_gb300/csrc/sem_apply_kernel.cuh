@@ -266,8 +266,8 @@ __host__ __device__ constexpr size_t apply_tile_bytes() {
 
 // Warp-per-element mode (WARP): each warp of the CTA owns one element and
 // synchronises with __syncwarp only, so the warps of an SM run their gather,
-// sweep, metric and scatter phases independently.  Used for the FP32 kernels,
-// which are bound by memory latency rather than by arithmetic.
+// sweep, metric and scatter phases independently.  Used for the FP32 mass operator up
+// to p = 4, which is bound by memory latency rather than by arithmetic.
 constexpr int kWarpsPerCta = kApplyThreads / 32;
 
 // Elements per warp in warp mode: G n^2 lines close to 32 lanes (p <= 4).
@@ -392,9 +392,9 @@ __device__ __forceinline__ void element_results(const KTab<P + 1, T>& tab, const
 }
 
 // The double-float kernel at p = 4 (the outer operator of the benchmark's mixed
-// step) is bound by issue and memory latency: 10 CTAs per SM at 48 registers, with
-// small spills (8 measure the same in the plain apply, 1 % slower with the inner
-// product; at p = 3, 5, 6 it would spill far more).
+// step) is bound by issue and memory latency: 10 CTAs per SM at 48 registers, without
+// spills (8 measure the same in the plain apply, 1 % slower with the inner product; at
+// p = 3, 5, 6, which take 90 to 124 registers, it would spill).
 template <int P, int QUAD, typename T, typename MT, bool DOT, bool MASS_ONLY, bool WARP = false>
 __global__ void __launch_bounds__(MASS_ONLY ? kApplyThreads : ApplyCta<P, T, DOT>::kThreads,
                                   (std::is_same<T, df>::value && !MASS_ONLY && P == 4)
@@ -442,9 +442,9 @@ __global__ void __launch_bounds__(MASS_ONLY ? kApplyThreads : ApplyCta<P, T, DOT
                    : "memory");
   }
 
-  // Gather and scatter loops.  Every launch of this kernel has kApplyThreads
-  // threads per CTA (a warp per element group in warp mode), so the loops of
-  // the plain apply have compile-time trip counts: they unroll and keep the
+  // Gather and scatter loops.  The threads of a CTA are fixed (256 or 128 by
+  // ApplyCta, 256 for the mass alone; a warp per element group in warp mode), so the
+  // loops of the plain apply have compile-time trip counts: they unroll and keep the
   // loads of all their iterations in flight at once.  The apply with the fused
   // inner product keeps the rolled loops (both measured faster that way).
   constexpr int NTH = WARP ? 32 : MASS_ONLY ? kApplyThreads : ApplyCta<P, T, DOT>::kThreads;

@@ -273,8 +273,14 @@ __global__ void __launch_bounds__(kThreads)
   cluster_sync();  // no CTA ends while another may write to its shared memory
 }
 
-// CTAs of the cluster: 8 up to 1,500 nodes (20 time steps of 765 nodes: 1.61 ms, 1.84 with
-// 16: cheaper barriers and sums), above and at p = 1 (most elements a node) the 16 SMs pay.
+// CTAs of the cluster: 8 up to 1,500 nodes (cheaper barriers and sums), above and at
+// p = 1 (most elements a node) 16.  A Jacobi step, 8 / 16, SEM-NI and SEM, us: p = 1 532
+// nodes 79 / 81 and 486 / 519, 1,350 94 / 93 and 705 / 576, 2,304 146 / 119 and 1,050 /
+// 746; p = 2 1,035 nodes 81 / 93 and 408 / 442, 1,485 96 / 106 and 430 / 437, 1,595 104 /
+// 104 and 440 / 426, 3,367 132 / 116 and 609 / 451; p = 3 1,120 nodes 103 / 114 and 354 /
+// 388, 2,821 117 / 117 and 475 / 444.  From p = 4 on (fewer, longer elements) 8 would stay
+// the faster to about 2,500 nodes (p = 4 2,145 nodes 131 / 143 and 480 / 513, p = 6 2,275
+// 156 / 168 and 539 / 570; even at 3,400 to 4,000); the line does not follow that.
 int small_ctas(const Level& L) { return L.p >= 2 && L.ndofs <= 1500 ? 8 : kCtasMax; }
 
 template <int P>
@@ -332,9 +338,15 @@ cudaError_t launch_small(const Level& L, const SmallArgs& a, cudaStream_t s) {
 
 // Whether the one-kernel solve takes a mesh on the current device: up to where it
 // measured even with the launches of cg_solve (us a time step, launches / one kernel):
-// p = 1 SEM-NI 177 / 173 at 4,816 nodes, SEM 768 / 791 at 3,108; p = 2 SEM-NI 213 / 216 at 9,405, SEM 600 / 594 at
-// 7,497; p = 3 SEM 749 / 781 at 10,450; p = 4 SEM 817 / 868 at 14,625; p = 6 SEM still
-// 1,172 / 661 at 8,113.
+//   SEM-NI  p = 1 175 / 146 at 3,920 nodes, 174 / 185 at 5,760; p = 2 216 / 181 at 7,497,
+//           209 / 211 at 9,063; p = 3 246 / 232 at 9,880, 257 / 274 at 13,420; p = 4 313 /
+//           243 at 11,529, 342 / 342 at 14,625; p = 5 376 / 296 at 12,936, 406 / 337 at
+//           15,246; p = 6 441 / 338 at 13,975
+//   SEM     p = 1 799 / 764 at 2,730, 808 / 939 at 3,920; p = 2 696 / 633 at 5,355, 679 /
+//           687 at 7,497; p = 3 744 / 517 at 6,517, 723 / 752 at 9,880; p = 4 849 / 674 at
+//           11,529, 827 / 871 at 14,625; p = 5 962 / 749 at 12,936, 967 / 814 at 15,246;
+//           p = 6 1,074 / 824 at 13,975
+// (p = 5 and 6: the nodes that the cluster's threads hold are the limit).
 bool cg_small_fits(const Level& L, int max_ctas) {
   static constexpr int64_t kNodes[2][kMaxP + 1] = {
       {0, 2500, 6000, 9000, 12000, 14000, 14000},    // SEM

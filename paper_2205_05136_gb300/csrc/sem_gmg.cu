@@ -1442,7 +1442,8 @@ double lanczos_lambda(const LanczosScalars& sc) {
 
 // Diagonals and eigenvalue estimates of every level for alpha.  All levels' estimates
 // are enqueued before the one host read (each step read two scalars back before: 1.8 ms
-// for the three levels of a 70,000-node hierarchy, now 0.64).
+// for the three levels of a 70,000-node hierarchy, now 0.64).  That read is also the full
+// dependency between the levels' metric conversions and the first applies (pdl_wait).
 int set_alpha(sem_ctx* ctx, Gmg& g, double alpha, cudaStream_t s) {
   if (g.alpha == alpha) return SEM_OK;
   const size_t nl = g.lv.size();

@@ -31,7 +31,7 @@ namespace sem {
 // (kind << 56) | (32-bit index) and returns 0, so no access leaves the vector.
 // The host reads and clears the word after the call (debug_check) and returns
 // SEM_ERR_ARG with the index.  In the normal build SEM_IDX is the index itself.
-constexpr unsigned kDbgGather = 1, kDbgScatter = 2, kDbgLine = 3, kDbgTransfer = 4;
+constexpr unsigned kDbgGather = 1, kDbgScatter = 2, kDbgLine = 3;
 #if defined(SEM_DEBUG) && defined(__CUDACC__)
 __device__ __forceinline__ int64_t dbg_index(int64_t g, int64_t n, unsigned long long* word, unsigned kind) {
   if (g >= 0 && g < n) return g;
@@ -68,9 +68,13 @@ __device__ __forceinline__ int64_t dbg_index(int64_t g, int64_t n, unsigned long
 // come free they spread evenly, and the launch latency is hidden all the same.
 // Measured with the plane kernel: V-cycle on 2.06 M nodes 404 us with triggers at
 // the start, 362 us at the end (476 us without the attribute).
-// Before pdl_wait() a kernel may read what only the set-up writes (map, metric):
-// those kernels and copies never call pdl_trigger, so they have completed before
-// any later kernel is scheduled.
+// Before pdl_wait() a kernel may read the map, the elements' first nodes and the
+// metric copies, which only the set-up writes, because a full dependency always lies
+// between them.  That the set-up kernels do not trigger is not enough: their blocks
+// have then ended before a kernel launched by launch_k starts, but their writes are
+// promised to it by its wait only.  The full dependency is a memset or a host
+// synchronisation: apply_fp32 clears y between the conversion and the apply, and the
+// multigrid set-up, first or after a tissue update, ends in set_alpha's synchronisation.
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }

@@ -62,7 +62,7 @@ constexpr int kSetupThreads = 256;
 __host__ __device__ constexpr int setup_elems(int n3) { return n3 < 1024 ? 1024 / n3 : 1; }
 
 // Metric of E elements per CTA, one quadrature point a thread and turn.  The trilinear
-// map x_d = c0 + c1 xi + c2 eta + c3 zeta + c4 xi eta + c5 eta zeta + c6 xi zeta +
+// map x_d = c0 + c1 xi + c2 eta + c3 xi eta + c4 zeta + c5 xi zeta + c6 eta zeta +
 // c7 xi eta zeta is kept by its coefficients, so a column of J takes three
 // multiply-adds an entry; with A = adj J = det J J^{-1} (rows the cross products of
 // J's columns), G = w / det A D_e A^T takes one division.  About 100 FP64 operations a

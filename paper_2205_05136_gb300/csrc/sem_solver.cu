@@ -254,9 +254,11 @@ static __device__ __noinline__ bool grid_wait(const volatile unsigned* gen, unsi
 // clock and SM): both sums share one shuffle tree (half the lanes each), the divisions
 // are one thread's, and the nodes are spread over all SMs.  A Jacobi-CG step, three
 // launches / one: p = 3 SEM 299 k nodes 2.15 / 2.05 ms, SEM-NI 1.55 / 1.43; p = 6 SEM
-// 267 k 2.63 / 2.49; p = 1 SEM-NI 287 k 1.81 / 1.74; 633 k nodes 4.16 / 4.15.  Below
-// kUpdateMin the programmatic launches hide as much (p = 1 SEM 46 k nodes 983 / 1007 us,
-// 99 k 1388 / 1394).  Cooperative, since its CTAs wait for one another; at most one CTA
+// 267 k 2.63 / 2.49; p = 1 SEM-NI 287 k 1.81 / 1.74; 633 k nodes 4.16 / 4.15.  kUpdateMin
+// is a cautious line: there the programmatic launches hide much of it (us, 100 k to 110 k
+// nodes: p = 1 SEM-NI 616 / 598, SEM 1518 / 1494; p = 2 533 / 510, 974 / 930; p = 3 686 /
+// 639, 1094 / 1043; p = 6 925 / 865, 1369 / 1304), at 45 k nodes nearly all or more (p = 1
+// SEM-NI 332 / 339, SEM 1069 / 1059; p = 3 357 / 343, 754 / 720).  Cooperative, since its CTAs wait for one another; at most one CTA
 // an SM.  No pdl_trigger: with it the apply's CTAs crowd on the SMs that come free first
 // (p = 3, 50 k nodes 361 -> 551 us a step).
 constexpr int kUpdThreads = 512, kUpdCtas = 152;
@@ -803,6 +805,7 @@ int apply_fp32(sem_ctx* ctx, double alpha, double beta, const float* u, float* y
     SEM_CK(cudaGetLastError());
     return SEM_OK;
   }
+  // also the full dependency that the kernels' early metric reads need (pdl_wait)
   SEM_CK(cudaMemsetAsync(y, 0, sizeof(float) * L.ndofs, s));
   const bool mass_only = beta == 0.0;
   const double bb = mass_only ? 1.0 : beta;

@@ -1,4 +1,4 @@
-"""The SEM_DEBUG build: index checks in the apply and transfer kernels.
+"""The SEM_DEBUG build: index checks in the apply kernels.
 
 That build checks every node index the kernels take from the element-to-DOF map
 against [0, ndofs), records the first one outside in a device word instead of
@@ -8,7 +8,7 @@ SEM_LIBRARY, plants an out-of-range entry in the map through
 sem_debug_set_map_entry, and checks that the FP64 apply, the FP32 smoother
 apply, a multigrid V-cycle and a CG solve all report it; with the entry
 restored the results are again those of the clean run.  The same child also
-holds back one metric copy of the pipelined apply (sem_debug_hold_copy): the
+holds back one metric copy of the plane kernel (sem_debug_hold_copy): the
 bounded wait for it runs out and the multigrid solve returns SEM_ERR_TIMEOUT,
 after which the context solves as before.  The normal build answers both
 debug entry points with SEM_ERR_UNSUPPORTED.
@@ -70,7 +70,7 @@ assert float(torch.linalg.norm(y1f - y0f) / torch.linalg.norm(y0f)) < 1e-6
 z1 = torch.empty_like(u)
 capi.sem_vcycle(g.ctx, 30.0, u, z1)
 assert float(torch.linalg.norm(z1 - z0) / torch.linalg.norm(z0)) < 1e-6
-# the timeout path: the fine level's pipelined apply leaves out the metric copy of
+# the timeout path: the fine level's plane kernel leaves out the metric copy of
 # element group 3, the wait for it runs out, the multigrid solve reports it, and
 # the context then solves as before
 xr = torch.zeros_like(u)
